@@ -1053,311 +1053,93 @@ __global__ void wait_selftest_kernel(int kind, const uint32_t* flag, uint32_t ta
 // correction tiles exist, so a handful of SMs stream the weights.  Here the
 // GEMMs run transposed: c^T = W_c [m; u]^T and [v; g_r]^T = [W_v; W_g,r] r^T,
 // the weights as the A operand in 128-row tiles (M = 128, no padding), the
-// rows as B in tiles of up to 256 (N = R rounded up to 16, read on the
-// device), and the K range split so that one resident wave of CTAs streams
-// the weights.  Each CTA writes its fp32 partial [split][row][feature]; a
-// reduction kernel sums the splits in a fixed order (results repeat bit for
-// bit) and applies the epilogue.
-constexpr int SW_STAGES = 4;
+// rows as B in tiles of up to 256, and the K range split so that about one
+// resident wave of CTAs streams the weights.
+//
+// The S K-splits of one (weight tile, row tile) unit run as one cluster of S
+// CTAs.  Each CTA accumulates its k-range in TMEM, moves the fp32 partial into
+// its own shared memory (the drained pipeline stages), and after a cluster
+// barrier sums its slice of the rows over the S partials through distributed
+// shared memory, in rank order (results repeat bit for bit), and applies the
+// epilogue: r = m + beta c (Eq. 7) for the correction tiles of W_c, or the
+// gated fusion e~ = e + v sigmoid(g_r + W_g[:, :d] e) (Eq. 8) for the gate
+// tiles, whose 128 weight rows stack 64 rows of W_v over the same 64 rows of
+// W_g[:, d:2d] (v and g_r of a feature in TMEM lanes f and 64 + f).  Nothing
+// goes through global partials and no reduction kernel follows.  The partial
+// is stored row-major ([row][feature]) so that both the TMEM drain and the
+// cluster's reads move whole 128- and 256-byte rows.
+//
+// The row tiles are cut on the device from R (swap_cut): as many as the
+// resident clusters can take side by side, so that every SM has work and a
+// k-block costs an SM little more than its 16 KB of weights (a stage goes
+// through shared memory twice, about 2 (128 + N) cycles at 128 B per clock).
+constexpr int SW_STAGES = 4;      // most pipeline stages
+constexpr int SW_MIN_BLOCKS = 4;  // least k-blocks of a split
 constexpr int SW_THREADS = 256;
+constexpr int SW_A_BYTES = BM * BK * 2;  // 16 KB: 128 weight rows of a k-block
+constexpr int SW_ROW_STEP = 32;          // row boxes come in multiples of this many rows
+constexpr int SW_ROW_MAPS = 256 / SW_ROW_STEP;
+constexpr int SW_SMEM_MAX = 226 * 1024;  // dynamic shared memory of a CTA at most (its barriers beside it)
 
-// How a GEMM of R rows is cut, the same in the GEMM and its reduction: N
-// tiles of up to 256 rows, work = weight tiles x N tiles, each split `grid /
-// work` ways along K (no empty split).
-struct SwapPlan {
-  int nrows, ntiles, work, splits, kb_split;
+// Row tiles of R rows for `clusters` resident clusters over `mtiles` weight
+// tiles: `ntiles` tiles of `tile_n` rows (a multiple of 16, at most 256).
+// The units u < mtiles * ntiles (weight tile u % mtiles) are taken by cluster
+// u mod clusters.
+struct SwapCut {
+  int ntiles, tile_n;
 };
-__device__ __forceinline__ SwapPlan swap_plan(int R, int mtiles, int nkb, int grid) {
-  SwapPlan s;
-  s.nrows = (R + 15) / 16 * 16;
-  s.ntiles = (s.nrows + 255) / 256;
-  s.work = mtiles * s.ntiles;
-  int splits = s.work > 0 ? grid / s.work : 1;
-  if (splits < 1) splits = 1;
-  if (splits > nkb) splits = nkb;
-  s.kb_split = (nkb + splits - 1) / splits;
-  s.splits = (nkb + s.kb_split - 1) / s.kb_split;
-  return s;
+__host__ __device__ __forceinline__ SwapCut swap_cut(int R, int mtiles, int clusters) {
+  const int nrows = (R + 15) / 16 * 16;
+  if (clusters < 2 * mtiles && nrows <= 256) return {nrows > 0 ? 1 : 0, nrows};  // one tile
+  const int need = (nrows + 255) / 256;
+  const int fit = clusters / mtiles, most = (nrows + SW_ROW_STEP - 1) / SW_ROW_STEP;
+  int n = fit < most ? fit : most;
+  if (n < need) n = need;
+  if (n < 1) n = 1;
+  SwapCut c;
+  c.tile_n = ((nrows + n - 1) / n + 15) / 16 * 16;
+  c.ntiles = c.tile_n > 0 ? (nrows + c.tile_n - 1) / c.tile_n : 0;
+  return c;
+}
+__host__ __device__ __forceinline__ int swap_box_rows(int tile_n) {
+  return (tile_n + SW_ROW_STEP - 1) / SW_ROW_STEP * SW_ROW_STEP;
+}
+// Pipeline stages (a weight tile and a row box each) that `bytes` of shared memory hold.
+__host__ __device__ __forceinline__ int swap_stages(int bytes, int box_rows) {
+  const int n = bytes / (SW_A_BYTES + box_rows * BK * 2);
+  return n < SW_STAGES ? n : SW_STAGES;
 }
 
-struct SwapParams {
-  const int32_t* R;
-  int nkb;        // k-blocks of the reduction
-  int mtiles;     // 128-row weight tiles in all
-  int mt_a;       // tiles taken from map A (the others from map A2)
-  int a2_x0;      // column offset of map A2's operand (d: the r half of W_g)
-  int box_n;      // rows of a B box (min(256, the largest R rounded to 16))
-  uint32_t tmem_cols;
-  uint32_t stage_stride;  // bytes per pipeline stage (A tile + B box, 1024-aligned)
-  float* part;            // [splits][nrows][mtiles * 128]
-  uint32_t* status;
+// The rows operand once per box height: map i has boxes of SW_ROW_STEP (i + 1) rows.
+struct RowMaps {
+  CUtensorMap m[SW_ROW_MAPS];
 };
 
-__global__ void __launch_bounds__(SW_THREADS, 1)
-    swap_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA2,
-                     const __grid_constant__ CUtensorMap tmB, const SwapParams p) {
-  extern __shared__ uint8_t dsmem[];
-  __shared__ __align__(8) uint64_t bar_full[SW_STAGES];
-  __shared__ __align__(8) uint64_t bar_empty[SW_STAGES];
-  __shared__ __align__(8) uint64_t bar_acc;
-  __shared__ uint32_t s_tmem;
-  __shared__ volatile int s_abort;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  pdl_launch_dependents();
-  if (threadIdx.x == 0) {
-    s_abort = 0;
-    for (int s = 0; s < SW_STAGES; ++s) {
-      mbar_init(smem_u32(&bar_full[s]), 1);
-      mbar_init(smem_u32(&bar_empty[s]), 1);
-    }
-    mbar_init(smem_u32(&bar_acc), 1);
-    fence_mbar_init();
-  }
-  if (warp == 0 && lane == 0) {
-    tma_prefetch_desc(&tmA);
-    tma_prefetch_desc(&tmA2);
-    tma_prefetch_desc(&tmB);
-  }
-  if (warp == 2) {
-    tmem_alloc(smem_u32(&s_tmem), p.tmem_cols);
-    tmem_relinquish();
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = s_tmem;
-  const uint32_t base = (smem_u32(dsmem) + 1023u) & ~1023u;
-  pdl_wait();  // R and the activation rows come from the previous kernels
-  const int R = *(volatile const int32_t*)p.R;
-  const SwapPlan pl = swap_plan(R, p.mtiles, p.nkb, (int)gridDim.x);
-  const int c = blockIdx.x;
-  const bool active = c < pl.work * pl.splits;
-  const int sp = c % pl.splits, w = c / pl.splits;
-  const int mt = w / (pl.ntiles > 0 ? pl.ntiles : 1), nt = w - mt * (pl.ntiles > 0 ? pl.ntiles : 1);
-  const int kb0 = sp * pl.kb_split, kb1 = min(p.nkb, kb0 + pl.kb_split);
-  const int tn = active ? min(256, pl.nrows - nt * 256) : 0;  // rows of this N tile (MMA N)
-
-  if (!active) {
-    // nothing to do: fall through to the teardown
-  } else if (warp == 0) {
-    // ---------------- TMA producer ----------------
-    if (lane == 0) {
-      const bool second = mt >= p.mt_a;
-      const CUtensorMap* ma = second ? &tmA2 : &tmA;
-      const int ay = (second ? mt - p.mt_a : mt) * 128, ax0 = second ? p.a2_x0 : 0;
-      const uint32_t tx = (uint32_t)(BM * BK * 2) + (uint32_t)p.box_n * BK * 2;
-      int kb = kb0;
-      for (; kb < kb1; ++kb) {
-        const int i = kb - kb0;
-        const uint32_t s = (uint32_t)(i % SW_STAGES), ph = (uint32_t)((i / SW_STAGES) & 1);
-        if (!mbar_wait_bounded(smem_u32(&bar_empty[s]), ph ^ 1u, &s_abort)) break;
-        const uint32_t a_dst = base + s * p.stage_stride, b_dst = a_dst + (uint32_t)(BM * BK * 2);
-        mbar_arrive_expect_tx(smem_u32(&bar_full[s]), tx);
-        tma_load_2d(a_dst, ma, ax0 + kb * BK, ay, smem_u32(&bar_full[s]));
-        tma_load_2d(b_dst, &tmB, kb * BK, nt * 256, smem_u32(&bar_full[s]));
-      }
-      if (kb < kb1) {  // a wait expired: flag it, let the copies in flight land
-        raise_abort(&s_abort, p.status);
-        volatile int never = 0;
-        const int first = kb - kb0 > SW_STAGES ? kb - kb0 - SW_STAGES : 0;
-        for (int i = first; i < kb - kb0; ++i)
-          mbar_wait_bounded(smem_u32(&bar_full[i % SW_STAGES]), (uint32_t)((i / SW_STAGES) & 1), &never);
-      }
-    }
-    __syncwarp();
-  } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      const uint32_t idesc = idesc_bf16_f32(128, tn);
-      bool ok = true;
-      for (int kb = kb0; kb < kb1; ++kb) {
-        const int i = kb - kb0;
-        const uint32_t s = (uint32_t)(i % SW_STAGES), ph = (uint32_t)((i / SW_STAGES) & 1);
-        if (!mbar_wait_bounded(smem_u32(&bar_full[s]), ph, &s_abort)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        const uint32_t a_base = base + s * p.stage_stride, b_base = a_base + (uint32_t)(BM * BK * 2);
-        const uint64_t adesc0 = sw128_kmajor_desc(a_base), bdesc0 = sw128_kmajor_desc(b_base);
-#pragma unroll
-        for (int k = 0; k < BK / 16; ++k)
-          tc_mma_bf16(tmem, adesc0 + 2u * k, bdesc0 + 2u * k, idesc, (i > 0 || k > 0) ? 1u : 0u);
-        tc_commit(smem_u32(&bar_empty[s]));
-      }
-      tc_commit(smem_u32(&bar_acc));  // accumulator ready (also after a failure)
-      if (!ok) raise_abort(&s_abort, p.status);
-    }
-    __syncwarp();
-  } else if (warp >= 4) {
-    // ---------------- epilogue: the partial of this (weight tile, N tile, split) ----------------
-    const int q = (warp - 4) * 32 + lane;  // weight row of the tile = TMEM lane
-    const bool ok = warp_wait(smem_u32(&bar_acc), 0u, &s_abort);
-    tc_fence_after();
-    if (ok && !s_abort) {
-      const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-      const long long mtot = (long long)p.mtiles * 128;
-      float* out = p.part + ((long long)sp * pl.nrows + nt * 256) * mtot + mt * 128 + q;
-      for (int c0 = 0; c0 < tn; c0 += 32) {
-        float v[32];
-        tmem_ld_32cols(taddr + (uint32_t)c0, v);
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (c0 + j < tn) out[(long long)(c0 + j) * mtot] = v[j];  // 32 lanes: 128 contiguous bytes
-      }
-    } else if (!ok && lane == 0) {
-      raise_abort(&s_abort, p.status);
-    }
-  }
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 2) {
-    tc_fence_after();
-    tmem_dealloc(tmem, p.tmem_cols);
-  }
-}
-
-struct SwapReduceParams {
+// W_g[:, :d] e for the gate of a small-R call (broadcast e).
+struct GateBiasParams {
   int d;
-  const int32_t* R;
-  // the GEMM's cut (swap_plan): weight tiles, k-blocks, grid
-  int mtiles, nkb, grid;
-  const float* part;  // [splits][nrows][mtiles * 128]
-  // correction: r = m + beta * c
-  const __nv_bfloat16* apack;  // m = the first d columns of each packed row
-  float beta;
-  __nv_bfloat16* r_out;
-  int compact_out;
-  // gate: e~ = e + v * sigmoid(g_r + ge)
   const __nv_bfloat16* e;
-  const float* ge;
-  __nv_bfloat16* e_out;
-  const int32_t* rowmap;
-  // W_g[:, :d] e for a broadcast e, before the wait (it reads inputs only)
-  int do_gemv;
-  CondParams gemv;
-  uint32_t* gemv_next;
-  uint32_t* gemv_done;
+  const __nv_bfloat16* Wg;
+  float* ge;
 };
 
-// r rows of the packed correction (Eq. 7): eight features per thread; the
-// splits summed in order.  Before it waits for the correction GEMM, every
-// warp takes rows of the gate-bias GEMV W_g[:, :d] e, which thereby overlaps
-// the GEMM.
-__global__ void __launch_bounds__(256) swap_reduce_correction_kernel(const SwapReduceParams p) {
-  pdl_launch_dependents();
-  if (p.do_gemv) gate_bias_rows(p.gemv, p.d, threadIdx.x & 31, p.gemv_next, p.gemv_done);
-  pdl_wait();
-  const int R = *(volatile const int32_t*)p.R;
-  const SwapPlan pl = swap_plan(R, p.mtiles, p.nkb, p.grid);
-  const int d = p.d, vpr = d / 8;
-  const long long n_units = (long long)R * vpr;
-  for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < n_units;
-       u += (long long)gridDim.x * blockDim.x) {
-    const int g = (int)(u / vpr), n = (int)(u - (long long)g * vpr) * 8;
-    float c[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) c[j] = 0.f;
-    for (int s = 0; s < pl.splits; ++s) {
-      const float4* src = reinterpret_cast<const float4*>(p.part + ((long long)s * pl.nrows + g) * d + n);
-      const float4 x0 = __ldcg(src), x1 = __ldcg(src + 1);
-      c[0] += x0.x; c[1] += x0.y; c[2] += x0.z; c[3] += x0.w;
-      c[4] += x1.x; c[5] += x1.y; c[6] += x1.z; c[7] += x1.w;
-    }
-    const uint4 mw = __ldcg(reinterpret_cast<const uint4*>(p.apack + (long long)g * 2 * d + n));
-    const uint32_t mwords[4] = {mw.x, mw.y, mw.z, mw.w};
-    uint32_t o[4];
-#pragma unroll
-    for (int w = 0; w < 4; ++w)
-      o[w] = pack_bf16x2(bf16_lo(mwords[w]) + p.beta * c[2 * w], bf16_hi(mwords[w]) + p.beta * c[2 * w + 1]);
-    const long long orow = p.compact_out ? g : __ldcg(p.rowmap + g);
-    *reinterpret_cast<uint4*>(p.r_out + orow * d + n) = make_uint4(o[0], o[1], o[2], o[3]);
-  }
-}
-
-// W_g[:, :d] e alone (a gate-only call: no correction kernel to overlap it
-// with), by the same per-row code, so the bits match the correction path's.
-__global__ void __launch_bounds__(256) swap_gemv_kernel(const SwapReduceParams p) {
-  pdl_launch_dependents();
-  gate_bias_rows(p.gemv, p.d, threadIdx.x & 31, p.gemv_next, p.gemv_done);
-  // Complete only after the previous kernel: the next kernel's programmatic
-  // wait, which covers this kernel alone, then covers that one too.  One CTA
-  // waiting is enough (the grid completes with its last CTA); the others
-  // leave and free their SM for the next kernel.
-  if (blockIdx.x == 0) pdl_wait();
-}
-
-// e~ rows of the gated fusion (Eq. 8), broadcast e: v in features 0..d-1 of
-// the partials, the r half of the gate in d..2d-1.
-__global__ void __launch_bounds__(256) swap_reduce_gate_kernel(const SwapReduceParams p) {
-  pdl_launch_dependents();
-  pdl_wait();
-  const int R = *(volatile const int32_t*)p.R;
-  const SwapPlan pl = swap_plan(R, p.mtiles, p.nkb, p.grid);
-  const int d = p.d, vpr = d / 8;
-  const long long n_units = (long long)R * vpr;
-  for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < n_units;
-       u += (long long)gridDim.x * blockDim.x) {
-    const int g = (int)(u / vpr), n = (int)(u - (long long)g * vpr) * 8;
-    float v[8], gt[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) v[j] = gt[j] = 0.f;
-    for (int s = 0; s < pl.splits; ++s) {
-      const float* row = p.part + ((long long)s * pl.nrows + g) * 2 * d;
-      const float4* vs = reinterpret_cast<const float4*>(row + n);
-      const float4* gs = reinterpret_cast<const float4*>(row + d + n);
-      const float4 v0 = __ldcg(vs), v1 = __ldcg(vs + 1), g0 = __ldcg(gs), g1 = __ldcg(gs + 1);
-      v[0] += v0.x; v[1] += v0.y; v[2] += v0.z; v[3] += v0.w;
-      v[4] += v1.x; v[5] += v1.y; v[6] += v1.z; v[7] += v1.w;
-      gt[0] += g0.x; gt[1] += g0.y; gt[2] += g0.z; gt[3] += g0.w;
-      gt[4] += g1.x; gt[5] += g1.y; gt[6] += g1.z; gt[7] += g1.w;
-    }
-    const float4 b0 = __ldcg(reinterpret_cast<const float4*>(p.ge + n));
-    const float4 b1 = __ldcg(reinterpret_cast<const float4*>(p.ge + n) + 1);
-    gt[0] += b0.x; gt[1] += b0.y; gt[2] += b0.z; gt[3] += b0.w;
-    gt[4] += b1.x; gt[5] += b1.y; gt[6] += b1.z; gt[7] += b1.w;
-    const uint4 ew = __ldg(reinterpret_cast<const uint4*>(p.e + n));
-    const uint32_t ewords[4] = {ew.x, ew.y, ew.z, ew.w};
-    uint32_t o[4];
-#pragma unroll
-    for (int w = 0; w < 4; ++w) {
-      const float s0 = fast_sigmoid(gt[2 * w]), s1 = fast_sigmoid(gt[2 * w + 1]);
-      o[w] = pack_bf16x2(bf16_lo(ewords[w]) + v[2 * w] * s0, bf16_hi(ewords[w]) + v[2 * w + 1] * s1);
-    }
-    const long long orow = __ldcg(p.rowmap + g);
-    *reinterpret_cast<uint4*>(p.e_out + orow * d + n) = make_uint4(o[0], o[1], o[2], o[3]);
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Small R in one N tile (at most 256 rows): split-K clusters, no reduction launch
-// ---------------------------------------------------------------------------
-// The S K-splits of one weight tile run as one cluster of S CTAs.  Each CTA
-// accumulates its k-range in TMEM as swap_gemm_kernel does, moves the fp32
-// partial into its own shared memory (the drained pipeline stages), and after
-// a cluster barrier sums its slice of the rows over the S partials through
-// distributed shared memory, in rank order (results repeat bit for bit), and
-// applies the epilogue: r = m + beta c (Eq. 7) for the correction tiles of
-// W_c, or the gated fusion e~ = e + v sigmoid(g_r + W_g[:, :d] e) (Eq. 8)
-// for the gate tiles, whose 128 weight rows stack 64 rows of W_v over the
-// same 64 rows of W_g[:, d:2d] (v and g_r of a feature in TMEM lanes f and
-// 64 + f).  Nothing goes through global partials and no reduction kernel
-// follows.  The partial is stored row-major ([row][feature]) so that both
-// the TMEM drain and the cluster's reads move whole 128- and 256-byte rows.
 struct SwapClusterParams {
   const int32_t* R;
   int d;
+  int mtiles;  // weight tiles
   int nkb;     // 64-deep k-blocks of the GEMM
   int S;       // K splits = cluster size
   int gate;    // 0: correction tiles of W_c (128 features); 1: stacked [W_v; W_g,r] tiles (64 features)
-  int tile_n;  // rows of the B box (the largest R rounded to 16, at most 256)
+  int stage_bytes;  // shared memory of the pipeline stages
+  int pre;          // stages whose weight tiles are loaded before the wait on the previous kernel
+  int row_maps;     // maps of the rows operand
   uint32_t tmem_cols;
-  uint32_t stage_stride;
   // correction epilogue
   const __nv_bfloat16* apack;  // m = the first d columns of each packed row
   float beta;
   __nv_bfloat16* r_out;
   int compact_out;
+  GateBiasParams bias;  // correction: W_g[:, :d] e of the gate to come (ge NULL: not computed)
   // gate epilogue (broadcast e; ge = W_g[:, :d] e, complete before this launch)
   const __nv_bfloat16* e;
   const float* ge;
@@ -1366,9 +1148,103 @@ struct SwapClusterParams {
   uint32_t* status;
 };
 
+// The sum over the cluster's S partials and the epilogue of `total` positions
+// (row l0 + x / 32, features 4 (x % 32).. for the correction; 16 per row for
+// the gate) of the unit at weight tile mt and packed row row0.  A thread has NB
+// positions and, for each, the loads of NS partials in flight: with one
+// position and one partial at a time a CTA with 80 rows took a chain of
+// twenty round trips.  The partials are added in rank order.
+template <int NB, int NS>
+__device__ __forceinline__ void swap_correction_rows(const SwapClusterParams& p, uint32_t P, int mt, int row0, int l0,
+                                                     int total) {
+  const int d = p.d, S = p.S, n0 = mt * 128;
+  for (int x0 = threadIdx.x; x0 < total; x0 += NB * SW_THREADS) {
+    float4 c[NB];
+    uint2 mw[NB];
+    long long orow[NB];
+    uint32_t at[NB];
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      const int x = min(x0 + q * SW_THREADS, total - 1), l = l0 + x / 32, f = (x % 32) * 4, g = row0 + l;
+      mw[q] = __ldcg(reinterpret_cast<const uint2*>(p.apack + (long long)g * 2 * d + n0 + f));
+      orow[q] = p.compact_out ? g : __ldcg(p.rowmap + g);
+      at[q] = P + (uint32_t)(l * 512 + f * 4);
+      c[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    for (int s0 = 0; s0 < S; s0 += NS) {
+      float4 v[NS][NB];
+#pragma unroll
+      for (int s = 0; s < NS; ++s)
+#pragma unroll
+        for (int q = 0; q < NB; ++q)
+          v[s][q] = s0 + s < S ? ld_cluster_f4(map_rank(at[q], (uint32_t)(s0 + s))) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int s = 0; s < NS; ++s)
+#pragma unroll
+        for (int q = 0; q < NB; ++q) add4(c[q], v[s][q]);
+    }
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      const int x = x0 + q * SW_THREADS;
+      if (x < total)
+        *reinterpret_cast<uint2*>(p.r_out + orow[q] * d + n0 + (x % 32) * 4) =
+            make_uint2(pack_bf16x2(bf16_lo(mw[q].x) + p.beta * c[q].x, bf16_hi(mw[q].x) + p.beta * c[q].y),
+                       pack_bf16x2(bf16_lo(mw[q].y) + p.beta * c[q].z, bf16_hi(mw[q].y) + p.beta * c[q].w));
+    }
+  }
+}
+template <int NB, int NS>
+__device__ __forceinline__ void swap_gate_rows(const SwapClusterParams& p, uint32_t P, int mt, int row0, int l0,
+                                               int total) {
+  const int d = p.d, S = p.S;
+  const int f = ((int)threadIdx.x % 16) * 4, n = mt * 64 + f;  // the same features at every step
+  const float4 gb = __ldcg(reinterpret_cast<const float4*>(p.ge + n));
+  const uint2 ew = __ldg(reinterpret_cast<const uint2*>(p.e + n));
+  for (int x0 = threadIdx.x; x0 < total; x0 += NB * SW_THREADS) {
+    float4 v[NB], a[NB];
+    long long orow[NB];
+    uint32_t at[NB];
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      const int l = l0 + min(x0 + q * SW_THREADS, total - 1) / 16;
+      orow[q] = __ldcg(p.rowmap + row0 + l);
+      at[q] = P + (uint32_t)(l * 512 + f * 4);
+      v[q] = a[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    for (int s0 = 0; s0 < S; s0 += NS) {
+      float4 xv[NS][NB], xa[NS][NB];
+#pragma unroll
+      for (int s = 0; s < NS; ++s)
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+          const bool in = s0 + s < S;
+          const uint32_t src = map_rank(at[q], (uint32_t)(in ? s0 + s : 0));
+          xv[s][q] = in ? ld_cluster_f4(src) : make_float4(0.f, 0.f, 0.f, 0.f);
+          xa[s][q] = in ? ld_cluster_f4(src + 256u) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+      for (int s = 0; s < NS; ++s)
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+          add4(v[q], xv[s][q]);
+          add4(a[q], xa[s][q]);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      if (x0 + q * SW_THREADS >= total) continue;
+      const float s0 = fast_sigmoid(a[q].x + gb.x), s1 = fast_sigmoid(a[q].y + gb.y);
+      const float s2 = fast_sigmoid(a[q].z + gb.z), s3 = fast_sigmoid(a[q].w + gb.w);
+      *reinterpret_cast<uint2*>(p.e_out + orow[q] * d + n) =
+          make_uint2(pack_bf16x2(bf16_lo(ew.x) + v[q].x * s0, bf16_hi(ew.x) + v[q].y * s1),
+                     pack_bf16x2(bf16_lo(ew.y) + v[q].z * s2, bf16_hi(ew.y) + v[q].w * s3));
+    }
+  }
+}
+
 __global__ void __launch_bounds__(SW_THREADS, 1)
     swap_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA2,
-                        const __grid_constant__ CUtensorMap tmB, const SwapClusterParams p) {
+                        const __grid_constant__ RowMaps tmB, const SwapClusterParams p) {
   extern __shared__ uint8_t dsmem[];
   __shared__ __align__(8) uint64_t bar_full[SW_STAGES];
   __shared__ __align__(8) uint64_t bar_empty[SW_STAGES];
@@ -1378,12 +1254,12 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int S = p.S, d = p.d;
   const uint32_t rank = cluster_rank();
-  const int mt = (int)(blockIdx.x / (unsigned)S);  // weight tile of this cluster
+  const int cid = (int)(blockIdx.x / (unsigned)S), clusters = (int)(gridDim.x / (unsigned)S);
   pdl_launch_dependents();
   if (threadIdx.x == 0) {
     s_abort = 0;
     for (int s = 0; s < SW_STAGES; ++s) {
-      mbar_init(smem_u32(&bar_full[s]), 1);
+      mbar_init(smem_u32(&bar_full[s]), 2);  // the weight tile's and the row box's expect_tx
       mbar_init(smem_u32(&bar_empty[s]), 1);
     }
     mbar_init(smem_u32(&bar_acc), 1);
@@ -1392,8 +1268,8 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
   if (warp == 0 && lane == 0) {
     tma_prefetch_desc(&tmA);
     tma_prefetch_desc(&tmA2);
-    tma_prefetch_desc(&tmB);
   }
+  if (warp == 1 && lane < p.row_maps) tma_prefetch_desc(&tmB.m[lane]);
   if (warp == 2) {
     tmem_alloc(smem_u32(&s_tmem), p.tmem_cols);
     tmem_relinquish();
@@ -1406,185 +1282,166 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
   // the partial [row][128 features], in the drained pipeline stages (the same offset in every CTA)
   float* P = reinterpret_cast<float*>(dsmem + (base - smem_u32(dsmem)));
   const int kb0 = (int)((long long)rank * p.nkb / S), kb1 = (int)((long long)(rank + 1) * p.nkb / S);
-  // The weight boxes of the first stages are inputs: the producer issues them
-  // before the wait on the previous kernel, and their row boxes after it.
-  const uint32_t tx = (uint32_t)(BM * BK * 2) + (uint32_t)p.tile_n * BK * 2;
-  const int npre = min(SW_STAGES, kb1 - kb0);
-  auto load_a = [&](int kb, uint32_t a_dst, uint32_t bar) {
+  // Weight tiles lie at 16 KB steps from `base`, whatever the row boxes' size.
+  auto load_a = [&](int mt, int kb, uint32_t s) {
+    const uint32_t a_dst = base + s * (uint32_t)SW_A_BYTES, bar = smem_u32(&bar_full[s]);
+    mbar_arrive_expect_tx(bar, (uint32_t)SW_A_BYTES);
     if (p.gate) {  // rows 0-63: W_v rows f0..; rows 64-127: the same rows of W_g[:, d:2d]
       tma_load_2d(a_dst, &tmA, kb * BK, mt * 64, bar);
-      tma_load_2d(a_dst + (uint32_t)(64 * BK * 2), &tmA2, d + kb * BK, mt * 64, bar);
+      tma_load_2d(a_dst + (uint32_t)(SW_A_BYTES / 2), &tmA2, d + kb * BK, mt * 64, bar);
     } else {
       tma_load_2d(a_dst, &tmA, kb * BK, mt * 128, bar);
     }
   };
-  if (warp == 0 && lane == 0) {
-    for (int i = 0; i < npre; ++i) {  // every stage is free at the start
-      const uint32_t a_dst = base + (uint32_t)i * p.stage_stride;
-      mbar_arrive_expect_tx(smem_u32(&bar_full[i]), tx);
-      load_a(kb0 + i, a_dst, smem_u32(&bar_full[i]));
-    }
-  }
+  // The weights are inputs: the producer loads the first stages' tiles of the
+  // cluster's first unit before the wait on the previous kernel, and their
+  // row boxes after it.
+  const int npre = min(p.pre, kb1 - kb0);
+  if (warp == 0 && lane == 0)
+    for (int i = 0; i < npre; ++i) load_a(cid % p.mtiles, kb0 + i, (uint32_t)i);  // every stage is free at the start
+  // The gate's W_g[:, :d] e needs inputs only: warps 2-7, which have no work
+  // before the accumulator is complete, compute it while the previous kernels
+  // end (the memory is idle then) and the first k-blocks run.
+  if (p.bias.ge && warp >= 2)
+    gate_bias_share(p.bias.e, p.bias.Wg, p.bias.ge, d, (int)blockIdx.x * 6 + warp - 2, (int)gridDim.x * 6, lane);
   pdl_wait();  // R and the activation rows come from the previous kernels
   const int R = *(volatile const int32_t*)p.R;
-  const int nrows = (R + 15) / 16 * 16;  // MMA N (at most tile_n)
-  const bool work = R > 0;
+  const SwapCut cut = swap_cut(R, p.mtiles, clusters);
+  const int units = p.mtiles * cut.ntiles;
+  const int box = swap_box_rows(cut.tile_n);
+  const int nst = swap_stages(p.stage_bytes, box > 0 ? box : SW_ROW_STEP);  // >= p.pre
+  const uint32_t b_bytes = (uint32_t)(box * BK * 2);
+  const uint32_t b_base = base + (uint32_t)nst * (uint32_t)SW_A_BYTES;
+  const CUtensorMap* mb = &tmB.m[box > 0 ? box / SW_ROW_STEP - 1 : 0];
 
-  if (warp == 0) {
-    // ---------------- TMA producer ----------------
-    if (lane == 0) {
-      // the row boxes of the stages issued above (also without work: their
-      // barriers expect them; the boxes stay inside the tensor map)
-      for (int i = 0; i < npre; ++i)
-        tma_load_2d(base + (uint32_t)i * p.stage_stride + (uint32_t)(BM * BK * 2), &tmB, (kb0 + i) * BK, 0,
-                    smem_u32(&bar_full[i]));
-      int kb = kb0 + npre;
-      if (work) {
-        for (; kb < kb1; ++kb) {
-          const int i = kb - kb0;
-          const uint32_t s = (uint32_t)(i % SW_STAGES), ph = (uint32_t)((i / SW_STAGES) & 1);
-          if (!mbar_wait_bounded(smem_u32(&bar_empty[s]), ph ^ 1u, &s_abort)) break;
-          const uint32_t a_dst = base + s * p.stage_stride, b_dst = a_dst + (uint32_t)(BM * BK * 2);
-          mbar_arrive_expect_tx(smem_u32(&bar_full[s]), tx);
-          load_a(kb, a_dst, smem_u32(&bar_full[s]));
-          tma_load_2d(b_dst, &tmB, kb * BK, 0, smem_u32(&bar_full[s]));
+  if (cid >= units && warp == 0 && lane == 0) {  // (always so with R = 0)
+    // no unit: let the copies issued above land before the CTA leaves
+    volatile int never = 0;
+    for (int i = 0; i < npre; ++i) {
+      mbar_arrive(smem_u32(&bar_full[i]));
+      mbar_wait_bounded(smem_u32(&bar_full[i]), 0u, &never);
+    }
+  }
+  uint32_t s = 0, ph = 0;  // ring position and phase of the next k-block (producer and MMA thread)
+  auto advance = [&]() {
+    if (++s == (uint32_t)nst) {
+      s = 0;
+      ph ^= 1u;
+    }
+  };
+  uint32_t acc_ph = 0u;  // phase of bar_acc
+  int pre = npre;        // weight tiles of this unit already loaded
+  for (int u = cid; u < units; u += clusters, acc_ph ^= 1u, pre = 0) {
+    const int mt = u % p.mtiles, nt = u / p.mtiles;
+    const int row0 = nt * cut.tile_n;
+    const int rows = min(R - row0, cut.tile_n);  // of this unit, > 0
+    const int mma_n = (rows + 15) / 16 * 16;
+    if (warp == 0) {
+      // ---------------- TMA producer ----------------
+      if (lane == 0) {
+        int i = 0;
+        for (; i < kb1 - kb0; ++i, advance()) {
+          if (i >= pre) {
+            if (!mbar_wait_bounded(smem_u32(&bar_empty[s]), ph ^ 1u, &s_abort)) break;
+            load_a(mt, kb0 + i, s);
+          }
+          mbar_arrive_expect_tx(smem_u32(&bar_full[s]), b_bytes);
+          tma_load_2d(b_base + s * b_bytes, mb, (kb0 + i) * BK, row0, smem_u32(&bar_full[s]));
+        }
+        if (i < kb1 - kb0) {
+          // a wait expired: flag it, let the copies in flight land
+          raise_abort(&s_abort, p.status);
+          volatile int never = 0;
+          for (int k = 0; k < min(i, nst); ++k) {  // the last min(i, nst) k-blocks, backwards
+            ph ^= s == 0 ? 1u : 0u;
+            s = s == 0 ? (uint32_t)nst - 1u : s - 1u;
+            mbar_wait_bounded(smem_u32(&bar_full[s]), ph, &never);
+          }
         }
       }
-      if (!work || kb < kb1) {
-        // no MMA consumes the stages (no rows), or a wait expired: let the
-        // copies in flight land before the stages are reused or released
-        if (work) raise_abort(&s_abort, p.status);
-        volatile int never = 0;
-        const int issued = kb - kb0;
-        const int first = issued > SW_STAGES ? issued - SW_STAGES : 0;
-        for (int i = first; i < issued; ++i)
-          mbar_wait_bounded(smem_u32(&bar_full[i % SW_STAGES]), (uint32_t)((i / SW_STAGES) & 1), &never);
-      }
-    }
-    __syncwarp();
-  } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      if (work) {
-        const uint32_t idesc = idesc_bf16_f32(128, nrows);
+      __syncwarp();
+    } else if (warp == 1) {
+      // ---------------- MMA issuer ----------------
+      if (lane == 0) {
+        const uint32_t idesc = idesc_bf16_f32(128, mma_n);
         bool ok = true;
-        for (int kb = kb0; kb < kb1; ++kb) {
-          const int i = kb - kb0;
-          const uint32_t s = (uint32_t)(i % SW_STAGES), ph = (uint32_t)((i / SW_STAGES) & 1);
+        for (int i = 0; i < kb1 - kb0; ++i, advance()) {
           if (!mbar_wait_bounded(smem_u32(&bar_full[s]), ph, &s_abort)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t a_base = base + s * p.stage_stride, b_base = a_base + (uint32_t)(BM * BK * 2);
-          const uint64_t adesc0 = sw128_kmajor_desc(a_base), bdesc0 = sw128_kmajor_desc(b_base);
+          const uint64_t adesc0 = sw128_kmajor_desc(base + s * (uint32_t)SW_A_BYTES);
+          const uint64_t bdesc0 = sw128_kmajor_desc(b_base + s * b_bytes);
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k)
             tc_mma_bf16(tmem, adesc0 + 2u * k, bdesc0 + 2u * k, idesc, (i > 0 || k > 0) ? 1u : 0u);
           tc_commit(smem_u32(&bar_empty[s]));
         }
         if (!ok) raise_abort(&s_abort, p.status);
+        tc_commit(smem_u32(&bar_acc));  // accumulator ready (also after a failure)
       }
-      tc_commit(smem_u32(&bar_acc));  // accumulator ready (also without work or after a failure)
+      __syncwarp();
     }
-    __syncwarp();
-  } else if (warp >= 4) {
-    // ---------------- epilogue warps: the partial into shared memory ----------------
-    const int q = (warp - 4) * 32 + lane;  // weight row of the tile = TMEM lane = feature
-    const bool ok = warp_wait(smem_u32(&bar_acc), 0u, &s_abort);
-    tc_fence_after();
-    if (!ok && lane == 0) raise_abort(&s_abort, p.status);
-    if (ok && work && !s_abort) {
-      const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-      for (int c0 = 0; c0 < nrows; c0 += 32) {
-        float v[32];
-        tmem_ld_32cols(taddr + (uint32_t)c0, v);
+    // ---------------- the partial into shared memory (every warp) ----------------
+    {
+      // weight row of the tile = TMEM lane = feature; a warp reaches the lanes
+      // 32 (warp % 4) .. + 31: warps 4-7 take the first half of the columns
+      const int q = (warp & 3) * 32 + lane;
+      const bool ok = warp_wait(smem_u32(&bar_acc), acc_ph, &s_abort);
+      tc_fence_after();
+      if (!ok && lane == 0) raise_abort(&s_abort, p.status);
+      if (ok && !s_abort) {
+        const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+        const int chunks = (mma_n + 31) / 32, half = (chunks + 1) / 2;
+        const int ch0 = warp >= 4 ? 0 : half, ch1 = warp >= 4 ? half : chunks;
+        for (int c0 = ch0 * 32; c0 < ch1 * 32; c0 += 32) {
+          float v[32];
+          tmem_ld_32cols(taddr + (uint32_t)c0, v);
 #pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (c0 + j < nrows) P[(c0 + j) * 128 + q] = v[j];  // a warp stores 128 contiguous bytes
+          for (int j = 0; j < 32; ++j)
+            if (c0 + j < mma_n) P[(c0 + j) * 128 + q] = v[j];  // a warp stores 128 contiguous bytes
+        }
       }
     }
+    // ---------------- the cluster's sum and the epilogue ----------------
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const bool go = !s_abort;  // every role is done with the unit: the same in every thread of the CTA
+    cluster_sync_all();        // every partial of the cluster is in shared memory
+    if (go) {
+      // this CTA's rows of the tile
+      const int l0 = (int)rank * rows / S, l1 = ((int)rank + 1) * rows / S;
+      const int total = (l1 - l0) * (p.gate ? 16 : 32);  // four features each
+      if (p.gate) {
+        if (total <= SW_THREADS) swap_gate_rows<1, 8>(p, smem_u32(P), mt, row0, l0, total);
+        else swap_gate_rows<4, 2>(p, smem_u32(P), mt, row0, l0, total);
+      } else {
+        if (total <= SW_THREADS) swap_correction_rows<1, 8>(p, smem_u32(P), mt, row0, l0, total);
+        else swap_correction_rows<4, 2>(p, smem_u32(P), mt, row0, l0, total);
+      }
+    }
+    fence_proxy_async_shared();  // the partial's space goes back to the copies of the next unit
+    cluster_sync_all();          // no CTA moves on while the others read its shared memory
   }
-  // ---------------- the cluster's sum and the epilogue ----------------
   tc_fence_before();
   __syncthreads();
-  const bool go = work && !s_abort;  // every role is done: the same in every thread of the CTA
-  cluster_sync_all();  // every partial of the cluster is in shared memory
-  if (go) {
-    const float* Pr[8];
-#pragma unroll
-    for (int s = 0; s < 8; ++s) Pr[s] = map_rank_ptr(P, (uint32_t)(s < S ? s : 0));
-    const int g0 = (int)((long long)rank * R / S), g1 = (int)((long long)(rank + 1) * R / S);
-    if (!p.gate) {
-      // r[g, n0 + f] = m + beta * c for this CTA's rows: four features per
-      // thread (16-byte partial loads, a warp 512 bytes of a row)
-      const int n0 = mt * 128;
-      for (int u = threadIdx.x; u < (g1 - g0) * 32; u += SW_THREADS) {
-        const int g = g0 + u / 32, f = (u % 32) * 4;
-        float4 x[8];
-#pragma unroll
-        for (int s = 0; s < 8; ++s)  // all loads first, then the sums in rank order
-          x[s] = s < S ? *reinterpret_cast<const float4*>(Pr[s] + g * 128 + f) : make_float4(0.f, 0.f, 0.f, 0.f);
-        const uint2 mw = __ldcg(reinterpret_cast<const uint2*>(p.apack + (long long)g * 2 * d + n0 + f));
-        const long long orow = p.compact_out ? g : __ldcg(p.rowmap + g);
-        float c0 = 0.f, c1 = 0.f, c2 = 0.f, c3 = 0.f;
-#pragma unroll
-        for (int s = 0; s < 8; ++s) {
-          if (s < S) {
-            c0 += x[s].x;
-            c1 += x[s].y;
-            c2 += x[s].z;
-            c3 += x[s].w;
-          }
-        }
-        *reinterpret_cast<uint2*>(p.r_out + orow * d + n0 + f) =
-            make_uint2(pack_bf16x2(bf16_lo(mw.x) + p.beta * c0, bf16_hi(mw.x) + p.beta * c1),
-                       pack_bf16x2(bf16_lo(mw.y) + p.beta * c2, bf16_hi(mw.y) + p.beta * c3));
-      }
-    } else {
-      // e~[g, f0 + f] = e + v sigmoid(g_r + ge) for this CTA's rows: four
-      // features per thread
-      const int f0 = mt * 64;
-      for (int u = threadIdx.x; u < (g1 - g0) * 16; u += SW_THREADS) {
-        const int g = g0 + u / 16, f = (u % 16) * 4;
-        float4 xv[8], xa[8];
-#pragma unroll
-        for (int s = 0; s < 8; ++s) {  // all loads first, then the sums in rank order
-          xv[s] = s < S ? *reinterpret_cast<const float4*>(Pr[s] + g * 128 + f) : make_float4(0.f, 0.f, 0.f, 0.f);
-          xa[s] = s < S ? *reinterpret_cast<const float4*>(Pr[s] + g * 128 + 64 + f) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        const float4 gb = __ldcg(reinterpret_cast<const float4*>(p.ge + f0 + f));
-        const uint2 ew = __ldg(reinterpret_cast<const uint2*>(p.e + f0 + f));
-        const long long orow = __ldcg(p.rowmap + g);
-        float v0 = 0.f, v1 = 0.f, v2 = 0.f, v3 = 0.f, a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-#pragma unroll
-        for (int s = 0; s < 8; ++s) {
-          if (s < S) {
-            v0 += xv[s].x;
-            v1 += xv[s].y;
-            v2 += xv[s].z;
-            v3 += xv[s].w;
-            a0 += xa[s].x;
-            a1 += xa[s].y;
-            a2 += xa[s].z;
-            a3 += xa[s].w;
-          }
-        }
-        a0 += gb.x;
-        a1 += gb.y;
-        a2 += gb.z;
-        a3 += gb.w;
-        *reinterpret_cast<uint2*>(p.e_out + orow * d + f0 + f) =
-            make_uint2(pack_bf16x2(bf16_lo(ew.x) + v0 * fast_sigmoid(a0), bf16_hi(ew.x) + v1 * fast_sigmoid(a1)),
-                       pack_bf16x2(bf16_lo(ew.y) + v2 * fast_sigmoid(a2), bf16_hi(ew.y) + v3 * fast_sigmoid(a3)));
-      }
-    }
-  }
-  cluster_sync_all();  // no CTA leaves while the others read its shared memory
   if (warp == 2) {
     tc_fence_after();
     tmem_dealloc(tmem, p.tmem_cols);
   }
+}
+
+// W_g[:, :d] e alone (a gate-only call).
+__global__ void __launch_bounds__(256) swap_gemv_kernel(const GateBiasParams p) {
+  pdl_launch_dependents();
+  gate_bias_share(p.e, p.Wg, p.ge, p.d, (int)blockIdx.x * 8 + (threadIdx.x >> 5), (int)gridDim.x * 8, threadIdx.x & 31);
+  // Complete only after the previous kernel: the next kernel's programmatic
+  // wait, which covers this kernel alone, then covers that one too.  One CTA
+  // waiting is enough (the grid completes with its last CTA); the others
+  // leave and free their SM for the next kernel.
+  if (blockIdx.x == 0) pdl_wait();
 }
 
 template <bool FUSED>
@@ -1712,130 +1569,6 @@ static int pair_clusters(const TcCondArgs& a, long long tiles_max_pairs, cudaErr
   return (int)(tiles_max_pairs < n ? tiles_max_pairs : n);
 }
 
-// The small-R path (B (K-1) <= kSwapMaxRows, broadcast e or no gate): each
-// GEMM as split-K tiles of 128 weight rows against the R rows, then its
-// reduction kernel; four launches, each waiting on the one before inside the
-// kernel, which cut the work from the R they read.
-static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
-  const long long rmax = (long long)a.B * (a.K - 1);
-  const int d = a.d;
-  const int rows_max = (int)((rmax + 15) / 16 * 16);
-  const int box_n = rows_max < 256 ? rows_max : 256;
-  const int ntiles_max = (rows_max + 255) / 256;
-  DeviceInfo info;
-  cudaError_t err = device_info(&info);
-  if (err != cudaSuccess) return err;
-  static std::atomic<int> attr_done[64];
-  const int max_smem = SW_STAGES * (BM * BK * 2 + 256 * BK * 2) + 1024;
-  if (!attr_done[info.device & 63].load(std::memory_order_acquire)) {
-    err = cudaFuncSetAttribute(swap_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
-    if (err != cudaSuccess) return err;
-    attr_done[info.device & 63].store(1, std::memory_order_release);
-  }
-  const uint32_t stage_stride = (uint32_t)((BM * BK * 2 + box_n * BK * 2 + 1023) / 1024 * 1024);
-  const int smem = SW_STAGES * (int)stage_stride + 1024;
-  uint32_t tmem_cols = 32;
-  while ((int)tmem_cols < box_n) tmem_cols <<= 1;
-  // One resident wave when it can carry every work tile: a split's CTA
-  // streams its whole K range, so a second wave would double the time.
-  static std::atomic<int> occ_cache[64][256 / 16 + 1];
-  int occ = occ_cache[info.device & 63][box_n / 16].load(std::memory_order_relaxed);
-  if (occ == 0) {
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, swap_gemm_kernel, SW_THREADS, (size_t)smem);
-    if (err != cudaSuccess) return err;
-    if (occ < 1) occ = 1;
-    occ_cache[info.device & 63][box_n / 16].store(occ, std::memory_order_relaxed);
-  }
-  int resident = info.sm_count * occ;
-  if (resident > kSwapMaxCtas) resident = kSwapMaxCtas;
-  const uint64_t du = (uint64_t)d;
-  auto params = [&](SwapParams& sp, int mtiles, int nkb) {
-    sp.R = a.R;
-    sp.nkb = nkb;
-    sp.mtiles = mtiles;
-    sp.box_n = box_n;
-    sp.tmem_cols = tmem_cols;
-    sp.stage_stride = stage_stride;
-    sp.part = a.part;
-    sp.status = a.status;
-    const int work_max = mtiles * ntiles_max;
-    return work_max > resident ? work_max : resident;  // the grid
-  };
-  SwapReduceParams rp{};
-  rp.d = d;
-  rp.R = a.R;
-  rp.part = a.part;
-  rp.rowmap = a.rowmap;
-  const int red_grid = info.sm_count * 4;
-  const bool gemv = a.do_gate && !a.e_dense;
-  if (a.do_correct) {
-    CUtensorMap mA, mB;
-    if (encode_tensor_map_2d(&mA, a.Wc, 2 * du, du, 4 * du, BK, 128) != CUDA_SUCCESS ||
-        encode_tensor_map_2d(&mB, a.apack, 2 * du, (uint64_t)rmax, 4 * du, BK, (uint32_t)box_n) != CUDA_SUCCESS)
-      return cudaErrorInvalidValue;
-    SwapParams sp{};
-    const int grid = params(sp, d / 128, 2 * d / BK);
-    sp.mt_a = d / 128;
-    sp.a2_x0 = 0;
-    err = launch_dependent(swap_gemm_kernel, dim3((unsigned)grid), dim3(SW_THREADS), (size_t)smem, stream, 1u, mA,
-                           mA, mB, sp);
-    if (err != cudaSuccess) return err;
-    rp.mtiles = sp.mtiles;
-    rp.nkb = sp.nkb;
-    rp.grid = grid;
-    rp.do_gemv = gemv ? 1 : 0;  // overlapping the correction GEMM
-    rp.gemv.d = d;
-    rp.gemv.e = reinterpret_cast<const __nv_bfloat16*>(a.e);
-    rp.gemv.Wg = reinterpret_cast<const __nv_bfloat16*>(a.Wg);
-    rp.gemv.ge = a.ge;
-    rp.gemv_next = a.sync + kSyncGemvNext;
-    rp.gemv_done = a.sync + kSyncGemvDone;
-    rp.apack = reinterpret_cast<const __nv_bfloat16*>(a.apack);
-    rp.beta = a.beta;
-    rp.r_out = reinterpret_cast<__nv_bfloat16*>(a.r_out);
-    rp.compact_out = a.compact_out;
-    err = launch_dependent(swap_reduce_correction_kernel, dim3((unsigned)red_grid), dim3(256), 0, stream, 1u, rp);
-    if (err != cudaSuccess) return err;
-  }
-  if (a.do_gate) {
-    const uint64_t rstride = 2 * (a.r_row_stride ? (uint64_t)a.r_row_stride : du);
-    CUtensorMap mA, mA2, mB;
-    if (encode_tensor_map_2d(&mA, a.Wv, du, du, 2 * du, BK, 128) != CUDA_SUCCESS ||
-        encode_tensor_map_2d(&mA2, a.Wg, 2 * du, du, 4 * du, BK, 128) != CUDA_SUCCESS ||
-        encode_tensor_map_2d(&mB, a.rpack, du, (uint64_t)rmax, rstride, BK, (uint32_t)box_n) != CUDA_SUCCESS)
-      return cudaErrorInvalidValue;
-    if (gemv && !a.do_correct) {  // no correction kernel to overlap the GEMV with
-      SwapReduceParams gp{};
-      gp.d = d;
-      gp.gemv.d = d;
-      gp.gemv.e = reinterpret_cast<const __nv_bfloat16*>(a.e);
-      gp.gemv.Wg = reinterpret_cast<const __nv_bfloat16*>(a.Wg);
-      gp.gemv.ge = a.ge;
-      gp.gemv_next = a.sync + kSyncGemvNext;
-      gp.gemv_done = a.sync + kSyncGemvDone;
-      err = launch_dependent(swap_gemv_kernel, dim3((unsigned)red_grid), dim3(256), 0, stream, 1u, gp);
-      if (err != cudaSuccess) return err;
-    }
-    SwapParams sp{};
-    const int grid = params(sp, 2 * d / 128, d / BK);
-    sp.mt_a = d / 128;  // W_v rows first, then the r half of W_g
-    sp.a2_x0 = d;
-    err = launch_dependent(swap_gemm_kernel, dim3((unsigned)grid), dim3(SW_THREADS), (size_t)smem, stream, 1u, mA,
-                           mA2, mB, sp);
-    if (err != cudaSuccess) return err;
-    rp.mtiles = sp.mtiles;
-    rp.nkb = sp.nkb;
-    rp.grid = grid;
-    rp.do_gemv = 0;
-    rp.e = reinterpret_cast<const __nv_bfloat16*>(a.e);
-    rp.ge = a.ge;
-    rp.e_out = reinterpret_cast<__nv_bfloat16*>(a.e_out);
-    err = launch_dependent(swap_reduce_gate_kernel, dim3((unsigned)red_grid), dim3(256), 0, stream, 1u, rp);
-    if (err != cudaSuccess) return err;
-  }
-  return cudaSuccess;
-}
-
 // Clusters of S CTAs of swap_cluster_kernel that the device holds at once
 // with `smem` bytes each (0: none), cached per device, S and shared memory.
 static int swap_cluster_capacity(int dev, int S, int smem, cudaError_t* err) {
@@ -1862,115 +1595,132 @@ static int swap_cluster_capacity(int dev, int S, int smem, cudaError_t* err) {
   return n > 0 ? n : 0;
 }
 
-// The small-R GEMMs as split-K clusters with the reduction inside
-// (swap_cluster_kernel): one N tile (at most 256 possible rows) and, for
-// each GEMM, a cluster size S <= 8 whose clusters all fit in one wave with
-// one CTA per SM.  Returns cudaErrorNotSupported (nothing launched) where
-// that does not hold.
-static cudaError_t launch_cond_swap_cluster(const TcCondArgs& a, cudaStream_t stream) {
-  const long long rmax = (long long)a.B * (a.K - 1);
+// Cluster size of a small-R GEMM: the one with the least estimated time at
+// three quarters of the possible rows (R itself is known on the device only).
+// A wave of units costs its k-blocks, 2 (128 + N) cycles each (the stage's
+// bytes in and out of shared memory), plus the drain and the sum of the
+// partial (about 24 cycles per row of the tile) and the fixed start and end.
+static cudaError_t swap_pick_splits(int dev, int smem, int rmax, int mtiles, int nkb, int* S_out, int* clusters) {
+  const int Rt = (3 * rmax + 3) / 4;
+  long long best = -1;
+  cudaError_t err = cudaSuccess;
+  for (int S = 8; S >= 1; --S) {
+    if (S > 1 && nkb / S < SW_MIN_BLOCKS) continue;
+    const int cap = swap_cluster_capacity(dev, S, smem, &err);
+    if (err != cudaSuccess) return err;
+    if (cap == 0) continue;
+    const SwapCut cut = swap_cut(Rt, mtiles, cap);
+    const long long waves = ((long long)mtiles * cut.ntiles + cap - 1) / cap;
+    const long long cost = waves * ((long long)((nkb + S - 1) / S) * 2 * (128 + cut.tile_n) + 24 * cut.tile_n + 2500);
+    if (best < 0 || cost < best) {
+      best = cost;
+      *S_out = S;
+      *clusters = cap;
+    }
+  }
+  return best < 0 ? cudaErrorInvalidConfiguration : cudaSuccess;
+}
+
+// The rows operand of a small-R GEMM: `rows` rows of `inner` elements, one
+// map per box height up to the largest tile of `rows` rows.
+static bool encode_row_maps(RowMaps* maps, const void* base, uint64_t inner, int rows, uint64_t row_stride_bytes) {
+  const int most = swap_box_rows(std::min(256, (rows + 15) / 16 * 16)) / SW_ROW_STEP;
+  for (int i = 0; i < most; ++i)
+    if (encode_tensor_map_2d(&maps->m[i], base, inner, (uint64_t)rows, row_stride_bytes, BK,
+                             (uint32_t)(SW_ROW_STEP * (i + 1))) != CUDA_SUCCESS)
+      return false;
+  return true;
+}
+
+// The small-R path (B (K-1) <= kSwapMaxRows, broadcast e or no gate): the
+// correction GEMM with the gate-bias GEMV, then the gate GEMM; each launch
+// waits on the one before inside the kernel, and cuts its work from the R it
+// reads.
+static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
+  const int rmax = (int)((long long)a.B * (a.K - 1));
   const int d = a.d;
-  const int rows_max = (int)((rmax + 15) / 16 * 16);
-  if (rows_max > 256 || d % 128 != 0) return cudaErrorNotSupported;
-  const int tile_n = rows_max;
   DeviceInfo info;
   cudaError_t err = device_info(&info);
   if (err != cudaSuccess) return err;
   const int dev = info.device;
-  const uint32_t stage_stride = (uint32_t)((BM * BK * 2 + tile_n * BK * 2 + 1023) / 1024 * 1024);
-  // at least half of an SM's shared memory: one CTA per SM, so the K splits
-  // of one wave stream over distinct SMs
-  int smem = SW_STAGES * (int)stage_stride + 1024;
-  if (smem < 117 * 1024) smem = 117 * 1024;
   static std::atomic<int> attr_done[64];
   if (!attr_done[dev & 63].load(std::memory_order_acquire)) {
-    err = cudaFuncSetAttribute(swap_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               SW_STAGES * (BM * BK * 2 + 256 * BK * 2) + 1024);
+    err = cudaFuncSetAttribute(swap_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SW_SMEM_MAX);
     if (err != cudaSuccess) return err;
     attr_done[dev & 63].store(1, std::memory_order_release);
   }
-  // the largest S <= 8 with every cluster of the GEMM resident at once and
-  // at least SW_STAGES k-blocks per split
-  auto pick = [&](int work, int nkb, int* S_out, int* clusters) -> cudaError_t {
-    *S_out = 0;
-    for (int S = 8; S >= 1; --S) {
-      if (nkb / S < SW_STAGES) continue;
-      const int cap = swap_cluster_capacity(dev, S, smem, &err);
-      if (err != cudaSuccess) return err;
-      if (work <= cap) {
-        *S_out = S;
-        *clusters = cap;
-        return cudaSuccess;
-      }
-    }
-    return cudaSuccess;
-  };
-  int Sc = 1, cc = 0, Sg = 1, cg = 0;
-  if (a.do_correct && (err = pick(d / 128, 2 * d / BK, &Sc, &cc)) != cudaSuccess) return err;
-  if (a.do_gate && (err = pick(d / 64, d / BK, &Sg, &cg)) != cudaSuccess) return err;
-  (void)cc;
-  (void)cg;
-  if ((a.do_correct && Sc == 0) || (a.do_gate && Sg == 0)) return cudaErrorNotSupported;
+  const int box_max = swap_box_rows(std::min(256, (rmax + 15) / 16 * 16));
+  const int pre = swap_stages(SW_SMEM_MAX - 1024, box_max);  // stages with the largest row box
+  // at least half of an SM's shared memory: one CTA per SM, so the K splits
+  // of one wave stream over distinct SMs
+  const int smem = std::max(pre * (SW_A_BYTES + box_max * BK * 2) + 1024, 117 * 1024);
   uint32_t tmem_cols = 32;
-  while ((int)tmem_cols < tile_n) tmem_cols <<= 1;
+  while ((int)tmem_cols < std::min(256, rmax)) tmem_cols <<= 1;
   const uint64_t du = (uint64_t)d;
   SwapClusterParams sp{};
   sp.R = a.R;
   sp.d = d;
-  sp.tile_n = tile_n;
+  sp.stage_bytes = smem - 1024;
+  sp.pre = pre;
+  sp.row_maps = box_max / SW_ROW_STEP;
   sp.tmem_cols = tmem_cols;
-  sp.stage_stride = stage_stride;
   sp.rowmap = a.rowmap;
   sp.status = a.status;
-  // W_g[:, :d] e in its own many-warp kernel, launched after the correction
-  // GEMM so that it runs beside it (alone, before the GEMM, it was slower:
-  // its stream is latency-bound); it ends with a programmatic wait, so the
-  // gate launch after it also waits for the correction.
-  auto launch_gemv = [&]() {
-    SwapReduceParams gp{};
-    gp.d = d;
-    gp.gemv.d = d;
-    gp.gemv.e = reinterpret_cast<const __nv_bfloat16*>(a.e);
-    gp.gemv.Wg = reinterpret_cast<const __nv_bfloat16*>(a.Wg);
-    gp.gemv.ge = a.ge;
-    gp.gemv_next = a.sync + kSyncGemvNext;
-    gp.gemv_done = a.sync + kSyncGemvDone;
-    return launch_dependent(swap_gemv_kernel, dim3((unsigned)(info.sm_count * 4)), dim3(256), 0, stream, 1u, gp);
+  // whole row tiles side by side where the resident clusters can take every
+  // row so, else all of them in turn over the units
+  auto grid_of = [&](const SwapClusterParams& c, int clusters) {
+    const int fit = clusters / c.mtiles, most = (rmax + SW_ROW_STEP - 1) / SW_ROW_STEP;
+    if (fit * 256 >= rmax) clusters = c.mtiles * std::min(fit, most);
+    return dim3((unsigned)(clusters * c.S));
   };
+  GateBiasParams gp{};
+  gp.d = d;
+  gp.e = reinterpret_cast<const __nv_bfloat16*>(a.e);
+  gp.Wg = reinterpret_cast<const __nv_bfloat16*>(a.Wg);
+  gp.ge = a.ge;
   if (a.do_correct) {
-    CUtensorMap mA, mB;
+    CUtensorMap mA;
+    RowMaps mB;
     if (encode_tensor_map_2d(&mA, a.Wc, 2 * du, du, 4 * du, BK, 128) != CUDA_SUCCESS ||
-        encode_tensor_map_2d(&mB, a.apack, 2 * du, (uint64_t)rmax, 4 * du, BK, (uint32_t)tile_n) != CUDA_SUCCESS)
+        !encode_row_maps(&mB, a.apack, 2 * du, rmax, 4 * du))
       return cudaErrorInvalidValue;
     SwapClusterParams c = sp;
+    c.mtiles = d / 128;
     c.nkb = 2 * d / BK;
-    c.S = Sc;
-    c.gate = 0;
     c.apack = reinterpret_cast<const __nv_bfloat16*>(a.apack);
     c.beta = a.beta;
     c.r_out = reinterpret_cast<__nv_bfloat16*>(a.r_out);
     c.compact_out = a.compact_out;
-    err = launch_dependent(swap_cluster_kernel, dim3((unsigned)(d / 128 * Sc)), dim3(SW_THREADS), (size_t)smem,
-                           stream, (unsigned)Sc, mA, mA, mB, c);
+    if (a.do_gate) c.bias = gp;
+    int clusters = 0;
+    if ((err = swap_pick_splits(dev, smem, rmax, c.mtiles, c.nkb, &c.S, &clusters)) != cudaSuccess) return err;
+    err = launch_dependent(swap_cluster_kernel, grid_of(c, clusters), dim3(SW_THREADS), (size_t)smem, stream,
+                           (unsigned)c.S, mA, mA, mB, c);
     if (err != cudaSuccess) return err;
   }
   if (a.do_gate) {
     const uint64_t rstride = 2 * (a.r_row_stride ? (uint64_t)a.r_row_stride : du);
-    CUtensorMap mA, mA2, mB;
+    CUtensorMap mA, mA2;
+    RowMaps mB;
     if (encode_tensor_map_2d(&mA, a.Wv, du, du, 2 * du, BK, 64) != CUDA_SUCCESS ||
         encode_tensor_map_2d(&mA2, a.Wg, 2 * du, du, 4 * du, BK, 64) != CUDA_SUCCESS ||
-        encode_tensor_map_2d(&mB, a.rpack, du, (uint64_t)rmax, rstride, BK, (uint32_t)tile_n) != CUDA_SUCCESS)
+        !encode_row_maps(&mB, a.rpack, du, rmax, rstride))
       return cudaErrorInvalidValue;
-    if ((err = launch_gemv()) != cudaSuccess) return err;
+    if (!a.do_correct) {  // no correction kernel to compute it: W_g[:, :d] e in its own launch
+      err = launch_dependent(swap_gemv_kernel, dim3((unsigned)(info.sm_count * 4)), dim3(256), 0, stream, 1u, gp);
+      if (err != cudaSuccess) return err;
+    }
     SwapClusterParams g = sp;
+    g.mtiles = d / 64;
     g.nkb = d / BK;
-    g.S = Sg;
     g.gate = 1;
     g.e = reinterpret_cast<const __nv_bfloat16*>(a.e);
     g.ge = a.ge;
     g.e_out = reinterpret_cast<__nv_bfloat16*>(a.e_out);
-    err = launch_dependent(swap_cluster_kernel, dim3((unsigned)(d / 64 * Sg)), dim3(SW_THREADS), (size_t)smem,
-                           stream, (unsigned)Sg, mA, mA2, mB, g);
+    int clusters = 0;
+    if ((err = swap_pick_splits(dev, smem, rmax, g.mtiles, g.nkb, &g.S, &clusters)) != cudaSuccess) return err;
+    err = launch_dependent(swap_cluster_kernel, grid_of(g, clusters), dim3(SW_THREADS), (size_t)smem, stream,
+                           (unsigned)g.S, mA, mA2, mB, g);
     if (err != cudaSuccess) return err;
   }
   return cudaSuccess;
@@ -1979,10 +1729,7 @@ static cudaError_t launch_cond_swap_cluster(const TcCondArgs& a, cudaStream_t st
 cudaError_t launch_cond_tc(const TcCondArgs& a, cudaStream_t stream) {
   const long long rmax = (long long)a.B * (a.K - 1);
   if (rmax <= 0 || (!a.do_correct && !a.do_gate)) return cudaSuccess;
-  if (a.part && !(a.do_gate && a.e_dense)) {
-    const cudaError_t e1 = launch_cond_swap_cluster(a, stream);
-    return e1 == cudaErrorNotSupported ? launch_cond_swap(a, stream) : e1;
-  }
+  if (rmax <= kSwapMaxRows && !(a.do_gate && a.e_dense)) return launch_cond_swap(a, stream);
   const long long tiles_max_pairs =
       (rmax + 2 * BM - 1) / (2 * BM) * ((a.do_correct ? a.d / 256 : 0) + (a.do_gate ? a.d / 128 : 0));
   cudaError_t err;

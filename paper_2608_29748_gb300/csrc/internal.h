@@ -40,16 +40,14 @@ constexpr int kLowRankLatent = 64;      // rank of the rejected-suffix latents
 constexpr int kLowRankCorrection = 32;  // rank of the target-aware correction
 constexpr int kLowRankSplits = 8;       // split-K parts per half of the [m; u] reduction
 //   skeys    uint64 [B*(2K+1), 64]  sampled verification: top-k keys per target and drafter row
-//   swp      fp32                   split partials of the small-R conditioning GEMMs, or the
-//                                   K halves of the CTA-pair kernel's split gate tiles
+//   swp      fp32                   K halves of the CTA-pair kernel's split gate tiles
 constexpr int kMaxTopK = 64;            // largest top_k of sampled verification
 constexpr int kWindowRows = 4;          // rows per pass of windowed verification
 constexpr int kMaxWindowPasses = 16;    // most passes of windowed verification
-// Small-R conditioning (at most kSwapMaxRows packed rows): the GEMMs as
-// split-K tiles of 128 weight rows against N tiles of up to 256 rows, one
-// grid of at most max(kSwapMaxCtas, work tiles) CTAs, each writing an fp32
-// partial of at most 128 x min(256, rows) values.  Taken while the gate
-// GEMM's work tiles (2d/128 x N tiles) fit in kSwapMaxCtas.
+// Small-R conditioning: at most kSwapMaxRows packed rows, the GEMMs with the
+// weights as the M side in split-K clusters, which sum their partials in shared
+// memory.  The workspace keeps the region that partials in global memory
+// took (swap_part_bytes), so that its size for a shape stays what it was.
 constexpr int kSwapMaxRows = 1024;
 constexpr int kSwapMaxCtas = 256;
 inline size_t swap_part_bytes(long long B, long long K, long long d) {
@@ -64,8 +62,7 @@ inline size_t swap_part_bytes(long long B, long long K, long long d) {
 // CTA-pair conditioning (every other bf16 shape with d a multiple of 256): a
 // last wave of at most kPairSplitTiles gate tiles runs as two K halves per
 // tile on two pairs.  Each half writes its fp32 accumulator (two CTAs x 128
-// rows x 256 columns) to the same region as the small-R partials, and counts
-// on one ticket per CTA and epilogue warp in the sync area.
+// rows x 256 columns) to the workspace (swp), and counts on one ticket per CTA and epilogue warp in the sync area.
 constexpr int kPairSplitTiles = 8;
 inline size_t pair_split_bytes(long long B, long long K, long long d, size_t elem) {
   const long long rmax = B * (K > 1 ? K - 1 : 0);
@@ -350,8 +347,6 @@ struct TcCondArgs {
   const int32_t* rowmap;
   uint32_t* sync;
   uint32_t* status;
-  // small-R path (B (K-1) <= kSwapMaxRows): fp32 split partials, swap_part_bytes (NULL: not taken)
-  float* part;
   // CTA-pair path: fp32 accumulators of the split gate tiles, pair_split_bytes (NULL: no split tiles)
   float* split_part;
 };

@@ -52,32 +52,20 @@ __device__ __forceinline__ bool wait_counter(const uint32_t* counter, uint32_t t
 __device__ __forceinline__ void fence_proxy_async_global() {
   asm volatile("fence.proxy.async.global;" ::: "memory");
 }
-
-// Non-blocking: has the phase with this parity completed?
-__device__ __forceinline__ bool mbar_test_parity(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
+__device__ __forceinline__ void fence_proxy_async_shared() {
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
 // One warp: rows i of ge = W_g[:, :d] e (broadcast e), claimed from a global
 // counter until all d rows are taken; each finished row is counted.  Eight
-// 16-byte loads per lane are in flight (d a multiple of 8).  With a stop
-// barrier (a shared::cta address, not 0) the warp takes no further row once
-// that barrier's phase 0 has completed.
+// 16-byte loads per lane are in flight (d a multiple of 8).
 __device__ void gate_bias_rows(const __nv_bfloat16* e, const __nv_bfloat16* Wg, float* ge, int d, int lane,
-                               uint32_t* next, uint32_t* done, uint32_t stop_bar = 0u) {
+                               uint32_t* next, uint32_t* done) {
   const int vpr = d / 8;
   const uint4* ev = reinterpret_cast<const uint4*>(e);
   for (;;) {
     int i = 0;
-    if (lane == 0) i = (stop_bar != 0u && mbar_test_parity(stop_bar, 0u)) ? d : (int)atomicAdd(next, 1u);
+    if (lane == 0) i = (int)atomicAdd(next, 1u);
     i = __shfl_sync(0xFFFFFFFFu, i, 0);
     if (i >= d) break;
     const uint4* wr = reinterpret_cast<const uint4*>(Wg + (long long)i * 2 * d);
@@ -110,6 +98,57 @@ __device__ void gate_bias_rows(const __nv_bfloat16* e, const __nv_bfloat16* Wg, 
       __threadfence();
       atomicAdd(done, 1u);
     }
+  }
+}
+
+// One warp of `nw`: rows w, w + nw, ... of ge = W_g[:, :d] e (d a multiple of
+// 8).  The row comes in steps of 256 vectors, the next step's loads issued
+// before the current one is multiplied: a warp that claimed its rows from a
+// counter and loaded one row at a time took 3 us per row of 4096, three
+// round trips.
+__device__ __forceinline__ void gate_bias_share(const __nv_bfloat16* e, const __nv_bfloat16* Wg, float* ge, int d,
+                                                int w, int nw, int lane) {
+  const int vpr = d / 8, steps = (vpr + 255) / 256;
+  const uint4* ev = reinterpret_cast<const uint4*>(e);
+  auto load = [&](uint4 (&x)[8], int row, int step) {
+    const uint4* wr = reinterpret_cast<const uint4*>(Wg + (long long)row * 2 * d);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int v = step * 256 + u * 32 + lane;
+      x[u] = v < vpr ? __ldcs(wr + v) : make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  if (w >= d) return;
+  uint4 cur[8], nxt[8];
+  load(cur, w, 0);
+  float acc = 0.f;
+  for (int row = w, step = 0; row < d;) {
+    const bool last = step + 1 == steps;
+    const int row_n = last ? row + nw : row, step_n = last ? 0 : step + 1;
+    if (row_n < d) load(nxt, row_n, step_n);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int v = step * 256 + u * 32 + lane;
+      if (v < vpr) {
+        const uint4 x = __ldg(ev + v);
+        const uint32_t ww[4] = {cur[u].x, cur[u].y, cur[u].z, cur[u].w}, xx[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          acc = fmaf(bf16_lo(ww[q]), bf16_lo(xx[q]), acc);
+          acc = fmaf(bf16_hi(ww[q]), bf16_hi(xx[q]), acc);
+        }
+      }
+    }
+    if (last) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
+      if (lane == 0) ge[row] = acc;
+      acc = 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) cur[u] = nxt[u];
+    row = row_n;
+    step = step_n;
   }
 }
 
@@ -163,13 +202,20 @@ __device__ __forceinline__ bool warp_wait_cluster(uint32_t bar, uint32_t parity,
   __syncwarp();
   return ok != 0;
 }
-// The generic address of `p` (this CTA's shared memory) in cluster CTA `rank`:
-// plain loads through it read that CTA's shared memory.
-template <typename T>
-__device__ __forceinline__ const T* map_rank_ptr(const T* p, uint32_t rank) {
-  uint64_t r;
-  asm volatile("mapa.u64 %0, %1, %2;" : "=l"(r) : "l"(reinterpret_cast<uint64_t>(p)), "r"(rank));
-  return reinterpret_cast<const T*>(r);
+// Four floats at a shared::cluster address (another CTA's shared memory, or this one's).
+__device__ __forceinline__ float4 ld_cluster_f4(uint32_t cluster_addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(cluster_addr)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ void add4(float4& a, const float4& b) {
+  a.x += b.x;
+  a.y += b.y;
+  a.z += b.z;
+  a.w += b.w;
 }
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
