@@ -273,9 +273,13 @@ retrace_status enqueue_conditioning(const ConditioningArgs& c, retrace_dtype dty
     if (phase_events) RT_CUDA(cudaEventRecord(phase_events[2], stream), "cudaEventRecord");
   } else {
     CorrectArgs ca{c.hD, c.hT, c.Wc, c.beta, B, K, d, rows, r_ws, 1, raw ? 1 : 0};
+    if (!c.e_dense) {
+      ca.Wg = c.Wg;
+      ca.e = c.e;
+      ca.ge = ge;
+    }
     RT_CUDA(launch_correct_simt(ca, dtype, stream), "correction kernel launch");
     if (phase_events) RT_CUDA(cudaEventRecord(phase_events[2], stream), "cudaEventRecord");
-    if (!c.e_dense) RT_CUDA(launch_gate_bias(c.Wg, c.e, d, ge, dtype, stream), "gate bias kernel launch");
     GateArgs ga{c.e, c.e_dense, r_ws, 1, c.Wv, c.Wg, c.e_dense ? nullptr : ge, B, K, d, rows, c.e_out};
     RT_CUDA(launch_gate_simt(ga, dtype, stream), "gate kernel launch");
   }

@@ -1,238 +1,136 @@
 // Conditioning projections on the CUDA cores (FFMA, fp32 accumulation).
 //
 // This path serves fp32 workloads (which must not use TF32) and bf16 shapes
-// the tensor-core kernels do not take (hidden size not a multiple of 256 or
-// unaligned tensors).  Same arithmetic as the tensor-core path:
+// the tensor-core kernels do not take.  Same arithmetic as the tensor-core
+// path:
 //   correction  r = m + beta * W_c [m; u]                (Eq. 6-7)
 //   gate        e~ = e + (W_v r) .* sigmoid(W_g [e; r])  (Eq. 8)
 // with the operand rows gathered through the device-side row plan.
 #include "common.cuh"
 #include "internal.h"
 #include "plan.cuh"
+#include "tc_pair.cuh"
 
 namespace retrace {
 namespace {
 
+// One kernel for both projections.  A unit is a tile of 64 weight rows (64
+// features of W_c; for the gate 32 rows of W_v and the same 32 of W_g, so that
+// v and the gate of a feature meet in one CTA) against a tile of up to 64
+// conditioned rows.  The reduction is cut into 32-deep chunks, and the chunks
+// of a unit are split over a cluster of S CTAs: with few rows a unit per 64
+// features would leave most SMs idle and walk thousands of products one
+// memory latency after another.  A chunk goes through a four-stage cp.async
+// ring; thread (ty, tx) of 16 x 16 owns rows ty + 16 i and weight rows
+// tx + 16 j (4 MR values) and reads both operands 16 bytes at a time along the
+// reduction (rows padded to 36 floats: conflict-free).  Each CTA then leaves
+// its partial tile in shared memory, and after a cluster barrier every CTA
+// sums its share of the rows over the S partials in rank order (results repeat
+// bit for bit) and applies the epilogue.  MR = rows of the tile / 16 is chosen
+// on the device from R.
 constexpr int kNT = 256;
-constexpr int TM = 32, TN = 64, TK = 32;
+constexpr int kTileRows = 64;              // most conditioned rows of a tile
+constexpr int TN = 64, TK = 32;            // weight rows and reduction depth of a chunk
+constexpr int kLd = TK + 4;                // floats between rows of a staged chunk
+constexpr int kSimtStages = 4;
+constexpr int kStageFloats = (kTileRows + TN) * kLd;
+constexpr int kSimtSmem = kSimtStages * kStageFloats * 4;
+static_assert(kTileRows * TN <= kSimtStages * kStageFloats, "the partial tile reuses the ring");
 
-struct SimtCorrectParams {
-  const void* hD;
-  const void* hT;
-  const void* Wc;
+struct SimtParams {
+  const void* a0;  // rows operand, part 0 and 1: hD, hT (correction); r, dense e (gate)
+  const void* a1;
+  const void* w;   // W_c (correction) or W_v (gate)
+  const void* wg;  // W_g
+  const void* e;
+  float* ge;       // W_g[:, :d] e for a broadcast e
   float beta;
   int B, K, d;
   RowSource rows;
   void* out;
-  int compact_out;
-  int raw;  // r = m: no accumulation, W_c not read
-};
-
-struct SimtGateParams {
-  const void* e;
+  int compact;     // the compact side of r: r_out rows (correction), r rows (gate)
+  int raw;         // correction: r = m, no reduction
   int e_dense;
-  const void* r;
-  int r_compact;
-  const void* Wv;
-  const void* Wg;
-  const float* ge;
-  int B, K, d;
-  RowSource rows;
-  void* out;
+  int S, ftiles;   // cluster size, feature tiles
+  int clusters;    // clusters with a unit; CTAs past them compute ge
+  int vec;         // 16-byte fp32 copies
 };
 
-// Threads form a 16 x 16 grid; thread (ty, tx) owns rows 2ty..2ty+1 and
-// columns 4tx..4tx+3 of the 32 x 64 output tile.
-template <typename T>
-__global__ void __launch_bounds__(kNT) simt_correct_kernel(const SimtCorrectParams p) {
-  __shared__ int s_b[TM], s_j[TM], s_nb[TM], s_scan[kNT / 32 + 1];
-  __shared__ long long s_m[TM], s_u[TM];
-  __shared__ float As[TM][TK + 1];
-  __shared__ float Bs[TN][TK + 1];
-
-  const long long m0 = (long long)blockIdx.x * TM;
-  const int n0 = blockIdx.y * TN;
-  const int R = plan_tile<kNT, TM>(p.rows, p.B, p.K, m0, s_b, s_j, s_nb, s_scan);
-  if (m0 >= R) return;
-  const int K = p.K, d = p.d, tid = threadIdx.x;
-  if (tid < TM) {
-    const int b = s_b[tid];
-    if (b >= 0) {
-      const int A = K - 1 - s_nb[tid];
-      s_m[tid] = ((long long)b * K + A + 1 + s_j[tid]) * d;  // m_j = hD[b, A+1+j]
-      s_u[tid] = ((long long)b * K + A + s_j[tid]) * d;      // u_j = hT[b, A+j]
-    } else {
-      s_m[tid] = -1;
-      s_u[tid] = -1;
-    }
+// Row numbers of the plan: the rows of this CTA's row tile nt, cut from R into
+// tiles of equal size (a multiple of 16, at most kTileRows).  Fills s_b (-1
+// past the last row), s_j, s_nb; returns R and the tile size and first row.
+__device__ int plan_row_tile(const RowSource& rs, int B, int K, int nt, int* s_b, int* s_j, int* s_nb, int* s_scan,
+                             int* tile, long long* m0) {
+  constexpr int NW = kNT / 32;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int total = 0, nb = 0;
+  for (int base = 0; base < B; base += kNT) {
+    nb = base + tid < B ? rows_of(rs, base + tid, K) : 0;
+    total += nb;
+  }
+  // inclusive sums over the threads (with B <= kNT: over the sequences)
+  int x = total;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int y = __shfl_up_sync(0xFFFFFFFFu, x, off);
+    if (lane >= off) x += y;
+  }
+  if (lane == 31) s_scan[warp] = x;
+  for (int q = tid; q < kTileRows; q += kNT) {
+    s_b[q] = -1;
+    s_j[q] = 0;
+    s_nb[q] = 0;
   }
   __syncthreads();
-  const T* hD = reinterpret_cast<const T*>(p.hD);
-  const T* hT = reinterpret_cast<const T*>(p.hT);
-  const T* Wc = reinterpret_cast<const T*>(p.Wc);
-  const int ty = tid / 16, tx = tid % 16;
-  float acc[2][4] = {};
-  const int K2 = 2 * d;
-  for (int k0 = 0; k0 < (p.raw ? 0 : K2); k0 += TK) {
-    for (int idx = tid; idx < TM * TK; idx += kNT) {
-      const int r = idx / TK, kk = idx % TK, k = k0 + kk;
-      float v = 0.f;
-      if (s_m[r] >= 0 && k < K2) v = (k < d) ? to_f32(hD[s_m[r] + k]) : to_f32(hT[s_u[r] + k - d]);
-      As[r][kk] = v;
-    }
-    for (int idx = tid; idx < TN * TK; idx += kNT) {
-      const int c = idx / TK, kk = idx % TK, k = k0 + kk, n = n0 + c;
-      Bs[c][kk] = (n < d && k < K2) ? to_f32(Wc[(long long)n * K2 + k]) : 0.f;
+  int before = 0, R = 0;
+#pragma unroll
+  for (int w = 0; w < NW; ++w) {
+    if (w < warp) before += s_scan[w];
+    R += s_scan[w];
+  }
+  const int ntiles = (R + kTileRows - 1) / kTileRows;
+  *tile = ntiles > 0 ? ((R + ntiles - 1) / ntiles + 15) / 16 * 16 : 16;
+  *m0 = (long long)nt * *tile;
+  if (*m0 >= R) return R;
+  if (B <= kNT) {
+    const long long off = before + x - nb;
+    const long long lo = off > *m0 ? off : *m0, end = *m0 + *tile;
+    const long long hi = off + nb < end ? off + nb : end;
+    for (long long g = lo; g < hi; ++g) {
+      const int q = (int)(g - *m0);
+      s_b[q] = tid;
+      s_j[q] = (int)(g - off);
+      s_nb[q] = nb;
     }
     __syncthreads();
-#pragma unroll 8
-    for (int kk = 0; kk < TK; ++kk) {
-      const float a0 = As[2 * ty][kk], a1 = As[2 * ty + 1][kk];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float bq = Bs[4 * tx + q][kk];
-        acc[0][q] = fmaf(a0, bq, acc[0][q]);
-        acc[1][q] = fmaf(a1, bq, acc[1][q]);
-      }
-    }
-    __syncthreads();
+  } else {
+    __syncthreads();  // s_scan is read to the end
+    plan_tile<kNT, kTileRows>(rs, B, K, *m0, s_b, s_j, s_nb, s_scan);
   }
-  T* out = reinterpret_cast<T*>(p.out);
-#pragma unroll
-  for (int rr = 0; rr < 2; ++rr) {
-    const int r = 2 * ty + rr;
-    const int b = s_b[r];
-    if (b < 0) continue;
-    const long long orow = p.compact_out ? (m0 + r) : ((long long)b * K + s_j[r]);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int n = n0 + 4 * tx + q;
-      if (n >= d) continue;
-      const T m = hD[s_m[r] + n];
-      out[orow * d + n] = p.raw ? m : from_f32<T>(to_f32(m) + p.beta * acc[rr][q]);
-    }
-  }
+  return R;
 }
 
+__device__ __forceinline__ void cp_async16_zfill(uint32_t smem_dst, const void* gsrc, bool in) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_dst), "l"(gsrc), "r"(in ? 16 : 0)
+               : "memory");
+}
+
+// Four consecutive elements src[k..k+3] of a row of d into staged floats; zeros
+// past the row's end (k >= d) or for a row that does not exist (src NULL).
 template <typename T>
-__global__ void __launch_bounds__(kNT) simt_gate_kernel(const SimtGateParams p) {
-  __shared__ int s_b[TM], s_j[TM], s_nb[TM], s_scan[kNT / 32 + 1];
-  __shared__ long long s_r[TM], s_e[TM];
-  __shared__ float As[TM][TK + 1];
-  __shared__ float Bv[TN][TK + 1];
-  __shared__ float Bg[TN][TK + 1];
-
-  const long long m0 = (long long)blockIdx.x * TM;
-  const int n0 = blockIdx.y * TN;
-  const int R = plan_tile<kNT, TM>(p.rows, p.B, p.K, m0, s_b, s_j, s_nb, s_scan);
-  if (m0 >= R) return;
-  const int K = p.K, d = p.d, tid = threadIdx.x;
-  if (tid < TM) {
-    const int b = s_b[tid];
-    if (b >= 0) {
-      const long long pos = (long long)b * K + s_j[tid];
-      s_r[tid] = (p.r_compact ? (m0 + tid) : pos) * d;
-      s_e[tid] = p.e_dense ? pos * d : 0;
-    } else {
-      s_r[tid] = -1;
-      s_e[tid] = 0;
+__device__ __forceinline__ void stage4(float* dst, const T* src, int k, int d, const void* any, bool vec) {
+  if constexpr (sizeof(T) == 4) {
+    if (vec) {
+      const bool in = src != nullptr && k < d;
+      cp_async16_zfill(smem_u32(dst), in ? static_cast<const void*>(src + k) : any, in);
+      return;
     }
   }
-  __syncthreads();
-  const T* r = reinterpret_cast<const T*>(p.r);
-  const T* e = reinterpret_cast<const T*>(p.e);
-  const T* Wv = reinterpret_cast<const T*>(p.Wv);
-  const T* Wg = reinterpret_cast<const T*>(p.Wg);
-  const int ty = tid / 16, tx = tid % 16;
-  const long long ldg = 2LL * d;
-  float av[2][4] = {}, ag[2][4] = {};
-  // v = W_v r and the r half of the gate, W_g[:, d:2d] r.
-  for (int k0 = 0; k0 < d; k0 += TK) {
-    for (int idx = tid; idx < TM * TK; idx += kNT) {
-      const int rr = idx / TK, kk = idx % TK, k = k0 + kk;
-      As[rr][kk] = (s_r[rr] >= 0 && k < d) ? to_f32(r[s_r[rr] + k]) : 0.f;
-    }
-    for (int idx = tid; idx < TN * TK; idx += kNT) {
-      const int c = idx / TK, kk = idx % TK, k = k0 + kk, n = n0 + c;
-      const bool ok = n < d && k < d;
-      Bv[c][kk] = ok ? to_f32(Wv[(long long)n * d + k]) : 0.f;
-      Bg[c][kk] = ok ? to_f32(Wg[(long long)n * ldg + d + k]) : 0.f;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int kk = 0; kk < TK; ++kk) {
-      const float a0 = As[2 * ty][kk], a1 = As[2 * ty + 1][kk];
+  float v[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float bv = Bv[4 * tx + q][kk], bg = Bg[4 * tx + q][kk];
-        av[0][q] = fmaf(a0, bv, av[0][q]);
-        av[1][q] = fmaf(a1, bv, av[1][q]);
-        ag[0][q] = fmaf(a0, bg, ag[0][q]);
-        ag[1][q] = fmaf(a1, bg, ag[1][q]);
-      }
-    }
-    __syncthreads();
-  }
-  // Per-position e: the e half of the gate, W_g[:, 0:d] e.
-  if (p.e_dense) {
-    for (int k0 = 0; k0 < d; k0 += TK) {
-      for (int idx = tid; idx < TM * TK; idx += kNT) {
-        const int rr = idx / TK, kk = idx % TK, k = k0 + kk;
-        As[rr][kk] = (s_r[rr] >= 0 && k < d) ? to_f32(e[s_e[rr] + k]) : 0.f;
-      }
-      for (int idx = tid; idx < TN * TK; idx += kNT) {
-        const int c = idx / TK, kk = idx % TK, k = k0 + kk, n = n0 + c;
-        Bg[c][kk] = (n < d && k < d) ? to_f32(Wg[(long long)n * ldg + k]) : 0.f;
-      }
-      __syncthreads();
-#pragma unroll 8
-      for (int kk = 0; kk < TK; ++kk) {
-        const float a0 = As[2 * ty][kk], a1 = As[2 * ty + 1][kk];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float bg = Bg[4 * tx + q][kk];
-          ag[0][q] = fmaf(a0, bg, ag[0][q]);
-          ag[1][q] = fmaf(a1, bg, ag[1][q]);
-        }
-      }
-      __syncthreads();
-    }
-  }
-  T* out = reinterpret_cast<T*>(p.out);
-#pragma unroll
-  for (int rr = 0; rr < 2; ++rr) {
-    const int row = 2 * ty + rr;
-    const int b = s_b[row];
-    if (b < 0) continue;
-    const long long orow = (long long)b * K + s_j[row];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int n = n0 + 4 * tx + q;
-      if (n >= d) continue;
-      const float g = ag[rr][q] + (p.e_dense ? 0.f : p.ge[n]);
-      const float ev = to_f32(e[s_e[row] + n]);
-      const float gate = 1.f / (1.f + expf(-g));
-      out[orow * d + n] = from_f32<T>(ev + av[rr][q] * gate);
-    }
-  }
+  for (int q = 0; q < 4; ++q) v[q] = (src != nullptr && k + q < d) ? to_f32(src[k + q]) : 0.f;
+  *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
 }
-
-// ---------------------------------------------------------------------------
-// Few rows (B (K-1) <= kRowsMax): one warp per output feature
-// ---------------------------------------------------------------------------
-// With a handful of rows the 32 x 64 tiles above leave all but d/64 SMs idle
-// and walk the reduction in 32-deep steps, one load latency each.  Here each
-// warp owns one output feature n and all rows: its lanes stride the
-// reduction index (coalesced loads of the weight row, the operand rows read
-// through L1), each lane keeps kRowGroup row sums, and a butterfly of
-// shuffles adds the lanes in a fixed order (results repeat bit for bit).
-// The rows are taken kRowGroup at a time (the weight row is re-read per
-// group), and each lane issues the loads of kBatch reduction steps for the
-// weight and every row of the group before it multiplies.
-constexpr int kRowsMax = 32;  // one plan tile
-constexpr int kRowGroup = 8;
-constexpr int kBatch = 4;  // reduction steps per lane with their loads issued together
-constexpr int kRowsWarps = kNT / 32;
 
 __device__ __forceinline__ float warp_sum(float s) {
 #pragma unroll
@@ -240,179 +138,215 @@ __device__ __forceinline__ float warp_sum(float s) {
   return s;
 }
 
+// W_g[i, :d] e by one warp: lanes stride the row, four loads in flight each.
 template <typename T>
-__global__ void __launch_bounds__(kNT) simt_rows_correct_kernel(const SimtCorrectParams p) {
-  __shared__ int s_b[kRowsMax], s_j[kRowsMax], s_nb[kRowsMax], s_scan[kNT / 32 + 1];
-  __shared__ long long s_m[kRowsMax], s_u[kRowsMax];
-  const int R = plan_tile<kNT, kRowsMax>(p.rows, p.B, p.K, 0, s_b, s_j, s_nb, s_scan);
-  const int K = p.K, d = p.d, tid = threadIdx.x, lane = tid & 31;
-  if (tid < kRowsMax) {
-    const int b = s_b[tid];
-    const int A = K - 1 - s_nb[tid];
-    s_m[tid] = b >= 0 ? ((long long)b * K + A + 1 + s_j[tid]) * d : 0;  // m_j = hD[b, A+1+j]
-    s_u[tid] = b >= 0 ? ((long long)b * K + A + s_j[tid]) * d : 0;      // u_j = hT[b, A+j]
+__device__ __forceinline__ float gate_bias_row(const T* Wg, const T* e, int i, int d, int lane) {
+  const T* w = Wg + (long long)i * 2 * d;
+  float s = 0.f;
+  for (int k0 = lane; k0 < d; k0 += 4 * 32) {
+    float a[4], b[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int k = k0 + 32 * q;
+      a[q] = k < d ? to_f32(w[k]) : 0.f;
+      b[q] = k < d ? to_f32(e[k]) : 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) s = fmaf(a[q], b[q], s);
   }
-  __syncthreads();
-  const int n = blockIdx.x * kRowsWarps + (tid >> 5);
-  if (n >= d) return;
-  const T* hD = reinterpret_cast<const T*>(p.hD);
-  const T* hT = reinterpret_cast<const T*>(p.hT);
-  const T* w = reinterpret_cast<const T*>(p.Wc) + (long long)n * 2 * d;
-  T* out = reinterpret_cast<T*>(p.out);
-  const int nrows = R < kRowsMax ? R : kRowsMax;
-  for (int g0 = 0; g0 < nrows; g0 += kRowGroup) {
-    const int gn = nrows - g0 < kRowGroup ? nrows - g0 : kRowGroup;
-    float acc[kRowGroup];
+  return warp_sum(s);
+}
+
+// The partial tile of this CTA: its chunks [c0, c1) of the unit with weight
+// tile n0, rows at s_off0 / s_off1 (-1: no row), into ring[] as [row][TN].
+template <typename T, bool GATE, int MR>
+__device__ __forceinline__ void simt_partial(const SimtParams& p, float* ring, const long long* s_off0,
+                                             const long long* s_off1, int n0, int c0, int c1) {
+  const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16, d = p.d;
+  const int per = (d + TK - 1) / TK;  // chunks per part
+  const T* A0 = reinterpret_cast<const T*>(p.a0);
+  const T* A1 = reinterpret_cast<const T*>(p.a1);
+  const T* W = reinterpret_cast<const T*>(p.w);
+  const T* Wg = reinterpret_cast<const T*>(p.wg);
+  const bool vec = p.vec != 0;
+  auto stage = [&](int c) {
+    if (c < c1) {
+      const int part = c >= per ? 1 : 0, kc = (c - part * per) * TK + (tid % 8) * 4;
+      float* As = ring + (c - c0) % kSimtStages * kStageFloats;
+      float* Bs = As + kTileRows * kLd;
 #pragma unroll
-    for (int q = 0; q < kRowGroup; ++q) acc[q] = 0.f;
-    if (!p.raw) {
-      // c = W_c [m; u]: the m half (k < d), then the u half
-      for (int half = 0; half < 2; ++half) {
-        const T* wh = w + half * d;
-        const T* src[kRowGroup];
-#pragma unroll
-        for (int q = 0; q < kRowGroup; ++q) {  // rows past the group repeat its first (discarded)
-          const int row = g0 + (q < gn ? q : 0);
-          src[q] = half == 0 ? hD + s_m[row] : hT + s_u[row];
+      for (int i = 0; i < (MR + 1) / 2; ++i) {
+        const int r = tid / 8 + 32 * i;
+        if (r < 16 * MR) {
+          const long long off = part ? s_off1[r] : s_off0[r];
+          stage4<T>(As + r * kLd + (tid % 8) * 4, off >= 0 ? (part ? A1 : A0) + off : nullptr, kc, d, W, vec);
         }
-        for (int k0 = lane; k0 < d; k0 += 32 * kBatch) {
-          float wk[kBatch], x[kRowGroup][kBatch];
+      }
 #pragma unroll
-          for (int u = 0; u < kBatch; ++u) {
-            const int k = k0 + 32 * u;
-            wk[u] = k < d ? to_f32(wh[k]) : 0.f;
-#pragma unroll
-            for (int q = 0; q < kRowGroup; ++q) x[q][u] = k < d ? to_f32(src[q][k]) : 0.f;
+      for (int i = 0; i < TN / 32; ++i) {
+        const int r = tid / 8 + 32 * i;
+        const T* src;
+        if constexpr (!GATE) {
+          const int n = n0 + r;
+          src = n < d ? W + (long long)n * 2 * d + (long long)part * d : nullptr;
+        } else {
+          const int n = n0 + (r & 31);  // i = 0: rows of W_v, i = 1: the same rows of W_g
+          if (i == 0) {
+            if (part) continue;  // the e part has a gate only
+            src = n < d ? W + (long long)n * d : nullptr;
+          } else {
+            src = n < d ? Wg + (long long)n * 2 * d + (part ? 0 : d) : nullptr;
           }
+        }
+        stage4<T>(Bs + r * kLd + (tid % 8) * 4, src, kc, d, W, vec);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  float acc[MR][4];
 #pragma unroll
-          for (int q = 0; q < kRowGroup; ++q)
+  for (int i = 0; i < MR; ++i)
 #pragma unroll
-            for (int u = 0; u < kBatch; ++u) acc[q] = fmaf(wk[u], x[q][u], acc[q]);
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+#pragma unroll
+  for (int q = 0; q < kSimtStages - 1; ++q) stage(c0 + q);
+  for (int c = c0; c < c1; ++c) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kSimtStages - 2) : "memory");
+    __syncthreads();  // chunk c is staged, and chunk c - 1's slot is read
+    stage(c + kSimtStages - 1);
+    const float* As = ring + (c - c0) % kSimtStages * kStageFloats + ty * kLd;
+    const float* Bs = ring + (c - c0) % kSimtStages * kStageFloats + (kTileRows + tx) * kLd;
+    const bool gate_only = GATE && c >= per;
+#pragma unroll
+    for (int k = 0; k < TK; k += 4) {
+      float4 a[MR], b[4];
+#pragma unroll
+      for (int i = 0; i < MR; ++i) a[i] = *reinterpret_cast<const float4*>(As + 16 * i * kLd + k);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4*>(Bs + 16 * j * kLd + k);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (j < 2 && gate_only) continue;  // weight rows tx, tx + 16: W_v
+#pragma unroll
+        for (int i = 0; i < MR; ++i) {
+          acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
+          acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
+          acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
+          acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
         }
       }
-#pragma unroll
-      for (int q = 0; q < kRowGroup; ++q) acc[q] = warp_sum(acc[q]);
-    }
-    if (lane < gn) {
-      float a = acc[0];
-#pragma unroll
-      for (int q = 1; q < kRowGroup; ++q)
-        if (lane == q) a = acc[q];
-      const int row = g0 + lane;
-      const long long orow = p.compact_out ? row : ((long long)s_b[row] * K + s_j[row]);
-      const T m = hD[s_m[row] + n];
-      out[orow * d + n] = p.raw ? m : from_f32<T>(to_f32(m) + p.beta * a);
     }
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();  // the ring becomes the partial tile
+#pragma unroll
+  for (int i = 0; i < MR; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) ring[(ty + 16 * i) * TN + tx + 16 * j] = acc[i][j];
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kNT) simt_rows_gate_kernel(const SimtGateParams p) {
-  __shared__ int s_b[kRowsMax], s_j[kRowsMax], s_nb[kRowsMax], s_scan[kNT / 32 + 1];
-  __shared__ long long s_r[kRowsMax], s_e[kRowsMax];
-  const int R = plan_tile<kNT, kRowsMax>(p.rows, p.B, p.K, 0, s_b, s_j, s_nb, s_scan);
-  const int K = p.K, d = p.d, tid = threadIdx.x, lane = tid & 31;
-  if (tid < kRowsMax) {
+template <typename T, bool GATE>
+__global__ void __launch_bounds__(kNT, 2) simt_cluster_kernel(const SimtParams p) {
+  extern __shared__ float4 simt_smem[];
+  __shared__ int s_b[kTileRows], s_j[kTileRows], s_nb[kTileRows], s_scan[kNT / 32 + 1];
+  __shared__ long long s_off0[kTileRows], s_off1[kTileRows];
+  float* ring = reinterpret_cast<float*>(simt_smem);
+  const int tid = threadIdx.x, S = p.S, K = p.K, d = p.d;
+  const int cid = (int)(blockIdx.x / (unsigned)S);
+  pdl_launch_dependents();
+  const T* e = reinterpret_cast<const T*>(p.e);
+  if (cid >= p.clusters) {  // the gate's broadcast-e half (inputs only: no wait)
+    const int first = ((int)blockIdx.x - p.clusters * S) * (kNT / 32) + tid / 32;
+    const int stride = ((int)gridDim.x - p.clusters * S) * (kNT / 32);
+    for (int i = first; i < d; i += stride) {
+      const float s = gate_bias_row<T>(reinterpret_cast<const T*>(p.wg), e, i, d, tid & 31);
+      if ((tid & 31) == 0) p.ge[i] = s;
+    }
+    return;
+  }
+  pdl_wait();  // the accepted lengths (and r) come from the previous kernels
+  int tile;
+  long long m0;
+  const int R = plan_row_tile(p.rows, p.B, K, cid / p.ftiles, s_b, s_j, s_nb, s_scan, &tile, &m0);
+  if (m0 >= R) return;  // the whole cluster
+  const int rows = (int)(R - m0 < tile ? R - m0 : tile);
+  if (tid < kTileRows) {
     const int b = s_b[tid];
-    const long long pos = b >= 0 ? (long long)b * K + s_j[tid] : 0;
-    s_r[tid] = (p.r_compact ? tid : pos) * d;
-    s_e[tid] = p.e_dense ? pos * d : 0;
+    const long long pos = (long long)b * K + s_j[tid];
+    const int A = K - 1 - s_nb[tid];
+    if (b < 0) {
+      s_off0[tid] = s_off1[tid] = -1;
+    } else if constexpr (!GATE) {
+      s_off0[tid] = (pos + A + 1) * d;  // m_j = hD[b, A+1+j]
+      s_off1[tid] = (pos + A) * d;      // u_j = hT[b, A+j]
+    } else {
+      s_off0[tid] = (p.compact ? m0 + tid : pos) * d;
+      s_off1[tid] = p.e_dense ? pos * d : 0;
+    }
   }
   __syncthreads();
-  const int n = blockIdx.x * kRowsWarps + (tid >> 5);
-  if (n >= d) return;
-  const T* r = reinterpret_cast<const T*>(p.r);
-  const T* e = reinterpret_cast<const T*>(p.e);
-  const T* wv = reinterpret_cast<const T*>(p.Wv) + (long long)n * d;
-  const T* wg = reinterpret_cast<const T*>(p.Wg) + (long long)n * 2 * d;
+  const uint32_t rank = cluster_rank();
+  constexpr int F = GATE ? 32 : 64;  // features of a unit
+  const int n0 = cid % p.ftiles * F;
+  const int per = (d + TK - 1) / TK;
+  const int chunks = GATE ? per * (p.e_dense ? 2 : 1) : (p.raw ? 0 : 2 * per);
+  const int c0 = (int)((long long)rank * chunks / S), c1 = (int)((long long)(rank + 1) * chunks / S);
+  if (tile == 16) simt_partial<T, GATE, 1>(p, ring, s_off0, s_off1, n0, c0, c1);
+  else if (tile == 32) simt_partial<T, GATE, 2>(p, ring, s_off0, s_off1, n0, c0, c1);
+  else if (tile == 48) simt_partial<T, GATE, 3>(p, ring, s_off0, s_off1, n0, c0, c1);
+  else simt_partial<T, GATE, 4>(p, ring, s_off0, s_off1, n0, c0, c1);
+  cluster_sync_all();  // every partial of the cluster is in shared memory
+  const int l0 = (int)rank * rows / S, l1 = ((int)rank + 1) * rows / S;  // this CTA's rows of the tile
+  const uint32_t P = smem_u32(ring);
   T* out = reinterpret_cast<T*>(p.out);
-  const int nrows = R < kRowsMax ? R : kRowsMax;
-  for (int g0 = 0; g0 < nrows; g0 += kRowGroup) {
-    const int gn = nrows - g0 < kRowGroup ? nrows - g0 : kRowGroup;
-    float av[kRowGroup], ag[kRowGroup];
+  for (int x = tid; x < (l1 - l0) * (F / 4); x += kNT) {
+    const int l = l0 + x / (F / 4), f = x % (F / 4) * 4;
+    const uint32_t at = P + (uint32_t)((l * TN + f) * 4);
+    float4 v[8], g[8];
 #pragma unroll
-    for (int q = 0; q < kRowGroup; ++q) av[q] = ag[q] = 0.f;
-    // v = W_v r and the r half of the gate, W_g[:, d:2d] r
-    const T* rs[kRowGroup];
-    const T* es[kRowGroup];
-#pragma unroll
-    for (int q = 0; q < kRowGroup; ++q) {  // rows past the group repeat its first (discarded)
-      const int row = g0 + (q < gn ? q : 0);
-      rs[q] = r + s_r[row];
-      es[q] = e + s_e[row];
-    }
-    for (int k0 = lane; k0 < d; k0 += 32 * kBatch) {
-      float wvk[kBatch], wgk[kBatch], x[kRowGroup][kBatch];
-#pragma unroll
-      for (int u = 0; u < kBatch; ++u) {
-        const int k = k0 + 32 * u;
-        wvk[u] = k < d ? to_f32(wv[k]) : 0.f;
-        wgk[u] = k < d ? to_f32(wg[d + k]) : 0.f;
-#pragma unroll
-        for (int q = 0; q < kRowGroup; ++q) x[q][u] = k < d ? to_f32(rs[q][k]) : 0.f;
-      }
-#pragma unroll
-      for (int q = 0; q < kRowGroup; ++q)
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
-          av[q] = fmaf(wvk[u], x[q][u], av[q]);
-          ag[q] = fmaf(wgk[u], x[q][u], ag[q]);
-        }
-    }
-    // per-position e: the e half of the gate, W_g[:, 0:d] e
-    if (p.e_dense) {
-      for (int k0 = lane; k0 < d; k0 += 32 * kBatch) {
-        float wk[kBatch], x[kRowGroup][kBatch];
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
-          const int k = k0 + 32 * u;
-          wk[u] = k < d ? to_f32(wg[k]) : 0.f;
-#pragma unroll
-          for (int q = 0; q < kRowGroup; ++q) x[q][u] = k < d ? to_f32(es[q][k]) : 0.f;
-        }
-#pragma unroll
-        for (int q = 0; q < kRowGroup; ++q)
-#pragma unroll
-          for (int u = 0; u < kBatch; ++u) ag[q] = fmaf(wk[u], x[q][u], ag[q]);
+    for (int s = 0; s < 8; ++s) {  // all loads first, then the sums in rank order
+      v[s] = g[s] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (s < S) {
+        const uint32_t src = map_rank(at, (uint32_t)s);
+        v[s] = ld_cluster_f4(src);
+        if constexpr (GATE) g[s] = ld_cluster_f4(src + 32 * 4);
       }
     }
 #pragma unroll
-    for (int q = 0; q < kRowGroup; ++q) {
-      av[q] = warp_sum(av[q]);
-      ag[q] = warp_sum(ag[q]);
+    for (int s = 1; s < 8; ++s) {
+      add4(v[0], v[s]);
+      if constexpr (GATE) add4(g[0], g[s]);
     }
-    if (lane < gn) {
-      float v = av[0], gs = ag[0];
+    const float vv[4] = {v[0].x, v[0].y, v[0].z, v[0].w}, gg[4] = {g[0].x, g[0].y, g[0].z, g[0].w};
+    const long long pos = (long long)s_b[l] * K + s_j[l];
+    const long long orow = (!GATE && p.compact) ? m0 + l : pos;
 #pragma unroll
-      for (int q = 1; q < kRowGroup; ++q)
-        if (lane == q) {
-          v = av[q];
-          gs = ag[q];
-        }
-      const int row = g0 + lane;
-      const long long orow = (long long)s_b[row] * K + s_j[row];
-      const float g = gs + (p.e_dense ? 0.f : p.ge[n]);
-      const float ev = to_f32(e[s_e[row] + n]);
-      const float gate = 1.f / (1.f + expf(-g));
-      out[orow * d + n] = from_f32<T>(ev + v * gate);
+    for (int q = 0; q < 4; ++q) {
+      const int n = n0 + f + q;
+      if (n >= d) break;
+      if constexpr (!GATE) {
+        const T m = reinterpret_cast<const T*>(p.a0)[s_off0[l] + n];
+        out[orow * d + n] = p.raw ? m : from_f32<T>(to_f32(m) + p.beta * vv[q]);
+      } else {
+        const float z = gg[q] + (p.e_dense ? 0.f : p.ge[n]);
+        const float ev = to_f32(e[s_off1[l] + n]);
+        const float gate = 1.f / (1.f + expf(-z));
+        out[orow * d + n] = from_f32<T>(ev + vv[q] * gate);
+      }
     }
   }
+  cluster_sync_all();  // no CTA leaves while the others read its shared memory
 }
 
-// ge[i] = sum_k W_g[i, k] e[k] over the e half (k < d), one warp per output.
+// ge = W_g[:, :d] e alone (a gate-only call), one warp per output.
 template <typename T>
 __global__ void __launch_bounds__(256) gate_bias_kernel(const T* __restrict__ Wg,
                                                         const T* __restrict__ e, int d,
                                                         float* __restrict__ ge) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i = blockIdx.x * 8 + warp;
+  const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (i >= d) return;
-  const T* w = Wg + (long long)i * 2 * d;
-  float s = 0.f;
-  for (int k = lane; k < d; k += 32) s = fmaf(to_f32(w[k]), to_f32(e[k]), s);
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, off);
-  if (lane == 0) ge[i] = s;
+  const float s = gate_bias_row<T>(Wg, e, i, d, threadIdx.x & 31);
+  if ((threadIdx.x & 31) == 0) ge[i] = s;
 }
 
 // One CTA per position (b, j): n_out[b], and rows j >= n_b of the zero / copy targets.
@@ -432,32 +366,78 @@ __global__ void __launch_bounds__(256) fill_rows_kernel(int B, int K, int d, Row
   }
 }
 
+// Launches a projection: one cluster of S CTAs per unit of the largest
+// possible R (those past the R found on the device leave at once) and, with
+// `gemv`, CTAs for W_g[:, :d] e behind them.  S: two CTAs per SM over the
+// units at three quarters of the possible rows, at most 8 and one chunk each.
+template <typename T, bool GATE>
+cudaError_t launch_simt(SimtParams& p, bool gemv, cudaStream_t stream) {
+  const long long rmax = (long long)p.B * (p.K - 1);
+  if (rmax <= 0) return cudaSuccess;
+  DeviceInfo info;
+  cudaError_t err = device_info(&info);
+  if (err != cudaSuccess) return err;
+  static std::atomic<int> attr_done[64];
+  if (!attr_done[info.device & 63].load(std::memory_order_acquire)) {
+    err = cudaFuncSetAttribute(simt_cluster_kernel<T, GATE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSimtSmem);
+    if (err != cudaSuccess) return err;
+    attr_done[info.device & 63].store(1, std::memory_order_release);
+  }
+  constexpr int F = GATE ? 32 : 64;
+  p.ftiles = (p.d + F - 1) / F;
+  const long long tiles = (3 * rmax / 4 + kTileRows) / kTileRows;
+  const int chunks = (p.d + TK - 1) / TK * (GATE ? (p.e_dense ? 2 : 1) : 2);
+  long long S = p.raw ? 1 : 2LL * info.sm_count / (p.ftiles * tiles);
+  S = std::min<long long>(std::min<long long>(S, 8), chunks);
+  p.S = S < 1 ? 1 : (int)S;
+  const long long clusters = (long long)p.ftiles * ((rmax + kTileRows - 1) / kTileRows);
+  const long long extra = gemv ? (p.d / 8 + p.S) / p.S : 0;  // clusters of the GEMV: about a warp per row
+  if ((clusters + extra) * p.S >= (1LL << 31)) return cudaErrorInvalidConfiguration;
+  p.clusters = (int)clusters;
+  const size_t es = sizeof(T);
+  auto al = [](const void* q) { return (uintptr_t)q % 16 == 0; };
+  p.vec = es == 4 && p.d % 4 == 0 && al(p.a0) && al(p.w) && (!GATE || al(p.wg)) && (!p.a1 || al(p.a1));
+  return launch_dependent(simt_cluster_kernel<T, GATE>, dim3((unsigned)((clusters + extra) * p.S)), dim3(kNT),
+                          (size_t)kSimtSmem, stream, (unsigned)p.S, p);
+}
+
 template <typename T>
 cudaError_t correct_typed(const CorrectArgs& a, cudaStream_t stream) {
-  SimtCorrectParams p{a.hD, a.hT, a.Wc, a.beta, a.B, a.K, a.d, a.rows, a.r_out, a.compact_out, a.raw};
-  const long long rmax = (long long)a.B * (a.K - 1);
-  if (rmax <= 0) return cudaSuccess;
-  if (rmax <= kRowsMax) {
-    simt_rows_correct_kernel<T><<<(unsigned)((a.d + kRowsWarps - 1) / kRowsWarps), kNT, 0, stream>>>(p);
-    return cudaGetLastError();
-  }
-  dim3 grid((unsigned)((rmax + TM - 1) / TM), (unsigned)((a.d + TN - 1) / TN));
-  simt_correct_kernel<T><<<grid, kNT, 0, stream>>>(p);
-  return cudaGetLastError();
+  SimtParams p{};
+  p.a0 = a.hD;
+  p.a1 = a.hT;
+  p.w = a.Wc;
+  p.wg = a.Wg;
+  p.e = a.e;
+  p.ge = a.ge;
+  p.beta = a.beta;
+  p.B = a.B;
+  p.K = a.K;
+  p.d = a.d;
+  p.rows = a.rows;
+  p.out = a.r_out;
+  p.compact = a.compact_out;
+  p.raw = a.raw;
+  return launch_simt<T, false>(p, a.ge != nullptr, stream);
 }
 
 template <typename T>
 cudaError_t gate_typed(const GateArgs& a, cudaStream_t stream) {
-  SimtGateParams p{a.e, a.e_dense, a.r, a.r_compact, a.Wv, a.Wg, a.ge, a.B, a.K, a.d, a.rows, a.e_out};
-  const long long rmax = (long long)a.B * (a.K - 1);
-  if (rmax <= 0) return cudaSuccess;
-  if (rmax <= kRowsMax) {
-    simt_rows_gate_kernel<T><<<(unsigned)((a.d + kRowsWarps - 1) / kRowsWarps), kNT, 0, stream>>>(p);
-    return cudaGetLastError();
-  }
-  dim3 grid((unsigned)((rmax + TM - 1) / TM), (unsigned)((a.d + TN - 1) / TN));
-  simt_gate_kernel<T><<<grid, kNT, 0, stream>>>(p);
-  return cudaGetLastError();
+  SimtParams p{};
+  p.a0 = a.r;
+  p.a1 = a.e_dense ? a.e : nullptr;
+  p.w = a.Wv;
+  p.wg = a.Wg;
+  p.e = a.e;
+  p.ge = const_cast<float*>(a.ge);
+  p.B = a.B;
+  p.K = a.K;
+  p.d = a.d;
+  p.rows = a.rows;
+  p.out = a.e_out;
+  p.compact = a.r_compact;
+  p.e_dense = a.e_dense;
+  return launch_simt<T, true>(p, false, stream);
 }
 
 }  // namespace

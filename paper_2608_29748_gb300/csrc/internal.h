@@ -264,6 +264,10 @@ struct CorrectArgs {
   void* r_out;        // compact [R, d] (compact_out) or [B, K, d]
   int compact_out;
   int raw;            // 1: r = m (no correction; W_c is not read)
+  // W_g[:, :d] e of the gate to come, by further CTAs (ge NULL: not computed)
+  const void* Wg;
+  const void* e;
+  float* ge;
 };
 cudaError_t launch_correct_simt(const CorrectArgs& a, retrace_dtype dtype, cudaStream_t stream);
 

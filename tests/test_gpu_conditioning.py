@@ -278,3 +278,43 @@ def test_small_r_rows(rt, B, K, d, R):
     e_full = np.broadcast_to(host_f64(x["e_vec"]), (B, K, d))
     want = oracle.gate_fuse(e_full, host_f64(r), n_host, host_f64(x["Wv"]), host_f64(x["Wg"]))
     assert_close(out, want, f"e~, R={R} d={d}")
+
+
+@pytest.mark.parametrize("dense_e", [False, True])
+@pytest.mark.parametrize("B,K,d,R,dtype", [
+    (5, 4, 33, 1, torch.float32),      # rows not 16-byte aligned: element copies
+    (9, 3, 36, 16, torch.float32),     # 16-byte copies, a last reduction chunk of 4
+    (9, 16, 100, 17, torch.float32),   # tiles of 16, 32, 48 and 64 rows on both sides of their edges
+    (9, 16, 68, 33, torch.float32),
+    (9, 16, 132, 49, torch.float32),
+    (9, 16, 64, 65, torch.float32),    # two row tiles of 48
+    (24, 16, 1000, 129, torch.float32),
+    (300, 3, 40, 300, torch.float32),  # more sequences than threads of a CTA
+    (9, 16, 65, 64, torch.bfloat16),   # bf16 with odd hidden sizes
+    (300, 2, 33, 257, torch.bfloat16),
+])
+def test_ffma_rows(rt, B, K, d, R, dtype, dense_e):
+    """Exactly R carried rows on the FFMA path: both calls against the oracle
+    and repeated bit for bit."""
+    x = make_inputs(B, K, d, dtype, seed=R + d, accept=accept_for_rows(B, K, R))
+    A = host_int(x["accept"])
+    n_host = oracle.carried_rows(A, K)
+    ws = rt.Workspace(B, K, 8, d, dtype)
+    e = x["e_dense"] if dense_e else x["e_vec"]
+    outs = []
+    for _ in range(2):
+        r = torch.full((B, K, d), 9.0, dtype=dtype, device="cuda")
+        n = torch.empty((B,), dtype=torch.int32, device="cuda")
+        rt.retrace_align_refine(x["hD"], x["hT"], x["accept"], x["Wc"], 0.5, r, n, ws)
+        out = torch.full((B, K, d), 7.0, dtype=dtype, device="cuda")
+        rt.retrace_gate_fuse(e, r, n, x["Wv"], x["Wg"], out, ws)
+        torch.cuda.synchronize()
+        outs.append((r, out))
+    assert ws.check() == 0
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
+    r, out = outs[0]
+    m, u = oracle.align(host_f64(x["hD"]), host_f64(x["hT"]), A)
+    assert_close(r, oracle.correct(m, u, host_f64(x["Wc"]), 0.5, round_r_bf16=False), f"r, R={R} d={d}")
+    want = oracle.gate_fuse(np.broadcast_to(host_f64(e), (B, K, d)), host_f64(r), n_host, host_f64(x["Wv"]),
+                            host_f64(x["Wg"]))
+    assert_close(out, want, f"e~, R={R} d={d}")
