@@ -25,19 +25,21 @@
 //        computed once by idle warps (W_g[:, :d] e, added in the epilogue)
 //        or, for per-position e, extra K blocks (Epack x W_g[:, :d])
 //        accumulated into the gate columns.
-//    Two kernels implement it:
-//    cond_pair_kernel   (broadcast e) clusters of two CTAs, 256-row tiles,
+//    Three kernels implement it:
+//    swap_cluster_kernel  (at most kSwapMaxRows possible rows; one launch per
+//                       projection instead) the weights as the M side;
+//    cond_pair_kernel   (more rows) clusters of two CTAs, 256-row tiles,
 //                       tcgen05.mma.cta_group::2 M256 N256 K16; each CTA
 //                       stages its own 128 rows and half of the weight tile
-//                       (described at the kernel);
-//    cond_kernel<false> (per-position e) one CTA per SM, 128-row tiles,
-//                       tcgen05.mma.cta_group::1 M128 N256 K16;
-//    cond_kernel<true>  the overlapped round: the same plus verification
-//                       streamed through shared memory (verify_stream.cuh).
+//                       (each described at the kernel);
+//    cond_overlap_kernel  the overlapped round: one CTA per SM, 128-row tiles,
+//                       tcgen05.mma.cta_group::1 M128 N256 K16, and
+//                       verification streamed through shared memory
+//                       (verify_stream.cuh).
 //
-// Warp roles of cond_kernel<false> (256 threads; the pair kernel's are alike):
+// Warp roles of the persistent kernels' GEMM part (256 threads):
 //   warp 0     tile scheduler + TMA producer (one elected lane);
-//   warp 1     MMA issuer (one lane): 4 x tcgen05.mma per 64-deep stage;
+//   warp 1     MMA issuer (one lane);
 //   warp 2     TMEM allocation: 2 accumulators x 256 fp32 columns = 512 columns;
 //   warps 2-3  the broadcast-e GEMV W_g[:, :d] e, rows claimed from a counter;
 //   warps 4-7  epilogue: tcgen05.ld of their 32 TMEM lanes (= tile rows).
@@ -56,14 +58,11 @@ namespace {
 
 constexpr int BM = 128;
 constexpr int BK = 64;  // 64 bf16 = 128 bytes = one swizzle row
-constexpr int STAGES = 4;
-constexpr int THREADS = 256;
-constexpr int THREADS_FUSED = 2 * THREADS + 32;  // + consumer warps 8-15 and the bookkeeper warp 16
+constexpr int THREADS_FUSED = 2 * 256 + 32;  // consumer warps 8-15 and the bookkeeper warp 16 beside the GEMM's eight
 constexpr int A_BYTES = BM * BK * 2;   // 16 KB
 constexpr int B_BYTES = 256 * BK * 2;  // 32 KB
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024;  // + slack for 1024-B alignment
-// The fused round kernel keeps three operand stages and gives the rest of the
+// The overlapped round's kernel keeps three operand stages and gives the rest of the
 // shared memory to the ring that streams the logits.
 constexpr int STAGES_FUSED = 3;
 constexpr int SMEM_BYTES_FUSED = STAGES_FUSED * STAGE_BYTES + kRingBufs * kChunkBytes + kStageBytes + 1024;
@@ -159,7 +158,7 @@ struct CondParams {
   __nv_bfloat16* e_out;
   uint32_t* sync;
   uint32_t* block_done;   // per 128-row block: correction epilogue warps finished
-  uint32_t* block_ready;  // per 128-row block: packed rows published (FUSED)
+  uint32_t* block_ready;  // per 128-row block: packed rows published (overlapped round)
   int max_blocks;         // 128-row blocks of the largest possible R
   // CTA-pair kernel: the gate tiles of a last wave of at most split_max
   // tiles run as two K halves on two pairs.  Each half writes its fp32
@@ -181,6 +180,8 @@ __device__ __forceinline__ void gate_bias_rows(const CondParams& p, int d, int l
 
 // Correction epilogue of one tile row (Eq. 7): r = m + beta * c for the 256
 // accumulator columns n0.., m = the first d columns of the packed row g.
+// GENERAL: d may end inside the tile (at a multiple of 8 columns).
+template <bool GENERAL>
 __device__ __forceinline__ void epilogue_correction(const CondParams& p, uint32_t taddr, int g, bool valid, int n0,
                                                     int d) {
   const __nv_bfloat16* mrow = p.apack + (long long)g * 2 * d;
@@ -194,6 +195,7 @@ __device__ __forceinline__ void epilogue_correction(const CondParams& p, uint32_
       uint4* ov = reinterpret_cast<uint4*>(p.r_out + orow * d + n);
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
+        if (GENERAL && n + v * 8 >= d) break;
         const uint4 mw = __ldcg(mv + v);
         const uint32_t mwords[4] = {mw.x, mw.y, mw.z, mw.w};
         uint32_t o[4];
@@ -215,6 +217,7 @@ __device__ __forceinline__ void epilogue_correction(const CondParams& p, uint32_
 // 32 values for every lane: one 16-byte broadcast load per four features).
 // With `other` (a split tile), the other K half's accumulator of this row is
 // added first: column c at other[128 c].
+template <bool GENERAL>
 __device__ __forceinline__ void epilogue_gate(const CondParams& p, uint32_t taddr, int g, bool valid, int n0, int d,
                                               const float* other = nullptr) {
   const long long orow = valid ? __ldcg(p.rowmap + g) : 0;
@@ -236,6 +239,7 @@ __device__ __forceinline__ void epilogue_gate(const CondParams& p, uint32_t tadd
         const float4* gb = reinterpret_cast<const float4*>(p.ge + n);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
+          if (GENERAL && n + 4 * j >= d) break;
           const float4 b = __ldcg(gb + j);
           gt[4 * j] += b.x;
           gt[4 * j + 1] += b.y;
@@ -247,6 +251,7 @@ __device__ __forceinline__ void epilogue_gate(const CondParams& p, uint32_t tadd
       uint4* ov = reinterpret_cast<uint4*>(p.e_out + orow * d + n);
 #pragma unroll
       for (int x = 0; x < 4; ++x) {
+        if (GENERAL && n + x * 8 >= d) break;
         const uint4 ew = __ldcg(ev + x);
         const uint32_t ewords[4] = {ew.x, ew.y, ew.z, ew.w};
         uint32_t o[4];
@@ -266,8 +271,7 @@ __device__ __forceinline__ void epilogue_gate(const CondParams& p, uint32_t tadd
 // T0 <= t < T0 + T1: gate tile (row block (t-T0) / nt1, 128 features).  Tiles
 // are handed out in this order by a global counter, so every gate tile's row
 // block was handed out (to a running CTA) before it.
-// FUSED: the same kernel also runs verification (verify_stream.cuh): warp 3
-// streams the logits into a shared-memory ring, warps 8-15 reduce it, warp 16 folds the keys.  Packed rows then become available while the
+// The kernel also runs verification (verify_stream.cuh): warp 3 streams the logits into a shared-memory ring, warps 8-15 reduce it, warp 16 folds the keys.  Packed rows then become available while the
 // kernel runs, so the tile queue is decoded in phases -- phase q holds the
 // correction tiles of row block q followed by the gate tiles of row block
 // q - kGateLag -- and the producer resolves each tile against the published
@@ -275,34 +279,28 @@ __device__ __forceinline__ void epilogue_gate(const CondParams& p, uint32_t tadd
 // known once every sequence is finalised.
 constexpr int kGateLag = 4;
 
-template <bool FUSED>
-__global__ void __launch_bounds__(FUSED ? THREADS_FUSED : THREADS, 1)
-    cond_kernel(const __grid_constant__ CUtensorMap tmApack, const __grid_constant__ CUtensorMap tmWc,
+__global__ void __launch_bounds__(THREADS_FUSED, 1)
+    cond_overlap_kernel(const __grid_constant__ CUtensorMap tmApack, const __grid_constant__ CUtensorMap tmWc,
                 const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmE,
                 const __grid_constant__ CUtensorMap tmWv, const __grid_constant__ CUtensorMap tmWg,
                 const CondParams p, const VerifyStreamParams vp) {
   extern __shared__ uint8_t dsmem[];
-  __shared__ __align__(8) uint64_t bar_full[STAGES];
-  __shared__ __align__(8) uint64_t bar_empty[STAGES];
+  __shared__ __align__(8) uint64_t bar_full[STAGES_FUSED];
+  __shared__ __align__(8) uint64_t bar_empty[STAGES_FUSED];
   __shared__ __align__(8) uint64_t bar_tfull[2];
   __shared__ __align__(8) uint64_t bar_tempty[2];
   __shared__ __align__(8) uint64_t bar_tile_full[TILE_SLOTS];
   __shared__ __align__(8) uint64_t bar_tile_empty[TILE_SLOTS];
   __shared__ int s_tile[TILE_SLOTS];
-  __shared__ int s_rows[TILE_SLOTS];  // valid rows of the tile (FUSED)
+  __shared__ int s_rows[TILE_SLOTS];  // valid rows of the tile
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_abort;
   __shared__ VerifyStreamSmem vsm;
 
-  constexpr int NST = FUSED ? STAGES_FUSED : STAGES;
+  constexpr int NST = STAGES_FUSED;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int d = p.d;
   const int nt0 = d / 256, nt1 = d / 128;
-  const int R = FUSED ? 0 : *(volatile const int32_t*)p.R;
-  const int tiles_m = (R + BM - 1) / BM;
-  const int T0 = FUSED ? 0 : (p.do_correct ? tiles_m * nt0 : 0);
-  const int T = FUSED ? 0 : T0 + (p.do_gate ? tiles_m * nt1 : 0);
-  if (!FUSED && T == 0) return;  // nothing to condition
   uint32_t* tile_queue = p.sync + kSyncTileQueue;
   uint32_t* gemv_next = p.sync + kSyncGemvNext;
   uint32_t* gemv_done = p.sync + kSyncGemvDone;
@@ -323,7 +321,7 @@ __global__ void __launch_bounds__(FUSED ? THREADS_FUSED : THREADS, 1)
       mbar_init(smem_u32(&bar_tile_full[a]), 1);
       mbar_init(smem_u32(&bar_tile_empty[a]), 5);  // MMA thread + four epilogue warps
     }
-    if constexpr (FUSED) vs_init(vsm);
+    vs_init(vsm);
     fence_mbar_init();
   }
   if (warp == 0 && lane == 0) {
@@ -358,14 +356,7 @@ __global__ void __launch_bounds__(FUSED ? THREADS_FUSED : THREADS, 1)
         const uint32_t slot = lt % TILE_SLOTS, sph = (lt / TILE_SLOTS) & 1u;
         int t, rows = BM, m0, n0;
         bool corr, done = false;
-        if (!FUSED) {
-          t = (int)atomicAdd(tile_queue, 1u);
-          done = t >= T;
-          corr = t < T0;
-          const int tt = corr ? t : t - T0;
-          m0 = (corr ? tt / nt0 : tt / nt1) * BM;
-          n0 = corr ? (tt % nt0) * 256 : (tt % nt1) * 128;
-        } else {
+        {
           // next valid tile of the phased queue
           for (;;) {
             t = (int)atomicAdd(tile_queue, 1u);
@@ -483,7 +474,7 @@ __global__ void __launch_bounds__(FUSED ? THREADS_FUSED : THREADS, 1)
         const int t = s_tile[slot];
         mbar_arrive(smem_u32(&bar_tile_empty[slot]));
         if (t < 0) break;
-        const bool corr = FUSED ? (t % (nt0 + nt1)) < nt0 : t < T0;
+        const bool corr = (t % (nt0 + nt1)) < nt0;
         const int nkb = corr ? 2 * kb_half : kb_half + (p.e_dense ? kb_half : 0);
         const uint32_t acc = lt & 1u, aph = (lt >> 1) & 1u;
         if (!mbar_wait_bounded(smem_u32(&bar_tempty[acc]), aph ^ 1u, &s_abort)) {
@@ -519,33 +510,28 @@ __global__ void __launch_bounds__(FUSED ? THREADS_FUSED : THREADS, 1)
       if (!ok) raise_abort(&s_abort, p.status);
     }
     __syncwarp();
-  } else if (FUSED && warp == 3) {
+  } else if (warp == 3) {
     // ---------------- logits stream into the verification ring ----------------
     if (lane == 0) vs_producer(vp, vsm, base + NST * STAGE_BYTES, &s_abort);
     __syncwarp();
-  } else if (FUSED && warp == 2) {
+  } else if (warp == 2) {
     // ---------------- sequence finaliser (bulk copies through staging) ----------------
     vs_finalizer(vp, vsm, base + NST * STAGE_BYTES + kRingBufs * kChunkBytes, blockIdx.x, gridDim.x, lane, &s_abort);
-  } else if (warp == 2 || warp == 3) {
-    // ---------------- W_g[:, :d] e for a broadcast e (idle warps) ----------------
-    if (need_ge) gate_bias_rows(p, d, lane, gemv_next, gemv_done);
   } else if (warp >= 16) {
-    // ---------------- verification bookkeeping (FUSED only) ----------------
-    if constexpr (FUSED)
-      if (lane == 0) vs_bookkeeper(vp, vsm, &s_abort);
+    // ---------------- verification bookkeeping ----------------
+    if (lane == 0) vs_bookkeeper(vp, vsm, &s_abort);
     __syncwarp();
   } else if (warp >= 8) {
-    // ---------------- verification (FUSED only: warps 8-15) ----------------
-    if constexpr (FUSED)
-      vs_consumer(vp, vsm, reinterpret_cast<const uint4*>(dsmem + (base + NST * STAGE_BYTES - smem_u32(dsmem))),
-                  warp - 8, lane, &s_abort);
+    // ---------------- verification (warps 8-15) ----------------
+    vs_consumer(vp, vsm, reinterpret_cast<const uint4*>(dsmem + (base + NST * STAGE_BYTES - smem_u32(dsmem))), warp - 8,
+                lane, &s_abort);
   } else if (warp >= 4) {
     // ---------------- epilogue ----------------
     const int q = (warp - 4) * 32 + lane;  // tile row = TMEM lane
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-    // In the fused kernel the epilogue warps have nothing to do until the
-    // first rows are packed: they compute W_g[:, :d] e meanwhile.
-    if (FUSED && need_ge) gate_bias_rows(p, d, lane, gemv_next, gemv_done);
+    // The epilogue warps have nothing to do until the first rows are packed:
+    // they compute W_g[:, :d] e meanwhile.
+    if (need_ge) gate_bias_rows(p, d, lane, gemv_next, gemv_done);
     bool have_ge = !need_ge;
     for (uint32_t lt = 0;; ++lt) {
       const uint32_t slot = lt % TILE_SLOTS, sph = (lt / TILE_SLOTS) & 1u;
@@ -561,17 +547,10 @@ __global__ void __launch_bounds__(FUSED ? THREADS_FUSED : THREADS, 1)
       if (t < 0) break;
       bool corr;
       int m0, n0;
-      if (FUSED) {
-        const int q2 = t / (nt0 + nt1), r = t % (nt0 + nt1);
-        corr = r < nt0;
-        m0 = (corr ? q2 : q2 - kGateLag) * BM;
-        n0 = corr ? r * 256 : (r - nt0) * 128;
-      } else {
-        corr = t < T0;
-        const int tt = corr ? t : t - T0;
-        m0 = (corr ? tt / nt0 : tt / nt1) * BM;
-        n0 = corr ? (tt % nt0) * 256 : (tt % nt1) * 128;
-      }
+      const int q2 = t / (nt0 + nt1), r2 = t % (nt0 + nt1);
+      corr = r2 < nt0;
+      m0 = (corr ? q2 : q2 - kGateLag) * BM;
+      n0 = corr ? r2 * 256 : (r2 - nt0) * 128;
       const uint32_t acc = lt & 1u, aph = (lt >> 1) & 1u;
       ok = warp_wait(smem_u32(&bar_tfull[acc]), aph, &s_abort);
       tc_fence_after();
@@ -591,10 +570,10 @@ __global__ void __launch_bounds__(FUSED ? THREADS_FUSED : THREADS, 1)
         have_ge = true;
       }
       const int g = m0 + q;
-      const bool valid = FUSED ? q < tile_rows : g < R;
+      const bool valid = q < tile_rows;
       const uint32_t taddr = tmem + acc * ACC_COLS + lane_base;
       if (corr) {
-        epilogue_correction(p, taddr, g, valid, n0, d);
+        epilogue_correction<false>(p, taddr, g, valid, n0, d);
         if (p.do_gate) {
           // Publish this warp's 32 rows of the (row block, column block) of r
           // to the gate tiles: one count per epilogue warp, no wait.
@@ -604,14 +583,12 @@ __global__ void __launch_bounds__(FUSED ? THREADS_FUSED : THREADS, 1)
           if (lane == 0) atomicAdd(block_done + m0 / BM, 1u);
         }
       } else {
-        epilogue_gate(p, taddr, g, valid, n0, d);
+        epilogue_gate<false>(p, taddr, g, valid, n0, d);
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&bar_tempty[acc]));
     }
-    // out of tiles: help finish W_g[:, :d] e (the rows left on the counter)
-    if (!FUSED && need_ge && !s_abort) gate_bias_rows(p, d, lane, gemv_next, gemv_done);
   }
   // ---------------- teardown ----------------
   tc_fence_before();
@@ -625,8 +602,7 @@ __global__ void __launch_bounds__(FUSED ? THREADS_FUSED : THREADS, 1)
 // ---------------------------------------------------------------------------
 // CTA-pair projections: tcgen05.mma.cta_group::2, M = 256 over two SMs
 // ---------------------------------------------------------------------------
-// The same tiles as cond_kernel<false> with twice the rows: a cluster of two
-// CTAs takes a 256-row pair tile, each CTA staging its own 128 rows of A and
+// A cluster of two CTAs takes a 256-row pair tile, each CTA staging its own 128 rows of A and
 // half of the N = 256 weight tile (correction: W_c rows n0.. and n0+128..;
 // gate: the W_v rows in the leader, the matching W_g[:, d:2d] rows in the
 // follower).  A stage is 128 deep in K (two 64-element swizzle boxes per
@@ -641,7 +617,9 @@ __global__ void __launch_bounds__(FUSED ? THREADS_FUSED : THREADS, 1)
 // barriers (multicast).  Stage-full barriers live in the leader and count the
 // bytes of both CTAs' copies.  The leader takes tiles from the global queue
 // and hands each to the follower through the follower's shared memory.  A
-// broadcast e only (per-position e takes cond_kernel).  Every wait is bounded.
+// per-position e adds k-blocks to the gate tiles: e rows against W_g[:, :d],
+// accumulated into the gate's 128 columns (M256 N128 MMAs).  Every wait is
+// bounded.
 constexpr int PSTAGES = 3;
 constexpr int P_THREADS = 256;
 constexpr int PBK = 2 * BK;                      // k-block depth of a stage: two swizzle boxes
@@ -651,6 +629,7 @@ constexpr int P_B_BYTES = 2 * P_BOX_BYTES;       // 32 KB: this CTA's half of th
 constexpr int P_STAGE_BYTES = P_A_BYTES + P_B_BYTES;
 constexpr int P_SMEM_BYTES = PSTAGES * P_STAGE_BYTES + 1024;  // + slack for 1024-B alignment
 constexpr uint32_t IDESC_M256_N256 = idesc_bf16_f32(256, 256);
+constexpr uint32_t IDESC_M256_N128 = idesc_bf16_f32(256, 128);
 // Pair blocks (256 packed rows) per group of the tile order: inside a group
 // the weight tile is the outer index, so the pairs that start together share
 // weight tiles as well as row blocks (measured: 260 against 264 us for
@@ -658,10 +637,15 @@ constexpr uint32_t IDESC_M256_N256 = idesc_bf16_f32(256, 256);
 constexpr int kGroupBlocks = 4;
 constexpr int P_TILE_SLOTS = 3;  // tile indices in flight: the leader publishes one tile ahead
 
+// GENERAL = false: d a multiple of 256, where every tile is whole, and a broadcast e.  With the
+// checks of the general form in its epilogue and MMA loop the kernel took
+// 285 instead of 241 us at B = 256 (d = 4096).
+template <bool GENERAL>
 __global__ void __launch_bounds__(P_THREADS, 1)
     cond_pair_kernel(const __grid_constant__ CUtensorMap tmApack, const __grid_constant__ CUtensorMap tmWc,
                      const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmWv,
-                     const __grid_constant__ CUtensorMap tmWg, const CondParams p) {
+                     const __grid_constant__ CUtensorMap tmWg, const __grid_constant__ CUtensorMap tmE,
+                     const __grid_constant__ CUtensorMap tmWge, const CondParams p) {
   extern __shared__ uint8_t dsmem[];
   __shared__ __align__(8) uint64_t bar_full[PSTAGES];             // leader: both CTAs' bytes of a stage
   __shared__ __align__(8) uint64_t bar_empty[PSTAGES];            // stage free (leader's commit, both CTAs)
@@ -676,13 +660,13 @@ __global__ void __launch_bounds__(P_THREADS, 1)
   const uint32_t rank = cluster_rank();
   const bool leader = rank == 0;  // issues the pair's MMAs and runs the tile queue
   const int d = p.d;
-  const int nt0 = d / 256, nt1 = d / 128;
+  const int nt0 = GENERAL ? (d + 255) / 256 : d / 256, nt1 = GENERAL ? (d + 127) / 128 : d / 128;
   pdl_launch_dependents();
   uint32_t* tile_queue = p.sync + kSyncTileQueue;
   uint32_t* gemv_next = p.sync + kSyncGemvNext;
   uint32_t* gemv_done = p.sync + kSyncGemvDone;
   uint32_t* block_done = p.block_done;
-  const bool need_ge = p.do_gate;  // broadcast e
+  const bool need_ge = p.do_gate && !(GENERAL && p.e_dense);
 
   if (tid == 0) {
     s_abort = 0;
@@ -709,6 +693,10 @@ __global__ void __launch_bounds__(P_THREADS, 1)
       tma_prefetch_desc(&tmR);
       tma_prefetch_desc(&tmWv);
       tma_prefetch_desc(&tmWg);
+      if (GENERAL && p.e_dense) {
+        tma_prefetch_desc(&tmE);
+        tma_prefetch_desc(&tmWge);
+      }
     }
   }
   if (warp == 2) {
@@ -721,7 +709,10 @@ __global__ void __launch_bounds__(P_THREADS, 1)
   tc_fence_after();
   const uint32_t tmem = s_tmem;
   const uint32_t base = (smem_u32(dsmem) + 1023u) & ~1023u;
-  const int kb_half = d / PBK;
+  // k-blocks of the correction (over [m; u], 2d long) and of the gate.  Past the
+  // operands' ends (GENERAL) the copies fill zeros.
+  const int nkb_g = GENERAL ? (d + PBK - 1) / PBK : d / PBK;
+  const int nkb_c = GENERAL ? (2 * d + PBK - 1) / PBK : 2 * nkb_g;
   // The set-up above may overlap the end of the previous kernel (programmatic
   // dependent launch).  R, the packed rows and the row map are its outputs:
   // every role that reads them waits here first.  The gate-bias GEMV (warps
@@ -737,7 +728,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
     // the last wave: work units (a gate tile's worth of MMAs) beyond the
     // whole waves of the pairs
     const int last_wave = (2 * T0 + T1) % (int)(gridDim.x / 2);
-    X = last_wave <= p.split_max ? min(last_wave, T1) : 0;
+    X = last_wave <= p.split_max && (!GENERAL || nkb_g > 1) ? min(last_wave, T1) : 0;
     T = T0 + T1 + X;
   }
   // Tile t: correction tiles first, then gate tiles; within each kind, groups
@@ -762,7 +753,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
     x.corr = t < T0;
     int tt = x.corr ? t : t - T0;
     x.kb0 = 0;
-    x.nkb = x.corr ? 2 * kb_half : kb_half;
+    x.nkb = x.corr ? nkb_c : (GENERAL && p.e_dense) ? 2 * nkb_g : nkb_g;
     x.split = -1;
     x.half = 0;
     if (!x.corr && tt >= T1 - X) {
@@ -770,8 +761,8 @@ __global__ void __launch_bounds__(P_THREADS, 1)
       x.split = j >> 1;
       x.half = j & 1;
       tt = T1 - X + x.split;
-      x.nkb = kb_half / 2;
-      x.kb0 = x.half * x.nkb;
+      x.kb0 = x.half ? nkb_g / 2 : 0;
+      x.nkb = x.half ? nkb_g - nkb_g / 2 : nkb_g / 2;
     }
     const int nt = x.corr ? nt0 : nt1;
     const int g = tt / (kGroupBlocks * nt), w = tt - g * kGroupBlocks * nt;
@@ -848,6 +839,18 @@ __global__ void __launch_bounds__(P_THREADS, 1)
           }
           const uint32_t a_dst = base + s * P_STAGE_BYTES, b_dst = a_dst + P_A_BYTES;
           const uint32_t full = leader_addr(&bar_full[s]);
+          if (GENERAL && !corr && kb >= nkb_g) {
+            // per-position e: the gate's e half, e rows against 128 rows of
+            // W_g[:, :d], 64 in each CTA
+            if (leader) mbar_arrive_expect_tx(smem_u32(&bar_full[s]), 2 * (P_A_BYTES + P_B_BYTES / 2));
+            const int xe = (kb - nkb_g) * PBK;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              tma_load_2d_pair(a_dst + (uint32_t)h * P_BOX_BYTES, &tmE, xe + h * BK, m0, full);
+              tma_load_2d_pair(b_dst + (uint32_t)h * P_BOX_BYTES, &tmWge, xe + h * BK, n0 + (int)rank * 64, full);
+            }
+            continue;
+          }
           if (leader) mbar_arrive_expect_tx(smem_u32(&bar_full[s]), 2 * P_STAGE_BYTES);  // both CTAs' bytes
           // [m; u] or r rows; this CTA's half of the weight tile: W_c rows n0..
           // (leader) or n0 + 128.. (follower), or the W_v rows (leader) and the
@@ -889,7 +892,9 @@ __global__ void __launch_bounds__(P_THREADS, 1)
         const int t = s_tile[slot];
         mbar_arrive(smem_u32(&bar_tile_empty[slot]));
         if (t < 0) break;
-        const int nkb = decode(t).nkb;
+        const Tile x = decode(t);
+        const int nkb = x.nkb;
+        const int nkb_full = GENERAL && !x.corr ? min(nkb, nkb_g) : nkb;  // the others: the gate's e half
         const uint32_t acc = lt & 1u, aph = (lt >> 1) & 1u;
         if (!mbar_wait_cluster_bounded(smem_u32(&bar_tempty[acc]), aph ^ 1u, &s_abort)) {
           ok = false;
@@ -912,7 +917,10 @@ __global__ void __launch_bounds__(P_THREADS, 1)
 #pragma unroll
           for (int k = 0; k < PBK / 16; ++k) {
             const uint64_t step = (uint64_t)((k / (BK / 16)) * (P_BOX_BYTES >> 4) + 2 * (k % (BK / 16)));
-            tc_mma_pair(d_tmem, adesc0 + step, bdesc0 + step, IDESC_M256_N256, (kb > 0 || k > 0) ? 1u : 0u);
+            if (!GENERAL || kb < nkb_full)
+              tc_mma_pair(d_tmem, adesc0 + step, bdesc0 + step, IDESC_M256_N256, (kb > 0 || k > 0) ? 1u : 0u);
+            else  // into the gate's columns only
+              tc_mma_pair(d_tmem + 128u, adesc0 + step, bdesc0 + step, IDESC_M256_N128, 1u);
           }
           tc_commit_pair(smem_u32(&bar_empty[s]));  // stage free in both CTAs
         }
@@ -969,7 +977,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
       const bool valid = g < R;
       const uint32_t taddr = tmem + acc * ACC_COLS + lane_base;
       if (corr) {
-        epilogue_correction(p, taddr, g, valid, n0, d);
+        epilogue_correction<GENERAL>(p, taddr, g, valid, n0, d);
         if (p.do_gate) {
           __threadfence();
           fence_proxy_async_global();
@@ -977,7 +985,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
           if (lane == 0) atomicAdd(block_done + m0 / BM, 1u);
         }
       } else if (x.split < 0) {
-        epilogue_gate(p, taddr, g, valid, n0, d);
+        epilogue_gate<GENERAL>(p, taddr, g, valid, n0, d);
       } else {
         // A K half: this row's accumulator goes to the half's slot ([column][row]
         // per CTA, so that a warp's stores are contiguous); the warp that counts
@@ -1002,7 +1010,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
         }
         before = __shfl_sync(0xFFFFFFFFu, before, 0);
         __syncwarp();
-        if (before == 1u) epilogue_gate(p, taddr, g, valid, n0, d, other);
+        if (before == 1u) epilogue_gate<GENERAL>(p, taddr, g, valid, n0, d, other);
       }
       tc_fence_before();
       __syncwarp();
@@ -1064,8 +1072,9 @@ __global__ void wait_selftest_kernel(int kind, const uint32_t* flag, uint32_t ta
 // epilogue: r = m + beta c (Eq. 7) for the correction tiles of W_c, or the
 // gated fusion e~ = e + v sigmoid(g_r + W_g[:, :d] e) (Eq. 8) for the gate
 // tiles, whose 128 weight rows stack 64 rows of W_v over the same 64 rows of
-// W_g[:, d:2d] (v and g_r of a feature in TMEM lanes f and 64 + f).  Nothing
-// goes through global partials and no reduction kernel follows.  The partial
+// W_g[:, d:2d] (v and g_r of a feature in TMEM lanes f and 64 + f); with a
+// per-position e further k-blocks add W_g[:, :d] e to the gate's lanes, their
+// W_v half filled with zeros by the copy.  Nothing goes through global partials and no reduction kernel follows.  The partial
 // is stored row-major ([row][feature]) so that both the TMEM drain and the
 // cluster's reads move whole 128- and 256-byte rows.
 //
@@ -1128,6 +1137,7 @@ struct SwapClusterParams {
   int d;
   int mtiles;  // weight tiles
   int nkb;     // 64-deep k-blocks of the GEMM
+  int nkb_r;   // those over the rows operand tmB; the others (gate, per-position e) are over tmE
   int S;       // K splits = cluster size
   int gate;    // 0: correction tiles of W_c (128 features); 1: stacked [W_v; W_g,r] tiles (64 features)
   int stage_bytes;  // shared memory of the pipeline stages
@@ -1140,7 +1150,8 @@ struct SwapClusterParams {
   __nv_bfloat16* r_out;
   int compact_out;
   GateBiasParams bias;  // correction: W_g[:, :d] e of the gate to come (ge NULL: not computed)
-  // gate epilogue (broadcast e; ge = W_g[:, :d] e, complete before this launch)
+  // gate epilogue.  Broadcast e: [d], and ge = W_g[:, :d] e, complete before
+  // this launch.  Per-position e (ge NULL): packed rows [R, d].
   const __nv_bfloat16* e;
   const float* ge;
   __nv_bfloat16* e_out;
@@ -1165,6 +1176,7 @@ __device__ __forceinline__ void swap_correction_rows(const SwapClusterParams& p,
     uint32_t at[NB];
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
+      // (features past d, in the last tile: d + 127 < 2 d keeps their loads inside the packed rows)
       const int x = min(x0 + q * SW_THREADS, total - 1), l = l0 + x / 32, f = (x % 32) * 4, g = row0 + l;
       mw[q] = __ldcg(reinterpret_cast<const uint2*>(p.apack + (long long)g * 2 * d + n0 + f));
       orow[q] = p.compact_out ? g : __ldcg(p.rowmap + g);
@@ -1186,7 +1198,7 @@ __device__ __forceinline__ void swap_correction_rows(const SwapClusterParams& p,
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
       const int x = x0 + q * SW_THREADS;
-      if (x < total)
+      if (x < total && n0 + (x % 32) * 4 < d)
         *reinterpret_cast<uint2*>(p.r_out + orow[q] * d + n0 + (x % 32) * 4) =
             make_uint2(pack_bf16x2(bf16_lo(mw[q].x) + p.beta * c[q].x, bf16_hi(mw[q].x) + p.beta * c[q].y),
                        pack_bf16x2(bf16_lo(mw[q].y) + p.beta * c[q].z, bf16_hi(mw[q].y) + p.beta * c[q].w));
@@ -1198,8 +1210,15 @@ __device__ __forceinline__ void swap_gate_rows(const SwapClusterParams& p, uint3
                                                int total) {
   const int d = p.d, S = p.S;
   const int f = ((int)threadIdx.x % 16) * 4, n = mt * 64 + f;  // the same features at every step
-  const float4 gb = __ldcg(reinterpret_cast<const float4*>(p.ge + n));
-  const uint2 ew = __ldg(reinterpret_cast<const uint2*>(p.e + n));
+  if (n >= d) return;  // past the last feature (no barrier below)
+  float4 gb = make_float4(0.f, 0.f, 0.f, 0.f);
+  uint2 ew[NB];
+  if (p.ge) {
+    gb = __ldcg(reinterpret_cast<const float4*>(p.ge + n));
+    ew[0] = __ldg(reinterpret_cast<const uint2*>(p.e + n));
+#pragma unroll
+    for (int q = 1; q < NB; ++q) ew[q] = ew[0];
+  }
   for (int x0 = threadIdx.x; x0 < total; x0 += NB * SW_THREADS) {
     float4 v[NB], a[NB];
     long long orow[NB];
@@ -1208,6 +1227,7 @@ __device__ __forceinline__ void swap_gate_rows(const SwapClusterParams& p, uint3
     for (int q = 0; q < NB; ++q) {
       const int l = l0 + min(x0 + q * SW_THREADS, total - 1) / 16;
       orow[q] = __ldcg(p.rowmap + row0 + l);
+      if (!p.ge) ew[q] = __ldcg(reinterpret_cast<const uint2*>(p.e + (long long)(row0 + l) * d + n));
       at[q] = P + (uint32_t)(l * 512 + f * 4);
       v[q] = a[q] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
@@ -1236,15 +1256,16 @@ __device__ __forceinline__ void swap_gate_rows(const SwapClusterParams& p, uint3
       const float s0 = fast_sigmoid(a[q].x + gb.x), s1 = fast_sigmoid(a[q].y + gb.y);
       const float s2 = fast_sigmoid(a[q].z + gb.z), s3 = fast_sigmoid(a[q].w + gb.w);
       *reinterpret_cast<uint2*>(p.e_out + orow[q] * d + n) =
-          make_uint2(pack_bf16x2(bf16_lo(ew.x) + v[q].x * s0, bf16_hi(ew.x) + v[q].y * s1),
-                     pack_bf16x2(bf16_lo(ew.y) + v[q].z * s2, bf16_hi(ew.y) + v[q].w * s3));
+          make_uint2(pack_bf16x2(bf16_lo(ew[q].x) + v[q].x * s0, bf16_hi(ew[q].x) + v[q].y * s1),
+                     pack_bf16x2(bf16_lo(ew[q].y) + v[q].z * s2, bf16_hi(ew[q].y) + v[q].w * s3));
     }
   }
 }
 
 __global__ void __launch_bounds__(SW_THREADS, 1)
     swap_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA2,
-                        const __grid_constant__ RowMaps tmB, const SwapClusterParams p) {
+                        const __grid_constant__ CUtensorMap tmA3, const __grid_constant__ RowMaps tmB,
+                        const __grid_constant__ RowMaps tmE, const SwapClusterParams p) {
   extern __shared__ uint8_t dsmem[];
   __shared__ __align__(8) uint64_t bar_full[SW_STAGES];
   __shared__ __align__(8) uint64_t bar_empty[SW_STAGES];
@@ -1269,7 +1290,10 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
     tma_prefetch_desc(&tmA);
     tma_prefetch_desc(&tmA2);
   }
-  if (warp == 1 && lane < p.row_maps) tma_prefetch_desc(&tmB.m[lane]);
+  if (warp == 1 && lane < p.row_maps) {
+    tma_prefetch_desc(&tmB.m[lane]);
+    if (p.nkb > p.nkb_r) tma_prefetch_desc(&tmE.m[lane]);
+  }
   if (warp == 2) {
     tmem_alloc(smem_u32(&s_tmem), p.tmem_cols);
     tmem_relinquish();
@@ -1286,7 +1310,11 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
   auto load_a = [&](int mt, int kb, uint32_t s) {
     const uint32_t a_dst = base + s * (uint32_t)SW_A_BYTES, bar = smem_u32(&bar_full[s]);
     mbar_arrive_expect_tx(bar, (uint32_t)SW_A_BYTES);
-    if (p.gate) {  // rows 0-63: W_v rows f0..; rows 64-127: the same rows of W_g[:, d:2d]
+    if (kb >= p.nkb_r) {
+      // the gate's e half: zeros (columns past W_v's end) over the rows of W_g[:, :d]
+      tma_load_2d(a_dst, &tmA, p.nkb_r * BK, mt * 64, bar);
+      tma_load_2d(a_dst + (uint32_t)(SW_A_BYTES / 2), &tmA3, (kb - p.nkb_r) * BK, mt * 64, bar);
+    } else if (p.gate) {  // rows 0-63: W_v rows f0..; rows 64-127: the same rows of W_g[:, d:2d]
       tma_load_2d(a_dst, &tmA, kb * BK, mt * 64, bar);
       tma_load_2d(a_dst + (uint32_t)(SW_A_BYTES / 2), &tmA2, d + kb * BK, mt * 64, bar);
     } else {
@@ -1313,6 +1341,7 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
   const uint32_t b_bytes = (uint32_t)(box * BK * 2);
   const uint32_t b_base = base + (uint32_t)nst * (uint32_t)SW_A_BYTES;
   const CUtensorMap* mb = &tmB.m[box > 0 ? box / SW_ROW_STEP - 1 : 0];
+  const CUtensorMap* me = &tmE.m[box > 0 ? box / SW_ROW_STEP - 1 : 0];
 
   if (cid >= units && warp == 0 && lane == 0) {  // (always so with R = 0)
     // no unit: let the copies issued above land before the CTA leaves
@@ -1346,7 +1375,9 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
             load_a(mt, kb0 + i, s);
           }
           mbar_arrive_expect_tx(smem_u32(&bar_full[s]), b_bytes);
-          tma_load_2d(b_base + s * b_bytes, mb, (kb0 + i) * BK, row0, smem_u32(&bar_full[s]));
+          const int kb = kb0 + i;
+          if (kb < p.nkb_r) tma_load_2d(b_base + s * b_bytes, mb, kb * BK, row0, smem_u32(&bar_full[s]));
+          else tma_load_2d(b_base + s * b_bytes, me, (kb - p.nkb_r) * BK, row0, smem_u32(&bar_full[s]));
         }
         if (i < kb1 - kb0) {
           // a wait expired: flag it, let the copies in flight land
@@ -1444,21 +1475,6 @@ __global__ void __launch_bounds__(256) swap_gemv_kernel(const GateBiasParams p) 
   if (blockIdx.x == 0) pdl_wait();
 }
 
-template <bool FUSED>
-cudaError_t ensure_smem_attr() {
-  static std::atomic<int> done[64];
-  int dev = 0;
-  cudaError_t err = cudaGetDevice(&dev);
-  if (err != cudaSuccess) return err;
-  if (!done[dev & 63].load(std::memory_order_acquire)) {
-    err = cudaFuncSetAttribute(cond_kernel<FUSED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               FUSED ? SMEM_BYTES_FUSED : SMEM_BYTES);
-    if (err != cudaSuccess) return err;
-    done[dev & 63].store(1, std::memory_order_release);
-  }
-  return cudaSuccess;
-}
-
 }  // namespace
 
 cudaError_t launch_wait_selftest(int kind, const uint32_t* flag, uint32_t target, uint32_t* status,
@@ -1468,7 +1484,7 @@ cudaError_t launch_wait_selftest(int kind, const uint32_t* flag, uint32_t target
 }
 
 bool tc_supported(retrace_dtype dtype, int d) {
-  return dtype == RETRACE_BF16 && d >= 256 && d % 256 == 0;
+  return dtype == RETRACE_BF16 && d >= 128 && d % 8 == 0;
 }
 
 cudaError_t launch_pack(const PackArgs& a, cudaStream_t stream) {
@@ -1494,18 +1510,21 @@ cudaError_t launch_pack(const PackArgs& a, cudaStream_t stream) {
 static cudaError_t launch_cond_pair(const TcCondArgs& a, int clusters, cudaStream_t stream) {
   const long long rmax = (long long)a.B * (a.K - 1);
   const uint64_t d = (uint64_t)a.d;
-  CUtensorMap mApack, mWc, mR, mWv, mWg;
+  CUtensorMap mApack, mWc, mR, mWv, mWg, mE, mWge;
   // Maps of operands a call does not use point at a used buffer (never read).
   const void* apack = a.do_correct ? a.apack : a.rpack;
   const void* wc = a.do_correct ? a.Wc : a.Wv;
   const void* rp = a.do_gate ? a.rpack : a.apack;
   const void* wv = a.do_gate ? a.Wv : a.Wc;
   const void* wg = a.do_gate ? a.Wg : a.Wc;
+  const void* erows = a.do_gate && a.e_dense ? a.epack : rp;
   if (encode_tensor_map_2d(&mApack, apack, a.do_correct ? 2 * d : d, (uint64_t)rmax, (a.do_correct ? 4 : 2) * d, BK, BM) != CUDA_SUCCESS ||
       encode_tensor_map_2d(&mWc, wc, a.do_correct ? 2 * d : d, d, (a.do_correct ? 4 : 2) * d, BK, 128) != CUDA_SUCCESS ||
       encode_tensor_map_2d(&mR, rp, d, (uint64_t)rmax, 2 * (a.r_row_stride ? (uint64_t)a.r_row_stride : d), BK, BM) != CUDA_SUCCESS ||
       encode_tensor_map_2d(&mWv, wv, a.do_gate ? d : 2 * d, d, (a.do_gate ? 2 : 4) * d, BK, 128) != CUDA_SUCCESS ||
-      encode_tensor_map_2d(&mWg, wg, 2 * d, d, 4 * d, BK, 128) != CUDA_SUCCESS)
+      encode_tensor_map_2d(&mWg, wg, 2 * d, d, 4 * d, BK, 128) != CUDA_SUCCESS ||
+      encode_tensor_map_2d(&mE, erows, d, (uint64_t)rmax, 2 * d, BK, BM) != CUDA_SUCCESS ||
+      encode_tensor_map_2d(&mWge, wg, d, d, 4 * d, BK, 64) != CUDA_SUCCESS)  // the e half: zeros past column d
     return cudaErrorInvalidValue;
   CondParams p{};
   p.d = a.d;
@@ -1517,8 +1536,8 @@ static cudaError_t launch_cond_pair(const TcCondArgs& a, int clusters, cudaStrea
   p.beta = a.beta;
   p.r_out = reinterpret_cast<__nv_bfloat16*>(a.r_out);
   p.compact_out = a.compact_out;
-  p.e = reinterpret_cast<const __nv_bfloat16*>(a.e);
-  p.e_dense = 0;
+  p.e = reinterpret_cast<const __nv_bfloat16*>(a.e_dense ? a.epack : a.e);
+  p.e_dense = a.e_dense;
   p.Wg = reinterpret_cast<const __nv_bfloat16*>(a.Wg);
   p.ge = a.ge;
   p.e_out = reinterpret_cast<__nv_bfloat16*>(a.e_out);
@@ -1527,26 +1546,26 @@ static cudaError_t launch_cond_pair(const TcCondArgs& a, int clusters, cudaStrea
   p.block_ready = a.sync + kSyncBlocks + blocks_max(a.B, a.K);
   p.split_part = a.split_part;
   p.split_ticket = a.sync + kSyncBlocks + 2 * blocks_max(a.B, a.K);
-  p.split_max = (a.split_part && a.do_gate) ? kPairSplitTiles : 0;
+  // (a K half over a per-position e would hold the gate's columns only)
+  p.split_max = (a.split_part && a.do_gate && !a.e_dense) ? kPairSplitTiles : 0;
   p.status = a.status;
   // clusters of two CTAs; set-up may overlap the previous kernel's end
-  return launch_dependent(cond_pair_kernel, dim3(2 * (unsigned)clusters), dim3(P_THREADS), P_SMEM_BYTES, stream, 2,
-                          mApack, mWc, mR, mWv, mWg, p);
+  return launch_dependent(d % 256 == 0 && !p.e_dense ? cond_pair_kernel<false> : cond_pair_kernel<true>, dim3(2 * (unsigned)clusters), dim3(P_THREADS), P_SMEM_BYTES, stream, 2,
+                          mApack, mWc, mR, mWv, mWg, mE, mWge, p);
 }
 
-// The CTA-pair kernel: broadcast e (or no gate), and a device that can keep
-// at least one pair of its CTAs resident.  Returns the pair count (0: use
-// cond_kernel).
-static int pair_clusters(const TcCondArgs& a, long long tiles_max_pairs, cudaError_t* err) {
-  *err = cudaSuccess;
-  if (a.do_gate && a.e_dense) return 0;
-  static std::atomic<int> max_clusters[64];  // per device; 0: not yet known; -1: none fits
+// Pairs of CTAs of cond_pair_kernel to launch: those the device keeps resident
+// (cached per device), or fewer when the call has fewer tiles.
+static int pair_clusters(const TcCondArgs& a, long long tiles_max, cudaError_t* err) {
+  static std::atomic<int> max_clusters[64];  // 0: not yet known
   int dev = 0;
   if ((*err = cudaGetDevice(&dev)) != cudaSuccess) return 0;
-  if (max_clusters[dev & 63].load(std::memory_order_acquire) == 0) {
-    if ((*err = cudaFuncSetAttribute(cond_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, P_SMEM_BYTES)) !=
-        cudaSuccess)
-      return 0;
+  int n = max_clusters[dev & 63].load(std::memory_order_acquire);
+  if (n == 0) {
+    // (the two forms of the kernel have the same threads and shared memory, one CTA per SM)
+    for (auto kern : {cond_pair_kernel<false>, cond_pair_kernel<true>})
+      if ((*err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, P_SMEM_BYTES)) != cudaSuccess)
+        return 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2, 1, 1);
     cfg.blockDim = dim3(P_THREADS, 1, 1);
@@ -1558,15 +1577,16 @@ static int pair_clusters(const TcCondArgs& a, long long tiles_max_pairs, cudaErr
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    int n = 0;
-    if ((*err = cudaOccupancyMaxActiveClusters(&n, cond_pair_kernel, &cfg)) != cudaSuccess) return 0;
-    max_clusters[dev & 63].store(n > 0 ? n : -1, std::memory_order_release);
+    if ((*err = cudaOccupancyMaxActiveClusters(&n, cond_pair_kernel<true>, &cfg)) != cudaSuccess) return 0;
+    if (n < 1) {
+      *err = cudaErrorInvalidConfiguration;
+      return 0;
+    }
+    max_clusters[dev & 63].store(n, std::memory_order_release);
   }
-  const int n = max_clusters[dev & 63].load(std::memory_order_acquire);
-  if (n <= 0) return 0;
   // every pair when the gate-bias GEMV is needed: pairs without tiles compute it
-  if (a.do_gate) return n;
-  return (int)(tiles_max_pairs < n ? tiles_max_pairs : n);
+  if (a.do_gate && !a.e_dense) return n;
+  return (int)(tiles_max < n ? tiles_max : n);
 }
 
 // Clusters of S CTAs of swap_cluster_kernel that the device holds at once
@@ -1632,10 +1652,11 @@ static bool encode_row_maps(RowMaps* maps, const void* base, uint64_t inner, int
   return true;
 }
 
-// The small-R path (B (K-1) <= kSwapMaxRows, broadcast e or no gate): the
+// The small-R path (B (K-1) <= kSwapMaxRows): the
 // correction GEMM with the gate-bias GEMV, then the gate GEMM; each launch
 // waits on the one before inside the kernel, and cuts its work from the R it
-// reads.
+// reads.  Past the operands' ends (d no multiple of the tiles) the copies fill
+// zeros and the epilogues store nothing.
 static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
   const int rmax = (int)((long long)a.B * (a.K - 1));
   const int d = a.d;
@@ -1685,42 +1706,45 @@ static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
         !encode_row_maps(&mB, a.apack, 2 * du, rmax, 4 * du))
       return cudaErrorInvalidValue;
     SwapClusterParams c = sp;
-    c.mtiles = d / 128;
-    c.nkb = 2 * d / BK;
+    c.mtiles = (d + 127) / 128;
+    c.nkb = c.nkb_r = (2 * d + BK - 1) / BK;
     c.apack = reinterpret_cast<const __nv_bfloat16*>(a.apack);
     c.beta = a.beta;
     c.r_out = reinterpret_cast<__nv_bfloat16*>(a.r_out);
     c.compact_out = a.compact_out;
-    if (a.do_gate) c.bias = gp;
+    if (a.do_gate && !a.e_dense) c.bias = gp;
     int clusters = 0;
     if ((err = swap_pick_splits(dev, smem, rmax, c.mtiles, c.nkb, &c.S, &clusters)) != cudaSuccess) return err;
     err = launch_dependent(swap_cluster_kernel, grid_of(c, clusters), dim3(SW_THREADS), (size_t)smem, stream,
-                           (unsigned)c.S, mA, mA, mB, c);
+                           (unsigned)c.S, mA, mA, mA, mB, mB, c);
     if (err != cudaSuccess) return err;
   }
   if (a.do_gate) {
     const uint64_t rstride = 2 * (a.r_row_stride ? (uint64_t)a.r_row_stride : du);
-    CUtensorMap mA, mA2;
-    RowMaps mB;
+    CUtensorMap mA, mA2, mA3;
+    RowMaps mB, mE;
     if (encode_tensor_map_2d(&mA, a.Wv, du, du, 2 * du, BK, 64) != CUDA_SUCCESS ||
         encode_tensor_map_2d(&mA2, a.Wg, 2 * du, du, 4 * du, BK, 64) != CUDA_SUCCESS ||
-        !encode_row_maps(&mB, a.rpack, du, rmax, rstride))
+        encode_tensor_map_2d(&mA3, a.Wg, du, du, 4 * du, BK, 64) != CUDA_SUCCESS ||  // the e half: zeros past column d
+        !encode_row_maps(&mB, a.rpack, du, rmax, rstride) ||
+        (a.e_dense && !encode_row_maps(&mE, a.epack, du, rmax, 2 * du)))
       return cudaErrorInvalidValue;
-    if (!a.do_correct) {  // no correction kernel to compute it: W_g[:, :d] e in its own launch
+    if (!a.do_correct && !a.e_dense) {  // no correction kernel to compute it: W_g[:, :d] e in its own launch
       err = launch_dependent(swap_gemv_kernel, dim3((unsigned)(info.sm_count * 4)), dim3(256), 0, stream, 1u, gp);
       if (err != cudaSuccess) return err;
     }
     SwapClusterParams g = sp;
-    g.mtiles = d / 64;
-    g.nkb = d / BK;
+    g.mtiles = (d + 63) / 64;
+    g.nkb_r = (d + BK - 1) / BK;
+    g.nkb = a.e_dense ? 2 * g.nkb_r : g.nkb_r;
     g.gate = 1;
-    g.e = reinterpret_cast<const __nv_bfloat16*>(a.e);
-    g.ge = a.ge;
+    g.e = reinterpret_cast<const __nv_bfloat16*>(a.e_dense ? a.epack : a.e);
+    g.ge = a.e_dense ? nullptr : a.ge;
     g.e_out = reinterpret_cast<__nv_bfloat16*>(a.e_out);
     int clusters = 0;
     if ((err = swap_pick_splits(dev, smem, rmax, g.mtiles, g.nkb, &g.S, &clusters)) != cudaSuccess) return err;
     err = launch_dependent(swap_cluster_kernel, grid_of(g, clusters), dim3(SW_THREADS), (size_t)smem, stream,
-                           (unsigned)g.S, mA, mA2, mB, g);
+                           (unsigned)g.S, mA, mA2, mA3, mB, a.e_dense ? mE : mB, g);
     if (err != cudaSuccess) return err;
   }
   return cudaSuccess;
@@ -1729,60 +1753,13 @@ static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
 cudaError_t launch_cond_tc(const TcCondArgs& a, cudaStream_t stream) {
   const long long rmax = (long long)a.B * (a.K - 1);
   if (rmax <= 0 || (!a.do_correct && !a.do_gate)) return cudaSuccess;
-  if (rmax <= kSwapMaxRows && !(a.do_gate && a.e_dense)) return launch_cond_swap(a, stream);
-  const long long tiles_max_pairs =
-      (rmax + 2 * BM - 1) / (2 * BM) * ((a.do_correct ? a.d / 256 : 0) + (a.do_gate ? a.d / 128 : 0));
+  if (rmax <= kSwapMaxRows) return launch_cond_swap(a, stream);
+  const long long tiles_max = (rmax + 2 * BM - 1) / (2 * BM) *
+                              ((a.do_correct ? (a.d + 255) / 256 : 0) + (a.do_gate ? (a.d + 127) / 128 : 0));
   cudaError_t err;
-  const int clusters = pair_clusters(a, tiles_max_pairs, &err);
+  const int clusters = pair_clusters(a, tiles_max, &err);
   if (err != cudaSuccess) return err;
-  if (clusters > 0) return launch_cond_pair(a, clusters, stream);
-  err = ensure_smem_attr<false>();
-  if (err != cudaSuccess) return err;
-  const uint64_t d = (uint64_t)a.d;
-  CUtensorMap mApack, mWc, mR, mE, mWv, mWg;
-  // Maps of operands a call does not use point at a used buffer (never read).
-  const void* apack = a.do_correct ? a.apack : a.rpack;
-  const void* wc = a.do_correct ? a.Wc : a.Wv;
-  const void* rp = a.do_gate ? a.rpack : a.apack;
-  const void* erows = (a.do_gate && a.e_dense) ? a.epack : rp;
-  const void* wv = a.do_gate ? a.Wv : a.Wc;
-  const void* wg = a.do_gate ? a.Wg : a.Wc;
-  if (encode_tensor_map_2d(&mApack, apack, a.do_correct ? 2 * d : d, (uint64_t)rmax, (a.do_correct ? 4 : 2) * d, BK, BM) != CUDA_SUCCESS ||
-      encode_tensor_map_2d(&mWc, wc, a.do_correct ? 2 * d : d, d, (a.do_correct ? 4 : 2) * d, BK, 256) != CUDA_SUCCESS ||
-      encode_tensor_map_2d(&mR, rp, d, (uint64_t)rmax, 2 * (a.r_row_stride ? (uint64_t)a.r_row_stride : d), BK, BM) != CUDA_SUCCESS ||
-      encode_tensor_map_2d(&mE, erows, d, (uint64_t)rmax, 2 * d, BK, BM) != CUDA_SUCCESS ||
-      encode_tensor_map_2d(&mWv, wv, a.do_gate ? d : 2 * d, d, (a.do_gate ? 2 : 4) * d, BK, 128) != CUDA_SUCCESS ||
-      encode_tensor_map_2d(&mWg, wg, 2 * d, d, 4 * d, BK, 128) != CUDA_SUCCESS)
-    return cudaErrorInvalidValue;
-  CondParams p{};
-  p.d = a.d;
-  p.do_correct = a.do_correct;
-  p.do_gate = a.do_gate;
-  p.R = a.R;
-  p.rowmap = a.rowmap;
-  p.apack = reinterpret_cast<const __nv_bfloat16*>(a.apack);
-  p.beta = a.beta;
-  p.r_out = reinterpret_cast<__nv_bfloat16*>(a.r_out);
-  p.compact_out = a.compact_out;
-  p.e = reinterpret_cast<const __nv_bfloat16*>(a.e_dense ? a.epack : a.e);
-  p.e_dense = a.e_dense;
-  p.Wg = reinterpret_cast<const __nv_bfloat16*>(a.Wg);
-  p.ge = a.ge;
-  p.e_out = reinterpret_cast<__nv_bfloat16*>(a.e_out);
-  p.sync = a.sync;
-  p.block_done = a.sync + kSyncBlocks;
-  p.block_ready = a.sync + kSyncBlocks + blocks_max(a.B, a.K);
-  p.status = a.status;
-  DeviceInfo info{0, 148};
-  err = device_info(&info);
-  if (err != cudaSuccess) return err;
-  const long long tiles_max = (rmax + BM - 1) / BM * ((a.do_correct ? a.d / 256 : 0) + (a.do_gate ? a.d / 128 : 0));
-  // every SM when the broadcast-e GEMV is needed: CTAs without tiles compute it
-  const bool need_ge = a.do_gate && !a.e_dense;
-  const unsigned grid = (unsigned)(need_ge || tiles_max >= info.sm_count ? info.sm_count : tiles_max);
-  VerifyStreamParams vp{};
-  cond_kernel<false><<<grid, THREADS, SMEM_BYTES, stream>>>(mApack, mWc, mR, mE, mWv, mWg, p, vp);
-  return cudaGetLastError();
+  return launch_cond_pair(a, clusters, stream);
 }
 
 }  // namespace retrace
@@ -1792,14 +1769,21 @@ namespace retrace {
 bool round_fused_supported(const TcRoundArgs& a) {
   // contiguous logits with rows of at least one stream chunk, so that a chunk
   // is one contiguous copy and spans at most two rows
-  return tc_supported(RETRACE_BF16, a.d) && 4 * a.d <= kStageBytes && ((uintptr_t)a.logits % 16 == 0) && a.V % 8 == 0 &&
+  return a.d >= 256 && a.d % 256 == 0 && 4 * a.d <= kStageBytes && ((uintptr_t)a.logits % 16 == 0) && a.V % 8 == 0 &&
          a.V >= 8 * kChunkSlots && a.row_stride == a.V && a.batch_stride == (long long)(a.K + 1) * a.V &&
          a.K >= 2 && (long long)a.B * (a.K + 1) * (a.V / 8) < (1ll << 32) - kChunkSlots;
 }
 
 cudaError_t launch_round_tc(const TcRoundArgs& a, cudaStream_t stream) {
-  cudaError_t err = ensure_smem_attr<true>();
+  DeviceInfo info;
+  cudaError_t err = device_info(&info);
   if (err != cudaSuccess) return err;
+  static std::atomic<int> attr_done[64];
+  if (!attr_done[info.device & 63].load(std::memory_order_acquire)) {
+    err = cudaFuncSetAttribute(cond_overlap_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES_FUSED);
+    if (err != cudaSuccess) return err;
+    attr_done[info.device & 63].store(1, std::memory_order_release);
+  }
   const uint64_t d = (uint64_t)a.d;
   const long long rmax = (long long)a.B * (a.K - 1);
   CUtensorMap mApack, mWc, mR, mE, mWv, mWg;
@@ -1865,9 +1849,6 @@ cudaError_t launch_round_tc(const TcRoundArgs& a, cudaStream_t stream) {
   vp.chunk_next = a.sync + kSyncChunkNext;
   vp.status = a.status;
 
-  DeviceInfo info{0, 148};
-  err = device_info(&info);
-  if (err != cudaSuccess) return err;
   const long long grid = info.sm_count;
   // Cooperative: every CTA's share of the logits feeds other CTAs' tiles, so
   // all CTAs must be resident together (one per SM); the launch fails
@@ -1882,7 +1863,7 @@ cudaError_t launch_round_tc(const TcRoundArgs& a, cudaStream_t stream) {
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, cond_kernel<true>, mApack, mWc, mR, mE, mWv, mWg, p, vp);
+  return cudaLaunchKernelEx(&cfg, cond_overlap_kernel, mApack, mWc, mR, mE, mWv, mWg, p, vp);
 }
 
 }  // namespace retrace

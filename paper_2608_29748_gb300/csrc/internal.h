@@ -59,7 +59,7 @@ inline size_t swap_part_bytes(long long B, long long K, long long d) {
   const long long box = rows < 256 ? rows : 256;
   return (size_t)(kSwapMaxCtas * 128 * box * 4);
 }
-// CTA-pair conditioning (every other bf16 shape with d a multiple of 256): a
+// CTA-pair conditioning (more rows): with d a multiple of 256 a
 // last wave of at most kPairSplitTiles gate tiles runs as two K halves per
 // tile on two pairs.  Each half writes its fp32 accumulator (two CTAs x 128
 // rows x 256 columns) to the workspace (swp), and counts on one ticket per CTA and epilogue warp in the sync area.
@@ -287,7 +287,7 @@ cudaError_t launch_gate_simt(const GateArgs& a, retrace_dtype dtype, cudaStream_
 cudaError_t launch_gate_bias(const void* Wg, const void* e, int d, float* ge, retrace_dtype dtype,
                              cudaStream_t stream);
 
-// Tensor-core path (bf16, d a multiple of 256).
+// Tensor-core path (bf16, d a multiple of 8, at least 128).
 struct PackArgs {
   int B, K, d;
   RowSource rows;

@@ -318,3 +318,37 @@ def test_ffma_rows(rt, B, K, d, R, dtype, dense_e):
     want = oracle.gate_fuse(np.broadcast_to(host_f64(e), (B, K, d)), host_f64(r), n_host, host_f64(x["Wv"]),
                             host_f64(x["Wg"]))
     assert_close(out, want, f"e~, R={R} d={d}")
+
+
+@pytest.mark.parametrize("dense_e", [False, True])
+@pytest.mark.parametrize("B,K,d,R", [
+    (3, 6, 136, 11),     # small-R kernel: a last feature tile of 8, k-blocks past the operands' ends
+    (9, 16, 264, 100),
+    (9, 16, 1160, 128),
+    (20, 16, 200, 257),  # two row tiles
+    (64, 17, 328, 1024),
+    (80, 16, 136, 1100),  # CTA-pair kernel
+    (80, 16, 392, 1023),
+    (80, 16, 512, 257),
+])
+def test_ragged_hidden_sizes(rt, B, K, d, R, dense_e):
+    """bf16 hidden sizes that are a multiple of 8 but not of the tiles, with a
+    broadcast and a per-position e, on the small-R and the CTA-pair kernels."""
+    dtype = torch.bfloat16
+    x = make_inputs(B, K, d, dtype, seed=R + d, accept=accept_for_rows(B, K, R))
+    A = host_int(x["accept"])
+    n_host = oracle.carried_rows(A, K)
+    ws = rt.Workspace(B, K, 8, d, dtype)
+    r = torch.full((B, K, d), 9.0, dtype=dtype, device="cuda")
+    n = torch.empty((B,), dtype=torch.int32, device="cuda")
+    rt.retrace_align_refine(x["hD"], x["hT"], x["accept"], x["Wc"], 0.5, r, n, ws)
+    e = x["e_dense"] if dense_e else x["e_vec"]
+    out = torch.full((B, K, d), 7.0, dtype=dtype, device="cuda")
+    rt.retrace_gate_fuse(e, r, n, x["Wv"], x["Wg"], out, ws)
+    torch.cuda.synchronize()
+    assert ws.check() == 0
+    m, u = oracle.align(host_f64(x["hD"]), host_f64(x["hT"]), A)
+    assert_close(r, oracle.correct(m, u, host_f64(x["Wc"]), 0.5, round_r_bf16=False), f"r, R={R} d={d}")
+    want = oracle.gate_fuse(np.broadcast_to(host_f64(e), (B, K, d)), host_f64(r), n_host, host_f64(x["Wv"]),
+                            host_f64(x["Wg"]))
+    assert_close(out, want, f"e~, R={R} d={d}")
