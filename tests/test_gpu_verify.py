@@ -161,3 +161,25 @@ def test_verify_empty_batch(rt):
     rt.retrace_verify(logits, torch.empty((0, 4), dtype=torch.int32, device="cuda"), z,
                       torch.empty((0, 5), dtype=torch.int32, device="cuda"), z, ws)
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("V,pad,offset", [(1, 0, 0), (3, 0, 1), (8, 1, 0), (9, 0, 0), (15, 0, 7), (16, 3, 5), (17, 0, 2),
+                                          (4099, 0, 0), (8191, 2, 3), (32003, 0, 0)])
+def test_verify_unaligned_rows(rt, V, pad, offset, dtype):
+    """Rows that begin and end off a 16-byte boundary (odd vocabularies, row
+    strides and bases): the maximum, or a tie of it, in the elements before
+    the first and after the last aligned vector."""
+    B, K = 6, 7
+    g = torch.Generator(device="cuda").manual_seed(V * 8 + offset)
+    stride = V + pad
+    buf = torch.randn(B * (K + 1) * stride + offset, generator=g, device="cuda").to(dtype)
+    logits = buf[offset:].as_strided((B, K + 1, V), ((K + 1) * stride, stride, 1))
+    for i in range(K + 1):  # the winner at the front, at the back, or tied between both
+        if i % 3 != 1:
+            logits[:, i, min(i, V - 1)] = 9.0
+        if i % 3 != 0:
+            logits[:, i, max(V - 1 - i, 0)] = 9.0
+    draft = torch.argmax(logits.float()[:, :K], dim=-1).to(torch.int32)
+    draft[torch.arange(B), torch.arange(B) % K] -= 1  # a mismatch somewhere (-1: no token)
+    check_against_oracle(rt, logits, draft)
