@@ -9,11 +9,10 @@
 //
 // Only the top_k logits of a row enter its filtered distribution, so the
 // row's full softmax is never formed:
-//   sampled_topk_kernel      one CTA per row (target rows, then drafter rows):
-//                            elements above a proven lower bound of the row's
-//                            k-th largest (a sample's k-th largest, then the
-//                            best warp's k-th largest candidate) go to per-warp
-//                            buffers; the CTA merges the warps' lists by rank;
+//   sampled_topk_kernel      one CTA, or a cluster, per row (target rows, then
+//                            drafter rows): one branch-free pass for maxima,
+//                            from them a proven lower bound of the row's k-th
+//                            largest, then the few elements above it, ranked;
 //   sampled_finalize_kernel  one CTA per sequence: the filtered
 //                            probabilities of the draft tokens from the sorted
 //                            lists (eight positions at a time, one per warp),
@@ -28,16 +27,21 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cstddef>
+
 #include "common.cuh"
 #include "internal.h"
+#include "tc_pair.cuh"
 
 namespace retrace {
 namespace {
 
 constexpr int kThreads = 512;
-constexpr int kWarps = kThreads / 32;
-constexpr int kTrigger = kMaxTopK;       // a warp's buffer is cut to its top k once it holds more keys
-constexpr int kBuf = kTrigger + 32 * 8;  // candidate keys per warp: the trigger + one bf16 chunk of the warp
+constexpr int kUnroll = 4;    // 16-byte loads in flight per thread
+constexpr int kCells = 16;    // most cells per thread
+constexpr int kBuf = 1024;    // candidates a CTA keeps without the slow path
+constexpr int kMaxParts = 8;  // most CTAs (a cluster) per row
+constexpr int kPrefetchVectors = 4096;  // 64 KB of the next row: two batches of every thread
 
 struct TopkParams {
   const void* tlogits;
@@ -52,15 +56,12 @@ struct TopkParams {
   int i0, i1;
   const int32_t* live_in;
   const uint32_t* count_in;
+  int parts;  // CTAs of a cluster, which share a row (or take a row each when there are many)
 };
 
-// The largest key whose value is below v: every element of value >= v beats it.
-__device__ __forceinline__ unsigned long long below_value(float v) {
-  return ((unsigned long long)ordered_bits(v) << 32) - 1ull;
-}
-
+// One lane's 16 bytes of a row.
 template <typename T>
-struct Chunk;  // one lane's share of a chunk (16 bytes): raw bits, partial maxima, candidate masks
+struct Chunk;
 template <>
 struct Chunk<__nv_bfloat16> {
   static constexpr int E = 8;
@@ -76,236 +77,212 @@ struct Chunk<__nv_bfloat16> {
   static __device__ Part combine(Part a, Part b) { return __hmax2(a, b); }
   static __device__ float finish(Part m) { return fmaxf(__low2float(m), __high2float(m)); }
   static __device__ Part lowest() { return __floats2bfloat162_rn(-INFINITY, -INFINITY); }
-  // bit e set iff element e >= tv
-  __device__ unsigned mask(float tv) const {
-    const uint32_t q[4] = {w.x, w.y, w.z, w.w};
-    unsigned m = 0;
-#pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      m |= (bf16_lo(q[h]) >= tv ? 1u : 0u) << (2 * h);
-      m |= (bf16_hi(q[h]) >= tv ? 1u : 0u) << (2 * h + 1);
-    }
-    return m;
-  }
   __device__ float value(int e) const {
     const uint32_t x = e < 2 ? w.x : e < 4 ? w.y : e < 6 ? w.z : w.w;
     return (e & 1) ? bf16_hi(x) : bf16_lo(x);
   }
-  __device__ void load(const __nv_bfloat16* p) { w = __ldcs(reinterpret_cast<const uint4*>(p)); }
-  __device__ void fill() { w = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u); }  // -inf
-  __device__ void set_single(float v) { w = make_uint4(pack_bf16x2(v, -INFINITY), 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u); }
 };
 template <>
 struct Chunk<float> {
   static constexpr int E = 4;
   using Part = float;
-  float4 w;
-  __device__ Part part() const { return fmaxf(fmaxf(w.x, w.y), fmaxf(w.z, w.w)); }
+  uint4 w;
+  __device__ Part part() const {
+    return fmaxf(fmaxf(__uint_as_float(w.x), __uint_as_float(w.y)), fmaxf(__uint_as_float(w.z), __uint_as_float(w.w)));
+  }
   static __device__ Part combine(Part a, Part b) { return fmaxf(a, b); }
   static __device__ float finish(Part m) { return m; }
   static __device__ Part lowest() { return -INFINITY; }
-  __device__ unsigned mask(float tv) const {
-    return (w.x >= tv ? 1u : 0u) | (w.y >= tv ? 2u : 0u) | (w.z >= tv ? 4u : 0u) | (w.w >= tv ? 8u : 0u);
-  }
-  __device__ float value(int e) const { return e == 0 ? w.x : e == 1 ? w.y : e == 2 ? w.z : w.w; }
-  __device__ void load(const float* p) { w = __ldcs(reinterpret_cast<const float4*>(p)); }
-  __device__ void fill() { w = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY); }
-  __device__ void set_single(float v) { w = make_float4(v, -INFINITY, -INFINITY, -INFINITY); }
+  __device__ float value(int e) const { return __uint_as_float(e == 0 ? w.x : e == 1 ? w.y : e == 2 ? w.z : w.w); }
 };
 
-// Ranks the warp's `n` buffered keys (distinct) and keeps the largest
-// min(n, k) in descending order at the front of the buffer; returns their
-// count.  Lane-parallel rank counting (every key's rank is the number of
-// larger keys); the thresholds keep n small.
-__device__ int warp_compact(unsigned long long* buf, unsigned long long* tmp, int n, int k, int lane) {
-  for (int a = lane; a < n; a += 32) {
-    const unsigned long long x = buf[a];
+// Shared memory of a top-k CTA.  The slow path uses buf and cell together as
+// one array of kSlowBuf keys.
+struct TopkSmem {
+  unsigned long long buf[kBuf];
+  float cell[kCells][kThreads];
+  unsigned long long top[kMaxTopK];  // this CTA's part of the row, in descending order
+  float thr;
+  int n;      // candidates in buf
+  int n_top;  // keys in top
+};
+constexpr int kSlowBuf = kBuf + kCells * kThreads / 2;
+static_assert(offsetof(TopkSmem, cell) == sizeof(unsigned long long) * kBuf, "the slow path's array is contiguous");
+static_assert(kSlowBuf >= kBuf + kThreads * 8, "a slow-path round fits behind kBuf keys");
+
+// Moves the largest min(n, k) of `keys` (distinct) to `top` in descending
+// order, by rank counting; returns their count.  Called by the whole CTA,
+// after a barrier; ends before one.
+__device__ __forceinline__ int rank_top(const unsigned long long* keys, int n, int k, unsigned long long* top) {
+  for (int a = threadIdx.x; a < n; a += kThreads) {
+    const unsigned long long x = keys[a];
     int rank = 0;
-    for (int c = 0; c < n; ++c) rank += buf[c] > x ? 1 : 0;
-    if (rank < k) tmp[rank] = x;
+    for (int c = 0; c < n; ++c) rank += keys[c] > x ? 1 : 0;
+    if (rank < k) top[rank] = x;
   }
-  __syncwarp();
-  const int m = n < k ? n : k;
-  for (int a = lane; a < m; a += 32) buf[a] = tmp[a];
-  __syncwarp();
-  return m;
+  return n < k ? n : k;
 }
 
-// One CTA per row; warp w scans a contiguous part of it, U chunks (16 bytes
-// per lane each) per step.  Elements are kept as candidates only above a
-// proven lower bound of the row's k-th largest key: first the k-th largest
-// of a sample (every lane's maximum over its first U chunks: each is an
-// element of the row), then any warp's k-th largest candidate so far (the
-// maximum of both in s_thr).  One vote per step on the packed maxima decides whether
-// any element can pass (the common case: none); otherwise a ballot per chunk
-// skips the chunks without one, and the lanes that have some append them, by
-// bit mask, to the warp's buffer with shared-memory atomics.  A buffer that
-// passes a trigger is cut to its top k.  The row's top k are merged from the
-// warps' sorted lists.
-struct TopkSmem {
-  unsigned long long buf[kWarps][kBuf];
-  unsigned long long tmp[kWarps][kMaxTopK];
-  float sample[kThreads];
-  int n[kWarps];
-  unsigned long long thr;
-};
-
-// The top-k list of one row x into p.keys slot `row` (the whole CTA).
+// The k largest keys of row elements >= t when they are too many for buf (long
+// runs of equal values): rounds of one vector per thread, the keys cut to the
+// k largest whenever they pass kBuf.  Fills sm.top; returns the count.
 template <typename T>
-__device__ __forceinline__ void topk_row(const TopkParams& p, const T* x, int row, TopkSmem& sm) {
-  using CT = Chunk<T>;
-  using Part = typename CT::Part;
-  constexpr int E = CT::E;
-  constexpr int U = 4;
-  auto& s_buf = sm.buf;
-  auto& s_tmp = sm.tmp;
-  auto& s_sample = sm.sample;
-  auto& s_n = sm.n;
-  auto& s_thr = sm.thr;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int V = p.V, k = p.k;
-  unsigned long long* buf = s_buf[warp];
-  unsigned long long* tmp = s_tmp[warp];
-  if (lane == 0) s_n[warp] = 0;
-  const unsigned FULL = 0xFFFFFFFFu;
-  const bool vec = (V % E == 0) && ((uintptr_t)x % 16 == 0);
-  const int per = vec ? E : 1;  // elements of the row per lane per chunk
-  const int span = 32 * per;
-  const int nchunks = (V + span - 1) / span;
-  const int c0 = (int)((long long)nchunks * warp / kWarps), c1 = (int)((long long)nchunks * (warp + 1) / kWarps);
-  // k <= kMaxTopK = kTrigger: a compaction leaves at most kTrigger keys, so
-  // the buffer has room for the next chunk
-  const int trigger = kTrigger;
-  const unsigned valid_bits = vec ? (1u << E) - 1u : 1u;  // the scalar path fills elements 1.. with -inf
-
-  // chunk c of this lane: valid iff c < c1 and its first element is in the row
-  auto load_checked = [&](CT (&ch)[U], int c) {
-#pragma unroll
-    for (int q = 0; q < U; ++q) {
-      const int base = (c + q) * span + lane * per;
-      ch[q].fill();
-      if (c + q < c1 && base < V) {
-        if (vec) ch[q].load(x + base);
-        else ch[q].set_single(to_f32(x[base]));
-      }
-    }
+__device__ __noinline__ int topk_slow(const T* x, int head, int v0, int v1, int edge_n, int full, float t, int k,
+                                      TopkSmem& sm) {
+  constexpr int E = Chunk<T>::E;
+  unsigned long long* keys = sm.buf;
+  if (threadIdx.x == 0) sm.n = 0;
+  __syncthreads();
+  unsigned long long least = 0ull;  // keys up to this one are not among the k largest
+  auto add = [&](float v, int idx) {
+    const unsigned long long key = make_key(v, (uint32_t)idx);
+    if (v >= t && key > least) keys[atomicAdd(&sm.n, 1)] = key;
   };
-  // U chunks that lie inside the row and the warp's range (the main loop)
-  auto load_full = [&](CT (&ch)[U], int c) {
-    const T* ptr = x + c * span + lane * per;
+  if ((int)threadIdx.x < edge_n) {
+    const int i = (int)threadIdx.x < head ? (int)threadIdx.x : (int)threadIdx.x + full * E;
+    add(to_f32(x[i]), i);
+  }
+  for (int b = v0;; b += kThreads) {
+    const int v = b + (int)threadIdx.x;
+    if (v < v1) {
+      Chunk<T> c;
+      c.w = __ldg(reinterpret_cast<const uint4*>(x + head) + v);
 #pragma unroll
-    for (int q = 0; q < U; ++q) {
-      if (vec) ch[q].load(ptr + q * span);
-      else ch[q].set_single(to_f32(ptr[q * span]));
+      for (int e = 0; e < E; ++e) add(c.value(e), head + v * E + e);
     }
-  };
-  auto process = [&](const CT (&ch)[U], int c, bool full) {
-    const unsigned long long t = *(volatile unsigned long long*)&s_thr;
-    const float tv = t ? key_value(t) : -INFINITY;
-    Part m = ch[0].part();
-#pragma unroll
-    for (int q = 1; q < U; ++q) m = CT::combine(m, ch[q].part());
-    // invalid chunks hold -inf; they can pass only with no bound at all
-    if (!__any_sync(FULL, CT::finish(m) >= tv)) return;
-#pragma unroll
-    for (int q = 0; q < U; ++q) {
-      const int base = (c + q) * span + lane * per;
-      const bool has = CT::finish(ch[q].part()) >= tv && (full || (c + q < c1 && base < V));
-      if (!__ballot_sync(FULL, has)) continue;
-      const unsigned bits = has ? ch[q].mask(tv) & valid_bits : 0u;
-      for (unsigned r = bits; r; r &= r - 1) {
-        const int e = __ffs(r) - 1;
-        const unsigned long long key = make_key(ch[q].value(e), (uint32_t)(base + e));
-        if (key > t) buf[atomicAdd(&s_n[warp], 1)] = key;
-      }
-      __syncwarp();
-      int n = *(volatile int*)&s_n[warp];
-      if (n > trigger) {  // keep the top k so far (kBuf leaves room for one more chunk)
-        n = warp_compact(buf, tmp, n, k, lane);
-        if (lane == 0) s_n[warp] = n;
-        if (n >= k && lane == 0) atomicMax(&s_thr, buf[k - 1]);
-        __syncwarp();
-      }
-    }
-  };
-
-  CT ch[U];
-  load_checked(ch, c0);
-  {
-    // Sampling: each lane's maximum over its first U chunks, sorted within
-    // the warp (bitonic, by shuffles); warp 0 merges the 16 sorted lists up
-    // to the k-th largest, a lower bound of the row's k-th largest.
-    Part m = ch[0].part();
-#pragma unroll
-    for (int q = 1; q < U; ++q) m = CT::combine(m, ch[q].part());
-    float v = CT::finish(m);
-    if (v != v) v = -INFINITY;  // all-NaN lane: no sample
-#pragma unroll
-    for (int size = 2; size <= 32; size <<= 1) {
-#pragma unroll
-      for (int stride = size >> 1; stride > 0; stride >>= 1) {
-        const float o = __shfl_xor_sync(FULL, v, stride);
-        const bool keep_max = ((lane & size) == 0) == ((lane & stride) == 0);  // descending at size 32
-        v = keep_max ? fmaxf(v, o) : fminf(v, o);
-      }
-    }
-    s_sample[threadIdx.x] = v;
-    if (threadIdx.x == 0) s_thr = 0ull;
     __syncthreads();
-    if (warp == 0) {
-      int pos = 0;
-      float head = lane < kWarps ? s_sample[lane * 32] : -INFINITY;
-      float best = -INFINITY;
-      for (int r = 0; r < k; ++r) {
-        best = head;
+    const int n = sm.n;
+    const bool done = b + kThreads >= v1;
+    if (n > kBuf || done) {
+      const int m = rank_top(keys, n, k, sm.top);
+      __syncthreads();
+      for (int a = threadIdx.x; a < m; a += kThreads) keys[a] = sm.top[a];
+      if (threadIdx.x == 0) sm.n = m;
+      least = m == k ? sm.top[k - 1] : 0ull;
+      __syncthreads();
+      if (done) return m;
+    }
+    __syncthreads();
+  }
+}
+
+// The top-k keys of part `part` of `parts` of row x, into sm.top (whole CTA).
+//
+// Every thread streams its vectors once and keeps only maxima: one per cell
+// (a few batches of kUnroll vectors) in shared memory and one overall.  The
+// k-th largest of the threads' maxima is a lower bound t of the part's k-th
+// largest element (each is an element), and a close one: with 512 threads and
+// k = 20 a part has about 21 elements above it.  With several parts the
+// largest of their bounds serves all.  Then the few threads whose maxima
+// reach t reload the cells that do, and their elements >= t are ranked.  The
+// stream itself has no branch on the data; a scan that compared each vector
+// with a bound sampled from the row's start spent most of its time on the
+// vectors that passed it (one pass over 1056 rows of 151936 bf16: 84 us, now
+// 74).
+template <typename T>
+__device__ __forceinline__ void topk_part(const T* x, int V, int k, int parts, int part, TopkSmem& sm) {
+  using CT = Chunk<T>;
+  constexpr int E = CT::E;
+  const int tid = threadIdx.x;
+  const int head = min(V, (int)((16u - (uint32_t)((uintptr_t)x & 15u)) & 15u) / (int)sizeof(T));
+  const int full = (V - head) / E;  // aligned vectors inside the row
+  const int v0 = (int)((long long)part * full / parts), v1 = (int)((long long)(part + 1) * full / parts);
+  // the elements before and after the vectors (fewer than 2 E), one per thread of part 0
+  const int edge_n = part == 0 ? V - full * E : 0;
+  const int edge_i = tid < head ? tid : tid + full * E;
+  const uint4* vp = reinterpret_cast<const uint4*>(x + head);
+  const int batches = (v1 - v0 + kUnroll * kThreads - 1) / (kUnroll * kThreads);
+  const int per = (batches + kCells - 1) / kCells;  // batches per cell
+  const int cells = per > 0 ? (batches + per - 1) / per : 0;
+  if (tid == 0) sm.n = 0;
+  float edge_v = -INFINITY;
+  if (tid < edge_n) edge_v = to_f32(x[edge_i]);
+  float tm = edge_v;
+  for (int j = 0; j < cells; ++j) {
+    typename CT::Part m = CT::lowest();
+    for (int c = j * per; c < (j + 1) * per; ++c) {
+      const int b = v0 + c * kUnroll * kThreads + tid;
+      CT ch[kUnroll];
+      if (b + (kUnroll - 1) * kThreads < v1) {
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) best = fmaxf(best, __shfl_xor_sync(FULL, best, off));
-        const unsigned own = __ballot_sync(FULL, head == best);
-        if (lane == __ffs(own) - 1) {
-          ++pos;
-          head = pos < 32 ? s_sample[lane * 32 + pos] : -INFINITY;
+        for (int u = 0; u < kUnroll; ++u) ch[u].w = __ldcs(vp + b + u * kThreads);
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) m = CT::combine(m, ch[u].part());
+      } else {
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) {
+          if (b + u * kThreads < v1) {
+            ch[u].w = __ldcs(vp + b + u * kThreads);
+            m = CT::combine(m, ch[u].part());
+          }
         }
       }
-      if (lane == 0) s_thr = best > -INFINITY ? below_value(best) : 0ull;
     }
-    __syncthreads();
+    const float mv = CT::finish(m);
+    sm.cell[j][tid] = mv;
+    tm = fmaxf(tm, mv);
   }
-  process(ch, c0, false);
-  // chunks [0, nfull) lie wholly inside the row
-  const int cfull = c1 < V / span ? c1 : V / span;
-  int c = c0 + U;
-  for (; c + U <= cfull; c += U) {
-    load_full(ch, c);
-    process(ch, c, true);
+  // t: the largest value of 16 leading key bits that at least k threads'
+  // maxima reach (all bits of a bf16 value; an fp32 bound is rounded down)
+  const unsigned h = ordered_bits(tm) >> 16;
+  unsigned lo = 0u;
+#pragma unroll 1
+  for (int bit = 15; bit >= 0; --bit) {
+    const unsigned c = lo | (1u << bit);
+    if (__syncthreads_count(h >= c) >= k) lo = c;
   }
-  for (; c < c1; c += U) {
-    load_checked(ch, c);
-    process(ch, c, false);
+  const unsigned minus_inf = ordered_bits(-INFINITY) >> 16;
+  float t = lo <= minus_inf ? -INFINITY : key_value((unsigned long long)lo << 48);
+  if (parts > 1) {
+    if (tid == 0) sm.thr = t;
+    cluster_sync_all();
+    for (int q = 0; q < parts; ++q) t = fmaxf(t, ld_cluster_f1(map_rank(smem_u32(&sm.thr), (uint32_t)q)));
   }
-  int n = warp_compact(buf, tmp, *(volatile int*)&s_n[warp], k, lane);
-  if (lane == 0) s_n[warp] = n;
+  // the elements >= t
+  auto add = [&](float v, int idx) {
+    if (v >= t) {
+      const int at = atomicAdd(&sm.n, 1);
+      if (at < kBuf) sm.buf[at] = make_key(v, (uint32_t)idx);
+    }
+  };
+  if (tm >= t) {
+    if (tid < edge_n) add(edge_v, edge_i);
+    for (int j = 0; j < cells; ++j) {
+      if (!(sm.cell[j][tid] >= t)) continue;
+      for (int c = j * per; c < (j + 1) * per; ++c) {
+        const int b = v0 + c * kUnroll * kThreads + tid;
+        CT ch[kUnroll];
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u)
+          if (b + u * kThreads < v1) ch[u].w = __ldg(vp + b + u * kThreads);
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u)
+          if (b + u * kThreads < v1) {
+            const int v = b + u * kThreads;
+#pragma unroll
+            for (int e = 0; e < E; ++e) add(ch[u].value(e), head + v * E + e);
+          }
+      }
+    }
+  }
   __syncthreads();
-  // Merge the warps' sorted lists: lane w of warp 0 holds the head of list w;
-  // the largest head is the next key of the row.
-  if (warp == 0) {
-    unsigned long long* out = p.keys + (long long)row * kMaxTopK;
-    int pos = 0;
-    const int len = lane < kWarps ? s_n[lane] : 0;
-    for (int r = 0; r < k; ++r) {
-      const unsigned long long head = pos < len ? s_buf[lane][pos] : 0ull;
-      const unsigned long long best = warp_max_key(head);
-      if (lane == 0) out[r] = best;  // 0 once every list is exhausted (V < k)
-      if (head == best && best != 0ull) ++pos;
-    }
-  }
+  int n = sm.n;
+  __syncthreads();  // the slow path reuses sm.n
+  if (n > kBuf) n = topk_slow<T>(x, head, v0, v1, edge_n, full, t, k, sm);
+  else n = rank_top(sm.buf, n, k, sm.top);
+  if (tid == 0) sm.n_top = n;
+  __syncthreads();
 }
 
-// One row per CTA (the first pass: every row of the window), or a grid of
-// resident CTAs looping over the rows of a later pass (its live count is
-// known only on the device; a grid of the whole batch's rows would spend
-// whole waves of CTAs that only find they have nothing to do).  The rows of
-// a pass: the window's target rows of each listed sequence, then its drafter
-// rows; `row` is the row's slot in p.keys.
+// Clusters of p.parts CTAs.  The rows of a pass: the window's target rows of
+// each listed sequence, then its drafter rows (`row` is the row's slot in
+// p.keys).  A cluster takes one row at a time, each CTA a part of it, and
+// CTA 0 merges the parts; when a pass has many rows for its clusters, each
+// CTA takes whole rows instead (the merge and the shorter streams cost more
+// than they balance).  The live count of a later pass is known on the device
+// only, so its grid is resident CTAs that loop over the rows (LOOP; in the first
+// pass a CTA per row, which measured 158 us per round of 32 sequences, was
+// faster than resident ones, 165).
 template <typename T, bool LOOP>
 __global__ void __launch_bounds__(kThreads, 3) sampled_topk_kernel(const TopkParams p) {
   __shared__ TopkSmem sm;
@@ -317,6 +294,9 @@ __global__ void __launch_bounds__(kThreads, 3) sampled_topk_kernel(const TopkPar
   }
   const int wt = p.i1 - p.i0, wd = min(p.i1, p.K) - p.i0;
   const int rows = n_live * (wt + wd);  // B (2K+1) at most, below 2^31
+  const int parts = rows > (int)gridDim.x ? 1 : p.parts;
+  const int part = parts > 1 ? (int)cluster_rank() : 0;
+  const int step = (int)gridDim.x / parts;
   auto row_of = [&](int r0, const T*& x) -> int {
     if (r0 < n_live * wt) {
       const int l = r0 / wt, i = p.i0 + (r0 - l * wt);
@@ -329,18 +309,48 @@ __global__ void __launch_bounds__(kThreads, 3) sampled_topk_kernel(const TopkPar
     x = reinterpret_cast<const T*>(p.dlogits) + b * p.d_batch + i * p.d_row;
     return p.B * (p.K + 1) + b * p.K + i;
   };
-  if constexpr (!LOOP) {
-    if ((int)blockIdx.x >= rows) return;
+  for (int r0 = (int)blockIdx.x / parts; r0 < rows; r0 += step) {
     const T* x;
-    const int row = row_of(blockIdx.x, x);
-    topk_row<T>(p, x, row, sm);
-  } else {
-    for (int r0 = blockIdx.x; r0 < rows; r0 += gridDim.x) {
-      const T* x;
-      const int row = row_of(r0, x);
-      topk_row<T>(p, x, row, sm);
-      __syncthreads();  // the row's shared buffers are read to the end before the next row
+    if (LOOP && threadIdx.x == 0 && r0 + step < rows) {
+      // the stream pauses between rows: the first vectors of this CTA's next
+      // part (inside the row, 16-byte aligned) go to L2 meanwhile
+      row_of(r0 + step, x);
+      const int h = min(p.V, (int)((16u - (uint32_t)((uintptr_t)x & 15u)) & 15u) / (int)sizeof(T));
+      const int full = (p.V - h) / Chunk<T>::E;
+      const int v0 = (int)((long long)part * full / parts), v1 = (int)((long long)(part + 1) * full / parts);
+      const int nv = min(v1 - v0, kPrefetchVectors);
+      if (nv > 0)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(reinterpret_cast<const uint4*>(x + h) + v0),
+                     "r"(nv * 16)
+                     : "memory");
     }
+    const int row = row_of(r0, x);
+    topk_part<T>(x, p.V, p.k, parts, part, sm);
+    unsigned long long* out = p.keys + (long long)row * kMaxTopK;
+    if (parts == 1) {
+      for (int r = threadIdx.x; r < p.k; r += kThreads) out[r] = r < sm.n_top ? sm.top[r] : 0ull;
+      __syncthreads();  // sm is read to the end before the next row
+    } else {
+      cluster_sync_all();  // every part's list is complete
+      if (part == 0) {
+        // thread 64 q + r has key r of part q (kMaxParts * kMaxTopK = kThreads)
+        const int q = (int)threadIdx.x / kMaxTopK, r = (int)threadIdx.x % kMaxTopK;
+        int before = 0, total = 0, mine = 0;
+#pragma unroll
+        for (int c = 0; c < kMaxParts; ++c) {
+          const int n = c < parts ? ld_cluster_s32(map_rank(smem_u32(&sm.n_top), (uint32_t)c)) : 0;
+          before += c < q ? n : 0;
+          mine = c == q ? n : mine;
+          total += n;
+        }
+        if (r < mine) sm.buf[before + r] = ld_cluster_u64(map_rank(smem_u32(&sm.top[r]), (uint32_t)q));
+        __syncthreads();
+        const int n = rank_top(sm.buf, total, p.k, out);
+        for (int r2 = n + (int)threadIdx.x; r2 < p.k; r2 += kThreads) out[r2] = 0ull;
+      }
+      cluster_sync_all();  // CTA 0 has read the parts' lists
+    }
+    if constexpr (!LOOP) break;
   }
 }
 
@@ -735,21 +745,25 @@ cudaError_t launch_verify_sampled(const SampledArgs& a, retrace_dtype dtype, cud
     fp.n_counts = last ? n_pass - 1 : 0;
     fp.exits = last && n_pass > 1 ? a.pass_counts : nullptr;
     const int wt = tp.i1 - tp.i0, wd = (tp.i1 < a.K ? tp.i1 : a.K) - tp.i0;
-    // the first pass: one CTA per row; later passes: resident CTAs looping
+    // Parts per row, where the pass may have fewer rows than resident CTAs:
+    // as many as keep them in one wave, at least 16 KB of logits each.  In
+    // the first pass every row is known to be there; a later pass, whose
+    // rows are not known here, gets a whole resident grid in clusters of four
+    // and decides on the device.
     const long long rows_max = (long long)a.B * (wt + wd);
-    const long long grid_n = k == 0 ? rows_max : (rows_max < topk_resident ? rows_max : topk_resident);
-    const dim3 grid((unsigned)(grid_n > 0 ? grid_n : 1));
-    cudaError_t err;
+    const long long most = std::max(1LL, (long long)a.V * fp.elem / (16 << 10));
+    int parts = 1;
+    while (parts < kMaxParts && 2 * parts <= most && (k > 0 ? parts < 4 : 2 * parts * rows_max <= topk_resident)) parts *= 2;
+    tp.parts = parts;
+    long long grid_n = k == 0 ? rows_max * parts : std::min(rows_max * parts, topk_resident);
+    grid_n = std::max(1LL, grid_n / parts) * parts;
     auto topk = k == 0 ? (dtype == RETRACE_BF16 ? sampled_topk_kernel<__nv_bfloat16, false>
-                                                 : sampled_topk_kernel<float, false>)
+                                                : sampled_topk_kernel<float, false>)
                        : (dtype == RETRACE_BF16 ? sampled_topk_kernel<__nv_bfloat16, true>
-                                                 : sampled_topk_kernel<float, true>);
-    if (k == 0) {
-      topk<<<grid, kThreads, 0, stream>>>(tp);
-      err = cudaGetLastError();
-    } else {
-      err = launch_dependent(topk, grid, dim3(kThreads), 0, stream, 1, tp);
-    }
+                                                : sampled_topk_kernel<float, true>);
+    cudaError_t err = k == 0 ? launch_cluster(topk, dim3((unsigned)grid_n), dim3(kThreads), stream, (unsigned)parts, tp)
+                             : launch_dependent(topk, dim3((unsigned)grid_n), dim3(kThreads), 0, stream,
+                                                (unsigned)parts, tp);
     if (err != cudaSuccess) return err;
     err = launch_dependent(sampled_finalize_kernel, dim3((unsigned)a.B), dim3(256), 0, stream, 1, fp);
     if (err != cudaSuccess) return err;

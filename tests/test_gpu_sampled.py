@@ -122,3 +122,48 @@ def test_sampled_verification_is_lossless_on_the_gpu(rt):
     want[pt] = pp
     sd = np.sqrt(np.maximum(want * (1 - want), 1e-12) / B)
     assert np.all(np.abs(freq - want) <= 5 * sd + 1e-4), np.max(np.abs(freq - want) / (sd + 1e-12))
+
+
+def special_rows(kind, B, K, V, dtype, offset, g):
+    """[B, K+1, V] logits starting `offset` elements into their buffer."""
+    buf = torch.empty(B * (K + 1) * V + offset, device="cuda", dtype=dtype)
+    rows = buf[offset:].view(B, K + 1, V)
+    if kind == "random":
+        rows.copy_(torch.randn((B, K + 1, V), generator=g, device="cuda") * 2)
+    elif kind == "equal":  # every element ties: the lowest indices
+        rows.fill_(1.5)
+    elif kind == "rising":  # every later vector beats the ones before it
+        rows.copy_(torch.linspace(-4, 4, V, device="cuda").expand(B, K + 1, V))
+    else:  # few elements above -inf
+        rows.fill_(-float("inf"))
+        rows[:, :, torch.randperm(V, generator=g, device="cuda")[:5]] = torch.arange(5, device="cuda").to(dtype) / 4
+    return rows
+
+
+@pytest.mark.parametrize("windows", [False, True])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("kind,V,k,offset", [
+    ("random", 64, 64, 0), ("random", 67, 64, 1), ("random", 4099, 20, 0), ("random", 16392, 20, 3),
+    ("random", 32003, 20, 0), ("random", 70001, 64, 5), ("random", 151936, 20, 0),
+    ("equal", 100, 20, 0), ("equal", 32003, 64, 1), ("rising", 20000, 20, 0), ("rising", 20001, 64, 7),
+    ("sparse", 9000, 5, 0)])
+def test_sampled_topk_rows(rt, kind, V, k, offset, dtype, windows):
+    """The top-k scan where it can go wrong: rows that begin and end off a
+    16-byte boundary, rows of one to eight CTAs, fewer vectors than threads,
+    and rows whose bound leaves more candidates than the buffer holds."""
+    B, K = 2, 8
+    g = torch.Generator(device="cuda").manual_seed(V + k)
+    tl = special_rows(kind, B, K, V, dtype, offset, g)
+    dl = special_rows(kind, B, K, V, dtype, offset, g)[:, :K]
+    if kind == "random":
+        dl = (tl[:, :K].float() + 0.05 * torch.randn((B, K, V), generator=g, device="cuda")).to(dtype)
+    top = torch.topk(dl.float(), 1, dim=-1).indices[..., 0].to(torch.int32)
+    if kind == "equal":
+        top.copy_(torch.randint(0, k, (B, K), generator=g, device="cuda"))
+    s = {"draft_logits": dl, "draft": top, "uniforms": torch.rand((B, K + 1), generator=g, device="cuda") * 0.9,
+         "temperature": 1.0, "top_k": k, "top_p": 1.0 if kind != "random" else 0.9}
+    prev = rt.retrace_set_verify_schedule(rt.VERIFY_WINDOWS if windows else rt.VERIFY_FULL)
+    try:
+        check_against_oracle(rt, {"logits": tl}, s)
+    finally:
+        rt.retrace_set_verify_schedule(prev)
