@@ -229,6 +229,45 @@ struct ConditioningArgs {
   void* e_out;
 };
 
+// The conditioning of a round without packed rows (direct_rows_supported),
+// after a verification that left the argmax keys (keys) or the accepted lengths
+// (keys NULL).
+retrace_status enqueue_direct_conditioning(const ConditioningArgs& c, int B, int K, int d, unsigned long long* keys,
+                                           const int32_t* draft, int32_t* accept_len, int32_t* committed,
+                                           int32_t* bonus, int32_t* n_out, void* ws, const WsLayout& L,
+                                           const cudaEvent_t* phase_events, cudaStream_t stream) {
+  char* w = reinterpret_cast<char*>(ws);
+  TcCondArgs a{};
+  a.B = B;
+  a.K = K;
+  a.d = d;
+  a.do_correct = a.do_gate = 1;
+  a.Wc = c.Wc;
+  a.beta = c.beta;
+  a.r_out = w + L.swp;
+  a.compact_out = 1;
+  a.rpack = w + L.swp;
+  a.e = c.e;
+  a.Wv = c.Wv;
+  a.Wg = c.Wg;
+  a.ge = reinterpret_cast<float*>(w + L.ge);
+  a.e_out = c.e_out;
+  a.status = status_word(ws);
+  a.direct = 1;
+  a.keys = keys;
+  a.draft = draft;
+  a.accept_len = accept_len;
+  a.committed = committed;
+  a.bonus = bonus;
+  a.n_out = n_out;
+  a.hD = c.hD;
+  a.hT = c.hT;
+  RT_CUDA(launch_cond_tc(a, stream), "conditioning kernel launch");
+  if (phase_events)
+    for (int k = 2; k < 4; ++k) RT_CUDA(cudaEventRecord(phase_events[k], stream), "cudaEventRecord");
+  return RETRACE_OK;
+}
+
 // Correction (Eq. 6-7) and gated fusion (Eq. 8) of the rows j < n_b, after a
 // verification kernel has written accept_len and the unconditioned rows of
 // e_out and, on the tensor-core path, packed the [m; u] rows.  Records
@@ -502,9 +541,14 @@ retrace_status retrace_round(const void* logits, int64_t logits_row_stride,
   int32_t* rowmap = reinterpret_cast<int32_t*>(w + L.rowmap);
 
   if (phase_events) RT_CUDA(cudaEventRecord(phase_events[0], stream), "cudaEventRecord");
-  // The verification kernel packs the conditioned rows as sequences finish;
+  // Few sequences verified in one pass: the conditioning reads the carried
+  // rows where they lie (the ablations, a per-position e and every row's argmax
+  // as an output take the general path).
+  const bool direct = tc && flags == 0 && !dense && !target_argmax && direct_rows_supported(B, K, d) &&
+                      verify_windows(B, K, V, (int)elem_size(dtype), true, false, nullptr) == 1;
+  // Otherwise verification packs the conditioned rows as sequences finish;
   // they claim packed rows from a counter that starts at zero.
-  if (tc) RT_CUDA(cudaMemsetAsync(sync, 0, L.sync_bytes, stream), "cudaMemsetAsync(sync)");
+  if (tc && !direct) RT_CUDA(cudaMemsetAsync(sync, 0, L.sync_bytes, stream), "cudaMemsetAsync(sync)");
   if (tc) {
     TcRoundArgs ra{};
     ra.logits = logits;
@@ -571,10 +615,11 @@ retrace_status retrace_round(const void* logits, int64_t logits_row_stride,
   va.e_out = e_out;
   va.d = d;
   va.hD = hD;
+  va.keys_only = direct ? 1 : 0;
   va.cond_copy = ablation == RETRACE_COND_NONE ? kCondCopyE
                  : ablation == RETRACE_COND_OVERWRITE ? kCondCopyM
                                                       : kCondCopyKeep;
-  if (tc) {
+  if (tc && !direct) {
     va.hT = hT;
     va.e_dense = dense;
     va.apack = w + L.apack;
@@ -593,6 +638,9 @@ retrace_status retrace_round(const void* logits, int64_t logits_row_stride,
     return RETRACE_OK;
   }
   ConditioningArgs c{hD, hT, e, e_batch_stride, e_pos_stride, dense, Wc, Wv, Wg, beta, e_out};
+  if (direct)
+    return enqueue_direct_conditioning(c, B, K, d, va.keys, draft, accept_len, committed, bonus, n_out, ws, L,
+                                       phase_events, stream);
   if ((st = enqueue_conditioning(c, dtype, B, K, d, tc, ablation == RETRACE_COND_RAW, accept_len, ws, L,
                                  phase_events, stream)) != RETRACE_OK)
     return st;
@@ -684,8 +732,9 @@ retrace_status retrace_round_sampled(const void* target_logits, int64_t target_r
   uint32_t* sync = reinterpret_cast<uint32_t*>(w + L.sync);
 
   if (phase_events) RT_CUDA(cudaEventRecord(phase_events[0], stream), "cudaEventRecord");
+  const bool direct = tc && !dense && direct_rows_supported(B, K, d);  // as in retrace_round
   // the finalize kernel packs the conditioned rows behind a counter at zero
-  if (tc) RT_CUDA(cudaMemsetAsync(sync, 0, L.sync_bytes, stream), "cudaMemsetAsync(sync)");
+  if (tc && !direct) RT_CUDA(cudaMemsetAsync(sync, 0, L.sync_bytes, stream), "cudaMemsetAsync(sync)");
   SampledArgs a{};
   a.tlogits = target_logits;
   a.t_row = target_row_stride;
@@ -710,9 +759,9 @@ retrace_status retrace_round_sampled(const void* target_logits, int64_t target_r
   a.e = e;
   a.e_batch_stride = e_batch_stride;
   a.e_pos_stride = e_pos_stride;
-  a.e_out = e_out;
+  a.e_out = direct ? nullptr : e_out;
   a.d = d;
-  if (tc) {
+  if (tc && !direct) {
     a.hD = hD;
     a.hT = hT;
     a.e_dense = dense;
@@ -724,6 +773,9 @@ retrace_status retrace_round_sampled(const void* target_logits, int64_t target_r
   RT_CUDA(launch_verify_sampled(a, dtype, stream), "sampled verification launch");
   if (phase_events) RT_CUDA(cudaEventRecord(phase_events[1], stream), "cudaEventRecord");
   ConditioningArgs c{hD, hT, e, e_batch_stride, e_pos_stride, dense, Wc, Wv, Wg, beta, e_out};
+  if (direct)
+    return enqueue_direct_conditioning(c, B, K, d, nullptr, draft, accept_len, nullptr, nullptr, nullptr, ws, L,
+                                       phase_events, stream);
   if ((st = enqueue_conditioning(c, dtype, B, K, d, tc, false, accept_len, ws, L, phase_events, stream)) !=
       RETRACE_OK)
     return st;

@@ -1132,6 +1132,69 @@ struct GateBiasParams {
   float* ge;
 };
 
+// A round of few sequences without packed rows (DIRECT).  Sequence b has the KP
+// tile rows from b KP on (KP = K - 1 rounded up to 8; those past n_b compute
+// nothing that is stored), so the row tile's size is known on the host, and
+// the correction reads the carried rows where they lie: m_j and u_j of a
+// sequence are consecutive rows of hD and hT, one box per sequence and k-block.
+// Every warp finds the accepted lengths for itself from the argmax keys, so
+// no kernel stands between verification and the correction.  Warps 2-7 of the
+// correction write the outputs of verification and the rows j >= n_b of e~, the
+// gate's first CTA zeroes the keys.
+struct DirectRows {
+  int B, K, KP;
+  unsigned long long* keys;  // argmax keys of the verification (NULL: accept_len is given)
+  const int32_t* draft;
+  int32_t* accept_len;
+  int32_t* committed;
+  int32_t* bonus;
+  int32_t* n_out;            // optional
+  const __nv_bfloat16* hD;   // m, for the correction's epilogue
+  const __nv_bfloat16* e;
+  __nv_bfloat16* e_out;
+};
+constexpr int kDirectChunks = 3;  // (sequence, row) pairs per lane: B K <= 32 * kDirectChunks
+
+// Accepted length of sequence `lane` (lanes below B; the others return K): the
+// whole warp.  Read from accept_len once decided, else from the keys: the
+// first of the K drafts that is not its row's argmax, from ballots over 32
+// (sequence, row) pairs at a time.  The draft tokens are inputs, read before
+// the wait on verification.
+struct DirectDrafts {
+  int tok[kDirectChunks];  // of (sequence, row) pair 32 c + lane
+};
+__device__ __forceinline__ DirectDrafts direct_drafts(const DirectRows& q, int lane) {
+  DirectDrafts t;
+#pragma unroll
+  for (int c = 0; c < kDirectChunks; ++c) t.tok[c] = c * 32 + lane < q.B * q.K ? __ldg(q.draft + c * 32 + lane) : -1;
+  return t;
+}
+__device__ __forceinline__ int direct_accepted(const DirectRows& q, const DirectDrafts& t, bool decided, int lane) {
+  const int B = q.B, K = q.K;
+  if (decided) {
+    const int A = lane < B ? __ldcg(q.accept_len + lane) : K;
+    return min(max(A, 0), K);
+  }
+  bool miss[kDirectChunks];
+#pragma unroll
+  for (int c = 0; c < kDirectChunks; ++c) {
+    const int x = c * 32 + lane, b = x / K;
+    miss[c] = x < B * K && (int)key_index(__ldcg(q.keys + (long long)b * (K + 1) + (x - b * K))) != t.tok[c];
+  }
+  int A = K;
+#pragma unroll
+  for (int c = 0; c < kDirectChunks; ++c) {
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, miss[c]);
+    const int lo = lane * K - c * 32, hi = lo + K;  // this sequence's rows in the chunk
+    if (lane < B && A == K && lo < 32 && hi > 0) {
+      const unsigned above = lo > 0 ? ~0u << lo : ~0u, below = hi < 32 ? (1u << hi) - 1u : ~0u;
+      const unsigned own = m & above & below;
+      if (own) A = __ffs(own) - 1 - lo;
+    }
+  }
+  return A;
+}
+
 struct SwapClusterParams {
   const int32_t* R;
   int d;
@@ -1157,6 +1220,7 @@ struct SwapClusterParams {
   __nv_bfloat16* e_out;
   const int32_t* rowmap;
   uint32_t* status;
+  DirectRows direct;  // DIRECT only
 };
 
 // The sum over the cluster's S partials and the epilogue of `total` positions
@@ -1165,9 +1229,9 @@ struct SwapClusterParams {
 // positions and, for each, the loads of NS partials in flight: with one
 // position and one partial at a time a CTA with 80 rows took a chain of
 // twenty round trips.  The partials are added in rank order.
-template <int NB, int NS>
+template <bool DIRECT, int NB, int NS>
 __device__ __forceinline__ void swap_correction_rows(const SwapClusterParams& p, uint32_t P, int mt, int row0, int l0,
-                                                     int total) {
+                                                     int total, const int* s_A) {
   const int d = p.d, S = p.S, n0 = mt * 128;
   for (int x0 = threadIdx.x; x0 < total; x0 += NB * SW_THREADS) {
     float4 c[NB];
@@ -1178,8 +1242,15 @@ __device__ __forceinline__ void swap_correction_rows(const SwapClusterParams& p,
     for (int q = 0; q < NB; ++q) {
       // (features past d, in the last tile: d + 127 < 2 d keeps their loads inside the packed rows)
       const int x = min(x0 + q * SW_THREADS, total - 1), l = l0 + x / 32, f = (x % 32) * 4, g = row0 + l;
-      mw[q] = __ldcg(reinterpret_cast<const uint2*>(p.apack + (long long)g * 2 * d + n0 + f));
-      orow[q] = p.compact_out ? g : __ldcg(p.rowmap + g);
+      if constexpr (DIRECT) {
+        const int b = l / p.direct.KP, j = l - b * p.direct.KP, A = s_A[b];
+        orow[q] = j < p.direct.K - 1 - A && n0 + f < d ? l : -1;
+        if (orow[q] >= 0)
+          mw[q] = __ldg(reinterpret_cast<const uint2*>(p.direct.hD + ((long long)b * p.direct.K + A + 1 + j) * d + n0 + f));
+      } else {
+        mw[q] = __ldcg(reinterpret_cast<const uint2*>(p.apack + (long long)g * 2 * d + n0 + f));
+        orow[q] = n0 + f >= d ? -1 : p.compact_out ? g : __ldcg(p.rowmap + g);
+      }
       at[q] = P + (uint32_t)(l * 512 + f * 4);
       c[q] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
@@ -1198,16 +1269,16 @@ __device__ __forceinline__ void swap_correction_rows(const SwapClusterParams& p,
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
       const int x = x0 + q * SW_THREADS;
-      if (x < total && n0 + (x % 32) * 4 < d)
+      if (x < total && orow[q] >= 0)
         *reinterpret_cast<uint2*>(p.r_out + orow[q] * d + n0 + (x % 32) * 4) =
             make_uint2(pack_bf16x2(bf16_lo(mw[q].x) + p.beta * c[q].x, bf16_hi(mw[q].x) + p.beta * c[q].y),
                        pack_bf16x2(bf16_lo(mw[q].y) + p.beta * c[q].z, bf16_hi(mw[q].y) + p.beta * c[q].w));
     }
   }
 }
-template <int NB, int NS>
+template <bool DIRECT, int NB, int NS>
 __device__ __forceinline__ void swap_gate_rows(const SwapClusterParams& p, uint32_t P, int mt, int row0, int l0,
-                                               int total) {
+                                               int total, const int* s_A) {
   const int d = p.d, S = p.S;
   const int f = ((int)threadIdx.x % 16) * 4, n = mt * 64 + f;  // the same features at every step
   if (n >= d) return;  // past the last feature (no barrier below)
@@ -1226,8 +1297,13 @@ __device__ __forceinline__ void swap_gate_rows(const SwapClusterParams& p, uint3
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
       const int l = l0 + min(x0 + q * SW_THREADS, total - 1) / 16;
-      orow[q] = __ldcg(p.rowmap + row0 + l);
-      if (!p.ge) ew[q] = __ldcg(reinterpret_cast<const uint2*>(p.e + (long long)(row0 + l) * d + n));
+      if constexpr (DIRECT) {
+        const int b = l / p.direct.KP, j = l - b * p.direct.KP;
+        orow[q] = j < p.direct.K - 1 - s_A[b] ? (long long)b * p.direct.K + j : -1;
+      } else {
+        orow[q] = __ldcg(p.rowmap + row0 + l);
+      }
+      if (!DIRECT && !p.ge) ew[q] = __ldcg(reinterpret_cast<const uint2*>(p.e + (long long)(row0 + l) * d + n));
       at[q] = P + (uint32_t)(l * 512 + f * 4);
       v[q] = a[q] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
@@ -1252,7 +1328,7 @@ __device__ __forceinline__ void swap_gate_rows(const SwapClusterParams& p, uint3
     }
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
-      if (x0 + q * SW_THREADS >= total) continue;
+      if (x0 + q * SW_THREADS >= total || (DIRECT && orow[q] < 0)) continue;
       const float s0 = fast_sigmoid(a[q].x + gb.x), s1 = fast_sigmoid(a[q].y + gb.y);
       const float s2 = fast_sigmoid(a[q].z + gb.z), s3 = fast_sigmoid(a[q].w + gb.w);
       *reinterpret_cast<uint2*>(p.e_out + orow[q] * d + n) =
@@ -1262,6 +1338,7 @@ __device__ __forceinline__ void swap_gate_rows(const SwapClusterParams& p, uint3
   }
 }
 
+template <bool DIRECT>
 __global__ void __launch_bounds__(SW_THREADS, 1)
     swap_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA2,
                         const __grid_constant__ CUtensorMap tmA3, const __grid_constant__ RowMaps tmB,
@@ -1272,6 +1349,7 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
   __shared__ __align__(8) uint64_t bar_acc;
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_abort;
+  __shared__ int s_A[32];  // DIRECT: the sequences' accepted lengths
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int S = p.S, d = p.d;
   const uint32_t rank = cluster_rank();
@@ -1310,7 +1388,10 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
   auto load_a = [&](int mt, int kb, uint32_t s) {
     const uint32_t a_dst = base + s * (uint32_t)SW_A_BYTES, bar = smem_u32(&bar_full[s]);
     mbar_arrive_expect_tx(bar, (uint32_t)SW_A_BYTES);
-    if (kb >= p.nkb_r) {
+    if (DIRECT && !p.gate) {  // W_c's m columns, then its u columns
+      const bool u = kb >= p.nkb_r;
+      tma_load_2d(a_dst, u ? &tmA2 : &tmA, (u ? kb - p.nkb_r : kb) * BK, mt * 128, bar);
+    } else if (kb >= p.nkb_r) {
       // the gate's e half: zeros (columns past W_v's end) over the rows of W_g[:, :d]
       tma_load_2d(a_dst, &tmA, p.nkb_r * BK, mt * 64, bar);
       tma_load_2d(a_dst + (uint32_t)(SW_A_BYTES / 2), &tmA3, (kb - p.nkb_r) * BK, mt * 64, bar);
@@ -1332,9 +1413,50 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
   // end (the memory is idle then) and the first k-blocks run.
   if (p.bias.ge && warp >= 2)
     gate_bias_share(p.bias.e, p.bias.Wg, p.bias.ge, d, (int)blockIdx.x * 6 + warp - 2, (int)gridDim.x * 6, lane);
+  DirectDrafts drafts;
+  if (DIRECT && !p.gate && p.direct.keys) drafts = direct_drafts(p.direct, lane);
   pdl_wait();  // R and the activation rows come from the previous kernels
-  const int R = *(volatile const int32_t*)p.R;
-  const SwapCut cut = swap_cut(R, p.mtiles, clusters);
+  int R;
+  SwapCut cut;
+  int my_A = 0, boxes = 0;  // DIRECT: accepted length of sequence `lane`; sequences with carried rows
+  if constexpr (DIRECT) {
+    const DirectRows& q = p.direct;
+    my_A = direct_accepted(q, drafts, p.gate || !q.keys, lane);
+    boxes = __popc(__ballot_sync(0xFFFFFFFFu, my_A < q.K - 1));
+    R = q.B * q.KP;
+    cut = {boxes > 0 ? 1 : 0, (R + 15) / 16 * 16};
+    if (warp == 0) s_A[lane] = my_A;  // for the epilogue, a block barrier later
+    if (warp >= 2) {
+      const int w = (int)blockIdx.x * 6 + warp - 2, nw = (int)gridDim.x * 6;
+      if (!p.gate) {
+        // the outputs of verification, and the rows of e~ that carry nothing
+        if (q.keys) {
+          for (int b = w; b < q.B; b += nw) {
+            const int A = __shfl_sync(0xFFFFFFFFu, my_A, b);
+            const unsigned long long* key = q.keys + (long long)b * (q.K + 1);
+            for (int i = lane; i <= q.K; i += 32) q.committed[(long long)b * (q.K + 1) + i] = i <= A ? (int)key_index(__ldcg(key + i)) : -1;
+            if (lane == 0) {
+              q.accept_len[b] = A;
+              q.bonus[b] = (int)key_index(__ldcg(key + A));
+              if (q.n_out) q.n_out[b] = max(0, q.K - 1 - A);
+            }
+          }
+        }
+        for (int x = w; x < q.B * q.K; x += nw) {
+          const int b = x / q.K, j = x - b * q.K;
+          if (j < q.K - 1 - __shfl_sync(0xFFFFFFFFu, my_A, b)) continue;  // the gate writes it
+          const uint4* src = reinterpret_cast<const uint4*>(q.e);
+          uint4* dst = reinterpret_cast<uint4*>(q.e_out + (long long)x * d);
+          for (int v = lane; v < d / 8; v += 32) dst[v] = __ldg(src + v);
+        }
+      } else if (blockIdx.x == 0 && q.keys) {
+        for (int x = threadIdx.x - 64; x < q.B * (q.K + 1); x += SW_THREADS - 64) q.keys[x] = 0ull;
+      }
+    }
+  } else {
+    R = *(volatile const int32_t*)p.R;
+    cut = swap_cut(R, p.mtiles, clusters);
+  }
   const int units = p.mtiles * cut.ntiles;
   const int box = swap_box_rows(cut.tile_n);
   const int nst = swap_stages(p.stage_bytes, box > 0 ? box : SW_ROW_STEP);  // >= p.pre
@@ -1367,9 +1489,29 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
     const int mma_n = (rows + 15) / 16 * 16;
     if (warp == 0) {
       // ---------------- TMA producer ----------------
-      if (lane == 0) {
+      if (lane == 0 || (DIRECT && !p.gate)) {
         int i = 0;
         for (; i < kb1 - kb0; ++i, advance()) {
+          if constexpr (DIRECT) {
+            if (!p.gate) {  // the whole warp: lane 0 the weights, lane b the rows of sequence b
+              int ok = 1;
+              if (lane == 0) {
+                if (i >= pre) {
+                  ok = mbar_wait_bounded(smem_u32(&bar_empty[s]), ph ^ 1u, &s_abort) ? 1 : 0;
+                  if (ok) load_a(mt, kb0 + i, s);
+                }
+                if (ok) mbar_arrive_expect_tx(smem_u32(&bar_full[s]), (uint32_t)(boxes * p.direct.KP * BK * 2));
+              }
+              if (!__shfl_sync(0xFFFFFFFFu, ok, 0)) break;
+              if (my_A < p.direct.K - 1) {  // (lanes past B have my_A = K)
+                const int kb = kb0 + i;
+                const bool u = kb >= p.nkb_r;
+                tma_load_2d(b_base + s * b_bytes + (uint32_t)(lane * p.direct.KP * BK * 2), &tmB.m[u ? 1 : 0],
+                            (u ? kb - p.nkb_r : kb) * BK, lane * p.direct.K + my_A + (u ? 0 : 1), smem_u32(&bar_full[s]));
+              }
+              continue;
+            }
+          }
           if (i >= pre) {
             if (!mbar_wait_bounded(smem_u32(&bar_empty[s]), ph ^ 1u, &s_abort)) break;
             load_a(mt, kb0 + i, s);
@@ -1379,7 +1521,7 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
           if (kb < p.nkb_r) tma_load_2d(b_base + s * b_bytes, mb, kb * BK, row0, smem_u32(&bar_full[s]));
           else tma_load_2d(b_base + s * b_bytes, me, (kb - p.nkb_r) * BK, row0, smem_u32(&bar_full[s]));
         }
-        if (i < kb1 - kb0) {
+        if (i < kb1 - kb0 && lane == 0) {
           // a wait expired: flag it, let the copies in flight land
           raise_abort(&s_abort, p.status);
           volatile int never = 0;
@@ -1446,11 +1588,11 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
       const int l0 = (int)rank * rows / S, l1 = ((int)rank + 1) * rows / S;
       const int total = (l1 - l0) * (p.gate ? 16 : 32);  // four features each
       if (p.gate) {
-        if (total <= SW_THREADS) swap_gate_rows<1, 8>(p, smem_u32(P), mt, row0, l0, total);
-        else swap_gate_rows<4, 2>(p, smem_u32(P), mt, row0, l0, total);
+        if (total <= SW_THREADS) swap_gate_rows<DIRECT, 1, 8>(p, smem_u32(P), mt, row0, l0, total, s_A);
+        else swap_gate_rows<DIRECT, 4, 2>(p, smem_u32(P), mt, row0, l0, total, s_A);
       } else {
-        if (total <= SW_THREADS) swap_correction_rows<1, 8>(p, smem_u32(P), mt, row0, l0, total);
-        else swap_correction_rows<4, 2>(p, smem_u32(P), mt, row0, l0, total);
+        if (total <= SW_THREADS) swap_correction_rows<DIRECT, 1, 8>(p, smem_u32(P), mt, row0, l0, total, s_A);
+        else swap_correction_rows<DIRECT, 4, 2>(p, smem_u32(P), mt, row0, l0, total, s_A);
       }
     }
     fence_proxy_async_shared();  // the partial's space goes back to the copies of the next unit
@@ -1485,6 +1627,14 @@ cudaError_t launch_wait_selftest(int kind, const uint32_t* flag, uint32_t target
 
 bool tc_supported(retrace_dtype dtype, int d) {
   return dtype == RETRACE_BF16 && d >= 128 && d % 8 == 0;
+}
+
+bool direct_rows_supported(int B, int K, int d) {
+  // K >= 5: the tile rows are at most twice the carried ones.  The corrected
+  // signal's tile rows lie in the swp region.
+  const long long rows = (long long)B * direct_tile_rows(K);
+  return K >= 5 && rows <= kDirectMaxRows && B <= 32 && (long long)B * K <= 32 * kDirectChunks &&
+         (size_t)(rows * d) * 2 <= swap_part_bytes(B, K, d);
 }
 
 cudaError_t launch_pack(const PackArgs& a, cudaStream_t stream) {
@@ -1608,7 +1758,7 @@ static int swap_cluster_capacity(int dev, int S, int smem, cudaError_t* err) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int m = 0;
-    if ((*err = cudaOccupancyMaxActiveClusters(&m, swap_cluster_kernel, &cfg)) != cudaSuccess) return 0;
+    if ((*err = cudaOccupancyMaxActiveClusters(&m, swap_cluster_kernel<false>, &cfg)) != cudaSuccess) return 0;
     n = m > 0 ? m : -1;
     slot.store(n, std::memory_order_release);
   }
@@ -1616,12 +1766,14 @@ static int swap_cluster_capacity(int dev, int S, int smem, cudaError_t* err) {
 }
 
 // Cluster size of a small-R GEMM: the one with the least estimated time at
-// three quarters of the possible rows (R itself is known on the device only).
+// three quarters of the possible rows (R itself is known on the device only;
+// direct rows: one tile of all the tile rows).
 // A wave of units costs its k-blocks, 2 (128 + N) cycles each (the stage's
 // bytes in and out of shared memory), plus the drain and the sum of the
 // partial (about 24 cycles per row of the tile) and the fixed start and end.
-static cudaError_t swap_pick_splits(int dev, int smem, int rmax, int mtiles, int nkb, int* S_out, int* clusters) {
-  const int Rt = (3 * rmax + 3) / 4;
+static cudaError_t swap_pick_splits(int dev, int smem, int rmax, bool direct, int mtiles, int nkb, int* S_out,
+                                    int* clusters) {
+  const int Rt = direct ? rmax : (3 * rmax + 3) / 4;
   long long best = -1;
   cudaError_t err = cudaSuccess;
   for (int S = 8; S >= 1; --S) {
@@ -1629,7 +1781,7 @@ static cudaError_t swap_pick_splits(int dev, int smem, int rmax, int mtiles, int
     const int cap = swap_cluster_capacity(dev, S, smem, &err);
     if (err != cudaSuccess) return err;
     if (cap == 0) continue;
-    const SwapCut cut = swap_cut(Rt, mtiles, cap);
+    const SwapCut cut = direct ? SwapCut{1, (Rt + 15) / 16 * 16} : swap_cut(Rt, mtiles, cap);
     const long long waves = ((long long)mtiles * cut.ntiles + cap - 1) / cap;
     const long long cost = waves * ((long long)((nkb + S - 1) / S) * 2 * (128 + cut.tile_n) + 24 * cut.tile_n + 2500);
     if (best < 0 || cost < best) {
@@ -1658,7 +1810,9 @@ static bool encode_row_maps(RowMaps* maps, const void* base, uint64_t inner, int
 // reads.  Past the operands' ends (d no multiple of the tiles) the copies fill
 // zeros and the epilogues store nothing.
 static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
-  const int rmax = (int)((long long)a.B * (a.K - 1));
+  const bool direct = a.direct;
+  // rows of the operands: tile rows (direct), or the most there can be
+  const int rmax = direct ? a.B * direct_tile_rows(a.K) : (int)((long long)a.B * (a.K - 1));
   const int d = a.d;
   DeviceInfo info;
   cudaError_t err = device_info(&info);
@@ -1666,8 +1820,11 @@ static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
   const int dev = info.device;
   static std::atomic<int> attr_done[64];
   if (!attr_done[dev & 63].load(std::memory_order_acquire)) {
-    err = cudaFuncSetAttribute(swap_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SW_SMEM_MAX);
-    if (err != cudaSuccess) return err;
+    // (the two forms have the same threads and, but for 128 bytes, shared memory)
+    for (auto kern : {swap_cluster_kernel<false>, swap_cluster_kernel<true>}) {
+      err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SW_SMEM_MAX);
+      if (err != cudaSuccess) return err;
+    }
     attr_done[dev & 63].store(1, std::memory_order_release);
   }
   const int box_max = swap_box_rows(std::min(256, (rmax + 15) / 16 * 16));
@@ -1687,11 +1844,16 @@ static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
   sp.tmem_cols = tmem_cols;
   sp.rowmap = a.rowmap;
   sp.status = a.status;
+  if (direct)
+    sp.direct = {a.B, a.K, direct_tile_rows(a.K), a.keys, a.draft, a.accept_len, a.committed, a.bonus, a.n_out,
+                 reinterpret_cast<const __nv_bfloat16*>(a.hD), reinterpret_cast<const __nv_bfloat16*>(a.e),
+                 reinterpret_cast<__nv_bfloat16*>(a.e_out)};
   // whole row tiles side by side where the resident clusters can take every
   // row so, else all of them in turn over the units
   auto grid_of = [&](const SwapClusterParams& c, int clusters) {
     const int fit = clusters / c.mtiles, most = (rmax + SW_ROW_STEP - 1) / SW_ROW_STEP;
-    if (fit * 256 >= rmax) clusters = c.mtiles * std::min(fit, most);
+    if (direct) clusters = std::min(clusters, c.mtiles);
+    else if (fit * 256 >= rmax) clusters = c.mtiles * std::min(fit, most);
     return dim3((unsigned)(clusters * c.S));
   };
   GateBiasParams gp{};
@@ -1700,23 +1862,38 @@ static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
   gp.Wg = reinterpret_cast<const __nv_bfloat16*>(a.Wg);
   gp.ge = a.ge;
   if (a.do_correct) {
-    CUtensorMap mA;
+    CUtensorMap mA, mA2;
     RowMaps mB;
-    if (encode_tensor_map_2d(&mA, a.Wc, 2 * du, du, 4 * du, BK, 128) != CUDA_SUCCESS ||
-        !encode_row_maps(&mB, a.apack, 2 * du, rmax, 4 * du))
-      return cudaErrorInvalidValue;
     SwapClusterParams c = sp;
     c.mtiles = (d + 127) / 128;
-    c.nkb = c.nkb_r = (2 * d + BK - 1) / BK;
+    if (direct) {
+      // the m and u halves apart: zeros past column d of either
+      const uint64_t all = (uint64_t)a.B * a.K;
+      const uint32_t box = (uint32_t)direct_tile_rows(a.K);
+      if (encode_tensor_map_2d(&mA, a.Wc, du, du, 4 * du, BK, 128) != CUDA_SUCCESS ||
+          encode_tensor_map_2d(&mA2, static_cast<const __nv_bfloat16*>(a.Wc) + d, du, du, 4 * du, BK, 128) != CUDA_SUCCESS ||
+          encode_tensor_map_2d(&mB.m[0], a.hD, du, all, 2 * du, BK, box) != CUDA_SUCCESS ||
+          encode_tensor_map_2d(&mB.m[1], a.hT, du, all, 2 * du, BK, box) != CUDA_SUCCESS)
+        return cudaErrorInvalidValue;
+      c.row_maps = 2;
+      c.nkb_r = (d + BK - 1) / BK;
+      c.nkb = 2 * c.nkb_r;
+    } else {
+      if (encode_tensor_map_2d(&mA, a.Wc, 2 * du, du, 4 * du, BK, 128) != CUDA_SUCCESS ||
+          !encode_row_maps(&mB, a.apack, 2 * du, rmax, 4 * du))
+        return cudaErrorInvalidValue;
+      mA2 = mA;
+      c.nkb = c.nkb_r = (2 * d + BK - 1) / BK;
+    }
     c.apack = reinterpret_cast<const __nv_bfloat16*>(a.apack);
     c.beta = a.beta;
     c.r_out = reinterpret_cast<__nv_bfloat16*>(a.r_out);
     c.compact_out = a.compact_out;
     if (a.do_gate && !a.e_dense) c.bias = gp;
     int clusters = 0;
-    if ((err = swap_pick_splits(dev, smem, rmax, c.mtiles, c.nkb, &c.S, &clusters)) != cudaSuccess) return err;
-    err = launch_dependent(swap_cluster_kernel, grid_of(c, clusters), dim3(SW_THREADS), (size_t)smem, stream,
-                           (unsigned)c.S, mA, mA, mA, mB, mB, c);
+    if ((err = swap_pick_splits(dev, smem, rmax, direct, c.mtiles, c.nkb, &c.S, &clusters)) != cudaSuccess) return err;
+    err = launch_dependent(direct ? swap_cluster_kernel<true> : swap_cluster_kernel<false>, grid_of(c, clusters),
+                           dim3(SW_THREADS), (size_t)smem, stream, (unsigned)c.S, mA, mA2, mA, mB, mB, c);
     if (err != cudaSuccess) return err;
   }
   if (a.do_gate) {
@@ -1742,9 +1919,10 @@ static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
     g.ge = a.e_dense ? nullptr : a.ge;
     g.e_out = reinterpret_cast<__nv_bfloat16*>(a.e_out);
     int clusters = 0;
-    if ((err = swap_pick_splits(dev, smem, rmax, g.mtiles, g.nkb, &g.S, &clusters)) != cudaSuccess) return err;
-    err = launch_dependent(swap_cluster_kernel, grid_of(g, clusters), dim3(SW_THREADS), (size_t)smem, stream,
-                           (unsigned)g.S, mA, mA2, mA3, mB, a.e_dense ? mE : mB, g);
+    if ((err = swap_pick_splits(dev, smem, rmax, direct, g.mtiles, g.nkb, &g.S, &clusters)) != cudaSuccess) return err;
+    err = launch_dependent(direct ? swap_cluster_kernel<true> : swap_cluster_kernel<false>, grid_of(g, clusters),
+                           dim3(SW_THREADS), (size_t)smem, stream, (unsigned)g.S, mA, mA2, mA3, mB,
+                           a.e_dense ? mE : mB, g);
     if (err != cudaSuccess) return err;
   }
   return cudaSuccess;
@@ -1753,7 +1931,7 @@ static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
 cudaError_t launch_cond_tc(const TcCondArgs& a, cudaStream_t stream) {
   const long long rmax = (long long)a.B * (a.K - 1);
   if (rmax <= 0 || (!a.do_correct && !a.do_gate)) return cudaSuccess;
-  if (rmax <= kSwapMaxRows) return launch_cond_swap(a, stream);
+  if (a.direct || rmax <= kSwapMaxRows) return launch_cond_swap(a, stream);
   const long long tiles_max = (rmax + 2 * BM - 1) / (2 * BM) *
                               ((a.do_correct ? (a.d + 255) / 256 : 0) + (a.do_gate ? (a.d + 127) / 128 : 0));
   cudaError_t err;

@@ -46,8 +46,8 @@ constexpr int kWindowRows = 4;          // rows per pass of windowed verificatio
 constexpr int kMaxWindowPasses = 16;    // most passes of windowed verification
 // Small-R conditioning: at most kSwapMaxRows packed rows, the GEMMs with the
 // weights as the M side in split-K clusters, which sum their partials in shared
-// memory.  The workspace keeps the region that partials in global memory
-// took (swap_part_bytes), so that its size for a shape stays what it was.
+// memory.  The region of swap_part_bytes in the workspace holds the corrected
+// signal of a round without packed rows (direct rows, below).
 constexpr int kSwapMaxRows = 1024;
 constexpr int kSwapMaxCtas = 256;
 inline size_t swap_part_bytes(long long B, long long K, long long d) {
@@ -69,6 +69,11 @@ inline size_t pair_split_bytes(long long B, long long K, long long d, size_t ele
   if (rmax <= 0 || elem != 2 || d <= 0 || d % 256 != 0 || swap_part_bytes(B, K, d) != 0) return 0;
   return (size_t)kPairSplitTiles * 2 * 2 * 128 * 256 * 4;
 }
+// A round of few sequences whose conditioning reads the carried rows where they
+// lie (described at DirectRows in cond_tc.cu): tile rows per sequence, and the
+// most tile rows of a call.
+inline int direct_tile_rows(int K) { return (K - 1 + 7) / 8 * 8; }
+constexpr int kDirectMaxRows = 64;
 struct WsLayout {
   size_t status, sync, sync_bytes, keys, tickets, live, poff, counts, ge, r, apack, epack, rowmap, lrz, lrt, lrrho, skeys, swp, total;
 };
@@ -209,6 +214,9 @@ struct VerifyArgs {
   // leaves them to the conditioning kernels, kCondCopyE writes e (no
   // conditioning), kCondCopyM writes m_j = hD[b, A_b+1+j] (overwrite).
   int cond_copy;
+  // One pass that only folds the argmax keys: a direct-rows conditioning
+  // decides the sequences, writes the outputs and zeroes the keys.
+  int keys_only;
 };
 constexpr int kCondCopyKeep = 0;
 constexpr int kCondCopyE = 1;
@@ -220,7 +228,7 @@ cudaError_t launch_verify(const VerifyArgs& a, retrace_dtype dtype, cudaStream_t
 cudaError_t launch_verify_copies(const VerifyArgs& a, retrace_dtype dtype, cudaStream_t stream);
 int set_verify_schedule(int mode);  // RETRACE_VERIFY_*; previous mode, or -1
 // Row windows greedy verification takes for this call: writes the window
-// starts (n + 1 entries, at most kMaxWindowPasses + 1) and returns the number
+// starts (n + 1 entries, at most kMaxWindowPasses + 1; start may be NULL) and returns the number
 // of passes n (1: the one-pass schedule).
 int verify_windows(int B, int K, int V, int elem_bytes, bool have_workspace, bool argmax_out, int* start);
 
@@ -369,10 +377,24 @@ struct TcCondArgs {
   const int32_t* rowmap;
   uint32_t* sync;
   uint32_t* status;
+  // Direct rows (direct_rows_supported): do_correct and do_gate, broadcast e,
+  // r_out = rpack in the swp region; the correction also writes the outputs of
+  // verification (from its keys; keys NULL: accept_len is given) and the rows
+  // j >= n_b of e_out.
+  int direct;
+  unsigned long long* keys;
+  const int32_t* draft;
+  int32_t* accept_len;
+  int32_t* committed;
+  int32_t* bonus;
+  int32_t* n_out;
+  const void* hD;
+  const void* hT;
   // CTA-pair path: fp32 accumulators of the split gate tiles, pair_split_bytes (NULL: no split tiles)
   float* split_part;
 };
 cudaError_t launch_cond_tc(const TcCondArgs& a, cudaStream_t stream);
+bool direct_rows_supported(int B, int K, int d);
 // The bounded waits of the pipelined kernels on a caller-controlled condition.
 cudaError_t launch_wait_selftest(int kind, const uint32_t* flag, uint32_t target, uint32_t* status,
                                  cudaStream_t stream);

@@ -700,6 +700,8 @@ inline int window_bounds(int K1, int* start) {
 
 int verify_windows(int B, int K, int V, int elem_bytes, bool have_workspace, bool argmax_out, int* start) {
   const int K1 = K + 1;
+  int bounds[kMaxWindowPasses + 1];
+  if (!start) start = bounds;
   const int n = window_bounds(K1, start);
   const int mode = g_schedule.load(std::memory_order_relaxed);
   const long long wave = (long long)B * V * elem_bytes;
@@ -826,6 +828,11 @@ cudaError_t launch_typed(const VerifyArgs& a, cudaStream_t stream) {
     // and verify_finish_kernel decides every sequence, writes the outputs
     // and does the copies over its grid (target_argmax, every row's argmax,
     // stays with the finalisers).
+    if (a.keys_only) {
+      p.windowed = 1;
+      verify_kernel<T><<<(unsigned)grid, kThreads, kCopyStageBytes, stream>>>(p);
+      return cudaGetLastError();
+    }
     const bool defer = a.R_count && a.B < info.sm_count;
     if (defer && !a.target_argmax && a.live && a.pass_counts && a.B <= kWindowMaxB) {
       p.windowed = 1;

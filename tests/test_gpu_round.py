@@ -322,3 +322,34 @@ def test_small_r_round_with_almost_nothing_to_condition(rt, R):
     for b in range(cfg.B):
         nb = int(want["n"][b])
         assert np.array_equal(got[b, nb:], np.broadcast_to(e, got[b, nb:].shape))
+
+
+@pytest.mark.parametrize("accept", ["mixed", "none", "all"])
+@pytest.mark.parametrize("B,K,V,d", [(1, 5, 515, 128), (1, 16, 1003, 2560), (1, 120, 64, 256), (2, 63, 200, 264), (3, 9, 640, 136),
+                                     (5, 12, 333, 1160), (8, 16, 4099, 512), (8, 17, 129, 256), (16, 6, 77, 512)])
+def test_round_of_few_sequences(rt, B, K, V, d, accept):
+    """Few sequences verified in one pass (no argmax output): the conditioning
+    decides them and reads the carried rows where they lie.  One to 16
+    sequences of 8 to 120 tile rows, all drafts accepted (nothing to
+    condition), none, and a mix with A = K-2, K-1 and K; twice on one workspace."""
+    cfg = CONFIGS[2].__class__("few", B, K, V, d, "bf16", 1.0, "uniform", seed_offset=B + K)
+    x = make_round_inputs(cfg, device="cuda")
+    top = torch.argmax(x["logits"][:, :K].float(), dim=-1).to(torch.int32)
+    x["draft"] = top.clone()
+    for b in range(B):
+        at = {"mixed": [0, K - 2, K - 1, K, 1][b % 5], "none": 0, "all": K}[accept]
+        if at < K:
+            x["draft"][b, at] = (top[b, at] + 1) % V
+    ws = rt.Workspace(B, K, V, d, torch.bfloat16)
+    want = oracle_round(x)
+    outs = [rt.run_round(x, ws) for _ in range(2)]
+    torch.cuda.synchronize()
+    assert ws.check() == 0
+    for out in outs:
+        assert_verify_exact(want, out.accept_len, out.committed, out.bonus)
+        np.testing.assert_array_equal(host_int(out.n), want["n"])
+        assert_close(out.e_out, want["e_tilde"], f"B={B} K={K} d={d}")
+        for b in range(B):
+            nb = int(want["n"][b])
+            assert torch.equal(out.e_out[b, nb:], x["e"].expand(K - nb, d))
+    assert torch.equal(outs[0].e_out, outs[1].e_out)
