@@ -117,6 +117,74 @@ __device__ __forceinline__ void copy_vectors(long long n, Load load, Store store
 }
 
 // ---------------------------------------------------------------------------
+// One warp of `nw`: rows w, w + nw, ... of ge = W_g[:, :d] e (d a multiple of
+// 8; W_g's rows `ld` elements apart).  The rows come in steps of 256 vectors
+// through two register buffers in turn, one loading while the other is
+// multiplied (a single buffer handed on by a copy waits for the copy: one
+// memory latency per step).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void gate_bias_share(const __nv_bfloat16* e, const __nv_bfloat16* Wg, float* ge, int d,
+                                                int ld, int w, int nw, int lane) {
+  const int vpr = d / 8, steps = (vpr + 255) / 256;
+  const uint4* ev = reinterpret_cast<const uint4*>(e);
+  struct Pos {
+    int row, step;
+  };
+  auto advance = [&](Pos& p) {
+    if (++p.step == steps) {
+      p.step = 0;
+      p.row += nw;
+    }
+  };
+  auto load = [&](uint4 (&x)[8], const Pos& p) {
+    if (p.row >= d) return;
+    const uint4* wr = reinterpret_cast<const uint4*>(Wg + (long long)p.row * ld);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int v = p.step * 256 + u * 32 + lane;
+      x[u] = v < vpr ? __ldcs(wr + v) : make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  float acc = 0.f;
+  auto use = [&](const uint4 (&x)[8], const Pos& p) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int v = p.step * 256 + u * 32 + lane;
+      if (v < vpr) {
+        const uint4 y = __ldg(ev + v);
+        const uint32_t xx[4] = {x[u].x, x[u].y, x[u].z, x[u].w}, yy[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          acc = fmaf(bf16_lo(xx[q]), bf16_lo(yy[q]), acc);
+          acc = fmaf(bf16_hi(xx[q]), bf16_hi(yy[q]), acc);
+        }
+      }
+    }
+    if (p.step + 1 == steps) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
+      if (lane == 0) ge[p.row] = acc;
+      acc = 0.f;
+    }
+  };
+  uint4 a[8], b[8];
+  Pos pa{w, 0}, pb{w, 0};
+  advance(pb);
+  load(a, pa);
+  while (pa.row < d) {
+    load(b, pb);
+    use(a, pa);
+    pa = pb;
+    advance(pa);
+    if (pb.row >= d) break;
+    load(a, pa);
+    use(b, pb);
+    pb = pa;
+    advance(pb);
+  }
+}
+
+// ---------------------------------------------------------------------------
 // Programmatic dependent launch: a kernel launched with the programmatic
 // stream-serialisation attribute may start once every CTA of the previous
 // kernel in the stream has called pdl_launch_dependents (or exited); it must

@@ -1412,7 +1412,7 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
   // before the accumulator is complete, compute it while the previous kernels
   // end (the memory is idle then) and the first k-blocks run.
   if (p.bias.ge && warp >= 2)
-    gate_bias_share(p.bias.e, p.bias.Wg, p.bias.ge, d, (int)blockIdx.x * 6 + warp - 2, (int)gridDim.x * 6, lane);
+    gate_bias_share(p.bias.e, p.bias.Wg, p.bias.ge, d, 2 * d, (int)blockIdx.x * 6 + warp - 2, (int)gridDim.x * 6, lane);
   DirectDrafts drafts;
   if (DIRECT && !p.gate && p.direct.keys) drafts = direct_drafts(p.direct, lane);
   pdl_wait();  // R and the activation rows come from the previous kernels
@@ -1609,7 +1609,7 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
 // W_g[:, :d] e alone (a gate-only call).
 __global__ void __launch_bounds__(256) swap_gemv_kernel(const GateBiasParams p) {
   pdl_launch_dependents();
-  gate_bias_share(p.e, p.Wg, p.ge, p.d, (int)blockIdx.x * 8 + (threadIdx.x >> 5), (int)gridDim.x * 8, threadIdx.x & 31);
+  gate_bias_share(p.e, p.Wg, p.ge, p.d, 2 * p.d, (int)blockIdx.x * 8 + (threadIdx.x >> 5), (int)gridDim.x * 8, threadIdx.x & 31);
   // Complete only after the previous kernel: the next kernel's programmatic
   // wait, which covers this kernel alone, then covers that one too.  One CTA
   // waiting is enough (the grid completes with its last CTA); the others

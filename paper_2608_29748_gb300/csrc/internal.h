@@ -422,7 +422,6 @@ struct LowRankArgs {
   float* zpart;
   float* tpart;
   void* rho;
-  uint32_t* gemv_next;  // zero before the call
   uint32_t* status;
 };
 bool lowrank_tc_supported(retrace_dtype dtype, int d);

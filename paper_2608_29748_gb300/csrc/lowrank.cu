@@ -16,9 +16,9 @@
 //                      fp32 partials per split;
 //   lr_finish_kernel   one warp per row: sums the partials in a fixed order
 //                      (bitwise repeatable), rounds z, adds B_c[:, :64] z and
-//                      forms rho (lanes over the latent and correction ranks);
-//                      then every warp takes rows of the GEMV W_g[:, :d] e from
-//                      a counter (the grid has at least two CTAs per SM);
+//                      forms rho (lanes over the latent and correction ranks),
+//                      after its share of the GEMV W_g[:, :d] e (the grid has at
+//                      least two CTAs per SM);
 //   lr_fuse_kernel     persistent over (128-row, 64-feature) tiles, two CTAs
 //                      per SM: rho [128, 64] against [W_v; W_g,rho] [128, 64]
 //                      in four K16 MMAs into one of two TMEM accumulators, the
@@ -67,11 +67,10 @@ struct LrParams {
   float* tpart;             // [H, R_max, 32]
   __nv_bfloat16* rho;       // [R_max, 64]
   long long rmax;
-  // W_g[:, :d] e in the projection's idle warps
+  // W_g[:, :d] e
   const __nv_bfloat16* Wg;  // [d, d + 64]
   const __nv_bfloat16* e;   // [d]
   float* ge;                // [d]
-  uint32_t* gemv_next;      // row counter, zero before the launch
   uint32_t* status;
 };
 
@@ -271,45 +270,6 @@ __device__ __forceinline__ void finish_rows(const LrParams& p, long long g, int 
   p.rho[g * L + 32 + lane] = __float2bfloat16_rn(z1 + p.beta * r1);
 }
 
-// W_g[:, :d] e, one row of W_g per claim from the counter; eight 16-byte loads
-// in flight per lane (d a multiple of 8).
-__device__ __forceinline__ void lr_gemv_rows(const LrParams& p, int d, int lane) {
-  const uint4* ev = reinterpret_cast<const uint4*>(p.e);
-  const int nv = d / 8;
-  for (;;) {
-    uint32_t i = 0;
-    if (lane == 0) i = atomicAdd(p.gemv_next, 1u);
-    i = __shfl_sync(0xFFFFFFFFu, i, 0);
-    if (i >= (uint32_t)d) return;
-    const uint4* wv = reinterpret_cast<const uint4*>(p.Wg + (long long)i * (d + L));
-    float acc = 0.f;
-    for (int k0 = 0; k0 < nv; k0 += 8 * 32) {
-      uint4 a[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int k = k0 + u * 32 + lane;
-        a[u] = k < nv ? __ldg(wv + k) : make_uint4(0u, 0u, 0u, 0u);
-      }
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int k = k0 + u * 32 + lane;
-        if (k < nv) {
-          const uint4 b = __ldg(ev + k);
-          const uint32_t aw[4] = {a[u].x, a[u].y, a[u].z, a[u].w}, bw[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-          for (int x = 0; x < 4; ++x) {
-            acc = fmaf(bf16_lo(aw[x]), bf16_lo(bw[x]), acc);
-            acc = fmaf(bf16_hi(aw[x]), bf16_hi(bw[x]), acc);
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, off);
-    if (lane == 0) p.ge[i] = acc;
-  }
-}
-
 // grid >= ceil(R_max / 8) and >= two CTAs per SM.  The GEMV reads only the
 // inputs, so it runs first, while the projection may still be running
 // (programmatic dependent launch); the rows wait for the projection's partials.
@@ -317,7 +277,7 @@ __global__ void __launch_bounds__(256) lr_finish_kernel(const LrParams p) {
   pdl_launch_dependents();
   const long long g = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int d = p.d, lane = threadIdx.x & 31;
-  lr_gemv_rows(p, d, lane);
+  gate_bias_share(p.e, p.Wg, p.ge, d, d + L, (int)blockIdx.x * 8 + (threadIdx.x >> 5), (int)gridDim.x * 8, lane);
   pdl_wait();
   const int R = *(volatile const int32_t*)p.R;
   if ((long long)blockIdx.x * 8 < R) finish_rows(p, g, R, d, lane);  // uniform over the CTA
@@ -623,7 +583,6 @@ cudaError_t launch_lowrank(const LowRankArgs& a, bool tc, cudaStream_t stream) {
   p.Wg = reinterpret_cast<const __nv_bfloat16*>(a.Wg);
   p.e = reinterpret_cast<const __nv_bfloat16*>(a.e);
   p.ge = a.ge;
-  p.gemv_next = a.gemv_next;
   p.status = a.status;
   // Each of the three kernels may start while the previous one finishes
   // (programmatic dependent launch), and waits for its outputs in the kernel.

@@ -101,57 +101,6 @@ __device__ void gate_bias_rows(const __nv_bfloat16* e, const __nv_bfloat16* Wg, 
   }
 }
 
-// One warp of `nw`: rows w, w + nw, ... of ge = W_g[:, :d] e (d a multiple of
-// 8).  The row comes in steps of 256 vectors, the next step's loads issued
-// before the current one is multiplied: a warp that claimed its rows from a
-// counter and loaded one row at a time took 3 us per row of 4096, three
-// round trips.
-__device__ __forceinline__ void gate_bias_share(const __nv_bfloat16* e, const __nv_bfloat16* Wg, float* ge, int d,
-                                                int w, int nw, int lane) {
-  const int vpr = d / 8, steps = (vpr + 255) / 256;
-  const uint4* ev = reinterpret_cast<const uint4*>(e);
-  auto load = [&](uint4 (&x)[8], int row, int step) {
-    const uint4* wr = reinterpret_cast<const uint4*>(Wg + (long long)row * 2 * d);
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int v = step * 256 + u * 32 + lane;
-      x[u] = v < vpr ? __ldcs(wr + v) : make_uint4(0u, 0u, 0u, 0u);
-    }
-  };
-  if (w >= d) return;
-  uint4 cur[8], nxt[8];
-  load(cur, w, 0);
-  float acc = 0.f;
-  for (int row = w, step = 0; row < d;) {
-    const bool last = step + 1 == steps;
-    const int row_n = last ? row + nw : row, step_n = last ? 0 : step + 1;
-    if (row_n < d) load(nxt, row_n, step_n);
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int v = step * 256 + u * 32 + lane;
-      if (v < vpr) {
-        const uint4 x = __ldg(ev + v);
-        const uint32_t ww[4] = {cur[u].x, cur[u].y, cur[u].z, cur[u].w}, xx[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          acc = fmaf(bf16_lo(ww[q]), bf16_lo(xx[q]), acc);
-          acc = fmaf(bf16_hi(ww[q]), bf16_hi(xx[q]), acc);
-        }
-      }
-    }
-    if (last) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
-      if (lane == 0) ge[row] = acc;
-      acc = 0.f;
-    }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) cur[u] = nxt[u];
-    row = row_n;
-    step = step_n;
-  }
-}
-
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
