@@ -15,7 +15,7 @@
 //                            largest, then the few elements above it, ranked;
 //   sampled_finalize_kernel  one CTA per sequence: the filtered
 //                            probabilities of the draft tokens from the sorted
-//                            lists (eight positions at a time, one per warp),
+//                            lists (16 positions at a time, one per warp),
 //                            the accept tests in order, the draw, and for a
 //                            round the copies and packing of e~ and [m; u].
 // The outputs depend only on the target rows 0..A_b and the drafter rows
@@ -354,6 +354,8 @@ __global__ void __launch_bounds__(kThreads, 3) sampled_topk_kernel(const TopkPar
   }
 }
 
+constexpr int kFinWarps = 16;  // warps of a finalize CTA: positions whose accept tests run together
+
 struct FinalizeParams {
   const unsigned long long* keys;
   int B, K, V, k;
@@ -504,14 +506,15 @@ __device__ int draw(const RowDist& r, const float wt[2], float u, int lane) {
 }
 
 // One CTA per sequence.  The accept tests need only p_i(x_i) and q_i(x_i):
-// the warps compute them for eight positions at a time, one position each,
+// the warps compute them for kFinWarps positions at a time, one position each,
 // and thread 0 takes the decisions in order, so the chain of dependent
 // distributions is one per chunk instead of one per position.  Warp 0 then
 // draws the appended token; every thread writes the outputs and, for a round,
 // copies and packs rows.
 __device__ void sampled_finalize_sequence(const FinalizeParams& p, int b) {
-  constexpr int kFinWarps = 8;
   __shared__ int s_A, s_y, s_off;
+  __shared__ int s_qtok[kMaxTopK];
+  __shared__ float s_qw[kMaxTopK];
   __shared__ float s_px[kFinWarps], s_qx[kFinWarps];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int K = p.K, K1 = K + 1;
@@ -565,19 +568,24 @@ __device__ void sampled_finalize_sequence(const FinalizeParams& p, int b) {
     if (A < K) {
       // residual max(0, p - q) over the target's kept tokens
       const RowDist qd = row_dist(p, dbase + A, lane);
-      float res[2];
+      // (the drafter's list in shared memory: 64 entries handed round by
+      // shuffles took longer than the two distributions)
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        // q of this lane's token: every lane looks it up in the drafter's list
-        float qw = 0.f;
-        for (int s2 = 0; s2 < 32; ++s2) {
-          const int t0 = __shfl_sync(0xFFFFFFFFu, qd.tok[0], s2), t1 = __shfl_sync(0xFFFFFFFFu, qd.tok[1], s2);
-          const float w0 = __shfl_sync(0xFFFFFFFFu, qd.w[0], s2), w1 = __shfl_sync(0xFFFFFFFFu, qd.w[1], s2);
-          if (pt.tok[h] >= 0 && t0 == pt.tok[h]) qw = w0;
-          if (pt.tok[h] >= 0 && t1 == pt.tok[h]) qw = w1;
-        }
-        res[h] = pt.tok[h] >= 0 ? fmaxf(0.f, pt.w[h] / pt.total - qw / qd.total) : 0.f;
+        s_qtok[32 * h + lane] = qd.tok[h];
+        s_qw[32 * h + lane] = qd.w[h];
       }
+      __syncwarp();
+      float qw[2] = {0.f, 0.f}, res[2];
+      for (int t = 0; t < p.k; ++t) {
+        const int tok = s_qtok[t];  // -1: cut off by top-p
+        const float w = s_qw[t];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          if (tok >= 0 && tok == pt.tok[h]) qw[h] = w;
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) res[h] = pt.tok[h] >= 0 ? fmaxf(0.f, pt.w[h] / pt.total - qw[h] / qd.total) : 0.f;
       float rs = res[0] + res[1];
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) rs += __shfl_xor_sync(0xFFFFFFFFu, rs, off);
@@ -658,7 +666,7 @@ __device__ void sampled_finalize_sequence(const FinalizeParams& p, int b) {
   }
 }
 
-__global__ void __launch_bounds__(256) sampled_finalize_kernel(const FinalizeParams p) {
+__global__ void __launch_bounds__(32 * kFinWarps) sampled_finalize_kernel(const FinalizeParams p) {
   pdl_launch_dependents();
   pdl_wait();  // the sorted lists come from the top-k kernel
   const int n_live = p.count_in ? (int)__ldcg(p.count_in) : p.B;
@@ -765,7 +773,7 @@ cudaError_t launch_verify_sampled(const SampledArgs& a, retrace_dtype dtype, cud
                              : launch_dependent(topk, dim3((unsigned)grid_n), dim3(kThreads), 0, stream,
                                                 (unsigned)parts, tp);
     if (err != cudaSuccess) return err;
-    err = launch_dependent(sampled_finalize_kernel, dim3((unsigned)a.B), dim3(256), 0, stream, 1, fp);
+    err = launch_dependent(sampled_finalize_kernel, dim3((unsigned)a.B), dim3(32 * kFinWarps), 0, stream, 1, fp);
     if (err != cudaSuccess) return err;
   }
   if (!defer) return cudaSuccess;
