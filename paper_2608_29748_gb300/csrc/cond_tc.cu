@@ -663,7 +663,6 @@ __global__ void __launch_bounds__(P_THREADS, 1)
   const int nt0 = GENERAL ? (d + 255) / 256 : d / 256, nt1 = GENERAL ? (d + 127) / 128 : d / 128;
   pdl_launch_dependents();
   uint32_t* tile_queue = p.sync + kSyncTileQueue;
-  uint32_t* gemv_next = p.sync + kSyncGemvNext;
   uint32_t* gemv_done = p.sync + kSyncGemvDone;
   uint32_t* block_done = p.block_done;
   const bool need_ge = p.do_gate && !(GENERAL && p.e_dense);
@@ -932,7 +931,14 @@ __global__ void __launch_bounds__(P_THREADS, 1)
     __syncwarp();
   } else if (warp == 2 || warp == 3) {
     // ---------------- W_g[:, :d] e for the broadcast e (idle warps) ----------------
-    if (need_ge) gate_bias_rows(p, d, lane, gemv_next, gemv_done);
+    if (need_ge) {
+      const int w = 2 * (int)blockIdx.x + warp - 2, nw = 2 * (int)gridDim.x;
+      gate_bias_share(p.e, p.Wg, p.ge, d, 2 * d, w, nw, lane);
+      pdl_wait();  // the counters are zero from here on
+      __threadfence();
+      __syncwarp();
+      if (lane == 0 && w < d) atomicAdd(gemv_done, (uint32_t)((d - w + nw - 1) / nw));
+    }
   } else {
     // ---------------- epilogue (warps 4-7 of both CTAs) ----------------
     const int q = (warp - 4) * 32 + lane;  // tile row = TMEM lane
@@ -1019,8 +1025,6 @@ __global__ void __launch_bounds__(P_THREADS, 1)
         else mbar_arrive_remote(leader_addr(&bar_tempty[acc]));
       }
     }
-    // out of tiles: help finish W_g[:, :d] e (the rows left on the counter)
-    if (need_ge && !s_abort) gate_bias_rows(p, d, lane, gemv_next, gemv_done);
   }
   // ---------------- teardown ----------------
   tc_fence_before();

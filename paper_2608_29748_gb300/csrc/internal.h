@@ -204,7 +204,8 @@ struct VerifyArgs {
   void* apack;     // [R_max, 2d]: [m; u] rows
   void* epack;     // [R_max, d]: e rows (dense e only)
   int32_t* rowmap; // [R_max]: packed row -> b*K + j
-  int32_t* R_count;
+  int32_t* R_count;   // word kSyncRowCount of the sync area: R
+  size_t sync_bytes;  // the sync area, zeroed but for R by the end of verification
   // Windowed schedule (NULL live: one pass over every row only): two live
   // lists of B sequences and the passes' counters, from the workspace.
   int32_t* live;
@@ -217,6 +218,7 @@ struct VerifyArgs {
   // One pass that only folds the argmax keys: a direct-rows conditioning
   // decides the sequences, writes the outputs and zeroes the keys.
   int keys_only;
+  int plain_first;  // the first kernel without programmatic dependence on what precedes it
 };
 constexpr int kCondCopyKeep = 0;
 constexpr int kCondCopyE = 1;
@@ -329,7 +331,8 @@ struct PackArgs {
 };
 cudaError_t launch_pack(const PackArgs& a, cudaStream_t stream);
 
-// Counters of one conditioning pass (uint32, zeroed before each pass):
+// Counters of one conditioning pass (uint32, zeroed before each pass: by the last
+// verification kernel, or a memset):
 //   [kSyncRowCount]   packed rows claimed / R
 //   [kSyncTileQueue]  next tile of the dynamic schedule
 //   [kSyncGemvNext]   next row of W_g[:, :d] e;  [kSyncGemvDone] rows written

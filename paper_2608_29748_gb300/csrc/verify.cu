@@ -80,6 +80,8 @@ struct VerifyParams {
   uint32_t* pass_counts;
   int n_counts;
   uint32_t* exits;           // CTAs out (zero between calls)
+  uint32_t* sync;            // verify_finish_kernel: counters of the conditioning, zeroed but for R_count
+  int sync_words;
   int defer_copies;          // the finaliser leaves the copies to verify_copy_kernel
   int32_t* pack_off;         // [B] first packed row of each sequence (deferred copies)
 };
@@ -452,7 +454,12 @@ __global__ void __launch_bounds__(kThreads, 2) verify_kernel(const VerifyParams 
   __shared__ int s_A[2];  // accepted length, packed-row offset
   __shared__ int s_last;
   extern __shared__ uint4 s_stage[];  // kCopyStage * kThreads vectors: row copies of the finaliser
-  pdl_launch_dependents();  // the next kernel may take SMs as this grid's CTAs finish
+  // The first kernel of a call waits at once: what precedes it in the stream
+  // (the logits' producer, the previous call) may still be running.  Only then
+  // may the next kernel start, whose work before its own wait thus follows the
+  // previous call's end.  It may take SMs as this grid's CTAs finish.
+  if (p.i0 == 0) pdl_wait();
+  pdl_launch_dependents();
 
   long long n_live = p.B;
   const int* s_list = nullptr;  // the pass's live sequences (NULL: 0..B-1)
@@ -604,7 +611,8 @@ __global__ void __launch_bounds__(kThreads, 2) verify_copy_kernel(const VerifyPa
 
 // The end of a windowed verification, after its last pass.  Decides the
 // sequences of the last window (decide_window over the last pass's live list,
-// the same in every CTA; their outputs spread over the CTAs), sets R, and the
+// the same in every CTA; their outputs spread over the CTAs), sets R and zeroes
+// the conditioning's other counters, and the
 // last CTA to finish with the keys zeroes them and the passes' counters for
 // the next call.  Then the row copies as in verify_copy_kernel: the
 // unconditioned rows of e~ and the packed [m; u] (and e) rows, each warp one
@@ -634,7 +642,9 @@ __global__ void __launch_bounds__(kThreads, 2) verify_finish_kernel(const Verify
     s_mapA[b] = p.i0 + min(s_first[l], K - p.i0);
     s_mapO[b] = s_off[l];
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0 && p.R_count) *p.R_count = base + rows;
+  if (blockIdx.x == 0 && p.R_count) {
+    for (int k = threadIdx.x; k < p.sync_words; k += kThreads) p.sync[k] = k == kSyncRowCount ? (uint32_t)(base + rows) : 0u;
+  }
   // every read of the keys above is done: the last CTA out resets them
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -803,6 +813,8 @@ cudaError_t launch_typed(const VerifyArgs& a, cudaStream_t stream) {
   p.pass_counts = nullptr;
   p.n_counts = 0;
   p.exits = nullptr;
+  p.sync = reinterpret_cast<uint32_t*>(a.R_count) - kSyncRowCount;  // R_count is a word of the sync area
+  p.sync_words = a.R_count ? (int)(a.sync_bytes / 4) : 0;
   p.defer_copies = 0;
   p.pack_off = a.pack_off;
   const int K1 = a.K + 1;
@@ -828,17 +840,21 @@ cudaError_t launch_typed(const VerifyArgs& a, cudaStream_t stream) {
     // and verify_finish_kernel decides every sequence, writes the outputs
     // and does the copies over its grid (target_argmax, every row's argmax,
     // stays with the finalisers).
+    auto launch_first = [&]() -> cudaError_t {
+      if (a.plain_first) {
+        verify_kernel<T><<<(unsigned)grid, kThreads, kCopyStageBytes, stream>>>(p);
+        return cudaGetLastError();
+      }
+      return launch_dependent(verify_kernel<T>, dim3((unsigned)grid), dim3(kThreads), kCopyStageBytes, stream, 1u, p);
+    };
     if (a.keys_only) {
       p.windowed = 1;
-      verify_kernel<T><<<(unsigned)grid, kThreads, kCopyStageBytes, stream>>>(p);
-      return cudaGetLastError();
+      return launch_first();
     }
     const bool defer = a.R_count && a.B < info.sm_count;
     if (defer && !a.target_argmax && a.live && a.pass_counts && a.B <= kWindowMaxB) {
       p.windowed = 1;
-      verify_kernel<T><<<(unsigned)grid, kThreads, kCopyStageBytes, stream>>>(p);
-      err = cudaGetLastError();
-      if (err != cudaSuccess) return err;
+      if ((err = launch_first()) != cudaSuccess) return err;
       p.i0 = 0;
       p.live_in = nullptr;  // every sequence, no packed rows claimed before
       p.count_in = nullptr;
@@ -851,8 +867,11 @@ cudaError_t launch_typed(const VerifyArgs& a, cudaStream_t stream) {
       return launch_finish<T>(a, p, fgrid < 1 ? 1 : fgrid, stream);
     }
     p.defer_copies = defer ? 1 : 0;
-    verify_kernel<T><<<(unsigned)grid, kThreads, kCopyStageBytes, stream>>>(p);
-    err = cudaGetLastError();
+    if (a.R_count) {  // the finalisers claim packed rows from a counter that starts at zero
+      err = cudaMemsetAsync(p.sync, 0, a.sync_bytes, stream);
+      if (err != cudaSuccess) return err;
+    }
+    err = launch_first();
     if (err != cudaSuccess || !defer) return err;
     const long long copy_grid = ((long long)a.B * a.K * 4 + 15) / 16;  // a warp per row segment
     return launch_copies<T>(a, p, copy_grid < grid_full ? copy_grid : grid_full, stream);
@@ -878,12 +897,12 @@ cudaError_t launch_typed(const VerifyArgs& a, cudaStream_t stream) {
     p.live_out = k == 0 ? nullptr : a.live + (size_t)(k & 1) * a.B;
     p.count_out = k == 0 ? nullptr : a.pass_counts + k;
     p.base_out = k == 0 ? nullptr : bases + k;
-    if (k == 0) {
+    if (k == 0 && a.plain_first) {
       verify_kernel<T><<<(unsigned)grid_full, kThreads, kCopyStageBytes, stream>>>(p);
       err = cudaGetLastError();
     } else {
-      err = launch_dependent(verify_kernel<T>, dim3((unsigned)grid_full), dim3(kThreads), kCopyStageBytes,
-                             stream, 1u, p);
+      err = launch_dependent(verify_kernel<T>, dim3((unsigned)grid_full), dim3(kThreads), kCopyStageBytes, stream, 1u,
+                             p);
     }
     if (err != cudaSuccess) return err;
   }
