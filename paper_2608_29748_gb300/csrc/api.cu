@@ -410,16 +410,14 @@ retrace_status retrace_align_refine(const void* hD, const void* hT, retrace_dtyp
   if ((st = check_ws(ws, ws_bytes, L.total)) != RETRACE_OK) return st;
   if ((st = prepare_ws(ws, ws_bytes, L, B, K, stream)) != RETRACE_OK) return st;
   const RowSource rows{accept_len, 1};
-  RT_CUDA(launch_fill_rows(B, K, d, rows, n_out, r_out, nullptr, 0, nullptr, dtype, stream),
-          "fill kernel launch");
   const bool tc = tc_supported(dtype, d) && aligned16(hD) && aligned16(hT) && aligned16(Wc) && aligned16(r_out);
   if (tc) {
     char* w = reinterpret_cast<char*>(ws);
     uint32_t* sync = reinterpret_cast<uint32_t*>(w + L.sync);
     int32_t* R = reinterpret_cast<int32_t*>(sync + kSyncRowCount);
     int32_t* rowmap = reinterpret_cast<int32_t*>(w + L.rowmap);
-    RT_CUDA(cudaMemsetAsync(sync, 0, L.sync_bytes, stream), "cudaMemsetAsync(sync)");
-    PackArgs pk{B, K, d, rows, 0, hD, hT, nullptr, 0, w + L.apack, nullptr, rowmap, R};
+    PackArgs pk{B, K, d, rows, 0, hD, hT, nullptr, 0, w + L.apack, nullptr, rowmap, sync, L.sync_bytes,
+                n_out, r_out, nullptr, nullptr};
     RT_CUDA(launch_pack(pk, stream), "pack kernel launch");
     TcCondArgs a{};
     a.B = B;
@@ -437,6 +435,8 @@ retrace_status retrace_align_refine(const void* hD, const void* hT, retrace_dtyp
     a.status = status_word(ws);
     RT_CUDA(launch_cond_tc(a, stream), "correction kernel launch");
   } else {
+    RT_CUDA(launch_fill_rows(B, K, d, rows, n_out, r_out, nullptr, 0, nullptr, dtype, stream),
+            "fill kernel launch");
     CorrectArgs a{hD, hT, Wc, beta, B, K, d, rows, r_out, 0};
     RT_CUDA(launch_correct_simt(a, dtype, stream), "correction kernel launch");
   }
@@ -459,22 +459,21 @@ retrace_status retrace_gate_fuse(const void* e, int64_t e_batch_stride, int64_t 
   char* w = reinterpret_cast<char*>(ws);
   float* ge = reinterpret_cast<float*>(w + L.ge);
   const RowSource rows{n, 0};
-  RT_CUDA(launch_fill_rows(B, K, d, rows, nullptr, nullptr, e, dense, e_out, dtype, stream),
-          "fill kernel launch");
   const bool tc = tc_supported(dtype, d) && aligned16(e) && aligned16(r) && aligned16(Wv) &&
                   aligned16(Wg) && aligned16(e_out);
   if (tc) {
     uint32_t* sync = reinterpret_cast<uint32_t*>(w + L.sync);
     int32_t* R = reinterpret_cast<int32_t*>(sync + kSyncRowCount);
     int32_t* rowmap = reinterpret_cast<int32_t*>(w + L.rowmap);
-    RT_CUDA(cudaMemsetAsync(sync, 0, L.sync_bytes, stream), "cudaMemsetAsync(sync)");
-    PackArgs pk{B, K, d, rows, 1, r, nullptr, e, dense, w + L.r, w + L.epack, rowmap, R};
+    PackArgs pk{B, K, d, rows, 1, r, nullptr, e, dense, w + L.r, w + L.epack, rowmap, sync, L.sync_bytes,
+                nullptr, e_out, Wg, ge};
     RT_CUDA(launch_pack(pk, stream), "pack kernel launch");
     TcCondArgs a{};
     a.B = B;
     a.K = K;
     a.d = d;
     a.do_gate = 1;
+    a.ge_ready = 1;
     a.rpack = w + L.r;
     a.e = e;
     a.epack = w + L.epack;
@@ -490,6 +489,8 @@ retrace_status retrace_gate_fuse(const void* e, int64_t e_batch_stride, int64_t 
     a.split_part = pair_split_bytes(B, K, d, 2) ? reinterpret_cast<float*>(w + L.swp) : nullptr;
     RT_CUDA(launch_cond_tc(a, stream), "gate kernel launch");
   } else {
+    RT_CUDA(launch_fill_rows(B, K, d, rows, nullptr, nullptr, e, dense, e_out, dtype, stream),
+            "fill kernel launch");
     if (!dense) RT_CUDA(launch_gate_bias(Wg, e, d, ge, dtype, stream), "gate bias kernel launch");
     GateArgs a{e, dense, r, 0, Wv, Wg, dense ? nullptr : ge, B, K, d, rows, e_out};
     RT_CUDA(launch_gate_simt(a, dtype, stream), "gate kernel launch");

@@ -2,8 +2,8 @@
 //
 // Two steps per projection family:
 //
-// 1. pack_rows_kernel lays the conditioned rows out contiguously, in sequence
-//    order (R = sum_b n_b rows, n_b = max(0, K-1-A_b)):
+// 1. pack_rows_kernel (standalone calls; in a round verification packs) lays
+//    the conditioned rows out contiguously, in sequence order (R = sum_b n_b rows, n_b = max(0, K-1-A_b)):
 //      correction operand  Apack[g] = [ hD[b, A_b+1+j] ; hT[b, A_b+j] ]  (Eq. 4-5),
 //      or the corrected signal rows r[b, j] for a standalone gate call,
 //      plus, for per-position e, Epack[g] = e[b, j];
@@ -74,6 +74,14 @@ constexpr uint32_t IDESC_N128 = idesc_bf16_f32(128, 128);
 // ---------------------------------------------------------------------------
 // Row packing
 // ---------------------------------------------------------------------------
+// W_g[:, :d] e for the gate of a small-R call (broadcast e).
+struct GateBiasParams {
+  int d;
+  const __nv_bfloat16* e;
+  const __nv_bfloat16* Wg;
+  float* ge;
+};
+
 struct PackParams {
   int B, K, d;
   RowSource rows;
@@ -85,56 +93,81 @@ struct PackParams {
   __nv_bfloat16* apack;
   __nv_bfloat16* epack;
   int32_t* rowmap;
-  int32_t* R_out;
+  int32_t* n_out;           // mode 0: n_b
+  __nv_bfloat16* rest;      // [B, K, d]: rows j >= n_b are zeroed (mode 0) or set to e (mode 1)
+  uint32_t* sync;           // counters of the projections: R, the others zeroed
+  int sync_words;
+  GateBiasParams bias;      // mode 1: W_g[:, :d] e (ge NULL: not computed)
 };
 
-// One CTA per sequence.  Its first packed row is the number of rows of all
-// earlier sequences (a block-wide sum), so the layout is the sequence order.
+// A warp copies n 16-byte vectors, eight loads in flight per lane; src NULL: zeros.
+__device__ __forceinline__ void warp_copy_row(__nv_bfloat16* dst, const __nv_bfloat16* src, int n, int lane) {
+  uint4* d4 = reinterpret_cast<uint4*>(dst);
+  const uint4* s4 = reinterpret_cast<const uint4*>(src);
+  for (int v0 = 0; v0 < n; v0 += 8 * 32) {
+    uint4 x[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int v = v0 + k * 32 + lane;
+      x[k] = src && v < n ? __ldg(s4 + v) : make_uint4(0u, 0u, 0u, 0u);
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int v = v0 + k * 32 + lane;
+      if (v < n) d4[v] = x[k];
+    }
+  }
+}
+
+// What precedes the projections of a standalone call, in one launch: the
+// packed rows with their row map and count (in sequence order: a warp's first
+// packed row is the number of rows of all earlier sequences, which it sums
+// itself), n_b, the rows that carry nothing, the projections' counters and,
+// before a gate, W_g[:, :d] e.  A warp takes consecutive positions (b, j), one
+// each at the usual sizes.  Bound by
+// latency at the sizes it runs at; as three launches (fill, memset, pack with
+// one CTA per sequence) it took 2.7 + 10.4 us at B = 24, K = 12, d = 1152.
 __global__ void __launch_bounds__(256) pack_rows_kernel(const PackParams p) {
-  __shared__ int s_red[8];
-  const int b = blockIdx.x, tid = threadIdx.x, K = p.K, d = p.d;
-  int part = 0;
-  for (int x = tid; x < b; x += 256) part += rows_of(p.rows, x, K);
+  pdl_wait();
+  pdl_launch_dependents();
+  const int lane = threadIdx.x & 31, K = p.K, d = p.d, vpr = d / 8;
+  const int w = (int)blockIdx.x * 8 + (int)(threadIdx.x >> 5), nw = (int)gridDim.x * 8;
+  if (blockIdx.x == 0)
+    for (int k = threadIdx.x; k < p.sync_words; k += 256)
+      if (k != kSyncRowCount) p.sync[k] = 0u;
+  const long long all = (long long)p.B * K, per = (all + nw - 1) / nw;
+  const int p0 = (int)min(w * per, all), p1 = (int)min(p0 + per, all);
+  int b = p0 / K, off = 0;  // rows of the sequences before b
+  for (int x0 = lane; x0 < b; x0 += 4 * 32) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xFFFFFFFFu, part, o);
-  if ((tid & 31) == 0) s_red[tid >> 5] = part;
-  __syncthreads();
-  int off = 0;
+    for (int q = 0; q < 4; ++q) off += x0 + 32 * q < b ? rows_of(p.rows, x0 + 32 * q, K) : 0;
+  }
 #pragma unroll
-  for (int w = 0; w < 8; ++w) off += s_red[w];
-  const int nb = rows_of(p.rows, b, K);
-  if (b == p.B - 1 && tid == 0) *p.R_out = off + nb;
-  if (nb == 0) return;
-  for (int j = tid; j < nb; j += 256) p.rowmap[off + j] = b * K + j;
-  const int vpr = d / 8;  // 16-byte vectors per d-wide row
-  const long long base = (long long)b * K;
-  if (p.mode == 0) {
-    const int A = K - 1 - nb;
-    const uint4* hD = reinterpret_cast<const uint4*>(p.src0);
-    const uint4* hT = reinterpret_cast<const uint4*>(p.src1);
-    uint4* out = reinterpret_cast<uint4*>(p.apack);
-    for (int i = tid; i < nb * 2 * vpr; i += 256) {
-      const int j = i / (2 * vpr), c = i % (2 * vpr);
-      const uint4 v = (c < vpr) ? __ldg(hD + (base + A + 1 + j) * vpr + c)   // m_j (Eq. 4)
-                                : __ldg(hT + (base + A + j) * vpr + c - vpr);  // u_j (Eq. 5)
-      out[(long long)(off + j) * 2 * vpr + c] = v;
+  for (int o = 16; o > 0; o >>= 1) off += __shfl_xor_sync(0xFFFFFFFFu, off, o);
+  for (int pos = p0; pos < p1; ++pos) {
+    if (pos == (b + 1) * K) off += rows_of(p.rows, b++, K);
+    const int j = pos - b * K, nb = rows_of(p.rows, b, K);
+    if (j == 0 && lane == 0) {
+      if (p.n_out) p.n_out[b] = nb;
+      if (b == p.B - 1) p.sync[kSyncRowCount] = (uint32_t)(off + nb);
     }
-  } else {
-    const uint4* r = reinterpret_cast<const uint4*>(p.src0);
-    uint4* out = reinterpret_cast<uint4*>(p.apack);
-    for (int i = tid; i < nb * vpr; i += 256) {
-      const int j = i / vpr, c = i % vpr;
-      out[(long long)(off + j) * vpr + c] = __ldg(r + (base + j) * vpr + c);
+    const long long row = (long long)pos * d;
+    if (j >= nb) {
+      warp_copy_row(p.rest + row, p.mode == 0 ? nullptr : p.e + (p.e_dense ? row : 0), vpr, lane);
+      continue;
+    }
+    const long long g = off + j;
+    if (lane == 0) p.rowmap[g] = pos;
+    if (p.mode == 0) {
+      const int A = K - 1 - nb;
+      warp_copy_row(p.apack + g * 2 * d, p.src0 + row + (long long)(A + 1) * d, vpr, lane);  // m_j (Eq. 4)
+      warp_copy_row(p.apack + g * 2 * d + d, p.src1 + row + (long long)A * d, vpr, lane);    // u_j (Eq. 5)
+    } else {
+      warp_copy_row(p.apack + g * d, p.src0 + row, vpr, lane);
+      if (p.e_dense) warp_copy_row(p.epack + g * d, p.e + row, vpr, lane);
     }
   }
-  if (p.e_dense) {
-    const uint4* e = reinterpret_cast<const uint4*>(p.e);
-    uint4* out = reinterpret_cast<uint4*>(p.epack);
-    for (int i = tid; i < nb * vpr; i += 256) {
-      const int j = i / vpr, c = i % vpr;
-      out[(long long)(off + j) * vpr + c] = __ldg(e + (base + j) * vpr + c);
-    }
-  }
+  if (p.bias.ge) gate_bias_share(p.bias.e, p.bias.Wg, p.bias.ge, d, 2 * d, w, nw, lane);
 }
 
 // ---------------------------------------------------------------------------
@@ -1128,14 +1161,6 @@ struct RowMaps {
   CUtensorMap m[SW_ROW_MAPS];
 };
 
-// W_g[:, :d] e for the gate of a small-R call (broadcast e).
-struct GateBiasParams {
-  int d;
-  const __nv_bfloat16* e;
-  const __nv_bfloat16* Wg;
-  float* ge;
-};
-
 // A round of few sequences without packed rows (DIRECT).  Sequence b has the KP
 // tile rows from b KP on (KP = K - 1 rounded up to 8; those past n_b compute
 // nothing that is stored), so the row tile's size is known on the host, and
@@ -1610,7 +1635,7 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
   }
 }
 
-// W_g[:, :d] e alone (a gate-only call).
+// W_g[:, :d] e alone (a round whose gate follows verification: the raw variant).
 __global__ void __launch_bounds__(256) swap_gemv_kernel(const GateBiasParams p) {
   pdl_launch_dependents();
   gate_bias_share(p.e, p.Wg, p.ge, p.d, 2 * p.d, (int)blockIdx.x * 8 + (threadIdx.x >> 5), (int)gridDim.x * 8, threadIdx.x & 31);
@@ -1643,7 +1668,10 @@ bool direct_rows_supported(int B, int K, int d) {
 
 cudaError_t launch_pack(const PackArgs& a, cudaStream_t stream) {
   if (a.B <= 0) return cudaSuccess;
-  PackParams p;
+  DeviceInfo info;
+  cudaError_t err = device_info(&info);
+  if (err != cudaSuccess) return err;
+  PackParams p{};
   p.B = a.B;
   p.K = a.K;
   p.d = a.d;
@@ -1656,9 +1684,17 @@ cudaError_t launch_pack(const PackArgs& a, cudaStream_t stream) {
   p.apack = reinterpret_cast<__nv_bfloat16*>(a.apack);
   p.epack = reinterpret_cast<__nv_bfloat16*>(a.epack);
   p.rowmap = a.rowmap;
-  p.R_out = a.R;
-  pack_rows_kernel<<<(unsigned)a.B, 256, 0, stream>>>(p);
-  return cudaGetLastError();
+  p.n_out = a.n_out;
+  p.rest = reinterpret_cast<__nv_bfloat16*>(a.rest);
+  p.sync = a.sync;
+  p.sync_words = (int)(a.sync_bytes / 4);
+  // the CTA-pair kernel computes W_g[:, :d] e itself
+  if (a.mode == 1 && !a.e_dense && (long long)a.B * (a.K - 1) <= kSwapMaxRows)
+    p.bias = {a.d, p.e, reinterpret_cast<const __nv_bfloat16*>(a.Wg), a.ge};
+  // a warp per position, four CTAs per SM at most; all of them for the GEMV
+  const long long most = 4LL * info.sm_count, ctas = ((long long)a.B * a.K + 7) / 8;
+  const unsigned grid = (unsigned)(p.bias.ge || ctas > most ? most : ctas);
+  return launch_dependent(pack_rows_kernel, dim3(grid), dim3(256), 0, stream, 1u, p);
 }
 
 static cudaError_t launch_cond_pair(const TcCondArgs& a, int clusters, cudaStream_t stream) {
@@ -1910,7 +1946,7 @@ static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
         !encode_row_maps(&mB, a.rpack, du, rmax, rstride) ||
         (a.e_dense && !encode_row_maps(&mE, a.epack, du, rmax, 2 * du)))
       return cudaErrorInvalidValue;
-    if (!a.do_correct && !a.e_dense) {  // no correction kernel to compute it: W_g[:, :d] e in its own launch
+    if (!a.do_correct && !a.e_dense && !a.ge_ready) {  // no correction kernel to compute it: W_g[:, :d] e in its own launch
       err = launch_dependent(swap_gemv_kernel, dim3((unsigned)(info.sm_count * 4)), dim3(256), 0, stream, 1u, gp);
       if (err != cudaSuccess) return err;
     }

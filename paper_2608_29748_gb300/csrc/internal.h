@@ -327,7 +327,12 @@ struct PackArgs {
   void* apack;       // mode 0: [R_max, 2d]; mode 1: [R_max, d]
   void* epack;       // [R_max, d]
   int32_t* rowmap;   // [R_max]
-  int32_t* R;        // row count out
+  uint32_t* sync;    // the sync area: R, every other counter zeroed
+  size_t sync_bytes;
+  int32_t* n_out;    // mode 0
+  void* rest;        // [B, K, d] output whose rows j >= n_b are zeroed (mode 0) or set to e (mode 1)
+  const void* Wg;    // mode 1, broadcast e: W_g[:, :d] e into ge (small R)
+  float* ge;
 };
 cudaError_t launch_pack(const PackArgs& a, cudaStream_t stream);
 
@@ -375,6 +380,7 @@ struct TcCondArgs {
   const void* Wv;
   const void* Wg;
   float* ge;  // [d] scratch for W_g[:, :d] e (broadcast e)
+  int ge_ready;  // small R: ge is computed already
   void* e_out;
   const int32_t* R;
   const int32_t* rowmap;
