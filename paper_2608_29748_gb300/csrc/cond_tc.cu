@@ -1109,9 +1109,12 @@ __global__ void wait_selftest_kernel(int kind, const uint32_t* flag, uint32_t ta
 // epilogue: r = m + beta c (Eq. 7) for the correction tiles of W_c, or the
 // gated fusion e~ = e + v sigmoid(g_r + W_g[:, :d] e) (Eq. 8) for the gate
 // tiles, whose 128 weight rows stack 64 rows of W_v over the same 64 rows of
-// W_g[:, d:2d] (v and g_r of a feature in TMEM lanes f and 64 + f); with a
-// per-position e further k-blocks add W_g[:, :d] e to the gate's lanes, their
-// W_v half filled with zeros by the copy.  Nothing goes through global partials and no reduction kernel follows.  The partial
+// W_g[:, d:2d] (v and g_r of a feature in TMEM lanes f and 64 + f).  With a
+// per-position e the gate has three products of d-long rows, W_v r, W_g,r r and
+// W_g,e e: a cluster then holds 128 features of all three, each product in
+// its own CTAs (S = 3 splits), and the sum adds the last two.  (As further
+// k-blocks of the stacked tiles, W_v's half zeros, a gate tile had twice the
+// k-blocks on as many CTAs: 36 us at B = 32, d = 2560.)  Nothing goes through global partials and no reduction kernel follows.  The partial
 // is stored row-major ([row][feature]) so that both the TMEM drain and the
 // cluster's reads move whole 128- and 256-byte rows.
 //
@@ -1224,14 +1227,16 @@ __device__ __forceinline__ int direct_accepted(const DirectRows& q, const Direct
   return A;
 }
 
+enum { kCorrect = 0, kGateStacked = 1, kGateParts = 2 };
 struct SwapClusterParams {
   const int32_t* R;
   int d;
   int mtiles;  // weight tiles
   int nkb;     // 64-deep k-blocks of the GEMM
-  int nkb_r;   // those over the rows operand tmB; the others (gate, per-position e) are over tmE
-  int S;       // K splits = cluster size
-  int gate;    // 0: correction tiles of W_c (128 features); 1: stacked [W_v; W_g,r] tiles (64 features)
+  int nkb_m;   // DIRECT correction: those of the m half
+  int S;       // cluster size: K splits, or 3 times them (kGateParts)
+  int gate;    // kCorrect: tiles of W_c (128 features); kGateStacked: [W_v; W_g,r] tiles (64 features);
+               // kGateParts: per-position e, W_v, W_g,r and W_g,e tiles (128 features each)
   int stage_bytes;  // shared memory of the pipeline stages
   int pre;          // stages whose weight tiles are loaded before the wait on the previous kernel
   int row_maps;     // maps of the rows operand
@@ -1242,8 +1247,8 @@ struct SwapClusterParams {
   __nv_bfloat16* r_out;
   int compact_out;
   GateBiasParams bias;  // correction: W_g[:, :d] e of the gate to come (ge NULL: not computed)
-  // gate epilogue.  Broadcast e: [d], and ge = W_g[:, :d] e, complete before
-  // this launch.  Per-position e (ge NULL): packed rows [R, d].
+  // gate epilogue.  kGateStacked: e [d], and ge = W_g[:, :d] e, complete before
+  // this launch; kGateParts: e packed rows [R, d].
   const __nv_bfloat16* e;
   const float* ge;
   __nv_bfloat16* e_out;
@@ -1311,14 +1316,8 @@ __device__ __forceinline__ void swap_gate_rows(const SwapClusterParams& p, uint3
   const int d = p.d, S = p.S;
   const int f = ((int)threadIdx.x % 16) * 4, n = mt * 64 + f;  // the same features at every step
   if (n >= d) return;  // past the last feature (no barrier below)
-  float4 gb = make_float4(0.f, 0.f, 0.f, 0.f);
-  uint2 ew[NB];
-  if (p.ge) {
-    gb = __ldcg(reinterpret_cast<const float4*>(p.ge + n));
-    ew[0] = __ldg(reinterpret_cast<const uint2*>(p.e + n));
-#pragma unroll
-    for (int q = 1; q < NB; ++q) ew[q] = ew[0];
-  }
+  const float4 gb = __ldcg(reinterpret_cast<const float4*>(p.ge + n));
+  const uint2 ew = __ldg(reinterpret_cast<const uint2*>(p.e + n));
   for (int x0 = threadIdx.x; x0 < total; x0 += NB * SW_THREADS) {
     float4 v[NB], a[NB];
     long long orow[NB];
@@ -1332,7 +1331,6 @@ __device__ __forceinline__ void swap_gate_rows(const SwapClusterParams& p, uint3
       } else {
         orow[q] = __ldcg(p.rowmap + row0 + l);
       }
-      if (!DIRECT && !p.ge) ew[q] = __ldcg(reinterpret_cast<const uint2*>(p.e + (long long)(row0 + l) * d + n));
       at[q] = P + (uint32_t)(l * 512 + f * 4);
       v[q] = a[q] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
@@ -1361,6 +1359,51 @@ __device__ __forceinline__ void swap_gate_rows(const SwapClusterParams& p, uint3
       const float s0 = fast_sigmoid(a[q].x + gb.x), s1 = fast_sigmoid(a[q].y + gb.y);
       const float s2 = fast_sigmoid(a[q].z + gb.z), s3 = fast_sigmoid(a[q].w + gb.w);
       *reinterpret_cast<uint2*>(p.e_out + orow[q] * d + n) =
+          make_uint2(pack_bf16x2(bf16_lo(ew.x) + v[q].x * s0, bf16_hi(ew.x) + v[q].y * s1),
+                     pack_bf16x2(bf16_lo(ew.y) + v[q].z * s2, bf16_hi(ew.y) + v[q].w * s3));
+    }
+  }
+}
+
+// kGateParts: v is the sum of the first third of the cluster's partials, the
+// gate that of the others.
+__device__ __forceinline__ void swap_parts_rows(const SwapClusterParams& p, uint32_t P, int mt, int row0, int l0,
+                                                int total) {
+  constexpr int NB = 4;
+  const int d = p.d, S = p.S;
+  for (int x0 = threadIdx.x; x0 < total; x0 += NB * SW_THREADS) {
+    float4 v[NB], a[NB];
+    uint2 ew[NB];
+    long long orow[NB];
+    uint32_t at[NB];
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      const int x = min(x0 + q * SW_THREADS, total - 1), l = l0 + x / 32, f = (x % 32) * 4, n = mt * 128 + f;
+      orow[q] = n < d ? __ldcg(p.rowmap + row0 + l) : -1;
+      ew[q] = n < d ? __ldcg(reinterpret_cast<const uint2*>(p.e + (long long)(row0 + l) * d + n)) : make_uint2(0u, 0u);
+      at[q] = P + (uint32_t)(l * 512 + f * 4);
+      v[q] = a[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    for (int s = 0; s < S / 3; ++s) {
+      float4 x[3][NB];
+#pragma unroll
+      for (int part = 0; part < 3; ++part)
+#pragma unroll
+        for (int q = 0; q < NB; ++q) x[part][q] = ld_cluster_f4(map_rank(at[q], (uint32_t)(part * (S / 3) + s)));
+#pragma unroll
+      for (int q = 0; q < NB; ++q) {
+        add4(v[q], x[0][q]);
+        add4(a[q], x[1][q]);
+        add4(a[q], x[2][q]);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      const int x = x0 + q * SW_THREADS;
+      if (x >= total || orow[q] < 0) continue;
+      const float s0 = fast_sigmoid(a[q].x), s1 = fast_sigmoid(a[q].y);
+      const float s2 = fast_sigmoid(a[q].z), s3 = fast_sigmoid(a[q].w);
+      *reinterpret_cast<uint2*>(p.e_out + orow[q] * d + mt * 128 + (x % 32) * 4) =
           make_uint2(pack_bf16x2(bf16_lo(ew[q].x) + v[q].x * s0, bf16_hi(ew[q].x) + v[q].y * s1),
                      pack_bf16x2(bf16_lo(ew[q].y) + v[q].z * s2, bf16_hi(ew[q].y) + v[q].w * s3));
     }
@@ -1399,7 +1442,7 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
   }
   if (warp == 1 && lane < p.row_maps) {
     tma_prefetch_desc(&tmB.m[lane]);
-    if (p.nkb > p.nkb_r) tma_prefetch_desc(&tmE.m[lane]);
+    if (p.gate == kGateParts) tma_prefetch_desc(&tmE.m[lane]);
   }
   if (warp == 2) {
     tmem_alloc(smem_u32(&s_tmem), p.tmem_cols);
@@ -1412,21 +1455,22 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
   const uint32_t base = (smem_u32(dsmem) + 1023u) & ~1023u;
   // the partial [row][128 features], in the drained pipeline stages (the same offset in every CTA)
   float* P = reinterpret_cast<float*>(dsmem + (base - smem_u32(dsmem)));
-  const int kb0 = (int)((long long)rank * p.nkb / S), kb1 = (int)((long long)(rank + 1) * p.nkb / S);
+  // this CTA's product (kGateParts) and k-blocks
+  const int splits = p.gate == kGateParts ? S / 3 : S;
+  const int part = (int)rank / splits, split = (int)rank - part * splits;
+  const int kb0 = (int)((long long)split * p.nkb / splits), kb1 = (int)((long long)(split + 1) * p.nkb / splits);
   // Weight tiles lie at 16 KB steps from `base`, whatever the row boxes' size.
   auto load_a = [&](int mt, int kb, uint32_t s) {
     const uint32_t a_dst = base + s * (uint32_t)SW_A_BYTES, bar = smem_u32(&bar_full[s]);
     mbar_arrive_expect_tx(bar, (uint32_t)SW_A_BYTES);
     if (DIRECT && !p.gate) {  // W_c's m columns, then its u columns
-      const bool u = kb >= p.nkb_r;
-      tma_load_2d(a_dst, u ? &tmA2 : &tmA, (u ? kb - p.nkb_r : kb) * BK, mt * 128, bar);
-    } else if (kb >= p.nkb_r) {
-      // the gate's e half: zeros (columns past W_v's end) over the rows of W_g[:, :d]
-      tma_load_2d(a_dst, &tmA, p.nkb_r * BK, mt * 64, bar);
-      tma_load_2d(a_dst + (uint32_t)(SW_A_BYTES / 2), &tmA3, (kb - p.nkb_r) * BK, mt * 64, bar);
-    } else if (p.gate) {  // rows 0-63: W_v rows f0..; rows 64-127: the same rows of W_g[:, d:2d]
+      const bool u = kb >= p.nkb_m;
+      tma_load_2d(a_dst, u ? &tmA2 : &tmA, (u ? kb - p.nkb_m : kb) * BK, mt * 128, bar);
+    } else if (p.gate == kGateStacked) {  // rows 0-63: W_v rows f0..; rows 64-127: the same rows of W_g[:, d:2d]
       tma_load_2d(a_dst, &tmA, kb * BK, mt * 64, bar);
       tma_load_2d(a_dst + (uint32_t)(SW_A_BYTES / 2), &tmA2, d + kb * BK, mt * 64, bar);
+    } else if (p.gate == kGateParts) {
+      tma_load_2d(a_dst, part == 0 ? &tmA : part == 1 ? &tmA2 : &tmA3, (part == 1 ? d : 0) + kb * BK, mt * 128, bar);
     } else {
       tma_load_2d(a_dst, &tmA, kb * BK, mt * 128, bar);
     }
@@ -1491,8 +1535,7 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
   const int nst = swap_stages(p.stage_bytes, box > 0 ? box : SW_ROW_STEP);  // >= p.pre
   const uint32_t b_bytes = (uint32_t)(box * BK * 2);
   const uint32_t b_base = base + (uint32_t)nst * (uint32_t)SW_A_BYTES;
-  const CUtensorMap* mb = &tmB.m[box > 0 ? box / SW_ROW_STEP - 1 : 0];
-  const CUtensorMap* me = &tmE.m[box > 0 ? box / SW_ROW_STEP - 1 : 0];
+  const CUtensorMap* mb = &(part == 2 ? tmE : tmB).m[box > 0 ? box / SW_ROW_STEP - 1 : 0];
 
   if (cid >= units && warp == 0 && lane == 0) {  // (always so with R = 0)
     // no unit: let the copies issued above land before the CTA leaves
@@ -1534,9 +1577,9 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
               if (!__shfl_sync(0xFFFFFFFFu, ok, 0)) break;
               if (my_A < p.direct.K - 1) {  // (lanes past B have my_A = K)
                 const int kb = kb0 + i;
-                const bool u = kb >= p.nkb_r;
+                const bool u = kb >= p.nkb_m;
                 tma_load_2d(b_base + s * b_bytes + (uint32_t)(lane * p.direct.KP * BK * 2), &tmB.m[u ? 1 : 0],
-                            (u ? kb - p.nkb_r : kb) * BK, lane * p.direct.K + my_A + (u ? 0 : 1), smem_u32(&bar_full[s]));
+                            (u ? kb - p.nkb_m : kb) * BK, lane * p.direct.K + my_A + (u ? 0 : 1), smem_u32(&bar_full[s]));
               }
               continue;
             }
@@ -1546,9 +1589,7 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
             load_a(mt, kb0 + i, s);
           }
           mbar_arrive_expect_tx(smem_u32(&bar_full[s]), b_bytes);
-          const int kb = kb0 + i;
-          if (kb < p.nkb_r) tma_load_2d(b_base + s * b_bytes, mb, kb * BK, row0, smem_u32(&bar_full[s]));
-          else tma_load_2d(b_base + s * b_bytes, me, (kb - p.nkb_r) * BK, row0, smem_u32(&bar_full[s]));
+          tma_load_2d(b_base + s * b_bytes, mb, (kb0 + i) * BK, row0, smem_u32(&bar_full[s]));
         }
         if (i < kb1 - kb0 && lane == 0) {
           // a wait expired: flag it, let the copies in flight land
@@ -1615,8 +1656,10 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
     if (go) {
       // this CTA's rows of the tile
       const int l0 = (int)rank * rows / S, l1 = ((int)rank + 1) * rows / S;
-      const int total = (l1 - l0) * (p.gate ? 16 : 32);  // four features each
-      if (p.gate) {
+      const int total = (l1 - l0) * (p.gate == kGateStacked ? 16 : 32);  // four features each
+      if (p.gate == kGateParts) {
+        if constexpr (!DIRECT) swap_parts_rows(p, smem_u32(P), mt, row0, l0, total);
+      } else if (p.gate) {
         if (total <= SW_THREADS) swap_gate_rows<DIRECT, 1, 8>(p, smem_u32(P), mt, row0, l0, total, s_A);
         else swap_gate_rows<DIRECT, 4, 2>(p, smem_u32(P), mt, row0, l0, total, s_A);
       } else {
@@ -1808,22 +1851,24 @@ static int swap_cluster_capacity(int dev, int S, int smem, cudaError_t* err) {
 // Cluster size of a small-R GEMM: the one with the least estimated time at
 // three quarters of the possible rows (R itself is known on the device only;
 // direct rows: one tile of all the tile rows).
+// A cluster holds `parts` products of the k-blocks.
 // A wave of units costs its k-blocks, 2 (128 + N) cycles each (the stage's
 // bytes in and out of shared memory), plus the drain and the sum of the
 // partial (about 24 cycles per row of the tile) and the fixed start and end.
-static cudaError_t swap_pick_splits(int dev, int smem, int rmax, bool direct, int mtiles, int nkb, int* S_out,
-                                    int* clusters) {
+static cudaError_t swap_pick_splits(int dev, int smem, int rmax, bool direct, int parts, int mtiles, int nkb,
+                                    int* S_out, int* clusters) {
   const int Rt = direct ? rmax : (3 * rmax + 3) / 4;
   long long best = -1;
   cudaError_t err = cudaSuccess;
-  for (int S = 8; S >= 1; --S) {
-    if (S > 1 && nkb / S < SW_MIN_BLOCKS) continue;
+  for (int S = 8 / parts * parts; S >= parts; S -= parts) {
+    const int splits = S / parts;
+    if (splits > 1 && nkb / splits < SW_MIN_BLOCKS) continue;
     const int cap = swap_cluster_capacity(dev, S, smem, &err);
     if (err != cudaSuccess) return err;
     if (cap == 0) continue;
     const SwapCut cut = direct ? SwapCut{1, (Rt + 15) / 16 * 16} : swap_cut(Rt, mtiles, cap);
     const long long waves = ((long long)mtiles * cut.ntiles + cap - 1) / cap;
-    const long long cost = waves * ((long long)((nkb + S - 1) / S) * 2 * (128 + cut.tile_n) + 24 * cut.tile_n + 2500);
+    const long long cost = waves * ((long long)((nkb + splits - 1) / splits) * 2 * (128 + cut.tile_n) + 24 * cut.tile_n + 2500);
     if (best < 0 || cost < best) {
       best = cost;
       *S_out = S;
@@ -1916,14 +1961,14 @@ static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
           encode_tensor_map_2d(&mB.m[1], a.hT, du, all, 2 * du, BK, box) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
       c.row_maps = 2;
-      c.nkb_r = (d + BK - 1) / BK;
-      c.nkb = 2 * c.nkb_r;
+      c.nkb_m = (d + BK - 1) / BK;
+      c.nkb = 2 * c.nkb_m;
     } else {
       if (encode_tensor_map_2d(&mA, a.Wc, 2 * du, du, 4 * du, BK, 128) != CUDA_SUCCESS ||
           !encode_row_maps(&mB, a.apack, 2 * du, rmax, 4 * du))
         return cudaErrorInvalidValue;
       mA2 = mA;
-      c.nkb = c.nkb_r = (2 * d + BK - 1) / BK;
+      c.nkb = (2 * d + BK - 1) / BK;
     }
     c.apack = reinterpret_cast<const __nv_bfloat16*>(a.apack);
     c.beta = a.beta;
@@ -1931,7 +1976,7 @@ static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
     c.compact_out = a.compact_out;
     if (a.do_gate && !a.e_dense) c.bias = gp;
     int clusters = 0;
-    if ((err = swap_pick_splits(dev, smem, rmax, direct, c.mtiles, c.nkb, &c.S, &clusters)) != cudaSuccess) return err;
+    if ((err = swap_pick_splits(dev, smem, rmax, direct, 1, c.mtiles, c.nkb, &c.S, &clusters)) != cudaSuccess) return err;
     err = launch_dependent(direct ? swap_cluster_kernel<true> : swap_cluster_kernel<false>, grid_of(c, clusters),
                            dim3(SW_THREADS), (size_t)smem, stream, (unsigned)c.S, mA, mA2, mA, mB, mB, c);
     if (err != cudaSuccess) return err;
@@ -1940,9 +1985,10 @@ static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
     const uint64_t rstride = 2 * (a.r_row_stride ? (uint64_t)a.r_row_stride : du);
     CUtensorMap mA, mA2, mA3;
     RowMaps mB, mE;
-    if (encode_tensor_map_2d(&mA, a.Wv, du, du, 2 * du, BK, 64) != CUDA_SUCCESS ||
-        encode_tensor_map_2d(&mA2, a.Wg, 2 * du, du, 4 * du, BK, 64) != CUDA_SUCCESS ||
-        encode_tensor_map_2d(&mA3, a.Wg, du, du, 4 * du, BK, 64) != CUDA_SUCCESS ||  // the e half: zeros past column d
+    const uint32_t box = a.e_dense ? 128 : 64;
+    if (encode_tensor_map_2d(&mA, a.Wv, du, du, 2 * du, BK, box) != CUDA_SUCCESS ||
+        encode_tensor_map_2d(&mA2, a.Wg, 2 * du, du, 4 * du, BK, box) != CUDA_SUCCESS ||
+        encode_tensor_map_2d(&mA3, a.Wg, du, du, 4 * du, BK, box) != CUDA_SUCCESS ||  // the e half: zeros past column d
         !encode_row_maps(&mB, a.rpack, du, rmax, rstride) ||
         (a.e_dense && !encode_row_maps(&mE, a.epack, du, rmax, 2 * du)))
       return cudaErrorInvalidValue;
@@ -1951,15 +1997,14 @@ static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
       if (err != cudaSuccess) return err;
     }
     SwapClusterParams g = sp;
-    g.mtiles = (d + 63) / 64;
-    g.nkb_r = (d + BK - 1) / BK;
-    g.nkb = a.e_dense ? 2 * g.nkb_r : g.nkb_r;
-    g.gate = 1;
+    g.mtiles = a.e_dense ? (d + 127) / 128 : (d + 63) / 64;
+    g.nkb = (d + BK - 1) / BK;
+    g.gate = a.e_dense ? kGateParts : kGateStacked;
     g.e = reinterpret_cast<const __nv_bfloat16*>(a.e_dense ? a.epack : a.e);
-    g.ge = a.e_dense ? nullptr : a.ge;
+    g.ge = a.ge;
     g.e_out = reinterpret_cast<__nv_bfloat16*>(a.e_out);
     int clusters = 0;
-    if ((err = swap_pick_splits(dev, smem, rmax, direct, g.mtiles, g.nkb, &g.S, &clusters)) != cudaSuccess) return err;
+    if ((err = swap_pick_splits(dev, smem, rmax, direct, a.e_dense ? 3 : 1, g.mtiles, g.nkb, &g.S, &clusters)) != cudaSuccess) return err;
     err = launch_dependent(direct ? swap_cluster_kernel<true> : swap_cluster_kernel<false>, grid_of(g, clusters),
                            dim3(SW_THREADS), (size_t)smem, stream, (unsigned)g.S, mA, mA2, mA3, mB,
                            a.e_dense ? mE : mB, g);
