@@ -94,9 +94,18 @@ def _ptr(t):
     return t.data_ptr()
 
 
+# The current stream's handle without building a torch Stream object (0.1
+# against 3 us of a call that takes 10 to 20 us to enqueue).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return s.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None or _current_device is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_current_device())
 
 
 def retrace_workspace_bytes(B: int, K: int, V: int, d: int, dtype: torch.dtype) -> int:
