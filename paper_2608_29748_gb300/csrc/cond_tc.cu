@@ -1605,25 +1605,25 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
       __syncwarp();
     } else if (warp == 1) {
       // ---------------- MMA issuer ----------------
-      if (lane == 0) {
-        const uint32_t idesc = idesc_bf16_f32(128, mma_n);
-        bool ok = true;
-        for (int i = 0; i < kb1 - kb0; ++i, advance()) {
-          if (!mbar_wait_bounded(smem_u32(&bar_full[s]), ph, &s_abort)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint64_t adesc0 = sw128_kmajor_desc(base + s * (uint32_t)SW_A_BYTES);
-          const uint64_t bdesc0 = sw128_kmajor_desc(b_base + s * b_bytes);
+      // (the whole warp waits, one lane issues: 1.5 % of a round against a loop in lane 0)
+      const uint32_t idesc = idesc_bf16_f32(128, mma_n);
+      bool ok = true;
+      for (int i = 0; i < kb1 - kb0; ++i, advance()) {
+        ok = __all_sync(0xFFFFFFFFu, mbar_wait_bounded(smem_u32(&bar_full[s]), ph, &s_abort));
+        if (!ok) break;
+        tc_fence_after();
+        const uint64_t adesc0 = sw128_kmajor_desc(base + s * (uint32_t)SW_A_BYTES);
+        const uint64_t bdesc0 = sw128_kmajor_desc(b_base + s * b_bytes);
+        if (elect_one()) {
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k)
             tc_mma_bf16(tmem, adesc0 + 2u * k, bdesc0 + 2u * k, idesc, (i > 0 || k > 0) ? 1u : 0u);
           tc_commit(smem_u32(&bar_empty[s]));
         }
-        if (!ok) raise_abort(&s_abort, p.status);
-        tc_commit(smem_u32(&bar_acc));  // accumulator ready (also after a failure)
+        __syncwarp();
       }
+      if (!ok && lane == 0) raise_abort(&s_abort, p.status);
+      if (elect_one()) tc_commit(smem_u32(&bar_acc));  // accumulator ready (also after a failure)
       __syncwarp();
     }
     // ---------------- the partial into shared memory (every warp) ----------------
