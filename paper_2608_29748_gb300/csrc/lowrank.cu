@@ -10,7 +10,8 @@
 // z and rho are rounded to bf16 where they are stored (bf16 workloads); e is
 // the broadcast mask embedding, so W_g[:, :d] e is one GEMV per call.
 //
-// Tensor-core path (bf16, d a multiple of 128), three launches:
+// Tensor-core path (bf16, d a multiple of 8, at least 64; past the operands'
+// ends the copies fill zeros), three launches:
 //   lr_project_kernel  split-K over the packed [m; u] rows: the m half against
 //                      P (N = 64), the u half against B_c's u columns (N = 32),
 //                      fp32 partials per split;
@@ -103,8 +104,9 @@ __device__ __forceinline__ float bf16_round(float x) { return __bfloat162float(_
 // grid (row blocks, 2H): blockIdx.y < H reduces over the m half against P,
 // the rest over the u half against B_c[:, 64:].
 __global__ void __launch_bounds__(256, 1)
-    lr_project_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmP,
-                      const __grid_constant__ CUtensorMap tmBc, const LrParams p) {
+    lr_project_kernel(const __grid_constant__ CUtensorMap tmM, const __grid_constant__ CUtensorMap tmU,
+                      const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CUtensorMap tmBc,
+                      const LrParams p) {
   extern __shared__ uint8_t dsmem[];
   __shared__ __align__(8) uint64_t bar_full[ST];
   __shared__ __align__(8) uint64_t bar_empty[ST];
@@ -120,7 +122,7 @@ __global__ void __launch_bounds__(256, 1)
   if (m0 >= R) return;
   const int d = p.d;
   const int half = (int)blockIdx.y / H, part = (int)blockIdx.y % H;
-  const int KB = d / BK;  // k-blocks per half
+  const int KB = (d + BK - 1) / BK;  // k-blocks per half
   const int kb0 = part * KB / H, kb1 = (part + 1) * KB / H;
   const int nkb = kb1 - kb0;
   const int N = half == 0 ? L : C;
@@ -157,7 +159,7 @@ __global__ void __launch_bounds__(256, 1)
         const uint32_t a_dst = base + s * STAGE_BYTES, b_dst = a_dst + A_BYTES;
         const int kb = kb0 + i;
         mbar_arrive_expect_tx(smem_u32(&bar_full[s]), A_BYTES + N * BK * 2);
-        tma_load_2d(a_dst, &tmA, half * d + kb * BK, m0, smem_u32(&bar_full[s]));
+        tma_load_2d(a_dst, half == 0 ? &tmM : &tmU, kb * BK, m0, smem_u32(&bar_full[s]));
         if (half == 0)
           tma_load_2d(b_dst, &tmP, kb * BK, 0, smem_u32(&bar_full[s]));
         else
@@ -303,7 +305,7 @@ __global__ void __launch_bounds__(kFuseThreads, 2)
   pdl_wait();  // rho and W_g[:, :d] e come from the finishing kernel
   const int R = *(volatile const int32_t*)p.R;
   const int d = p.d;
-  const int nb = d / kFuseFeat;
+  const int nb = (d + kFuseFeat - 1) / kFuseFeat;
   const int tiles = (R + BM - 1) / BM * nb;
   if ((int)blockIdx.x >= tiles) return;
   const int my_tiles = (tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
@@ -412,6 +414,7 @@ __global__ void __launch_bounds__(kFuseThreads, 2)
         uint4* ov = reinterpret_cast<uint4*>(p.e_out + orow * d + n);
 #pragma unroll
         for (int x = 0; x < 4; ++x) {
+          if (n + x * 8 >= d) break;  // past the last feature
           const uint4 ew = __ldg(ev + x);
           const float4 ga = __ldg(gv + 2 * x), gb = __ldg(gv + 2 * x + 1);
           const float gw[8] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w};
@@ -486,21 +489,44 @@ __global__ void __launch_bounds__(256) lr_simt_kernel(const LowRankArgs a) {
   const T* Wv = reinterpret_cast<const T*>(a.Wv);
   const T* Wg = reinterpret_cast<const T*>(a.Wg);
   const T* e = reinterpret_cast<const T*>(a.e);
-  for (int i = warp; i < L; i += 8) {  // z = P m
-    float s = 0.f;
-    for (int k = lane; k < d; k += 32) s = fmaf(to_f32(P[(long long)i * d + k]), to_f32(m[k]), s);
+  // z = P m, eight rows of P per warp at a time (one at a time, a warp walked
+  // eight reductions of d / 32 dependent loads one after another)
+  {
+    constexpr int N = L / 8;
+    float s[N];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, off);
-    if (lane == 0) s_z[i] = rnd ? bf16_round(s) : s;
+    for (int r = 0; r < N; ++r) s[r] = 0.f;
+#pragma unroll 2
+    for (int k = lane; k < d; k += 32) {
+      const float mk = to_f32(m[k]);
+#pragma unroll
+      for (int r = 0; r < N; ++r) s[r] = fmaf(to_f32(P[(long long)(warp * N + r) * d + k]), mk, s[r]);
+    }
+#pragma unroll
+    for (int r = 0; r < N; ++r) {
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) s[r] += __shfl_xor_sync(0xFFFFFFFFu, s[r], off);
+      if (lane == 0) s_z[warp * N + r] = rnd ? bf16_round(s[r]) : s[r];
+    }
   }
   __syncthreads();
-  for (int c = warp; c < C; c += 8) {  // t = B_c [z; u]
-    const T* brow = Bc + (long long)c * (L + d);
-    float s = 0.f;
-    for (int k = lane; k < L + d; k += 32) s = fmaf(to_f32(brow[k]), k < L ? s_z[k] : to_f32(u[k - L]), s);
+  {  // t = B_c [z; u], four rows of B_c per warp at a time
+    constexpr int N = C / 8;
+    float s[N];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, off);
-    if (lane == 0) s_t[c] = s;
+    for (int r = 0; r < N; ++r) s[r] = 0.f;
+#pragma unroll 4
+    for (int k = lane; k < L + d; k += 32) {
+      const float x = k < L ? s_z[k] : to_f32(u[k - L]);
+#pragma unroll
+      for (int r = 0; r < N; ++r) s[r] = fmaf(to_f32(Bc[(long long)(warp * N + r) * (L + d) + k]), x, s[r]);
+    }
+#pragma unroll
+    for (int r = 0; r < N; ++r) {
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) s[r] += __shfl_xor_sync(0xFFFFFFFFu, s[r], off);
+      if (lane == 0) s_t[warp * N + r] = s[r];
+    }
   }
   __syncthreads();
   if (threadIdx.x < L) {  // rho = z + beta A_c t
@@ -526,7 +552,7 @@ __global__ void __launch_bounds__(256) lr_simt_kernel(const LowRankArgs a) {
 
 }  // namespace
 
-bool lowrank_tc_supported(retrace_dtype dtype, int d) { return dtype == RETRACE_BF16 && d % kFuseFeat == 0; }
+bool lowrank_tc_supported(retrace_dtype dtype, int d) { return dtype == RETRACE_BF16 && d % 8 == 0 && d >= 64; }
 
 cudaError_t launch_lowrank(const LowRankArgs& a, bool tc, cudaStream_t stream) {
   const long long rmax = (long long)a.B * (a.K > 1 ? a.K - 1 : 0);
@@ -561,8 +587,10 @@ cudaError_t launch_lowrank(const LowRankArgs& a, bool tc, cudaStream_t stream) {
     attr_done[info.device & 63].store(1, std::memory_order_release);
   }
   const uint64_t d = (uint64_t)a.d;
-  CUtensorMap mA, mP, mBc, mRho, mWv, mWg;
-  if (encode_tensor_map_2d(&mA, a.apack, 2 * d, (uint64_t)rmax, 4 * d, BK, BM) != CUDA_SUCCESS ||
+  CUtensorMap mM, mU, mP, mBc, mRho, mWv, mWg;
+  // the m and u halves of the packed rows apart: zeros past column d of either
+  if (encode_tensor_map_2d(&mM, a.apack, d, (uint64_t)rmax, 4 * d, BK, BM) != CUDA_SUCCESS ||
+      encode_tensor_map_2d(&mU, static_cast<const __nv_bfloat16*>(a.apack) + d, d, (uint64_t)rmax, 4 * d, BK, BM) != CUDA_SUCCESS ||
       encode_tensor_map_2d(&mP, a.P, d, L, 2 * d, BK, L) != CUDA_SUCCESS ||
       encode_tensor_map_2d(&mBc, a.Bc, L + d, C, 2 * (L + d), BK, C) != CUDA_SUCCESS ||
       encode_tensor_map_2d(&mRho, a.rho, L, (uint64_t)rmax, 2 * L, BK, BM) != CUDA_SUCCESS ||
@@ -586,7 +614,7 @@ cudaError_t launch_lowrank(const LowRankArgs& a, bool tc, cudaStream_t stream) {
   p.status = a.status;
   // Each of the three kernels may start while the previous one finishes
   // (programmatic dependent launch), and waits for its outputs in the kernel.
-  if ((err = launch_dependent(lr_project_kernel, dim3(mt, 2 * H), dim3(256), SMEM_PROJECT, stream, 1, mA, mP, mBc,
+  if ((err = launch_dependent(lr_project_kernel, dim3(mt, 2 * H), dim3(256), SMEM_PROJECT, stream, 1, mM, mU, mP, mBc,
                               p)) != cudaSuccess)
     return err;
   const long long fgrid = (rmax + 7) / 8 > 2LL * info.sm_count ? (rmax + 7) / 8 : 2LL * info.sm_count;
@@ -600,7 +628,7 @@ cudaError_t launch_lowrank(const LowRankArgs& a, bool tc, cudaStream_t stream) {
   f.ge = a.ge;
   f.e_out = reinterpret_cast<__nv_bfloat16*>(a.e_out);
   f.status = a.status;
-  const long long tiles_max = (long long)mt * (a.d / kFuseFeat);
+  const long long tiles_max = (long long)mt * ((a.d + kFuseFeat - 1) / kFuseFeat);
   const long long slots = 2LL * info.sm_count;  // two CTAs per SM
   const unsigned grid = (unsigned)(tiles_max < slots ? tiles_max : slots);
   return launch_dependent(lr_fuse_kernel, dim3(grid), dim3(kFuseThreads), SMEM_FUSE, stream, 1, mRho, mWv, mWg, f);

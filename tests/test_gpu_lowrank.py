@@ -122,3 +122,17 @@ def test_lowrank_repeatable_bitwise_and_graph(rt):
     torch.cuda.synchronize()
     assert torch.equal(out.e_out, first.e_out)
     assert ws.check() == 0
+
+
+@pytest.mark.parametrize("d,dtype", [(72, "bf16"), (136, "bf16"), (1176, "bf16"),  # tensor cores, a ragged last block
+                                     (68, "bf16"), (33, "f32"), (260, "f32")])  # FFMA
+def test_lowrank_hidden_sizes(rt, d, dtype):
+    """Hidden sizes that are no multiple of the kernels' blocks, on both paths."""
+    cfg = CONFIGS[2].__class__("lowrank", 11, 9, 515, d, dtype, 1.0, "uniform", seed_offset=d)
+    x = make_round_inputs(cfg, device="cuda")
+    w = make_lowrank_weights(cfg, device="cuda")
+    out, targ, ws = run(rt, x, w)
+    assert ws.check() == 0
+    want = oracle_lowrank(x, w)
+    assert_verify_exact(want, out.accept_len, out.committed, out.bonus, targ)
+    assert_close(out.e_out, want["e_tilde"], f"low-rank e~, d={d}")
