@@ -157,8 +157,38 @@ __device__ __forceinline__ float gate_bias_row(const T* Wg, const T* e, int i, i
   return warp_sum(s);
 }
 
+// Stages the weight rows of chunk c (of chunks [c0, c1)) of the unit at n0.
+template <typename T, bool GATE>
+__device__ __forceinline__ void stage_weights(const SimtParams& p, float* ring, int n0, int c, int c0) {
+  const int tid = threadIdx.x, d = p.d, per = (d + TK - 1) / TK;  // chunks per part
+  const int part = c >= per ? 1 : 0, kc = (c - part * per) * TK + (tid % 8) * 4;
+  const T* W = reinterpret_cast<const T*>(p.w);
+  const T* Wg = reinterpret_cast<const T*>(p.wg);
+  float* Bs = ring + (c - c0) % kSimtStages * kStageFloats + kTileRows * kLd;
+#pragma unroll
+  for (int i = 0; i < TN / 32; ++i) {
+    const int r = tid / 8 + 32 * i;
+    const T* src;
+    if constexpr (!GATE) {
+      const int n = n0 + r;
+      src = n < d ? W + (long long)n * 2 * d + (long long)part * d : nullptr;
+    } else {
+      const int n = n0 + (r & 31);  // i = 0: rows of W_v, i = 1: the same rows of W_g
+      if (i == 0) {
+        if (part) continue;  // the e part has a gate only
+        src = n < d ? W + (long long)n * d : nullptr;
+      } else {
+        src = n < d ? Wg + (long long)n * 2 * d + (part ? 0 : d) : nullptr;
+      }
+    }
+    stage4<T>(Bs + r * kLd + (tid % 8) * 4, src, kc, d, W, p.vec != 0);
+  }
+}
+constexpr int kSimtAhead = kSimtStages - 1;  // chunks staged ahead
+
 // The partial tile of this CTA: its chunks [c0, c1) of the unit with weight
 // tile n0, rows at s_off0 / s_off1 (-1: no row), into ring[] as [row][TN].
+// The weights of the first kSimtAhead chunks are staged already.
 template <typename T, bool GATE, int MR>
 __device__ __forceinline__ void simt_partial(const SimtParams& p, float* ring, const long long* s_off0,
                                              const long long* s_off1, int n0, int c0, int c1) {
@@ -166,40 +196,19 @@ __device__ __forceinline__ void simt_partial(const SimtParams& p, float* ring, c
   const int per = (d + TK - 1) / TK;  // chunks per part
   const T* A0 = reinterpret_cast<const T*>(p.a0);
   const T* A1 = reinterpret_cast<const T*>(p.a1);
-  const T* W = reinterpret_cast<const T*>(p.w);
-  const T* Wg = reinterpret_cast<const T*>(p.wg);
-  const bool vec = p.vec != 0;
-  auto stage = [&](int c) {
+  auto stage = [&](int c, bool weights) {
     if (c < c1) {
       const int part = c >= per ? 1 : 0, kc = (c - part * per) * TK + (tid % 8) * 4;
       float* As = ring + (c - c0) % kSimtStages * kStageFloats;
-      float* Bs = As + kTileRows * kLd;
 #pragma unroll
       for (int i = 0; i < (MR + 1) / 2; ++i) {
         const int r = tid / 8 + 32 * i;
         if (r < 16 * MR) {
           const long long off = part ? s_off1[r] : s_off0[r];
-          stage4<T>(As + r * kLd + (tid % 8) * 4, off >= 0 ? (part ? A1 : A0) + off : nullptr, kc, d, W, vec);
+          stage4<T>(As + r * kLd + (tid % 8) * 4, off >= 0 ? (part ? A1 : A0) + off : nullptr, kc, d, p.w, p.vec != 0);
         }
       }
-#pragma unroll
-      for (int i = 0; i < TN / 32; ++i) {
-        const int r = tid / 8 + 32 * i;
-        const T* src;
-        if constexpr (!GATE) {
-          const int n = n0 + r;
-          src = n < d ? W + (long long)n * 2 * d + (long long)part * d : nullptr;
-        } else {
-          const int n = n0 + (r & 31);  // i = 0: rows of W_v, i = 1: the same rows of W_g
-          if (i == 0) {
-            if (part) continue;  // the e part has a gate only
-            src = n < d ? W + (long long)n * d : nullptr;
-          } else {
-            src = n < d ? Wg + (long long)n * 2 * d + (part ? 0 : d) : nullptr;
-          }
-        }
-        stage4<T>(Bs + r * kLd + (tid % 8) * 4, src, kc, d, W, vec);
-      }
+      if (weights) stage_weights<T, GATE>(p, ring, n0, c, c0);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
@@ -209,11 +218,11 @@ __device__ __forceinline__ void simt_partial(const SimtParams& p, float* ring, c
 #pragma unroll
     for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
 #pragma unroll
-  for (int q = 0; q < kSimtStages - 1; ++q) stage(c0 + q);
+  for (int q = 0; q < kSimtAhead; ++q) stage(c0 + q, false);
   for (int c = c0; c < c1; ++c) {
-    asm volatile("cp.async.wait_group %0;" ::"n"(kSimtStages - 2) : "memory");
+    asm volatile("cp.async.wait_group %0;" ::"n"(kSimtAhead - 1) : "memory");
     __syncthreads();  // chunk c is staged, and chunk c - 1's slot is read
-    stage(c + kSimtStages - 1);
+    stage(c + kSimtAhead, true);
     const float* As = ring + (c - c0) % kSimtStages * kStageFloats + ty * kLd;
     const float* Bs = ring + (c - c0) % kSimtStages * kStageFloats + (kTileRows + tx) * kLd;
     const bool gate_only = GATE && c >= per;
@@ -264,11 +273,26 @@ __global__ void __launch_bounds__(kNT, 2) simt_cluster_kernel(const SimtParams p
     }
     return;
   }
+  // The weights are inputs: those of this CTA's first chunks come while the
+  // previous kernel ends and the rows are planned.
+  const uint32_t rank = cluster_rank();
+  constexpr int F = GATE ? 32 : 64;  // features of a unit
+  const int n0 = cid % p.ftiles * F;
+  const int per = (d + TK - 1) / TK;
+  const int chunks = GATE ? per * (p.e_dense ? 2 : 1) : (p.raw ? 0 : 2 * per);
+  const int c0 = (int)((long long)rank * chunks / S), c1 = (int)((long long)(rank + 1) * chunks / S);
+#pragma unroll
+  for (int q = 0; q < kSimtAhead; ++q)
+    if (c0 + q < c1) stage_weights<T, GATE>(p, ring, n0, c0 + q, c0);
+  asm volatile("cp.async.commit_group;" ::: "memory");
   pdl_wait();  // the accepted lengths (and r) come from the previous kernels
   int tile;
   long long m0;
   const int R = plan_row_tile(p.rows, p.B, K, cid / p.ftiles, s_b, s_j, s_nb, s_scan, &tile, &m0);
-  if (m0 >= R) return;  // the whole cluster
+  if (m0 >= R) {  // the whole cluster
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    return;
+  }
   const int rows = (int)(R - m0 < tile ? R - m0 : tile);
   if (tid < kTileRows) {
     const int b = s_b[tid];
@@ -285,12 +309,6 @@ __global__ void __launch_bounds__(kNT, 2) simt_cluster_kernel(const SimtParams p
     }
   }
   __syncthreads();
-  const uint32_t rank = cluster_rank();
-  constexpr int F = GATE ? 32 : 64;  // features of a unit
-  const int n0 = cid % p.ftiles * F;
-  const int per = (d + TK - 1) / TK;
-  const int chunks = GATE ? per * (p.e_dense ? 2 : 1) : (p.raw ? 0 : 2 * per);
-  const int c0 = (int)((long long)rank * chunks / S), c1 = (int)((long long)(rank + 1) * chunks / S);
   if (tile == 16) simt_partial<T, GATE, 1>(p, ring, s_off0, s_off1, n0, c0, c1);
   else if (tile == 32) simt_partial<T, GATE, 2>(p, ring, s_off0, s_off1, n0, c0, c1);
   else if (tile == 48) simt_partial<T, GATE, 3>(p, ring, s_off0, s_off1, n0, c0, c1);
