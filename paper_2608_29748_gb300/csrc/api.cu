@@ -832,6 +832,13 @@ retrace_status retrace_round_lowrank(const void* logits, int64_t logits_row_stri
   va.d = d;
   va.hD = hD;
   va.cond_copy = kCondCopyKeep;
+  int ge_ready = 0;
+  if (tc) {
+    va.gate_W = Wg;
+    va.gate_ge = reinterpret_cast<float*>(w + Lw.ge);
+    va.gate_ld = d + RETRACE_LOWRANK_LATENT;
+    va.gate_done = &ge_ready;
+  }
   va.plain_first = 1;  // measured: 79-81 us against 87 with the next round's CTAs waiting beside lr_fuse_kernel's
   if (tc) {  // the finalising CTA of each sequence packs its [m; u] rows
     va.hT = hT;
@@ -861,6 +868,7 @@ retrace_status retrace_round_lowrank(const void* logits, int64_t logits_row_stri
   la.accept_len = accept_len;
   la.e_out = e_out;
   la.ge = reinterpret_cast<float*>(w + Lw.ge);
+  la.ge_ready = ge_ready;
   la.apack = w + Lw.apack;
   la.rowmap = rowmap;
   la.R = R;

@@ -184,6 +184,37 @@ __device__ __forceinline__ void gate_bias_share(const __nv_bfloat16* e, const __
   }
 }
 
+// The same with four loads in flight and few registers, for kernels that have
+// many warps and a row or two for each.
+__device__ __forceinline__ void gate_bias_share_small(const __nv_bfloat16* e, const __nv_bfloat16* Wg, float* ge, int d,
+                                                      int ld, int w, int nw, int lane) {
+  const int vpr = d / 8;
+  const uint4* ev = reinterpret_cast<const uint4*>(e);
+  for (int row = w; row < d; row += nw) {
+    const uint4* wr = reinterpret_cast<const uint4*>(Wg + (long long)row * ld);
+    float acc = 0.f;
+    for (int v0 = lane; v0 < vpr; v0 += 4 * 32) {
+      uint4 x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) x[u] = v0 + u * 32 < vpr ? __ldcs(wr + v0 + u * 32) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (v0 + u * 32 >= vpr) continue;
+        const uint4 y = __ldg(ev + v0 + u * 32);
+        const uint32_t xx[4] = {x[u].x, x[u].y, x[u].z, x[u].w}, yy[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          acc = fmaf(bf16_lo(xx[q]), bf16_lo(yy[q]), acc);
+          acc = fmaf(bf16_hi(xx[q]), bf16_hi(yy[q]), acc);
+        }
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
+    if (lane == 0) ge[row] = acc;
+  }
+}
+
 // ---------------------------------------------------------------------------
 // Programmatic dependent launch: a kernel launched with the programmatic
 // stream-serialisation attribute may start once every CTA of the previous

@@ -218,6 +218,13 @@ struct VerifyArgs {
   // One pass that only folds the argmax keys: a direct-rows conditioning
   // decides the sequences, writes the outputs and zeroes the keys.
   int keys_only;
+  // The gate's W_g[:, :d] e (W_g's rows gate_ld elements apart), by the finish
+  // kernel while the last pass ends; *gate_done tells whether the schedule has
+  // that kernel (gate_ge NULL: not wanted).
+  const void* gate_W;
+  float* gate_ge;
+  int gate_ld;
+  int* gate_done;
   int plain_first;  // the first kernel without programmatic dependence on what precedes it
 };
 constexpr int kCondCopyKeep = 0;
@@ -424,6 +431,7 @@ struct LowRankArgs {
   const int32_t* accept_len;
   void* e_out;
   float* ge;  // [d]: W_g[:, :d] e
+  int ge_ready;  // computed already
   // tensor-core path: rows packed by the verification kernel
   const void* apack;
   const int32_t* rowmap;

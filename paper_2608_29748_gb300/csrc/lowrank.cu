@@ -68,7 +68,7 @@ struct LrParams {
   float* tpart;             // [H, R_max, 32]
   __nv_bfloat16* rho;       // [R_max, 64]
   long long rmax;
-  // W_g[:, :d] e
+  // W_g[:, :d] e (ge NULL: computed already)
   const __nv_bfloat16* Wg;  // [d, d + 64]
   const __nv_bfloat16* e;   // [d]
   float* ge;                // [d]
@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(256) lr_finish_kernel(const LrParams p) {
   pdl_launch_dependents();
   const long long g = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int d = p.d, lane = threadIdx.x & 31;
-  gate_bias_share(p.e, p.Wg, p.ge, d, d + L, (int)blockIdx.x * 8 + (threadIdx.x >> 5), (int)gridDim.x * 8, lane);
+  if (p.ge) gate_bias_share(p.e, p.Wg, p.ge, d, d + L, (int)blockIdx.x * 8 + (threadIdx.x >> 5), (int)gridDim.x * 8, lane);
   pdl_wait();
   const int R = *(volatile const int32_t*)p.R;
   if ((long long)blockIdx.x * 8 < R) finish_rows(p, g, R, d, lane);  // uniform over the CTA
@@ -610,7 +610,7 @@ cudaError_t launch_lowrank(const LowRankArgs& a, bool tc, cudaStream_t stream) {
   p.rmax = rmax;
   p.Wg = reinterpret_cast<const __nv_bfloat16*>(a.Wg);
   p.e = reinterpret_cast<const __nv_bfloat16*>(a.e);
-  p.ge = a.ge;
+  p.ge = a.ge_ready ? nullptr : a.ge;
   p.status = a.status;
   // Each of the three kernels may start while the previous one finishes
   // (programmatic dependent launch), and waits for its outputs in the kernel.

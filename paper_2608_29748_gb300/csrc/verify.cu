@@ -80,6 +80,9 @@ struct VerifyParams {
   uint32_t* pass_counts;
   int n_counts;
   uint32_t* exits;           // CTAs out (zero between calls)
+  const void* gate_W;        // verify_finish_kernel: W_g[:, :d] e into gate_ge (NULL: not computed)
+  float* gate_ge;
+  int gate_ld;
   uint32_t* sync;            // verify_finish_kernel: counters of the conditioning, zeroed but for R_count
   int sync_words;
   int defer_copies;          // the finaliser leaves the copies to verify_copy_kernel
@@ -625,6 +628,12 @@ __global__ void __launch_bounds__(kThreads, 2) verify_finish_kernel(const Verify
   __shared__ int s_warp[kThreads / 32 + 1];
   __shared__ int s_last;
   pdl_launch_dependents();
+  if constexpr (sizeof(T) == 2) {
+    if (p.gate_ge)  // inputs only: while the last pass ends
+      gate_bias_share_small(reinterpret_cast<const __nv_bfloat16*>(p.e), reinterpret_cast<const __nv_bfloat16*>(p.gate_W),
+                            p.gate_ge, p.d, p.gate_ld, (int)blockIdx.x * (kThreads / 32) + (int)(threadIdx.x >> 5),
+                            (int)gridDim.x * (kThreads / 32), threadIdx.x & 31);
+  }
   pdl_wait();
   const int B = p.B, K = p.K, K1 = K + 1;
   // after a single pass (no live lists) every sequence is decided here
@@ -813,6 +822,9 @@ cudaError_t launch_typed(const VerifyArgs& a, cudaStream_t stream) {
   p.pass_counts = nullptr;
   p.n_counts = 0;
   p.exits = nullptr;
+  p.gate_W = a.gate_W;
+  p.gate_ge = a.gate_ge;
+  p.gate_ld = a.gate_ld;
   p.sync = reinterpret_cast<uint32_t*>(a.R_count) - kSyncRowCount;  // R_count is a word of the sync area
   p.sync_words = a.R_count ? (int)(a.sync_bytes / 4) : 0;
   p.defer_copies = 0;
@@ -863,7 +875,8 @@ cudaError_t launch_typed(const VerifyArgs& a, cudaStream_t stream) {
       p.n_counts = 2 * kMaxWindowPasses + 1;
       p.exits = a.pass_counts;
       long long fgrid = ((long long)a.B * a.K * 3 + 15) / 16;  // about a warp per row segment
-      if (fgrid > grid_full) fgrid = grid_full;
+      if (fgrid > grid_full || a.gate_ge) fgrid = grid_full;
+      if (a.gate_done) *a.gate_done = 1;
       return launch_finish<T>(a, p, fgrid < 1 ? 1 : fgrid, stream);
     }
     p.defer_copies = defer ? 1 : 0;
@@ -914,6 +927,7 @@ cudaError_t launch_typed(const VerifyArgs& a, cudaStream_t stream) {
   p.pass_counts = a.pass_counts + 1;
   p.n_counts = 2 * kMaxWindowPasses + 1;  // every live count and base after the exit counter
   p.exits = a.pass_counts;
+  if (a.gate_done) *a.gate_done = 1;
   return launch_finish<T>(a, p, grid_full, stream);
 }
 
