@@ -32,10 +32,11 @@
 //                       tcgen05.mma.cta_group::2 M256 N256 K16; each CTA
 //                       stages its own 128 rows and half of the weight tile
 //                       (each described at the kernel);
-//    cond_overlap_kernel  the overlapped round: one CTA per SM, 128-row tiles,
-//                       tcgen05.mma.cta_group::1 M128 N256 K16, and
-//                       verification streamed through shared memory
-//                       (verify_stream.cuh).
+//    cond_kernel<false> (more rows, per-position e, d a multiple of 256) one
+//                       CTA per SM, 128-row tiles, tcgen05.mma.cta_group::1
+//                       M128 N256 K16;
+//    cond_kernel<true>  the overlapped round: the same plus verification
+//                       streamed through shared memory (verify_stream.cuh).
 //
 // Warp roles of the persistent kernels' GEMM part (256 threads):
 //   warp 0     tile scheduler + TMA producer (one elected lane);
@@ -58,10 +59,13 @@ namespace {
 
 constexpr int BM = 128;
 constexpr int BK = 64;  // 64 bf16 = 128 bytes = one swizzle row
-constexpr int THREADS_FUSED = 2 * 256 + 32;  // consumer warps 8-15 and the bookkeeper warp 16 beside the GEMM's eight
+constexpr int STAGES = 4;
+constexpr int THREADS = 256;
+constexpr int THREADS_FUSED = 2 * THREADS + 32;  // + consumer warps 8-15 and the bookkeeper warp 16
 constexpr int A_BYTES = BM * BK * 2;   // 16 KB
 constexpr int B_BYTES = 256 * BK * 2;  // 32 KB
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
+constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024;  // + slack for 1024-B alignment
 // The overlapped round's kernel keeps three operand stages and gives the rest of the
 // shared memory to the ring that streams the logits.
 constexpr int STAGES_FUSED = 3;
@@ -304,33 +308,40 @@ __device__ __forceinline__ void epilogue_gate(const CondParams& p, uint32_t tadd
 // T0 <= t < T0 + T1: gate tile (row block (t-T0) / nt1, 128 features).  Tiles
 // are handed out in this order by a global counter, so every gate tile's row
 // block was handed out (to a running CTA) before it.
-// The kernel also runs verification (verify_stream.cuh): warp 3 streams the logits into a shared-memory ring, warps 8-15 reduce it, warp 16 folds the keys.  Packed rows then become available while the
-// kernel runs, so the tile queue is decoded in phases -- phase q holds the
-// correction tiles of row block q followed by the gate tiles of row block
-// q - kGateLag -- and the producer resolves each tile against the published
-// per-block row counts before loading it.  R (and the last partial block) is
-// known once every sequence is finalised.
+// FUSED: the same kernel also runs verification (verify_stream.cuh): warp 3
+// streams the logits into a shared-memory ring, warps 8-15 reduce it, warp 16
+// folds the keys.  Packed rows then become available while the kernel runs, so
+// the tile queue is decoded in phases -- phase q holds the correction tiles of
+// row block q followed by the gate tiles of row block q - kGateLag -- and the
+// producer resolves each tile against the published per-block row counts
+// before loading it.  R (and the last partial block) is known once every
+// sequence is finalised.
+// Not FUSED: a per-position e only.  Its 128-row tiles fill the last wave
+// better than the pair kernel's, whose gate tiles are long with the e half
+// added (a round, d = 2560, 1821 rows: 170 us here, 206 on pairs; d = 4096,
+// 1821: 337 / 365; 2802: 445 / 445).
 constexpr int kGateLag = 4;
 
-__global__ void __launch_bounds__(THREADS_FUSED, 1)
-    cond_overlap_kernel(const __grid_constant__ CUtensorMap tmApack, const __grid_constant__ CUtensorMap tmWc,
+template <bool FUSED>
+__global__ void __launch_bounds__(FUSED ? THREADS_FUSED : THREADS, 1)
+    cond_kernel(const __grid_constant__ CUtensorMap tmApack, const __grid_constant__ CUtensorMap tmWc,
                 const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmE,
                 const __grid_constant__ CUtensorMap tmWv, const __grid_constant__ CUtensorMap tmWg,
                 const CondParams p, const VerifyStreamParams vp) {
   extern __shared__ uint8_t dsmem[];
-  __shared__ __align__(8) uint64_t bar_full[STAGES_FUSED];
-  __shared__ __align__(8) uint64_t bar_empty[STAGES_FUSED];
+  __shared__ __align__(8) uint64_t bar_full[STAGES];
+  __shared__ __align__(8) uint64_t bar_empty[STAGES];
   __shared__ __align__(8) uint64_t bar_tfull[2];
   __shared__ __align__(8) uint64_t bar_tempty[2];
   __shared__ __align__(8) uint64_t bar_tile_full[TILE_SLOTS];
   __shared__ __align__(8) uint64_t bar_tile_empty[TILE_SLOTS];
   __shared__ int s_tile[TILE_SLOTS];
-  __shared__ int s_rows[TILE_SLOTS];  // valid rows of the tile
+  __shared__ int s_rows[TILE_SLOTS];  // valid rows of the tile (FUSED)
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_abort;
   __shared__ VerifyStreamSmem vsm;
 
-  constexpr int NST = STAGES_FUSED;
+  constexpr int NST = FUSED ? STAGES_FUSED : STAGES;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int d = p.d;
   const int nt0 = d / 256, nt1 = d / 128;
@@ -338,7 +349,7 @@ __global__ void __launch_bounds__(THREADS_FUSED, 1)
   uint32_t* gemv_next = p.sync + kSyncGemvNext;
   uint32_t* gemv_done = p.sync + kSyncGemvDone;
   uint32_t* block_done = p.block_done;
-  const bool need_ge = p.do_gate && !p.e_dense;
+  const bool need_ge = FUSED && p.do_gate && !p.e_dense;
 
   if (tid == 0) {
     s_abort = 0;
@@ -354,7 +365,7 @@ __global__ void __launch_bounds__(THREADS_FUSED, 1)
       mbar_init(smem_u32(&bar_tile_full[a]), 1);
       mbar_init(smem_u32(&bar_tile_empty[a]), 5);  // MMA thread + four epilogue warps
     }
-    vs_init(vsm);
+    if constexpr (FUSED) vs_init(vsm);
     fence_mbar_init();
   }
   if (warp == 0 && lane == 0) {
@@ -379,6 +390,16 @@ __global__ void __launch_bounds__(THREADS_FUSED, 1)
   const uint32_t tmem = s_tmem;
   const uint32_t base = (smem_u32(dsmem) + 1023u) & ~1023u;
   const int kb_half = d / BK;
+  // The set-up above may overlap the end of the previous kernel; R, the packed
+  // rows and the row map are its outputs.
+  int R = 0, T0 = 0, T = 0;
+  if (!FUSED) {
+    pdl_wait();
+    R = *(volatile const int32_t*)p.R;
+    const int tiles_m = (R + BM - 1) / BM;
+    T0 = p.do_correct ? tiles_m * nt0 : 0;
+    T = T0 + (p.do_gate ? tiles_m * nt1 : 0);
+  }
 
   if (warp == 0) {
     // ---------------- tile scheduler + TMA producer ----------------
@@ -389,7 +410,14 @@ __global__ void __launch_bounds__(THREADS_FUSED, 1)
         const uint32_t slot = lt % TILE_SLOTS, sph = (lt / TILE_SLOTS) & 1u;
         int t, rows = BM, m0, n0;
         bool corr, done = false;
-        {
+        if (!FUSED) {
+          t = (int)atomicAdd(tile_queue, 1u);
+          done = t >= T;
+          corr = t < T0;
+          const int tt = corr ? t : t - T0;
+          m0 = (corr ? tt / nt0 : tt / nt1) * BM;
+          n0 = corr ? (tt % nt0) * 256 : (tt % nt1) * 128;
+        } else {
           // next valid tile of the phased queue
           for (;;) {
             t = (int)atomicAdd(tile_queue, 1u);
@@ -507,7 +535,7 @@ __global__ void __launch_bounds__(THREADS_FUSED, 1)
         const int t = s_tile[slot];
         mbar_arrive(smem_u32(&bar_tile_empty[slot]));
         if (t < 0) break;
-        const bool corr = (t % (nt0 + nt1)) < nt0;
+        const bool corr = FUSED ? (t % (nt0 + nt1)) < nt0 : t < T0;
         const int nkb = corr ? 2 * kb_half : kb_half + (p.e_dense ? kb_half : 0);
         const uint32_t acc = lt & 1u, aph = (lt >> 1) & 1u;
         if (!mbar_wait_bounded(smem_u32(&bar_tempty[acc]), aph ^ 1u, &s_abort)) {
@@ -543,27 +571,29 @@ __global__ void __launch_bounds__(THREADS_FUSED, 1)
       if (!ok) raise_abort(&s_abort, p.status);
     }
     __syncwarp();
-  } else if (warp == 3) {
+  } else if (FUSED && warp == 3) {
     // ---------------- logits stream into the verification ring ----------------
     if (lane == 0) vs_producer(vp, vsm, base + NST * STAGE_BYTES, &s_abort);
     __syncwarp();
-  } else if (warp == 2) {
+  } else if (FUSED && warp == 2) {
     // ---------------- sequence finaliser (bulk copies through staging) ----------------
     vs_finalizer(vp, vsm, base + NST * STAGE_BYTES + kRingBufs * kChunkBytes, blockIdx.x, gridDim.x, lane, &s_abort);
   } else if (warp >= 16) {
-    // ---------------- verification bookkeeping ----------------
-    if (lane == 0) vs_bookkeeper(vp, vsm, &s_abort);
+    // ---------------- verification bookkeeping (FUSED only) ----------------
+    if constexpr (FUSED)
+      if (lane == 0) vs_bookkeeper(vp, vsm, &s_abort);
     __syncwarp();
   } else if (warp >= 8) {
-    // ---------------- verification (warps 8-15) ----------------
-    vs_consumer(vp, vsm, reinterpret_cast<const uint4*>(dsmem + (base + NST * STAGE_BYTES - smem_u32(dsmem))), warp - 8,
-                lane, &s_abort);
+    // ---------------- verification (FUSED only: warps 8-15) ----------------
+    if constexpr (FUSED)
+      vs_consumer(vp, vsm, reinterpret_cast<const uint4*>(dsmem + (base + NST * STAGE_BYTES - smem_u32(dsmem))),
+                  warp - 8, lane, &s_abort);
   } else if (warp >= 4) {
     // ---------------- epilogue ----------------
     const int q = (warp - 4) * 32 + lane;  // tile row = TMEM lane
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-    // The epilogue warps have nothing to do until the first rows are packed:
-    // they compute W_g[:, :d] e meanwhile.
+    // In the overlapped round the epilogue warps have nothing to do until the
+    // first rows are packed: they compute W_g[:, :d] e meanwhile.
     if (need_ge) gate_bias_rows(p, d, lane, gemv_next, gemv_done);
     bool have_ge = !need_ge;
     for (uint32_t lt = 0;; ++lt) {
@@ -580,10 +610,17 @@ __global__ void __launch_bounds__(THREADS_FUSED, 1)
       if (t < 0) break;
       bool corr;
       int m0, n0;
-      const int q2 = t / (nt0 + nt1), r2 = t % (nt0 + nt1);
-      corr = r2 < nt0;
-      m0 = (corr ? q2 : q2 - kGateLag) * BM;
-      n0 = corr ? r2 * 256 : (r2 - nt0) * 128;
+      if (FUSED) {
+        const int q2 = t / (nt0 + nt1), r2 = t % (nt0 + nt1);
+        corr = r2 < nt0;
+        m0 = (corr ? q2 : q2 - kGateLag) * BM;
+        n0 = corr ? r2 * 256 : (r2 - nt0) * 128;
+      } else {
+        corr = t < T0;
+        const int tt = corr ? t : t - T0;
+        m0 = (corr ? tt / nt0 : tt / nt1) * BM;
+        n0 = corr ? (tt % nt0) * 256 : (tt % nt1) * 128;
+      }
       const uint32_t acc = lt & 1u, aph = (lt >> 1) & 1u;
       ok = warp_wait(smem_u32(&bar_tfull[acc]), aph, &s_abort);
       tc_fence_after();
@@ -603,7 +640,7 @@ __global__ void __launch_bounds__(THREADS_FUSED, 1)
         have_ge = true;
       }
       const int g = m0 + q;
-      const bool valid = q < tile_rows;
+      const bool valid = FUSED ? q < tile_rows : g < R;
       const uint32_t taddr = tmem + acc * ACC_COLS + lane_base;
       if (corr) {
         epilogue_correction<false>(p, taddr, g, valid, n0, d);
@@ -2013,10 +2050,58 @@ static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
   return cudaSuccess;
 }
 
+// A per-position e with many rows (d a multiple of 256).
+static cudaError_t launch_cond_one_sm(const TcCondArgs& a, cudaStream_t stream) {
+  DeviceInfo info;
+  cudaError_t err = device_info(&info);
+  if (err != cudaSuccess) return err;
+  static std::atomic<int> attr_done[64];
+  if (!attr_done[info.device & 63].load(std::memory_order_acquire)) {
+    err = cudaFuncSetAttribute(cond_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    if (err != cudaSuccess) return err;
+    attr_done[info.device & 63].store(1, std::memory_order_release);
+  }
+  const long long rmax = (long long)a.B * (a.K - 1);
+  const uint64_t d = (uint64_t)a.d;
+  CUtensorMap mApack, mWc, mR, mE, mWv, mWg;
+  // Maps of operands a call does not use point at a used buffer (never read).
+  const void* apack = a.do_correct ? a.apack : a.rpack;
+  const void* wc = a.do_correct ? a.Wc : a.Wv;
+  if (encode_tensor_map_2d(&mApack, apack, a.do_correct ? 2 * d : d, (uint64_t)rmax, (a.do_correct ? 4 : 2) * d, BK, BM) != CUDA_SUCCESS ||
+      encode_tensor_map_2d(&mWc, wc, a.do_correct ? 2 * d : d, d, (a.do_correct ? 4 : 2) * d, BK, a.do_correct ? 256 : 128) != CUDA_SUCCESS ||
+      encode_tensor_map_2d(&mR, a.rpack, d, (uint64_t)rmax, 2 * (a.r_row_stride ? (uint64_t)a.r_row_stride : d), BK, BM) != CUDA_SUCCESS ||
+      encode_tensor_map_2d(&mE, a.epack, d, (uint64_t)rmax, 2 * d, BK, BM) != CUDA_SUCCESS ||
+      encode_tensor_map_2d(&mWv, a.Wv, d, d, 2 * d, BK, 128) != CUDA_SUCCESS ||
+      encode_tensor_map_2d(&mWg, a.Wg, 2 * d, d, 4 * d, BK, 128) != CUDA_SUCCESS)
+    return cudaErrorInvalidValue;
+  CondParams p{};
+  p.d = a.d;
+  p.do_correct = a.do_correct;
+  p.do_gate = 1;
+  p.R = a.R;
+  p.rowmap = a.rowmap;
+  p.apack = reinterpret_cast<const __nv_bfloat16*>(a.apack);
+  p.beta = a.beta;
+  p.r_out = reinterpret_cast<__nv_bfloat16*>(a.r_out);
+  p.compact_out = a.compact_out;
+  p.e = reinterpret_cast<const __nv_bfloat16*>(a.epack);
+  p.e_dense = 1;
+  p.e_out = reinterpret_cast<__nv_bfloat16*>(a.e_out);
+  p.sync = a.sync;
+  p.block_done = a.sync + kSyncBlocks;
+  p.status = a.status;
+  const long long tiles_max = (rmax + BM - 1) / BM * ((a.do_correct ? a.d / 256 : 0) + a.d / 128);
+  const unsigned grid = (unsigned)std::min<long long>(tiles_max, info.sm_count);
+  const VerifyStreamParams vp{};
+  return launch_dependent(cond_kernel<false>, dim3(grid), dim3(THREADS), (size_t)SMEM_BYTES, stream, 1u, mApack, mWc,
+                          mR, mE, mWv, mWg, p, vp);
+}
+
 cudaError_t launch_cond_tc(const TcCondArgs& a, cudaStream_t stream) {
   const long long rmax = (long long)a.B * (a.K - 1);
   if (rmax <= 0 || (!a.do_correct && !a.do_gate)) return cudaSuccess;
   if (a.direct || rmax <= kSwapMaxRows) return launch_cond_swap(a, stream);
+  if (a.do_gate && a.e_dense && a.d % 256 == 0) return launch_cond_one_sm(a, stream);
   const long long tiles_max = (rmax + 2 * BM - 1) / (2 * BM) *
                               ((a.do_correct ? (a.d + 255) / 256 : 0) + (a.do_gate ? (a.d + 127) / 128 : 0));
   cudaError_t err;
@@ -2043,7 +2128,7 @@ cudaError_t launch_round_tc(const TcRoundArgs& a, cudaStream_t stream) {
   if (err != cudaSuccess) return err;
   static std::atomic<int> attr_done[64];
   if (!attr_done[info.device & 63].load(std::memory_order_acquire)) {
-    err = cudaFuncSetAttribute(cond_overlap_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES_FUSED);
+    err = cudaFuncSetAttribute(cond_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES_FUSED);
     if (err != cudaSuccess) return err;
     attr_done[info.device & 63].store(1, std::memory_order_release);
   }
@@ -2126,7 +2211,7 @@ cudaError_t launch_round_tc(const TcRoundArgs& a, cudaStream_t stream) {
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, cond_overlap_kernel, mApack, mWc, mR, mE, mWv, mWg, p, vp);
+  return cudaLaunchKernelEx(&cfg, cond_kernel<true>, mApack, mWc, mR, mE, mWv, mWg, p, vp);
 }
 
 }  // namespace retrace
