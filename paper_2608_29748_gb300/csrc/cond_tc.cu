@@ -26,8 +26,8 @@
 //        or, for per-position e, extra K blocks (Epack x W_g[:, :d])
 //        accumulated into the gate columns.
 //    Three kernels implement it:
-//    swap_cluster_kernel  (at most kSwapMaxRows possible rows; one launch per
-//                       projection instead) the weights as the M side;
+//    swap_cluster_kernel  (few rows, cond_small_r; one launch per projection
+//                       instead) the weights as the M side;
 //    cond_pair_kernel   (more rows) clusters of two CTAs, 256-row tiles,
 //                       tcgen05.mma.cta_group::2 M256 N256 K16; each CTA
 //                       stages its own 128 rows and half of the weight tile
@@ -1129,7 +1129,7 @@ __global__ void wait_selftest_kernel(int kind, const uint32_t* flag, uint32_t ta
 }
 
 // ---------------------------------------------------------------------------
-// Small R (B (K-1) <= kSwapMaxRows conditioned rows): the weights on the M side
+// Small R (cond_small_r): the weights on the M side
 // ---------------------------------------------------------------------------
 // With few rows the 256-row pair tiles are mostly padding and only d/256
 // correction tiles exist, so a handful of SMs stream the weights.  Here the
@@ -1769,7 +1769,7 @@ cudaError_t launch_pack(const PackArgs& a, cudaStream_t stream) {
   p.sync = a.sync;
   p.sync_words = (int)(a.sync_bytes / 4);
   // the CTA-pair kernel computes W_g[:, :d] e itself
-  if (a.mode == 1 && !a.e_dense && (long long)a.B * (a.K - 1) <= kSwapMaxRows)
+  if (a.mode == 1 && !a.e_dense && cond_small_r(a.B, a.K, a.d))
     p.bias = {a.d, p.e, reinterpret_cast<const __nv_bfloat16*>(a.Wg), a.ge};
   // a warp per position, four CTAs per SM at most; all of them for the GEMV
   const long long most = 4LL * info.sm_count, ctas = ((long long)a.B * a.K + 7) / 8;
@@ -1885,27 +1885,39 @@ static int swap_cluster_capacity(int dev, int S, int smem, cudaError_t* err) {
   return n > 0 ? n : 0;
 }
 
-// Cluster size of a small-R GEMM: the one with the least estimated time at
-// three quarters of the possible rows (R itself is known on the device only;
-// direct rows: one tile of all the tile rows).
-// A cluster holds `parts` products of the k-blocks.
-// A wave of units costs its k-blocks, 2 (128 + N) cycles each (the stage's
-// bytes in and out of shared memory), plus the drain and the sum of the
-// partial (about 24 cycles per row of the tile) and the fixed start and end.
+// Cluster size of a small-R GEMM, `parts` products of S / parts K splits each:
+// the one with the least estimated time.  R itself is known on the device only,
+// so the estimate is the sum of two, at a half and at three quarters of the
+// possible rows (direct rows: one tile of all the tile rows).  A wave of units
+// costs its k-blocks (measured: 750 cycles each at N = 160, 830 at 177, 1070 at
+// 250; the issue of the MMAs and the stage's handshake make most of a small
+// one), 60 cycles per row of the tile (the drain and the sum over the splits),
+// 4000 to start and end, and with packed rows 700 per CTA of the cluster (they
+// wait for each other).  Packed rows take four K splits at most: larger
+// clusters are not all placed at once beside the last CTAs of the kernel before
+// (a round, V = 2048, d = 3584, B = 32, 384 rows: 108 us with S = 5 for the
+// correction, which one wave should hold, 72 with S = 2).  Over 160 rounds of
+// d = 1024 to 4096 and 64 to 733 rows, and 33 pairs of standalone calls, each
+// timed with every S, the choice takes 1.5 % more than the best S of each (11 %
+// at most); one estimate at three quarters, 2 (128 + N) cycles per k-block, 24
+// per row, any S: 6 % (32 % at most).
 static cudaError_t swap_pick_splits(int dev, int smem, int rmax, bool direct, int parts, int mtiles, int nkb,
                                     int* S_out, int* clusters) {
-  const int Rt = direct ? rmax : (3 * rmax + 3) / 4;
   long long best = -1;
   cudaError_t err = cudaSuccess;
-  for (int S = 8 / parts * parts; S >= parts; S -= parts) {
-    const int splits = S / parts;
+  for (int splits = std::min(direct ? 8 : 4, 8 / parts); splits >= 1; --splits) {
+    const int S = splits * parts;
     if (splits > 1 && nkb / splits < SW_MIN_BLOCKS) continue;
     const int cap = swap_cluster_capacity(dev, S, smem, &err);
     if (err != cudaSuccess) return err;
     if (cap == 0) continue;
-    const SwapCut cut = direct ? SwapCut{1, (Rt + 15) / 16 * 16} : swap_cut(Rt, mtiles, cap);
-    const long long waves = ((long long)mtiles * cut.ntiles + cap - 1) / cap;
-    const long long cost = waves * ((long long)((nkb + splits - 1) / splits) * 2 * (128 + cut.tile_n) + 24 * cut.tile_n + 2500);
+    long long cost = 0;
+    for (const int rows : {(rmax + 1) / 2, (3 * rmax + 3) / 4}) {
+      const SwapCut cut = direct ? SwapCut{1, (rmax + 15) / 16 * 16} : swap_cut(rows, mtiles, cap);
+      const long long waves = ((long long)mtiles * cut.ntiles + cap - 1) / cap;
+      const int block = std::max(750, 17 * cut.tile_n / 4);
+      cost += waves * ((long long)((nkb + splits - 1) / splits) * block + 60 * cut.tile_n + 4000 + (direct ? 0 : 700 * S));
+    }
     if (best < 0 || cost < best) {
       best = cost;
       *S_out = S;
@@ -1926,11 +1938,10 @@ static bool encode_row_maps(RowMaps* maps, const void* base, uint64_t inner, int
   return true;
 }
 
-// The small-R path (B (K-1) <= kSwapMaxRows): the
-// correction GEMM with the gate-bias GEMV, then the gate GEMM; each launch
-// waits on the one before inside the kernel, and cuts its work from the R it
-// reads.  Past the operands' ends (d no multiple of the tiles) the copies fill
-// zeros and the epilogues store nothing.
+// The small-R path (cond_small_r): the correction GEMM with the gate-bias GEMV,
+// then the gate GEMM; each launch waits on the one before inside the kernel,
+// and cuts its work from the R it reads.  Past the operands' ends (d no multiple
+// of the tiles) the copies fill zeros and the epilogues store nothing.
 static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
   const bool direct = a.direct;
   // rows of the operands: tile rows (direct), or the most there can be
@@ -2100,7 +2111,7 @@ static cudaError_t launch_cond_one_sm(const TcCondArgs& a, cudaStream_t stream) 
 cudaError_t launch_cond_tc(const TcCondArgs& a, cudaStream_t stream) {
   const long long rmax = (long long)a.B * (a.K - 1);
   if (rmax <= 0 || (!a.do_correct && !a.do_gate)) return cudaSuccess;
-  if (a.direct || rmax <= kSwapMaxRows) return launch_cond_swap(a, stream);
+  if (a.direct || cond_small_r(a.B, a.K, a.d)) return launch_cond_swap(a, stream);
   if (a.do_gate && a.e_dense && a.d % 256 == 0) return launch_cond_one_sm(a, stream);
   const long long tiles_max = (rmax + 2 * BM - 1) / (2 * BM) *
                               ((a.do_correct ? (a.d + 255) / 256 : 0) + (a.do_gate ? (a.d + 127) / 128 : 0));

@@ -44,10 +44,25 @@ constexpr int kLowRankSplits = 8;       // split-K parts per half of the [m; u] 
 constexpr int kMaxTopK = 64;            // largest top_k of sampled verification
 constexpr int kWindowRows = 4;          // rows per pass of windowed verification
 constexpr int kMaxWindowPasses = 16;    // most passes of windowed verification
-// Small-R conditioning: at most kSwapMaxRows packed rows, the GEMMs with the
-// weights as the M side in split-K clusters, which sum their partials in shared
-// memory.  The region of swap_part_bytes in the workspace holds the corrected
-// signal of a round without packed rows (direct rows, below).
+// Small-R conditioning: the GEMMs with the weights as the M side in split-K
+// clusters, which sum their partials in shared memory (swap_cluster_kernel), for
+// at most kSmallRWork rows times features.  Rounds on it and on the kernels for
+// more rows (CTA pairs; per-position e: one-SM tiles), V = 2048, K = 16, rows of
+// geometric 0.2, us: d = 1024, B = 72 / 128 / 256: 41 / 54 / 88 against 56 / 67 /
+// 94; d = 2048, B = 72 / 128 / 152 / 192: 59 / 93 / 100 / 111 against 74 / 95 / 99
+// / 108; d = 2560, B = 72 / 104 / 152: 90 / 101 / 116 against 96 / 102 / 113; d =
+// 4096, B = 64 / 72 / 104: 131 / 133 / 205 against 129 / 129 / 161; per-position e,
+// d = 2048, B = 104 / 128 / 192: 97 / 131 / 180 against 125 / 130 / 142; d = 4096,
+// B = 72 / 88: 201 / 254 against 199 / 203.  With uniform acceptance (fewer rows)
+// the lines cross later.  No more than kSmallRRows rows were measured.
+constexpr long long kSmallRWork = 1ll << 22;
+constexpr long long kSmallRRows = 4096;
+inline bool cond_small_r(long long B, long long K, long long d) {
+  const long long rmax = B * (K > 1 ? K - 1 : 0);
+  return rmax > 0 && rmax <= kSmallRRows && rmax * d <= kSmallRWork;
+}
+// The region of swap_part_bytes in the workspace holds the corrected signal of a
+// round without packed rows (direct rows, below).
 constexpr int kSwapMaxRows = 1024;
 constexpr int kSwapMaxCtas = 256;
 inline size_t swap_part_bytes(long long B, long long K, long long d) {
@@ -59,10 +74,11 @@ inline size_t swap_part_bytes(long long B, long long K, long long d) {
   const long long box = rows < 256 ? rows : 256;
   return (size_t)(kSwapMaxCtas * 128 * box * 4);
 }
-// CTA-pair conditioning (more rows): with d a multiple of 256 a
-// last wave of at most kPairSplitTiles gate tiles runs as two K halves per
-// tile on two pairs.  Each half writes its fp32 accumulator (two CTAs x 128
-// rows x 256 columns) to the workspace (swp), and counts on one ticket per CTA and epilogue warp in the sync area.
+// CTA-pair conditioning (more rows): with d a multiple of 256 a last wave of at
+// most kPairSplitTiles gate tiles runs as two K halves per tile on two pairs.
+// Each half writes its fp32 accumulator (two CTAs x 128 rows x 256 columns) to
+// the workspace (swp), and counts on one ticket per CTA and epilogue warp in the
+// sync area.
 constexpr int kPairSplitTiles = 8;
 inline size_t pair_split_bytes(long long B, long long K, long long d, size_t elem) {
   const long long rmax = B * (K > 1 ? K - 1 : 0);

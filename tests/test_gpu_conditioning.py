@@ -352,3 +352,46 @@ def test_ragged_hidden_sizes(rt, B, K, d, R, dense_e):
     want = oracle.gate_fuse(np.broadcast_to(host_f64(e), (B, K, d)), host_f64(r), n_host, host_f64(x["Wv"]),
                             host_f64(x["Wg"]))
     assert_close(out, want, f"e~, R={R} d={d}")
+
+
+@pytest.mark.parametrize("dense_e", [False, True])
+@pytest.mark.parametrize("B,K,d,R", [
+    # small-R kernel above 1024 possible rows
+    (80, 16, 1024, 1057),
+    (273, 16, 256, 4095),
+    (200, 16, 392, 1500),
+    # more than 4096 possible rows: CTA pairs (the gate's last wave in K halves), and one-SM tiles for a
+    # per-position e where d is a multiple of 256
+    (274, 16, 256, 1),
+    (274, 16, 256, 127),
+    (274, 16, 256, 129),
+    (274, 16, 256, 256),
+    (274, 16, 256, 257),
+    (274, 16, 256, 1200),
+    (274, 16, 256, 4110),
+    (274, 16, 264, 130),
+    (274, 16, 264, 4110),
+    # more than 2^22 rows times features
+    (70, 16, 4096, 129),
+])
+def test_many_rows(rt, B, K, d, R, dense_e):
+    """Either side of the lines between the small-R kernel and those for more
+    rows, at the edges of their row tiles."""
+    dtype = torch.bfloat16
+    x = make_inputs(B, K, d, dtype, seed=R + d, accept=accept_for_rows(B, K, R))
+    A = host_int(x["accept"])
+    n_host = oracle.carried_rows(A, K)
+    ws = rt.Workspace(B, K, 8, d, dtype)
+    r = torch.full((B, K, d), 9.0, dtype=dtype, device="cuda")
+    n = torch.empty((B,), dtype=torch.int32, device="cuda")
+    rt.retrace_align_refine(x["hD"], x["hT"], x["accept"], x["Wc"], 0.5, r, n, ws)
+    e = x["e_dense"] if dense_e else x["e_vec"]
+    out = torch.full((B, K, d), 7.0, dtype=dtype, device="cuda")
+    rt.retrace_gate_fuse(e, r, n, x["Wv"], x["Wg"], out, ws)
+    torch.cuda.synchronize()
+    assert ws.check() == 0
+    m, u = oracle.align(host_f64(x["hD"]), host_f64(x["hT"]), A)
+    assert_close(r, oracle.correct(m, u, host_f64(x["Wc"]), 0.5, round_r_bf16=False), f"r, R={R} d={d}")
+    want = oracle.gate_fuse(np.broadcast_to(host_f64(e), (B, K, d)), host_f64(r), n_host, host_f64(x["Wv"]),
+                            host_f64(x["Wg"]))
+    assert_close(out, want, f"e~, R={R} d={d}")
