@@ -1159,13 +1159,13 @@ __global__ void wait_selftest_kernel(int kind, const uint32_t* flag, uint32_t ta
 // resident clusters can take side by side, so that every SM has work and a
 // k-block costs an SM little more than its 16 KB of weights (a stage goes
 // through shared memory twice, about 2 (128 + N) cycles at 128 B per clock).
-constexpr int SW_STAGES = 4;      // most pipeline stages
+constexpr int SW_STAGES = 8;      // most pipeline stages
 constexpr int SW_MIN_BLOCKS = 4;  // least k-blocks of a split
 constexpr int SW_THREADS = 256;
 constexpr int SW_A_BYTES = BM * BK * 2;  // 16 KB: 128 weight rows of a k-block
 constexpr int SW_ROW_STEP = 32;          // row boxes come in multiples of this many rows
 constexpr int SW_ROW_MAPS = 256 / SW_ROW_STEP;
-constexpr int SW_SMEM_MAX = 226 * 1024;  // dynamic shared memory of a CTA at most (its barriers beside it)
+constexpr int SW_SMEM_MAX = 198 * 1024;  // dynamic shared memory of a CTA at most: four stages with a box of 256 rows
 
 // Row tiles of R rows for `clusters` resident clusters over `mtiles` weight
 // tiles: `ntiles` tiles of `tile_n` rows (a multiple of 16, at most 256).
@@ -1464,13 +1464,13 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
   const uint32_t rank = cluster_rank();
   const int cid = (int)(blockIdx.x / (unsigned)S), clusters = (int)(gridDim.x / (unsigned)S);
   pdl_launch_dependents();
-  if (threadIdx.x == 0) {
-    s_abort = 0;
-    for (int s = 0; s < SW_STAGES; ++s) {
-      mbar_init(smem_u32(&bar_full[s]), 2);  // the weight tile's and the row box's expect_tx
-      mbar_init(smem_u32(&bar_empty[s]), 1);
+  if (threadIdx.x < SW_STAGES) {
+    mbar_init(smem_u32(&bar_full[threadIdx.x]), 2);  // the weight tile's and the row box's expect_tx
+    mbar_init(smem_u32(&bar_empty[threadIdx.x]), 1);
+    if (threadIdx.x == 0) {
+      s_abort = 0;
+      mbar_init(smem_u32(&bar_acc), 1);
     }
-    mbar_init(smem_u32(&bar_acc), 1);
     fence_mbar_init();
   }
   if (warp == 0 && lane == 0) {
@@ -1961,7 +1961,13 @@ static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
     attr_done[dev & 63].store(1, std::memory_order_release);
   }
   const int box_max = swap_box_rows(std::min(256, (rmax + 15) / 16 * 16));
-  const int pre = swap_stages(SW_SMEM_MAX - 1024, box_max);  // stages with the largest row box
+  // Stages with the largest row box, their weight tiles loaded before the wait.
+  // (The kernel runs as many as fit with the box it needs.)  With a gate-bias
+  // GEMV before that wait, four: it has the memory busy (rounds at d = 4096, B =
+  // 8: 61.7 us with four, 64.1 with six).  Else all that fit (per-position e, V =
+  // 2048, d = 4096, B = 8: 64.0 -> 58.5 us; d = 2560: 43.0 -> 40.9).
+  int pre = swap_stages(SW_SMEM_MAX - 1024, box_max);
+  if (!(a.do_gate && a.e_dense)) pre = std::min(pre, 4);
   // at least half of an SM's shared memory: one CTA per SM, so the K splits
   // of one wave stream over distinct SMs
   const int smem = std::max(pre * (SW_A_BYTES + box_max * BK * 2) + 1024, 117 * 1024);
