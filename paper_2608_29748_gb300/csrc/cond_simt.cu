@@ -25,9 +25,15 @@ namespace {
 // tx + 16 j (4 MR values) and reads both operands 16 bytes at a time along the
 // reduction (rows padded to 36 floats: conflict-free).  Each CTA then leaves
 // its partial tile in shared memory, and after a cluster barrier every CTA
-// sums its share of the rows over the S partials in rank order (results repeat
-// bit for bit) and applies the epilogue.  MR = rows of the tile / 16 is chosen
-// on the device from R.
+// sums its share of the rows over the S partials in a fixed order (results
+// repeat bit for bit) and applies the epilogue.  MR = rows of the tile / 16 is
+// chosen on the device from R.
+//
+// Products are summed by eights, by chunk, by split, and the splits in pairs.
+// One chain over the split took 42.4 us instead of 43.2 for a round of B = 8, K =
+// 8, d = 1024, but had two to four times the rounding error (relative to 64 bits
+// there 3.4e-7, now 1.4e-7; B = 1, K = 16, d = 2048: 5.6e-7, now 1.6e-7; a warp per
+// feature with its lanes along the reduction 2.5e-7).
 constexpr int kNT = 256;
 constexpr int kTileRows = 64;              // most conditioned rows of a tile
 constexpr int TN = 64, TK = 32;            // weight rows and reduction depth of a chunk
@@ -226,24 +232,36 @@ __device__ __forceinline__ void simt_partial(const SimtParams& p, float* ring, c
     const float* As = ring + (c - c0) % kSimtStages * kStageFloats + ty * kLd;
     const float* Bs = ring + (c - c0) % kSimtStages * kStageFloats + (kTileRows + tx) * kLd;
     const bool gate_only = GATE && c >= per;
+    float sum[MR][4];  // of this chunk
 #pragma unroll
-    for (int k = 0; k < TK; k += 4) {
-      float4 a[MR], b[4];
+    for (int k0 = 0; k0 < TK; k0 += 8) {
+      float t[MR][4];
 #pragma unroll
-      for (int i = 0; i < MR; ++i) a[i] = *reinterpret_cast<const float4*>(As + 16 * i * kLd + k);
+      for (int k = k0; k < k0 + 8; k += 4) {
+        float4 a[MR], b[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4*>(Bs + 16 * j * kLd + k);
+        for (int i = 0; i < MR; ++i) a[i] = *reinterpret_cast<const float4*>(As + 16 * i * kLd + k);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (j < 2 && gate_only) continue;  // weight rows tx, tx + 16: W_v
+        for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4*>(Bs + 16 * j * kLd + k);
 #pragma unroll
-        for (int i = 0; i < MR; ++i) {
-          acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
-          acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
-          acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
-          acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
+        for (int j = 0; j < 4; ++j) {
+          if (j < 2 && gate_only) continue;  // weight rows tx, tx + 16: W_v
+#pragma unroll
+          for (int i = 0; i < MR; ++i) {
+            t[i][j] = k == k0 ? a[i].x * b[j].x : fmaf(a[i].x, b[j].x, t[i][j]);
+            t[i][j] = fmaf(a[i].y, b[j].y, t[i][j]);
+            t[i][j] = fmaf(a[i].z, b[j].z, t[i][j]);
+            t[i][j] = fmaf(a[i].w, b[j].w, t[i][j]);
+            if (k > k0) sum[i][j] = k0 == 0 ? t[i][j] : sum[i][j] + t[i][j];
+          }
         }
       }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (j < 2 && gate_only) continue;
+#pragma unroll
+      for (int i = 0; i < MR; ++i) acc[i][j] += sum[i][j];
     }
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -322,7 +340,7 @@ __global__ void __launch_bounds__(kNT, 2) simt_cluster_kernel(const SimtParams p
     const uint32_t at = P + (uint32_t)((l * TN + f) * 4);
     float4 v[8], g[8];
 #pragma unroll
-    for (int s = 0; s < 8; ++s) {  // all loads first, then the sums in rank order
+    for (int s = 0; s < 8; ++s) {  // all loads first, then the sums, in pairs of ranks
       v[s] = g[s] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (s < S) {
         const uint32_t src = map_rank(at, (uint32_t)s);
@@ -331,10 +349,12 @@ __global__ void __launch_bounds__(kNT, 2) simt_cluster_kernel(const SimtParams p
       }
     }
 #pragma unroll
-    for (int s = 1; s < 8; ++s) {
-      add4(v[0], v[s]);
-      if constexpr (GATE) add4(g[0], g[s]);
-    }
+    for (int h = 1; h < 8; h *= 2)
+#pragma unroll
+      for (int s = 0; s + h < 8; s += 2 * h) {
+        add4(v[s], v[s + h]);
+        if constexpr (GATE) add4(g[s], g[s + h]);
+      }
     const float vv[4] = {v[0].x, v[0].y, v[0].z, v[0].w}, gg[4] = {g[0].x, g[0].y, g[0].z, g[0].w};
     const long long pos = (long long)s_b[l] * K + s_j[l];
     const long long orow = (!GATE && p.compact) ? m0 + l : pos;
