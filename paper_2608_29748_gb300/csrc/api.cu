@@ -227,6 +227,7 @@ struct ConditioningArgs {
   const void* Wg;
   float beta;
   void* e_out;
+  int last = 0;  // TcCondArgs::last
 };
 
 // The conditioning of a round without packed rows (direct_rows_supported),
@@ -296,6 +297,7 @@ retrace_status enqueue_conditioning(const ConditioningArgs& c, retrace_dtype dty
     // raw: r = m is the first half of each packed [m; u] row
     a.rpack = raw ? w + L.apack : r_ws;
     a.r_row_stride = raw ? 2LL * d : 0;
+    a.last = c.last;
     a.e = c.e;
     a.epack = w + L.epack;
     a.e_dense = c.e_dense;
@@ -771,7 +773,7 @@ retrace_status retrace_round_sampled(const void* target_logits, int64_t target_r
   }
   RT_CUDA(launch_verify_sampled(a, dtype, stream), "sampled verification launch");
   if (phase_events) RT_CUDA(cudaEventRecord(phase_events[1], stream), "cudaEventRecord");
-  ConditioningArgs c{hD, hT, e, e_batch_stride, e_pos_stride, dense, Wc, Wv, Wg, beta, e_out};
+  ConditioningArgs c{hD, hT, e, e_batch_stride, e_pos_stride, dense, Wc, Wv, Wg, beta, e_out, 1};
   if (direct)
     return enqueue_direct_conditioning(c, B, K, d, nullptr, draft, accept_len, nullptr, nullptr, nullptr, ws, L,
                                        phase_events, stream);

@@ -1165,7 +1165,13 @@ constexpr int SW_THREADS = 256;
 constexpr int SW_A_BYTES = BM * BK * 2;  // 16 KB: 128 weight rows of a k-block
 constexpr int SW_ROW_STEP = 32;          // row boxes come in multiples of this many rows
 constexpr int SW_ROW_MAPS = 256 / SW_ROW_STEP;
-constexpr int SW_SMEM_MAX = 198 * 1024;  // dynamic shared memory of a CTA at most: four stages with a box of 256 rows
+// Dynamic shared memory of a CTA at most (its barriers beside it): four stages
+// with a box of 256 rows.  With more, CTAs that sit beside verification's leave
+// it too little L1 and room (rounds of B = 64, d = 2560: 102 us, 110 at 208 KB and
+// above), though their own loop gains from a fifth stage at 192 rows.
+constexpr int SW_SMEM_RING = 198 * 1024;
+// The gate's where no verification kernel is launched ahead beside it.
+constexpr int SW_SMEM_MAX = 222 * 1024;
 
 // Row tiles of R rows for `clusters` resident clusters over `mtiles` weight
 // tiles: `ntiles` tiles of `tile_n` rows (a multiple of 16, at most 256).
@@ -1966,7 +1972,7 @@ static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
   // GEMV before that wait, four: it has the memory busy (rounds at d = 4096, B =
   // 8: 61.7 us with four, 64.1 with six).  Else all that fit (per-position e, V =
   // 2048, d = 4096, B = 8: 64.0 -> 58.5 us; d = 2560: 43.0 -> 40.9).
-  int pre = swap_stages(SW_SMEM_MAX - 1024, box_max);
+  int pre = swap_stages(SW_SMEM_RING - 1024, box_max);
   if (!(a.do_gate && a.e_dense)) pre = std::min(pre, 4);
   // at least half of an SM's shared memory: one CTA per SM, so the K splits
   // of one wave stream over distinct SMs
@@ -2057,10 +2063,15 @@ static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
     g.e = reinterpret_cast<const __nv_bfloat16*>(a.e_dense ? a.epack : a.e);
     g.ge = a.ge;
     g.e_out = reinterpret_cast<__nv_bfloat16*>(a.e_out);
+    // all the shared memory where it buys stages and no verification follows
+    // ahead: temperature-1 rounds, d = 4096, B = 32: 152.8 -> 150.2 us; per-position
+    // e, V = 32000, B = 48: 205 -> 196
+    const int gsmem = a.last && rmax > 256 ? SW_SMEM_MAX : smem;
+    g.stage_bytes = gsmem - 1024;
     int clusters = 0;
-    if ((err = swap_pick_splits(dev, smem, rmax, direct, a.e_dense ? 3 : 1, g.mtiles, g.nkb, &g.S, &clusters)) != cudaSuccess) return err;
+    if ((err = swap_pick_splits(dev, gsmem, rmax, direct, a.e_dense ? 3 : 1, g.mtiles, g.nkb, &g.S, &clusters)) != cudaSuccess) return err;
     err = launch_dependent(direct ? swap_cluster_kernel<true> : swap_cluster_kernel<false>, grid_of(g, clusters),
-                           dim3(SW_THREADS), (size_t)smem, stream, (unsigned)g.S, mA, mA2, mA3, mB,
+                           dim3(SW_THREADS), (size_t)gsmem, stream, (unsigned)g.S, mA, mA2, mA3, mB,
                            a.e_dense ? mE : mB, g);
     if (err != cudaSuccess) return err;
   }

@@ -404,6 +404,7 @@ struct TcCondArgs {
   const void* Wg;
   float* ge;  // [d] scratch for W_g[:, :d] e (broadcast e)
   int ge_ready;  // small R: ge is computed already
+  int last;      // small R: the kernel that follows this call is not launched ahead (a temperature-1 round's first)
   void* e_out;
   const int32_t* R;
   const int32_t* rowmap;
