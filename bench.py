@@ -54,7 +54,6 @@ from paper_2608_29748_gb300.workloads import CONFIGS, PROFILE_CONFIG, RoundConfi
 METRIC = "verify+ReTrace rounds/sec at 1 GB300; logits HBM GB/s and % of roofline"
 UNIT = "rounds/s"
 KERNELS_PER_ROUND_FUSED = 1  # cond_kernel<FUSED>: the whole round
-KERNELS_PER_ROUND = 2  # one-pass verify_kernel (+ row packing), cond_kernel (both projections + gate-bias GEMV)
 L2_FLUSH_BYTES = 256 << 20
 # DRAM traffic per round (ncu dram__bytes_read.sum + dram__bytes_write.sum,
 # summed over the kernels of the phase) of the phase a roofline object names,
@@ -62,9 +61,9 @@ L2_FLUSH_BYTES = 256 << 20
 # kernel sources it was measured on: `sources` is kernel_sources_hash() at the
 # time, and the line reports null traffic once the sources differ.
 TRAFFIC = {
-    ("verify", "qwen3-8b-B256-K16"): {"bytes": 311308288 + 2800384 + 184310272 + 138752 + 55403264 + 0
-                                      + 47179520 + 4033792, "sources": "c403a58964d4ce6e"},
-    ("conditioning", "qwen3-8b-B256-K16"): {"bytes": 509979136 + 37198080, "sources": "c403a58964d4ce6e"},
+    ("verify", "qwen3-8b-B256-K16"): {"bytes": 311305216 + 2984192 + 184312320 + 76800 + 55402240 + 0
+                                      + 47182848 + 4213248, "sources": "2e90788d1d34cc87"},
+    ("conditioning", "qwen3-8b-B256-K16"): {"bytes": 518159360 + 37841408, "sources": "2e90788d1d34cc87"},
 }
 
 
@@ -454,23 +453,21 @@ def run_gpu(args) -> dict | None:
     # one greedy pass that packs rows for the tensor-core projections hands the
     # decisions and copies to a second kernel when there are fewer sequences
     # than SMs (the finish kernel; the copy kernel at temperature 1)
-    packs = cfg.dtype == "bf16" and (cfg.d % 64 == 0 if args.lowrank
-                                     else cfg.d % 256 == 0 and (args.sampled or args.variant in ("corrected", "raw")))
+    tensor_cores = cfg.dtype == "bf16" and cfg.d % 8 == 0 and cfg.d >= (64 if args.lowrank else 128)
+    rows = cfg.B * (cfg.K - 1)
+    # few sequences (at most 64 tile rows): the conditioning reads the carried
+    # rows where they lie, after a verification that packs nothing
+    direct = (tensor_cores and not args.lowrank and args.variant == "corrected" and cfg.K >= 5
+              and cfg.B * ((cfg.K - 1 + 7) // 8 * 8) <= 64)
+    packs = tensor_cores and not direct and (args.lowrank or args.sampled or args.variant in ("corrected", "raw"))
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     if n_pass == 1 and not fused and packs and cfg.B < sms:
         verify_launches += 1
-    # conditioning launches of the greedy and temperature-1 rounds, by path
-    rows = (cfg.B * (cfg.K - 1) + 15) // 16 * 16
-    small_r = 0 < rows <= 1024 and (2 * cfg.d // 128) * ((rows + 255) // 256) <= 256
-    if cfg.dtype != "bf16" or cfg.d % 256:
-        cond_launches = 3  # correction, gate bias, gate (FFMA)
-    elif small_r and rows <= 256:
-        # split-K clusters: correction, gate-bias GEMV, gate (raw: GEMV, gate)
-        cond_launches = 3 if args.variant == "corrected" else 2
-    elif small_r:
-        cond_launches = 4 if args.variant == "corrected" else 3  # GEMM + reduction each; raw: GEMV, GEMM, reduction
-    else:
-        cond_launches = 1  # cond_pair_kernel
+    # conditioning launches of the greedy and temperature-1 rounds, by path:
+    # small R (split-K clusters: correction with the gate-bias GEMV, then gate;
+    # raw: GEMV, gate) and FFMA (the same) two, CTA pairs one
+    small_r = tensor_cores and 0 < rows <= 4096 and rows * cfg.d <= 1 << 22
+    cond_launches = 2 if not tensor_cores or small_r else 1
     step_avg_s = statistics.mean(step_ms) / 1e3
     cflops = (lowrank_flops(cfg, R) if args.lowrank
               else conditioning_flops(cfg, R, dense_e=False, variant=args.variant))
@@ -502,8 +499,7 @@ def run_gpu(args) -> dict | None:
                       "tensor_view": {"achieved_tflops": round(cflops / step_avg_s / 1e12, 2),
                                       "frac": round(t_tc / step_avg_s, 4)}}
     else:
-        packs_rows = cfg.dtype == "bf16" and cfg.d % 256 == 0  # tensor-core path: verify packs the rows
-        vbytes = verify_bytes(cfg, n, packs_rows and args.variant in ("corrected", "raw"), args.variant, accept)
+        vbytes = verify_bytes(cfg, n, packs and args.variant in ("corrected", "raw"), args.variant, accept)
         rbytes = vbytes - needed_logits_bytes(cfg, accept) + read_logits_bytes(cfg, accept, windows)
         v_avg_s = statistics.mean(verify_ms) / 1e3
         c_avg_s = statistics.mean(cond_ms) / 1e3
@@ -587,15 +583,14 @@ def run_gpu(args) -> dict | None:
                 "traffic": None if args.sampled else measured_traffic("conditioning", cfg.name, args.variant),
                 "traffic_source": "ncu dram read+write of one launch on this workload",
             }
-            if cfg.dtype != "bf16" or cfg.d % 256:
+            if not tensor_cores:
                 # fp32 (no TF32) or shapes the tensor-core kernels do not take: plain FFMA
                 props = torch.cuda.get_device_properties(dev)
                 max_mhz = (clocks.summary() or {}).get("sm_max_mhz") or 2070.0
                 ffma_peak = props.multi_processor_count * 128 * 2 * max_mhz * 1e6 / 1e12
                 c_roof.update({
-                    "kernel": ("FFMA path: simt_rows_correct_kernel, gate_bias_kernel, simt_rows_gate_kernel (a warp per "
-                               "feature)" if cfg.B * (cfg.K - 1) <= 32 else
-                               "FFMA path: simt_correct_kernel, gate_bias_kernel, simt_gate_kernel"),
+                    "kernel": "FFMA path: simt_cluster_kernel for each projection (split-K clusters, the gate-bias GEMV in "
+                              "further CTAs of the first)",
                     "bound": "alu", "peak": round(ffma_peak, 1), "frac": round(c_tflops / ffma_peak, 4),
                     "peak_source": "derived: SMs x 128 FP32 lanes x 2 flop per FMA x maximum SM clock",
                     "frac_of_sustained": None, "traffic": None})
@@ -604,11 +599,9 @@ def run_gpu(args) -> dict | None:
                 es, d = cfg.elem_bytes, cfg.d
                 cbytes = 5 * d * d * es + R * (2 * d + d + d) * es + R * d * 2
                 c_roof.update({
-                    "kernel": ("small-R GEMMs: swap_cluster_kernel (tcgen05, weights as the 128-row side, split-K "
-                               "over a cluster whose partials are summed in distributed shared memory) for each "
-                               "projection, swap_gemv_kernel beside the correction" if rows <= 256 else
-                               "small-R GEMMs: swap_gemm_kernel (tcgen05, weights as the 128-row side, split-K) for "
-                               "each projection, each followed by its reduction kernel"),
+                    "kernel": "small-R GEMMs: swap_cluster_kernel (tcgen05, weights as the 128-row side, split-K over a "
+                              "cluster whose partials are summed in distributed shared memory) for each projection, "
+                              "the gate-bias GEMV in the correction's idle warps",
                     "bound": "hbm", "achieved": round(cbytes / c_avg_s / 1e9, 1), "peak": peaks["hbm_gbs"],
                     "unit": "GB/s", "frac": round(cbytes / c_avg_s / 1e9 / peaks["hbm_gbs"], 4),
                     "peak_source": peaks["source"] + " HBM copy bandwidth",

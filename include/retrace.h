@@ -47,8 +47,9 @@
  *               library allocates no device memory.  Scratch comes from the
  *               caller's workspace `ws` (size from retrace_workspace_bytes).
  *   Layout      row-major, last dimension contiguous.  16-byte alignment of
- *               every tensor base enables the vector paths; unaligned inputs
- *               take a scalar path on the GPU.  Outputs must not overlap inputs.
+ *               every conditioning tensor's base enables its tensor-core path
+ *               (else: FFMA); logits rows of any alignment stream in 16-byte
+ *               loads.  Outputs must not overlap inputs.
  *   Async       all work is enqueued on `stream` (NULL = legacy default stream);
  *               no entry point synchronises the host except
  *               retrace_workspace_check.
@@ -303,9 +304,9 @@ retrace_status retrace_verify_sampled(const void* target_logits, int64_t target_
  * speculative sampling; the paper evaluates at T = 1).  Arguments are those of
  * retrace_verify_sampled followed by those of retrace_round; there is no
  * target_argmax output and no flags.  The finalize kernel writes the rows
- * j >= n_b of e_out and, on the tensor-core path (bf16, d a multiple of 256,
- * 16-byte aligned tensors), packs the conditioned rows for one persistent
- * conditioning launch.
+ * j >= n_b of e_out and, on the tensor-core path (bf16, d a multiple of 8
+ * and at least 128, 16-byte aligned tensors), packs the conditioned rows for
+ * the conditioning launches.
  *   phase_events  optional 4 events: before verification, after it, after the
  *                 correction (after both projections on the tensor-core
  *                 path), after the gated fusion.
@@ -346,7 +347,7 @@ retrace_status retrace_round_sampled(const void* target_logits, int64_t target_r
  *         row-major.
  *   phase_events  optional 4 events: before verification, after it, after
  *         the latent projections, after the fusion.
- * Tensor cores for bf16 with d a multiple of 128 and 16-byte aligned tensors;
+ * Tensor cores for bf16 with d >= 64 a multiple of 8 and 16-byte aligned tensors;
  * an FFMA kernel otherwise.  K >= 1, V >= 1, d >= 1. */
 retrace_status retrace_round_lowrank(const void* logits, int64_t logits_row_stride,
                                      int64_t logits_batch_stride, const int32_t* draft,
