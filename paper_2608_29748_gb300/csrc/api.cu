@@ -841,7 +841,11 @@ retrace_status retrace_round_lowrank(const void* logits, int64_t logits_row_stri
     va.gate_ld = d + RETRACE_LOWRANK_LATENT;
     va.gate_done = &ge_ready;
   }
-  va.plain_first = 1;  // measured: 79-81 us against 87 with the next round's CTAs waiting beside lr_fuse_kernel's
+  // With several row blocks the next round's CTAs, launched ahead, take the room
+  // of lr_fuse_kernel's (B = 32 / 64, d = 2560, V = 151936: 60 / 77 us against 55 /
+  // 70); with one (128 rows) or on the FFMA kernel launching ahead wins (B = 1 /
+  // 8, d = 2560: 26.9 / 34.7 against 28.5 / 35.0; d = 1024, fp32, B = 4: 100.0 / 101.7).
+  va.plain_first = tc && (long long)B * (K - 1) > 128;
   if (tc) {  // the finalising CTA of each sequence packs its [m; u] rows
     va.hT = hT;
     va.apack = w + Lw.apack;
