@@ -61,9 +61,9 @@ L2_FLUSH_BYTES = 256 << 20
 # kernel sources it was measured on: `sources` is kernel_sources_hash() at the
 # time, and the line reports null traffic once the sources differ.
 TRAFFIC = {
-    ("verify", "qwen3-8b-B256-K16"): {"bytes": 311305216 + 2984192 + 184312320 + 76800 + 55402240 + 0
-                                      + 47182848 + 4213248, "sources": "2e90788d1d34cc87"},
-    ("conditioning", "qwen3-8b-B256-K16"): {"bytes": 518159360 + 37841408, "sources": "2e90788d1d34cc87"},
+    ("verify", "qwen3-8b-B256-K16"): {"bytes": 311310080 + 2837248 + 184313856 + 146176 + 55402496 + 3840
+                                      + 47182336 + 4024320, "sources": "6513f6d371864d1a"},
+    ("conditioning", "qwen3-8b-B256-K16"): {"bytes": 486870528 + 36317184, "sources": "6513f6d371864d1a"},
 }
 
 
