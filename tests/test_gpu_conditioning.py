@@ -327,13 +327,14 @@ def test_ffma_rows(rt, B, K, d, R, dtype, dense_e):
     (9, 16, 1160, 128),
     (20, 16, 200, 257),  # two row tiles
     (64, 17, 328, 1024),
-    (80, 16, 136, 1100),  # CTA-pair kernel
+    (80, 16, 136, 1100),  # more than 1024 possible rows
     (80, 16, 392, 1023),
     (80, 16, 512, 257),
 ])
 def test_ragged_hidden_sizes(rt, B, K, d, R, dense_e):
     """bf16 hidden sizes that are a multiple of 8 but not of the tiles, with a
-    broadcast and a per-position e, on the small-R and the CTA-pair kernels."""
+    broadcast and a per-position e, on the small-R kernel (test_many_rows: on
+    the kernels for more rows)."""
     dtype = torch.bfloat16
     x = make_inputs(B, K, d, dtype, seed=R + d, accept=accept_for_rows(B, K, R))
     A = host_int(x["accept"])
@@ -362,21 +363,16 @@ def test_ragged_hidden_sizes(rt, B, K, d, R, dense_e):
     (200, 16, 392, 1500),
     # more than 4096 possible rows: CTA pairs (the gate's last wave in K halves), and one-SM tiles for a
     # per-position e where d is a multiple of 256
-    (274, 16, 256, 1),
-    (274, 16, 256, 127),
-    (274, 16, 256, 129),
-    (274, 16, 256, 256),
-    (274, 16, 256, 257),
-    (274, 16, 256, 1200),
-    (274, 16, 256, 4110),
+    *[(274, 16, 256, R) for R in (1, 17, 127, 129, 241, 256, 257, 513, 1023, 1200, 4110)],
     (274, 16, 264, 130),
     (274, 16, 264, 4110),
     # more than 2^22 rows times features
     (70, 16, 4096, 129),
 ])
 def test_many_rows(rt, B, K, d, R, dense_e):
-    """Either side of the lines between the small-R kernel and those for more
-    rows, at the edges of their row tiles."""
+    """Either side of the lines between the small-R kernel (rows times features
+    up to 2^22, at most 4096 rows) and those for more rows, at the edges of
+    their row tiles (the CTA-pair kernel's 128 and 256 rows)."""
     dtype = torch.bfloat16
     x = make_inputs(B, K, d, dtype, seed=R + d, accept=accept_for_rows(B, K, R))
     A = host_int(x["accept"])
