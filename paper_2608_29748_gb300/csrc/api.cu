@@ -340,11 +340,10 @@ int retrace_set_verify_schedule(int mode) { return set_verify_schedule(mode); }
 
 int retrace_verify_plan(int B, int K, int V, retrace_dtype dtype, int target_argmax, int* window_starts) {
   if (B < 0 || K < 0 || V < 1 || K > kMaxK || (dtype != RETRACE_BF16 && dtype != RETRACE_F32)) return -1;
-  int start[kMaxWindowPasses + 1];
-  const int n = verify_windows(B, K, V, (int)elem_size(dtype), true, target_argmax != 0, start);
+  const RowWindows w = verify_windows(B, K, V, (int)elem_size(dtype), true, target_argmax != 0);
   if (window_starts)
-    for (int k = 0; k <= n; ++k) window_starts[k] = start[k];
-  return n;
+    for (int k = 0; k <= w.n; ++k) window_starts[k] = w.start[k];
+  return w.n;
 }
 
 size_t retrace_workspace_bytes(int B, int K, int V, int d, retrace_dtype dtype) {
@@ -383,6 +382,7 @@ retrace_status retrace_verify(const void* logits, retrace_dtype dtype, int B, in
   if ((st = check_ws(ws, ws_bytes, L.ge)) != RETRACE_OK) return st;
   if ((st = prepare_ws(ws, ws_bytes, L, B, K, stream)) != RETRACE_OK) return st;
   VerifyArgs a{};
+  a.windows = verify_windows(B, K, V, (int)elem_size(dtype), true, target_argmax != nullptr);
   a.logits = logits;
   a.B = B;
   a.K = K;
@@ -547,8 +547,8 @@ retrace_status retrace_round(const void* logits, int64_t logits_row_stride,
   // Few sequences verified in one pass: the conditioning reads the carried
   // rows where they lie (the ablations, a per-position e and every row's argmax
   // as an output take the general path).
-  const bool direct = tc && flags == 0 && !dense && !target_argmax && direct_rows_supported(B, K, d) &&
-                      verify_windows(B, K, V, (int)elem_size(dtype), true, false, nullptr) == 1;
+  const RowWindows windows = verify_windows(B, K, V, (int)elem_size(dtype), true, target_argmax != nullptr);
+  const bool direct = tc && flags == 0 && !dense && !target_argmax && direct_rows_supported(B, K, d) && windows.n == 1;
   // Otherwise verification packs the conditioned rows as sequences finish.
   if (flags & RETRACE_ROUND_OVERLAP) {
     RT_CUDA(cudaMemsetAsync(sync, 0, L.sync_bytes, stream), "cudaMemsetAsync(sync)");
@@ -596,6 +596,7 @@ retrace_status retrace_round(const void* logits, int64_t logits_row_stride,
     return RETRACE_OK;
   }
   VerifyArgs va{};
+  va.windows = windows;
   va.logits = logits;
   va.B = B;
   va.K = K;
@@ -679,6 +680,7 @@ retrace_status retrace_verify_sampled(const void* target_logits, int64_t target_
   if ((st = check_ws(ws, ws_bytes, Lw.total)) != RETRACE_OK) return st;
   if ((st = prepare_ws(ws, ws_bytes, Lw, B, K, stream)) != RETRACE_OK) return st;
   SampledArgs a{};
+  a.windows = verify_windows(B, K, V, (int)elem_size(dtype), true, false);
   a.tlogits = target_logits;
   a.t_row = target_row_stride;
   a.t_batch = target_batch_stride;
@@ -737,6 +739,7 @@ retrace_status retrace_round_sampled(const void* target_logits, int64_t target_r
   // the finalize kernel packs the conditioned rows behind a counter at zero
   if (tc && !direct) RT_CUDA(cudaMemsetAsync(sync, 0, L.sync_bytes, stream), "cudaMemsetAsync(sync)");
   SampledArgs a{};
+  a.windows = verify_windows(B, K, V, (int)elem_size(dtype), true, false);
   a.tlogits = target_logits;
   a.t_row = target_row_stride;
   a.t_batch = target_batch_stride;
@@ -814,6 +817,7 @@ retrace_status retrace_round_lowrank(const void* logits, int64_t logits_row_stri
 
   if (phase_events) RT_CUDA(cudaEventRecord(phase_events[0], stream), "cudaEventRecord");
   VerifyArgs va{};
+  va.windows = verify_windows(B, K, V, (int)elem_size(dtype), true, target_argmax != nullptr);
   va.logits = logits;
   va.B = B;
   va.K = K;

@@ -194,7 +194,19 @@ struct DeviceInfo {
 cudaError_t device_info(DeviceInfo* out);
 
 // ---- verification -----------------------------------------------------------
+// Row windows of one call: pass k of `n` reads rows [start[k], start[k + 1]).
+// Taken once per call, by the entry point: the schedule is process-wide and
+// another thread may set it meanwhile, so what the call chooses by the number of
+// passes and what it launches go by the same copy.
+struct RowWindows {
+  int n;  // 1: the one-pass schedule
+  int start[kMaxWindowPasses + 1];
+};
+// The windows a call takes under the current schedule.
+RowWindows verify_windows(int B, int K, int V, int elem_bytes, bool have_workspace, bool argmax_out);
+
 struct VerifyArgs {
+  RowWindows windows;
   const void* logits;
   int B, K, V;
   long long row_stride, batch_stride;  // elements
@@ -252,14 +264,11 @@ cudaError_t launch_verify(const VerifyArgs& a, retrace_dtype dtype, cudaStream_t
 // the copy fields of `a` (B, K, d, accept_len, e..., cond_copy, pack_off).
 cudaError_t launch_verify_copies(const VerifyArgs& a, retrace_dtype dtype, cudaStream_t stream);
 int set_verify_schedule(int mode);  // RETRACE_VERIFY_*; previous mode, or -1
-// Row windows greedy verification takes for this call: writes the window
-// starts (n + 1 entries, at most kMaxWindowPasses + 1; start may be NULL) and returns the number
-// of passes n (1: the one-pass schedule).
-int verify_windows(int B, int K, int V, int elem_bytes, bool have_workspace, bool argmax_out, int* start);
 
 // Stochastic verification (speculative sampling on top-k / top-p filtered
 // distributions at temperature T).
 struct SampledArgs {
+  RowWindows windows;
   const void* tlogits;  // [B, K+1, V]
   long long t_row, t_batch;
   const void* dlogits;  // [B, K, V]

@@ -717,19 +717,20 @@ inline int window_bounds(int K1, int* start) {
 
 }  // namespace
 
-int verify_windows(int B, int K, int V, int elem_bytes, bool have_workspace, bool argmax_out, int* start) {
+RowWindows verify_windows(int B, int K, int V, int elem_bytes, bool have_workspace, bool argmax_out) {
   const int K1 = K + 1;
-  int bounds[kMaxWindowPasses + 1];
-  if (!start) start = bounds;
-  const int n = window_bounds(K1, start);
+  RowWindows w{};
+  const int n = window_bounds(K1, w.start);
   const int mode = g_schedule.load(std::memory_order_relaxed);
   const long long wave = (long long)B * V * elem_bytes;
   const bool windowed = have_workspace && !argmax_out && B > 0 && B <= kWindowMaxB && n > 1 &&
                         (mode == RETRACE_VERIFY_WINDOWS || (mode == RETRACE_VERIFY_AUTO && wave >= kWindowMinBatchRowBytes));
-  if (windowed) return n;
-  start[0] = 0;
-  start[1] = K1;
-  return 1;
+  w.n = n;
+  if (!windowed) {
+    w.n = 1;
+    w.start[1] = K1;
+  }
+  return w;
 }
 
 namespace {
@@ -830,8 +831,8 @@ cudaError_t launch_typed(const VerifyArgs& a, cudaStream_t stream) {
   p.defer_copies = 0;
   p.pack_off = a.pack_off;
   const int K1 = a.K + 1;
-  int start[kMaxWindowPasses + 1];
-  const int n_pass = verify_windows(a.B, a.K, a.V, (int)sizeof(T), a.live != nullptr, a.target_argmax != nullptr, start);
+  const int n_pass = a.windows.n;
+  const int* start = a.windows.start;
   const bool windowed = n_pass > 1;
   const long long grid_full = (long long)info.sm_count * occ;
   if (!windowed) {

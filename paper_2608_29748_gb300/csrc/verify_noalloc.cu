@@ -145,6 +145,7 @@ extern "C" retrace_status retrace_verify_noalloc(const void* logits, retrace_dty
   a.B = B;
   a.K = K;
   a.V = V;
+  a.windows = verify_windows(B, K, V, dtype == RETRACE_BF16 ? 2 : 4, false, target_argmax != nullptr);
   a.row_stride = logits_row_stride;
   a.batch_stride = logits_batch_stride;
   a.draft = draft;

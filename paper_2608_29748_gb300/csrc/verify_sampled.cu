@@ -730,8 +730,8 @@ cudaError_t launch_verify_sampled(const SampledArgs& a, retrace_dtype dtype, cud
   // 0..min(A_b, K-1): the same row windows as greedy verification.  Pass k
   // scans the window's rows of the sequences that accepted every earlier
   // draft (top-k kernel), then runs their accept tests (finalize kernel).
-  int start[kMaxWindowPasses + 1];
-  const int n_pass = verify_windows(a.B, a.K, a.V, (int)fp.elem, a.live != nullptr, false, start);
+  const int n_pass = a.windows.n;
+  const int* start = a.windows.start;
   DeviceInfo info;
   cudaError_t e0 = device_info(&info);
   if (e0 != cudaSuccess) return e0;

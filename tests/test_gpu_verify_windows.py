@@ -298,3 +298,57 @@ def test_round_copies_in_finalisers_equal_copy_kernel(rt, flags):
         for name in ("accept_len", "committed", "bonus", "n", "e_out"):
             assert torch.equal(getattr(o, name), getattr(outs[0], name)), name
     assert ws.check() == 0
+
+
+SWITCHER = """
+typedef int (*set_schedule)(int);
+void switch_schedules(set_schedule set, int a, int b, volatile int* stop) {
+  while (!*stop) {
+    set(a);
+    set(b);
+  }
+}
+"""
+
+
+def test_schedule_set_by_another_thread_during_rounds(rt, tmp_path):
+    """The schedule is process-wide, and another thread may set it between any
+    two steps of a call: each call goes by one reading of it.  Rounds of few
+    sequences (whose conditioning decides the sequences itself after one pass
+    over every row, and leaves that to verification in row windows) while a
+    native thread switches between the two as fast as it can."""
+    import ctypes
+    import subprocess
+    import threading
+
+    (tmp_path / "switcher.c").write_text(SWITCHER)
+    so = str(tmp_path / "switcher.so")
+    subprocess.run(["gcc", "-O1", "-shared", "-fPIC", "-o", so, str(tmp_path / "switcher.c")], check=True)
+    switcher = ctypes.CDLL(so)
+    set_schedule = ctypes.cast(rt.lib.retrace_set_verify_schedule, ctypes.c_void_p)
+    stop = ctypes.c_int(0)
+
+    cfg = CONFIGS[2].__class__("few", 2, 16, 515, 256, "bf16", 1.0, "uniform", seed_offset=3)
+    x = make_round_inputs(cfg, device="cuda")
+    ws = rt.Workspace(cfg.B, cfg.K, cfg.V, cfg.d, cfg.torch_dtype)
+    prev = rt.retrace_set_verify_schedule(rt.VERIFY_WINDOWS)
+    want_windows = rt.run_round(x, ws)
+    rt.retrace_set_verify_schedule(rt.VERIFY_FULL)
+    want = rt.run_round(x, ws)
+    thread = threading.Thread(target=switcher.switch_schedules,
+                              args=(set_schedule, rt.VERIFY_WINDOWS, rt.VERIFY_FULL, ctypes.byref(stop)))
+    thread.start()
+    try:
+        outs = [rt.run_round(x, ws) for _ in range(1000)]
+    finally:
+        stop.value = 1
+        thread.join()
+        rt.retrace_set_verify_schedule(prev)
+    torch.cuda.synchronize()
+    assert ws.check() == 0
+    for out in outs:
+        assert torch.equal(out.accept_len, want.accept_len)
+        assert torch.equal(out.committed, want.committed)
+        assert torch.equal(out.bonus, want.bonus)
+        # the two conditioning paths add in different orders
+        assert torch.equal(out.e_out, want.e_out) or torch.equal(out.e_out, want_windows.e_out)
