@@ -117,14 +117,14 @@ __device__ __forceinline__ void copy_vectors(long long n, Load load, Store store
 }
 
 // ---------------------------------------------------------------------------
-// One warp of `nw`: rows w, w + nw, ... of ge = W_g[:, :d] e (d a multiple of
-// 8; W_g's rows `ld` elements apart).  The rows come in steps of 256 vectors
+// One warp of `nw`: rows w, w + nw, ... below `end` of ge = W_g[:, :d] e (d a
+// multiple of 8; W_g's rows `ld` elements apart).  The rows come in steps of 256 vectors
 // through two register buffers in turn, one loading while the other is
 // multiplied (a single buffer handed on by a copy waits for the copy: one
 // memory latency per step).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void gate_bias_share(const __nv_bfloat16* e, const __nv_bfloat16* Wg, float* ge, int d,
-                                                int ld, int w, int nw, int lane) {
+                                                int ld, int w, int nw, int lane, int end) {
   const int vpr = d / 8, steps = (vpr + 255) / 256;
   const uint4* ev = reinterpret_cast<const uint4*>(e);
   struct Pos {
@@ -137,7 +137,7 @@ __device__ __forceinline__ void gate_bias_share(const __nv_bfloat16* e, const __
     }
   };
   auto load = [&](uint4 (&x)[8], const Pos& p) {
-    if (p.row >= d) return;
+    if (p.row >= end) return;
     const uint4* wr = reinterpret_cast<const uint4*>(Wg + (long long)p.row * ld);
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
@@ -171,17 +171,22 @@ __device__ __forceinline__ void gate_bias_share(const __nv_bfloat16* e, const __
   Pos pa{w, 0}, pb{w, 0};
   advance(pb);
   load(a, pa);
-  while (pa.row < d) {
+  while (pa.row < end) {
     load(b, pb);
     use(a, pa);
     pa = pb;
     advance(pa);
-    if (pb.row >= d) break;
+    if (pb.row >= end) break;
     load(a, pa);
     use(b, pb);
     pb = pa;
     advance(pb);
   }
+}
+
+__device__ __forceinline__ void gate_bias_share(const __nv_bfloat16* e, const __nv_bfloat16* Wg, float* ge, int d,
+                                                int ld, int w, int nw, int lane) {
+  gate_bias_share(e, Wg, ge, d, ld, w, nw, lane, d);
 }
 
 // The same with four loads in flight and few registers, for kernels that have

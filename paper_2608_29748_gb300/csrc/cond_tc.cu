@@ -215,6 +215,13 @@ __device__ __forceinline__ void gate_bias_rows(const CondParams& p, int d, int l
   gate_bias_rows(p.e, p.Wg, p.ge, d, lane, next, done);
 }
 
+// One warp: ge for the 128 features from n0, in the order of a share's rows, so
+// that the bits are the same whoever computes them.
+__device__ __noinline__ void gate_bias_features(const CondParams& p, int d, int n0, int lane) {
+  gate_bias_share(p.e, p.Wg, p.ge, d, 2 * d, n0, 1, lane, min(n0 + 128, d));
+  __syncwarp();  // the warp reads the values back
+}
+
 // Correction epilogue of one tile row (Eq. 7): r = m + beta * c for the 256
 // accumulator columns n0.., m = the first d columns of the packed row g.
 // GENERAL: d may end inside the tile (at a multiple of 8 columns).
@@ -706,6 +713,12 @@ constexpr uint32_t IDESC_M256_N128 = idesc_bf16_f32(256, 128);
 // row-block-major order at config 5).
 constexpr int kGroupBlocks = 4;
 constexpr int P_TILE_SLOTS = 3;  // tile indices in flight: the leader publishes one tile ahead
+// A gate tile waits this long for W_g[:, :d] e, of which every CTA of the grid
+// computes a share, before its epilogue computes the 128 values of its features
+// itself: a share's CTA may not be on an SM yet where kernels of another stream
+// hold some, so a tile must not depend on it.  With the GPU to itself the grid is
+// resident and the shares take 10 to 50 us (d = 4096 to 8192).
+constexpr unsigned long long kGateBiasPatienceNs = 1000000ull;
 
 // GENERAL = false: d a multiple of 256, where every tile is whole, and a broadcast e.  With the
 // checks of the general form in its epilogue and MMA loop the kernel took
@@ -1014,6 +1027,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
     const int q = (warp - 4) * 32 + lane;  // tile row = TMEM lane
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
     bool have_ge = !need_ge;
+    unsigned long long patience = kGateBiasPatienceNs;
     for (uint32_t lt = 0;; ++lt) {
       const uint32_t slot = lt % P_TILE_SLOTS, sph = (lt / P_TILE_SLOTS) & 1u;
       bool ok = warp_wait_cluster(smem_u32(&bar_tile_full[slot]), sph, &s_abort);
@@ -1041,13 +1055,14 @@ __global__ void __launch_bounds__(P_THREADS, 1)
       if (s_abort) break;
       if (!corr && !have_ge) {
         int got = 1;
-        if (lane == 0) got = wait_counter(gemv_done, (uint32_t)d, &s_abort) ? 1 : 0;
-        got = __shfl_sync(0xFFFFFFFFu, got, 0);
-        if (!got) {
-          if (lane == 0) raise_abort(&s_abort, p.status);
-          break;
+        if (lane == 0) got = wait_counter(gemv_done, (uint32_t)d, &s_abort, patience) ? 1 : 0;
+        have_ge = __shfl_sync(0xFFFFFFFFu, got, 0) != 0;
+        if (!have_ge) {
+          if (__shfl_sync(0xFFFFFFFFu, s_abort, 0)) break;
+          patience = 0ull;  // of this warp's later tiles
+          // (every warp of the tile, and the share's owner, write the same bits)
+          gate_bias_features(p, d, n0, lane);
         }
-        have_ge = true;
       }
       const int g = m0 + q;
       const bool valid = g < R;

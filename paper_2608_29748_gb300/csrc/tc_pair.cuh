@@ -34,9 +34,9 @@ __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
 }
 
 // Waits until *counter >= target (written by other CTAs of this grid).
-// Bounded like every other wait: false after kWaitLimitNs or on abort.
-__device__ __forceinline__ bool wait_counter(const uint32_t* counter, uint32_t target,
-                                             volatile int* abort) {
+// Bounded like every other wait: false after limit_ns or on abort.
+__device__ __forceinline__ bool wait_counter(const uint32_t* counter, uint32_t target, volatile int* abort,
+                                             unsigned long long limit_ns = kWaitLimitNs) {
   if (ld_acquire(counter) >= target) return true;
   const unsigned long long t0 = global_ns();
   for (uint32_t it = 1;; ++it) {
@@ -44,7 +44,7 @@ __device__ __forceinline__ bool wait_counter(const uint32_t* counter, uint32_t t
     if (ld_acquire(counter) >= target) return true;
     if ((it & 63u) == 0u) {
       if (*abort) return false;
-      if (global_ns() - t0 > kWaitLimitNs) return false;
+      if (global_ns() - t0 > limit_ns) return false;
     }
   }
 }

@@ -353,3 +353,25 @@ def test_round_of_few_sequences(rt, B, K, V, d, accept):
             nb = int(want["n"][b])
             assert torch.equal(out.e_out[b, nb:], x["e"].expand(K - nb, d))
     assert torch.equal(outs[0].e_out, outs[1].e_out)
+
+
+@pytest.mark.parametrize("B,d", [(70, 4096), (140, 2056)])
+def test_rounds_on_two_streams(rt, B, d):
+    """Rounds of many rows, one workspace each, on two streams at once: neither
+    round's kernels may need SMs that the other's hold to finish (every wait
+    inside them is for work of CTAs that run)."""
+    K, V = 16, 2048
+    streams = [torch.cuda.Stream(priority=p) for p in (0, -1)]
+    cfgs = [CONFIGS[2].__class__("two", B, K, V, d, "bf16", 1.0, "uniform", seed_offset=i) for i in range(2)]
+    xs = [make_round_inputs(cfg, device="cuda") for cfg in cfgs]
+    wss = [rt.Workspace(B, K, V, d, torch.bfloat16) for _ in cfgs]
+    want = [rt.run_round(x, ws) for x, ws in zip(xs, wss)]
+    outs = [rt.RoundBuffers(B, K, d, torch.bfloat16) for _ in cfgs]
+    torch.cuda.synchronize()
+    for _ in range(25):
+        for x, ws, out, s in zip(xs, wss, outs, streams):
+            rt.run_round(x, ws, out=out, stream=s)
+    torch.cuda.synchronize()
+    for ws, out, w in zip(wss, outs, want):
+        assert ws.check() == 0
+        assert torch.equal(out.accept_len, w.accept_len) and torch.equal(out.e_out, w.e_out)
