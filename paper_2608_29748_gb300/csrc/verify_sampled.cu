@@ -27,6 +27,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cfloat>
 #include <cstddef>
 
 #include "common.cuh"
@@ -40,6 +41,7 @@ constexpr int kThreads = 512;
 constexpr int kUnroll = 4;    // 16-byte loads in flight per thread
 constexpr int kCells = 16;    // most cells per thread
 constexpr int kBuf = 1024;    // candidates a CTA keeps without the slow path
+constexpr int kTieThreads = 128;  // threads that reach the bound from which a row counts as tied there
 constexpr int kMaxParts = 8;  // most CTAs (a cluster) per row
 constexpr int kPrefetchVectors = 4096;  // 64 KB of the next row: two batches of every thread
 
@@ -96,19 +98,30 @@ struct Chunk<float> {
   __device__ float value(int e) const { return __uint_as_float(e == 0 ? w.x : e == 1 ? w.y : e == 2 ? w.z : w.w); }
 };
 
-// Shared memory of a top-k CTA.  The slow path uses buf and cell together as
-// one array of kSlowBuf keys.
+// Shared memory of a top-k CTA.  The slow path and topk_tied use buf and cell
+// together as one array of kSlowBuf keys.
 struct TopkSmem {
   unsigned long long buf[kBuf];
   float cell[kCells][kThreads];
   unsigned long long top[kMaxTopK];  // this CTA's part of the row, in descending order
   float thr;
+  int warp_n[kThreads / 32];
   int n;      // candidates in buf
   int n_top;  // keys in top
 };
 constexpr int kSlowBuf = kBuf + kCells * kThreads / 2;
 static_assert(offsetof(TopkSmem, cell) == sizeof(unsigned long long) * kBuf, "the slow path's array is contiguous");
 static_assert(kSlowBuf >= kBuf + kThreads * 8, "a slow-path round fits behind kBuf keys");
+
+// Cells of the vectors [v0, v1): batches of kUnroll * kThreads per cell, and cells.
+__device__ __forceinline__ int cell_batches(int v0, int v1) {
+  const int batches = (v1 - v0 + kUnroll * kThreads - 1) / (kUnroll * kThreads);
+  return (batches + kCells - 1) / kCells;
+}
+__device__ __forceinline__ int cell_count(int v0, int v1) {
+  const int batches = (v1 - v0 + kUnroll * kThreads - 1) / (kUnroll * kThreads), per = cell_batches(v0, v1);
+  return per > 0 ? (batches + per - 1) / per : 0;
+}
 
 // Moves the largest min(n, k) of `keys` (distinct) to `top` in descending
 // order, by rank counting; returns their count.  Called by the whole CTA,
@@ -123,9 +136,9 @@ __device__ __forceinline__ int rank_top(const unsigned long long* keys, int n, i
   return n < k ? n : k;
 }
 
-// The k largest keys of row elements >= t when they are too many for buf (long
-// runs of equal values): rounds of one vector per thread, the keys cut to the
-// k largest whenever they pass kBuf.  Fills sm.top; returns the count.
+// The k largest keys of row elements >= t when they are too many for buf: rounds
+// of one vector per thread, the keys cut to the k largest whenever they pass kBuf.
+// Fills sm.top; returns the count.
 template <typename T>
 __device__ __noinline__ int topk_slow(const T* x, int head, int v0, int v1, int edge_n, int full, float t, int k,
                                       TopkSmem& sm) {
@@ -166,7 +179,114 @@ __device__ __noinline__ int topk_slow(const T* x, int head, int v0, int v1, int 
   }
 }
 
+// The top-k keys of a part where many threads' maxima are the bound t itself: a
+// row masked with a finite value that leaves fewer than k tokens, or coarse
+// logits.  At most k - 1 threads hold anything larger, and of the elements equal
+// to t the first by index are enough, which a scan in index order finds in its
+// first rounds.  A verification of 1056 rows of 151936 bf16 masked so takes 109 us
+// (where nothing ties 88; with every masked element a candidate for topk_slow
+// 2585).  Nothing here is unrolled: with unrolled loops in this function the
+// kernel's rows that never call it took 2 % longer.  Fills sm.top; returns the
+// count.
+template <typename T>
+__device__ __noinline__ int topk_tied(const T* x, int head, int v0, int v1, int edge_n, int full, float t, int k,
+                                      TopkSmem& sm) {
+  using CT = Chunk<T>;
+  constexpr int E = CT::E;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint4* vp = reinterpret_cast<const uint4*>(x + head);
+  const int per = cell_batches(v0, v1), cells = cell_count(v0, v1);
+  const int edge_i = tid < head ? tid : tid + full * E;
+  float tm = tid < edge_n ? to_f32(x[edge_i]) : -INFINITY;  // this thread's maximum
+  for (int j = 0; j < cells; ++j) tm = fmaxf(tm, sm.cell[j][tid]);
+  if (tid == 0) sm.n = 0;
+  __syncthreads();
+  if constexpr (sizeof(T) == 4) {  // the bound's other 16 bits
+    const unsigned h = ordered_bits(tm);
+    unsigned b = ordered_bits(t) & 0xFFFF0000u;
+#pragma unroll 1
+    for (int bit = 15; bit >= 0; --bit) {
+      const unsigned c = b | (1u << bit);
+      if (__syncthreads_count(h >= c) >= k) b = c;
+    }
+    t = fmaxf(t, key_value((unsigned long long)b << 32));
+  }
+  // the elements > t
+  auto above = [&](float v, int idx) {
+    if (v > t) {
+      const int at = atomicAdd(&sm.n, 1);
+      if (at < kBuf) sm.buf[at] = make_key(v, (uint32_t)idx);
+    }
+  };
+  if (tm > t) {
+    if (tid < edge_n) above(to_f32(x[edge_i]), edge_i);
+    for (int j = 0; j < cells; ++j) {
+      if (!(sm.cell[j][tid] > t)) continue;
+      for (int c = j * per; c < (j + 1) * per; ++c)
+        for (int u = 0; u < kUnroll; ++u) {
+          const int v = v0 + (c * kUnroll + u) * kThreads + tid;
+          if (v >= v1) continue;
+          CT ch;
+          ch.w = __ldg(vp + v);
+#pragma unroll 1
+          for (int e = 0; e < E; ++e) above(ch.value(e), head + v * E + e);
+        }
+    }
+  }
+  __syncthreads();
+  const int n_above = sm.n;
+  __syncthreads();
+  if (n_above > kBuf) return topk_slow<T>(x, head, v0, v1, edge_n, full, t, k, sm);
+  // the elements equal to t in index order: before the vectors, the vectors, after them
+  const int limit = max(n_above, k);
+  int have = n_above;
+  for (int b = v0 - kThreads; have < limit; b += kThreads) {
+    unsigned equal = 0u;
+    int idx = 0;
+    if (b < v0) {
+      if (edge_n > 0 && tid < head) {
+        idx = tid;
+        equal = to_f32(x[idx]) == t ? 1u : 0u;
+      }
+    } else if (b < v1) {
+      const int v = b + tid;
+      if (v < v1) {
+        CT ch;
+        ch.w = __ldg(vp + v);
+        idx = head + v * E;
+#pragma unroll 1
+        for (int e = 0; e < E; ++e) equal |= ch.value(e) == t ? 1u << e : 0u;
+      }
+    } else if (tid < edge_n - head) {
+      idx = head + full * E + tid;
+      equal = to_f32(x[idx]) == t ? 1u : 0u;
+    }
+    const int count = __popc(equal);
+    int incl = count;
+#pragma unroll 1
+    for (int off = 1; off < 32; off <<= 1) {
+      const int y = __shfl_up_sync(0xFFFFFFFFu, incl, off);
+      if (lane >= off) incl += y;
+    }
+    if (lane == 31) sm.warp_n[warp] = incl;
+    __syncthreads();
+    int at = have + incl - count;
+#pragma unroll 1
+    for (int w = 0; w < kThreads / 32; ++w) {
+      const int n = sm.warp_n[w];
+      at += w < warp ? n : 0;
+      have += n;
+    }
+    for (; equal != 0u && at < limit; equal &= equal - 1u, ++at)
+      sm.buf[at] = make_key(t, (uint32_t)(idx + __ffs((int)equal) - 1));
+    __syncthreads();
+    if (b >= v1) break;
+  }
+  return rank_top(sm.buf, min(have, limit), k, sm.top);
+}
+
 // The top-k keys of part `part` of `parts` of row x, into sm.top (whole CTA).
+// Elements at -infinity carry no weight and get no key.
 //
 // Every thread streams its vectors once and keeps only maxima: one per cell
 // (a few batches of kUnroll vectors) in shared memory and one overall.  The
@@ -189,11 +309,9 @@ __device__ __forceinline__ void topk_part(const T* x, int V, int k, int parts, i
   const int v0 = (int)((long long)part * full / parts), v1 = (int)((long long)(part + 1) * full / parts);
   // the elements before and after the vectors (fewer than 2 E), one per thread of part 0
   const int edge_n = part == 0 ? V - full * E : 0;
+  const int per = cell_batches(v0, v1), cells = cell_count(v0, v1);
   const int edge_i = tid < head ? tid : tid + full * E;
   const uint4* vp = reinterpret_cast<const uint4*>(x + head);
-  const int batches = (v1 - v0 + kUnroll * kThreads - 1) / (kUnroll * kThreads);
-  const int per = (batches + kCells - 1) / kCells;  // batches per cell
-  const int cells = per > 0 ? (batches + per - 1) / per : 0;
   if (tid == 0) sm.n = 0;
   float edge_v = -INFINITY;
   if (tid < edge_n) edge_v = to_f32(x[edge_i]);
@@ -232,7 +350,9 @@ __device__ __forceinline__ void topk_part(const T* x, int V, int k, int parts, i
     if (__syncthreads_count(h >= c) >= k) lo = c;
   }
   const unsigned minus_inf = ordered_bits(-INFINITY) >> 16;
-  float t = lo <= minus_inf ? -INFINITY : key_value((unsigned long long)lo << 48);
+  // (a negative value's key has its low bits set)
+  const unsigned low = sizeof(T) == 2 && !(lo & 0x8000u) ? 0xFFFFu : 0u;
+  float t = lo <= minus_inf ? -FLT_MAX : key_value((unsigned long long)(lo << 16 | low) << 32);
   if (parts > 1) {
     if (tid == 0) sm.thr = t;
     cluster_sync_all();
@@ -245,7 +365,9 @@ __device__ __forceinline__ void topk_part(const T* x, int V, int k, int parts, i
       if (at < kBuf) sm.buf[at] = make_key(v, (uint32_t)idx);
     }
   };
-  if (tm >= t) {
+  if (__syncthreads_count(h >= lo) > kTieThreads && lo > minus_inf) {
+    sm.n = kBuf + 1;  // for topk_tied
+  } else if (tm >= t) {
     if (tid < edge_n) add(edge_v, edge_i);
     for (int j = 0; j < cells; ++j) {
       if (!(sm.cell[j][tid] >= t)) continue;
@@ -267,8 +389,8 @@ __device__ __forceinline__ void topk_part(const T* x, int V, int k, int parts, i
   }
   __syncthreads();
   int n = sm.n;
-  __syncthreads();  // the slow path reuses sm.n
-  if (n > kBuf) n = topk_slow<T>(x, head, v0, v1, edge_n, full, t, k, sm);
+  __syncthreads();  // topk_tied reuses sm.n
+  if (n > kBuf) n = topk_tied<T>(x, head, v0, v1, edge_n, full, t, k, sm);
   else n = rank_top(sm.buf, n, k, sm.top);
   if (tid == 0) sm.n_top = n;
   __syncthreads();

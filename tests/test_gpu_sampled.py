@@ -167,3 +167,77 @@ def test_sampled_topk_rows(rt, kind, V, k, offset, dtype, windows):
         check_against_oracle(rt, {"logits": tl}, s)
     finally:
         rt.retrace_set_verify_schedule(prev)
+
+
+def masked_rows(mask, tokens, B, K, V, dtype, offset, g):
+    """[B, K+1, V] logits at `mask` but for `tokens` of them, the same in every row."""
+    buf = torch.full((B * (K + 1) * V + offset,), mask, device="cuda", dtype=torch.float32).to(dtype)
+    rows = buf[offset:].view(B, K + 1, V)
+    at = torch.randperm(V, generator=g, device="cuda")[:tokens]
+    rows[:, :, at] = (torch.rand((B, K + 1, tokens), generator=g, device="cuda") * 3 + 0.5).to(dtype)
+    return rows
+
+
+MASKS = ["-inf", "lowest", -1e4, 0.0]
+
+
+def mask_value(mask, dtype):
+    return {"-inf": -float("inf"), "lowest": torch.finfo(dtype).min}.get(mask, mask)
+
+
+@pytest.mark.parametrize("windows", [False, True])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("tokens,V,k,offset", [(1, 9000, 20, 0), (5, 20001, 20, 7), (5, 151936, 20, 0), (19, 70001, 64, 3), (300, 32003, 64, 0)])
+@pytest.mark.parametrize("mask", MASKS)
+def test_sampled_masked_rows(rt, mask, tokens, V, k, offset, dtype, windows):
+    """Constrained decoding: a mask of -inf or of a finite value that leaves
+    fewer tokens than top_k (and one that leaves more).  At mask 0 the masked
+    tokens carry weight, the lowest indices first."""
+    B, K = 2, 6
+    g = torch.Generator(device="cuda").manual_seed(V + tokens)
+    value = mask_value(mask, dtype)
+    tl = masked_rows(value, tokens, B, K, V, dtype, offset, g)
+    dl = masked_rows(value, 0, B, K, V, dtype, offset, g)[:, :K]
+    kept = tl[:, :K] != value
+    dl[kept] = (tl[:, :K][kept].float() + 0.3 * torch.randn(int(kept.sum()), generator=g, device="cuda")).to(dtype)
+    s = {"draft_logits": dl, "draft": torch.topk(dl.float(), 1, dim=-1).indices[..., 0].to(torch.int32),
+         "uniforms": torch.rand((B, K + 1), generator=g, device="cuda") * 0.9, "temperature": 1.0, "top_k": k, "top_p": 0.9}
+    prev = rt.retrace_set_verify_schedule(rt.VERIFY_WINDOWS if windows else rt.VERIFY_FULL)
+    try:
+        check_against_oracle(rt, {"logits": tl}, s)
+    finally:
+        rt.retrace_set_verify_schedule(prev)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_sampled_masked_rows_cost_no_more(rt, dtype):
+    """The scan of masked rows, and of rows of one value, takes about the time
+    of plain rows (the bound, twice that, is a fifth of what ranking every
+    masked element took)."""
+    B, K, V = 8, 16, 151936
+    g = torch.Generator(device="cuda").manual_seed(9)
+    ws = rt.Workspace(B, K, V, 1, dtype)
+    outs = [torch.empty(B, dtype=torch.int32, device="cuda"), torch.empty((B, K + 1), dtype=torch.int32, device="cuda"),
+            torch.empty(B, dtype=torch.int32, device="cuda")]
+    u = torch.rand((B, K + 1), generator=g, device="cuda")
+
+    def cost(tl):
+        dl = tl[:, :K].clone()
+        draft = torch.argmax(dl.float(), dim=-1).to(torch.int32)
+        best = float("inf")
+        for _ in range(6):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda._sleep(1_000_000)  # the calls are enqueued before the first starts
+            a.record()
+            for _ in range(5):
+                rt.retrace_verify_sampled(tl, dl, draft, u, 1.0, 20, 0.95, *outs, ws)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        return best
+
+    plain = cost((torch.randn((B, K + 1, V), generator=g, device="cuda") * 2).to(dtype))
+    for mask in MASKS:
+        masked = cost(masked_rows(mask_value(mask, dtype), 5, B, K, V, dtype, 0, g))
+        assert masked <= 2 * plain, (mask, masked, plain)
+    assert cost(torch.full((B, K + 1, V), 1.5, device="cuda", dtype=dtype)) <= 2 * plain
