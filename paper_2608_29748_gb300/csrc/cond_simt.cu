@@ -33,7 +33,12 @@ namespace {
 // One chain over the split took 42.4 us instead of 43.2 for a round of B = 8, K =
 // 8, d = 1024, but had two to four times the rounding error (relative to 64 bits
 // there 3.4e-7, now 1.4e-7; B = 1, K = 16, d = 2048: 5.6e-7, now 1.6e-7; a warp per
-// feature with its lanes along the reduction 2.5e-7).
+// feature with its lanes along the reduction 2.5e-7).  FINE (fine_sums) adds by
+// fours and in pairs up to the chunk, and the splits with their rounding errors:
+// by eights, short reductions over few rows had up to 8 % more error than that
+// warp per feature, whose lanes held a few products each (r / e~ at B = 2, K = 16,
+// d = 64: 6.50e-8 / 1.16e-7 against 6.20e-8 / 1.12e-7, now 5.78e-8 / 1.08e-7; d = 72:
+// 6.68e-8 / 1.19e-7 against 6.27e-8 / 1.12e-7, now 5.69e-8 / 1.06e-7).
 constexpr int kNT = 256;
 constexpr int kTileRows = 64;              // most conditioned rows of a tile
 constexpr int TN = 64, TK = 32;            // weight rows and reduction depth of a chunk
@@ -61,6 +66,11 @@ struct SimtParams {
   int clusters;    // clusters with a unit; CTAs past them compute ge
   int vec;         // 16-byte fp32 copies
 };
+
+// Whether a projection of at most `rows` rows takes FINE sums.  From d = 224 on
+// the sums by eights have less error than a warp per feature too, and above 32
+// rows that was never the alternative.
+inline bool fine_sums(long long rows, int d) { return rows <= 32 && d < 224; }
 
 // Row numbers of the plan: the rows of this CTA's row tile nt, cut from R into
 // tiles of equal size (a multiple of 16, at most kTileRows).  Fills s_b (-1
@@ -192,10 +202,30 @@ __device__ __forceinline__ void stage_weights(const SimtParams& p, float* ring, 
 }
 constexpr int kSimtAhead = kSimtStages - 1;  // chunks staged ahead
 
+// v[0] = the sum of v[0..7], each addition's rounding error added at the end
+// (Knuth's two-sum; the error of an infinite sum is no number and is left out).
+__device__ __forceinline__ void sum_exactly(float4 (&v)[8]) {
+  float4 lost = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto add = [](float& s, float& c, float x) {
+    const float t = s + x, z = t - s;
+    c += (s - (t - z)) + (x - z);
+    s = t;
+  };
+#pragma unroll
+  for (int s = 1; s < 8; ++s) {
+    add(v[0].x, lost.x, v[s].x);
+    add(v[0].y, lost.y, v[s].y);
+    add(v[0].z, lost.z, v[s].z);
+    add(v[0].w, lost.w, v[s].w);
+  }
+  auto finite = [](float c) { return fabsf(c) < INFINITY ? c : 0.f; };
+  add4(v[0], make_float4(finite(lost.x), finite(lost.y), finite(lost.z), finite(lost.w)));
+}
+
 // The partial tile of this CTA: its chunks [c0, c1) of the unit with weight
 // tile n0, rows at s_off0 / s_off1 (-1: no row), into ring[] as [row][TN].
 // The weights of the first kSimtAhead chunks are staged already.
-template <typename T, bool GATE, int MR>
+template <typename T, bool GATE, int MR, bool FINE>
 __device__ __forceinline__ void simt_partial(const SimtParams& p, float* ring, const long long* s_off0,
                                              const long long* s_off1, int n0, int c0, int c1) {
   const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16, d = p.d;
@@ -232,10 +262,10 @@ __device__ __forceinline__ void simt_partial(const SimtParams& p, float* ring, c
     const float* As = ring + (c - c0) % kSimtStages * kStageFloats + ty * kLd;
     const float* Bs = ring + (c - c0) % kSimtStages * kStageFloats + (kTileRows + tx) * kLd;
     const bool gate_only = GATE && c >= per;
-    float sum[MR][4];  // of this chunk
+    float sum[MR][4], s16[MR][4];  // of this chunk, and of half of it (FINE)
 #pragma unroll
     for (int k0 = 0; k0 < TK; k0 += 8) {
-      float t[MR][4];
+      float t[MR][4], t4[MR][4];
 #pragma unroll
       for (int k = k0; k < k0 + 8; k += 4) {
         float4 a[MR], b[4];
@@ -248,6 +278,18 @@ __device__ __forceinline__ void simt_partial(const SimtParams& p, float* ring, c
           if (j < 2 && gate_only) continue;  // weight rows tx, tx + 16: W_v
 #pragma unroll
           for (int i = 0; i < MR; ++i) {
+            if constexpr (FINE) {
+              float& x = k == k0 ? t4[i][j] : t[i][j];
+              x = a[i].x * b[j].x;
+              x = fmaf(a[i].y, b[j].y, x);
+              x = fmaf(a[i].z, b[j].z, x);
+              x = fmaf(a[i].w, b[j].w, x);
+              if (k == k0) continue;
+              x += t4[i][j];
+              s16[i][j] = k0 % 16 == 0 ? x : s16[i][j] + x;
+              if (k0 % 16 == 8) sum[i][j] = k0 == 8 ? s16[i][j] : sum[i][j] + s16[i][j];
+              continue;
+            }
             t[i][j] = k == k0 ? a[i].x * b[j].x : fmaf(a[i].x, b[j].x, t[i][j]);
             t[i][j] = fmaf(a[i].y, b[j].y, t[i][j]);
             t[i][j] = fmaf(a[i].z, b[j].z, t[i][j]);
@@ -272,7 +314,7 @@ __device__ __forceinline__ void simt_partial(const SimtParams& p, float* ring, c
     for (int j = 0; j < 4; ++j) ring[(ty + 16 * i) * TN + tx + 16 * j] = acc[i][j];
 }
 
-template <typename T, bool GATE>
+template <typename T, bool GATE, bool FINE>
 __global__ void __launch_bounds__(kNT, 2) simt_cluster_kernel(const SimtParams p) {
   extern __shared__ float4 simt_smem[];
   __shared__ int s_b[kTileRows], s_j[kTileRows], s_nb[kTileRows], s_scan[kNT / 32 + 1];
@@ -327,10 +369,14 @@ __global__ void __launch_bounds__(kNT, 2) simt_cluster_kernel(const SimtParams p
     }
   }
   __syncthreads();
-  if (tile == 16) simt_partial<T, GATE, 1>(p, ring, s_off0, s_off1, n0, c0, c1);
-  else if (tile == 32) simt_partial<T, GATE, 2>(p, ring, s_off0, s_off1, n0, c0, c1);
-  else if (tile == 48) simt_partial<T, GATE, 3>(p, ring, s_off0, s_off1, n0, c0, c1);
-  else simt_partial<T, GATE, 4>(p, ring, s_off0, s_off1, n0, c0, c1);
+  if (tile == 16) {
+    simt_partial<T, GATE, 1, FINE>(p, ring, s_off0, s_off1, n0, c0, c1);
+  } else if (FINE || tile == 32) {
+    simt_partial<T, GATE, 2, FINE>(p, ring, s_off0, s_off1, n0, c0, c1);
+  } else if constexpr (!FINE) {
+    if (tile == 48) simt_partial<T, GATE, 3, false>(p, ring, s_off0, s_off1, n0, c0, c1);
+    else simt_partial<T, GATE, 4, false>(p, ring, s_off0, s_off1, n0, c0, c1);
+  }
   cluster_sync_all();  // every partial of the cluster is in shared memory
   const int l0 = (int)rank * rows / S, l1 = ((int)rank + 1) * rows / S;  // this CTA's rows of the tile
   const uint32_t P = smem_u32(ring);
@@ -348,13 +394,18 @@ __global__ void __launch_bounds__(kNT, 2) simt_cluster_kernel(const SimtParams p
         if constexpr (GATE) g[s] = ld_cluster_f4(src + 32 * 4);
       }
     }
+    if constexpr (FINE) {
+      sum_exactly(v);
+      if constexpr (GATE) sum_exactly(g);
+    } else {
 #pragma unroll
-    for (int h = 1; h < 8; h *= 2)
+      for (int h = 1; h < 8; h *= 2)
 #pragma unroll
-      for (int s = 0; s + h < 8; s += 2 * h) {
-        add4(v[s], v[s + h]);
-        if constexpr (GATE) add4(g[s], g[s + h]);
-      }
+        for (int s = 0; s + h < 8; s += 2 * h) {
+          add4(v[s], v[s + h]);
+          if constexpr (GATE) add4(g[s], g[s + h]);
+        }
+    }
     const float vv[4] = {v[0].x, v[0].y, v[0].z, v[0].w}, gg[4] = {g[0].x, g[0].y, g[0].z, g[0].w};
     const long long pos = (long long)s_b[l] * K + s_j[l];
     const long long orow = (!GATE && p.compact) ? m0 + l : pos;
@@ -408,16 +459,15 @@ __global__ void __launch_bounds__(256) fill_rows_kernel(int B, int K, int d, Row
 // possible R (those past the R found on the device leave at once) and, with
 // `gemv`, CTAs for W_g[:, :d] e behind them.  S: two CTAs per SM over the
 // units at three quarters of the possible rows, at most 8 and one chunk each.
-template <typename T, bool GATE>
+template <typename T, bool GATE, bool FINE>
 cudaError_t launch_simt(SimtParams& p, bool gemv, cudaStream_t stream) {
   const long long rmax = (long long)p.B * (p.K - 1);
-  if (rmax <= 0) return cudaSuccess;
   DeviceInfo info;
   cudaError_t err = device_info(&info);
   if (err != cudaSuccess) return err;
   static std::atomic<int> attr_done[64];
   if (!attr_done[info.device & 63].load(std::memory_order_acquire)) {
-    err = cudaFuncSetAttribute(simt_cluster_kernel<T, GATE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSimtSmem);
+    err = cudaFuncSetAttribute(simt_cluster_kernel<T, GATE, FINE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSimtSmem);
     if (err != cudaSuccess) return err;
     attr_done[info.device & 63].store(1, std::memory_order_release);
   }
@@ -435,8 +485,15 @@ cudaError_t launch_simt(SimtParams& p, bool gemv, cudaStream_t stream) {
   const size_t es = sizeof(T);
   auto al = [](const void* q) { return (uintptr_t)q % 16 == 0; };
   p.vec = es == 4 && p.d % 4 == 0 && al(p.a0) && al(p.w) && (!GATE || al(p.wg)) && (!p.a1 || al(p.a1));
-  return launch_dependent(simt_cluster_kernel<T, GATE>, dim3((unsigned)((clusters + extra) * p.S)), dim3(kNT),
+  return launch_dependent(simt_cluster_kernel<T, GATE, FINE>, dim3((unsigned)((clusters + extra) * p.S)), dim3(kNT),
                           (size_t)kSimtSmem, stream, (unsigned)p.S, p);
+}
+
+template <typename T, bool GATE>
+cudaError_t launch_simt(SimtParams& p, bool gemv, cudaStream_t stream) {
+  const long long rmax = (long long)p.B * (p.K - 1);
+  if (rmax <= 0) return cudaSuccess;
+  return fine_sums(rmax, p.d) ? launch_simt<T, GATE, true>(p, gemv, stream) : launch_simt<T, GATE, false>(p, gemv, stream);
 }
 
 template <typename T>
