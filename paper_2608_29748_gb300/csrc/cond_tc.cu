@@ -1846,9 +1846,9 @@ static cudaError_t launch_cond_pair(const TcCondArgs& a, int clusters, cudaStrea
 }
 
 // Pairs of CTAs of cond_pair_kernel to launch: those the device keeps resident
-// (cached per device), or fewer when the call has fewer tiles.
+// (cached per device; 0: none fits), or fewer when the call has fewer tiles.
 static int pair_clusters(const TcCondArgs& a, long long tiles_max, cudaError_t* err) {
-  static std::atomic<int> max_clusters[64];  // 0: not yet known
+  static std::atomic<int> max_clusters[64];  // 0: not yet known, -1: none
   int dev = 0;
   if ((*err = cudaGetDevice(&dev)) != cudaSuccess) return 0;
   int n = max_clusters[dev & 63].load(std::memory_order_acquire);
@@ -1869,12 +1869,10 @@ static int pair_clusters(const TcCondArgs& a, long long tiles_max, cudaError_t* 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if ((*err = cudaOccupancyMaxActiveClusters(&n, cond_pair_kernel<true>, &cfg)) != cudaSuccess) return 0;
-    if (n < 1) {
-      *err = cudaErrorInvalidConfiguration;
-      return 0;
-    }
+    if (n < 1) n = -1;
     max_clusters[dev & 63].store(n, std::memory_order_release);
   }
+  if (n < 0) return 0;
   // every pair when the gate-bias GEMV is needed: pairs without tiles compute it
   if (a.do_gate && !a.e_dense) return n;
   return (int)(tiles_max < n ? tiles_max : n);
@@ -2143,14 +2141,20 @@ static cudaError_t launch_cond_one_sm(const TcCondArgs& a, cudaStream_t stream) 
 cudaError_t launch_cond_tc(const TcCondArgs& a, cudaStream_t stream) {
   const long long rmax = (long long)a.B * (a.K - 1);
   if (rmax <= 0 || (!a.do_correct && !a.do_gate)) return cudaSuccess;
-  if (a.direct || cond_small_r(a.B, a.K, a.d)) return launch_cond_swap(a, stream);
-  if (a.do_gate && a.e_dense && a.d % 256 == 0) return launch_cond_one_sm(a, stream);
+  auto path = [&](int pairs) {
+    return cond_path(a.B, a.K, a.d, a.direct != 0, a.do_gate && a.e_dense, pairs);
+  };
+  if (path(1) == kCondSwap) return launch_cond_swap(a, stream);
+  if (path(1) == kCondOneSm) return launch_cond_one_sm(a, stream);
   const long long tiles_max = (rmax + 2 * BM - 1) / (2 * BM) *
                               ((a.do_correct ? (a.d + 255) / 256 : 0) + (a.do_gate ? (a.d + 127) / 128 : 0));
   cudaError_t err;
   const int clusters = pair_clusters(a, tiles_max, &err);
   if (err != cudaSuccess) return err;
-  return launch_cond_pair(a, clusters, stream);
+  if (path(clusters) == kCondPair) return launch_cond_pair(a, clusters, stream);
+  TcCondArgs b = a;
+  b.ge_ready = 0;  // launch_pack leaves it to the CTA-pair kernel above the small-R line
+  return launch_cond_swap(b, stream);
 }
 
 }  // namespace retrace

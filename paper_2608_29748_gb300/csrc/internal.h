@@ -61,6 +61,17 @@ inline bool cond_small_r(long long B, long long K, long long d) {
   const long long rmax = B * (K > 1 ? K - 1 : 0);
   return rmax > 0 && rmax <= kSmallRRows && rmax * d <= kSmallRWork;
 }
+// The kernels of a tensor-core conditioning call (described in cond_tc.cu):
+// split-K clusters for few rows and for direct ones, one-SM tiles for a
+// per-position e with d a multiple of 256, CTA pairs otherwise.  A device (or a
+// partition of one) that holds no pair of CTAs, `pairs` = 0, takes the split-K
+// clusters, whose cluster size may be one, for any number of rows.
+enum CondPath { kCondSwap, kCondOneSm, kCondPair };
+inline CondPath cond_path(long long B, long long K, long long d, bool direct, bool gate_dense_e, int pairs) {
+  if (direct || cond_small_r(B, K, d)) return kCondSwap;
+  if (gate_dense_e && d % 256 == 0) return kCondOneSm;
+  return pairs > 0 ? kCondPair : kCondSwap;
+}
 // The region of swap_part_bytes in the workspace holds the corrected signal of a
 // round without packed rows (direct rows, below).
 constexpr int kSwapMaxRows = 1024;
