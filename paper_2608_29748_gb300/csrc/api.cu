@@ -530,15 +530,24 @@ retrace_status retrace_round(const void* logits, int64_t logits_row_stride,
   if ((st = e_mode(e_batch_stride, e_pos_stride, K, d, &dense)) != RETRACE_OK) return st;
   const WsLayout L = ws_layout(B, K, d, elem_size(dtype));
   if ((st = check_ws(ws, ws_bytes, L.total)) != RETRACE_OK) return st;
+  const bool tc = need_gate && tc_supported(dtype, d) && aligned16(hD) && aligned16(hT) &&
+                  aligned16(Wc) && aligned16(Wv) && aligned16(Wg) && aligned16(e) && aligned16(e_out);
+  TcRoundArgs ra{};  // the overlapped round
+  if (flags & RETRACE_ROUND_OVERLAP) {
+    ra.logits = logits;
+    ra.B = B;
+    ra.K = K;
+    ra.V = V;
+    ra.d = d;
+    ra.row_stride = logits_row_stride;
+    ra.batch_stride = logits_batch_stride;
+    if (!tc || !round_fused_supported(ra))
+      return fail(RETRACE_ERR_UNSUPPORTED, "RETRACE_ROUND_OVERLAP: shape or layout outside the overlapped kernel");
+  }
   if ((st = prepare_ws(ws, ws_bytes, L, B, K, stream)) != RETRACE_OK) return st;
   char* w = reinterpret_cast<char*>(ws);
   float* ge = reinterpret_cast<float*>(w + L.ge);
   void* r_ws = w + L.r;
-
-  const bool tc = need_gate && tc_supported(dtype, d) && aligned16(hD) && aligned16(hT) &&
-                  aligned16(Wc) && aligned16(Wv) && aligned16(Wg) && aligned16(e) && aligned16(e_out);
-  if ((flags & RETRACE_ROUND_OVERLAP) && !tc)
-    return fail(RETRACE_ERR_UNSUPPORTED, "RETRACE_ROUND_OVERLAP: bf16 with d a multiple of 256 and 16-byte aligned tensors only");
   uint32_t* sync = reinterpret_cast<uint32_t*>(w + L.sync);
   int32_t* R = reinterpret_cast<int32_t*>(sync + kSyncRowCount);
   int32_t* rowmap = reinterpret_cast<int32_t*>(w + L.rowmap);
@@ -552,14 +561,6 @@ retrace_status retrace_round(const void* logits, int64_t logits_row_stride,
   // Otherwise verification packs the conditioned rows as sequences finish.
   if (flags & RETRACE_ROUND_OVERLAP) {
     RT_CUDA(cudaMemsetAsync(sync, 0, L.sync_bytes, stream), "cudaMemsetAsync(sync)");
-    TcRoundArgs ra{};
-    ra.logits = logits;
-    ra.B = B;
-    ra.K = K;
-    ra.V = V;
-    ra.d = d;
-    ra.row_stride = logits_row_stride;
-    ra.batch_stride = logits_batch_stride;
     ra.draft = draft;
     ra.accept_len = accept_len;
     ra.committed = committed;
@@ -586,8 +587,6 @@ retrace_status retrace_round(const void* logits, int64_t logits_row_stride,
     ra.rowmap = rowmap;
     ra.sync = sync;
     ra.status = status_word(ws);
-    if (!round_fused_supported(ra))
-      return fail(RETRACE_ERR_UNSUPPORTED, "RETRACE_ROUND_OVERLAP: shape or layout outside the overlapped kernel");
     // verification and both projections overlap inside one launch
     RT_CUDA(launch_round_tc(ra, stream), "round kernel launch");
     if (phase_events) {

@@ -129,6 +129,27 @@ def test_round_flag_errors(lib):
         assert _round(lib, flags) == OK  # B = 0: nothing to do
 
 
+def test_overlapped_round_refuses_before_any_cuda_call(lib):
+    """RETRACE_ROUND_OVERLAP outside the overlapped kernel's shapes: UNSUPPORTED, and nothing was enqueued (here any
+    CUDA call would fail first, with another status)."""
+    P, I64, sz = ctypes.c_void_p, ctypes.c_int64, ctypes.c_size_t
+
+    def call(d=256, V=4096, stride=None, e=16):
+        ws = lib.retrace_workspace_bytes(2, 4, V, d, BF16)
+        rs = stride or V
+        return lib.retrace_round(P(16), I64(rs), I64(5 * rs), P(16), P(16), P(16), P(e), I64(0), I64(0), P(16), P(16), P(16),
+                                 ctypes.c_float(1.0), BF16, 2, 4, V, d, P(16), P(16), P(16), None, None, P(16),
+                                 P(1 << 30), sz(ws), ctypes.c_uint32(0x1), None, None)
+
+    assert call(d=264) == UNSUPPORTED           # tensor cores, but no multiple of 256
+    assert call(d=100) == UNSUPPORTED
+    assert call(V=4000) == UNSUPPORTED          # rows shorter than a stream chunk
+    assert call(V=4100) == UNSUPPORTED          # no multiple of 8
+    assert call(stride=4104) == UNSUPPORTED     # rows apart
+    assert call(e=8) == UNSUPPORTED             # not 16-byte aligned
+    assert b"OVERLAP" in lib.retrace_last_error()
+
+
 def test_round_header_documents_the_flags():
     text = open(HEADER).read()
     for name, value in (("RETRACE_ROUND_OVERLAP", 0x1), ("RETRACE_COND_RAW", 0x2),
