@@ -465,9 +465,11 @@ def run_gpu(args) -> dict | None:
         verify_launches += 1
     # conditioning launches of the greedy and temperature-1 rounds, by path:
     # small R (split-K clusters: correction with the gate-bias GEMV, then gate;
-    # raw: GEMV, gate) and FFMA (the same) two, CTA pairs one
+    # the GEMV by itself above d = 4096; raw: GEMV, gate) and FFMA two, CTA pairs one
     small_r = tensor_cores and 0 < rows <= 4096 and rows * cfg.d <= 1 << 22
     cond_launches = 2 if not tensor_cores or small_r else 1
+    if small_r and cfg.d > 4096 and args.variant == "corrected":
+        cond_launches = 3
     step_avg_s = statistics.mean(step_ms) / 1e3
     cflops = (lowrank_flops(cfg, R) if args.lowrank
               else conditioning_flops(cfg, R, dense_e=False, variant=args.variant))

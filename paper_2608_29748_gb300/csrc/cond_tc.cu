@@ -1187,6 +1187,13 @@ constexpr int SW_ROW_MAPS = 256 / SW_ROW_STEP;
 constexpr int SW_SMEM_RING = 198 * 1024;
 // The gate's where no verification kernel is launched ahead beside it.
 constexpr int SW_SMEM_MAX = 222 * 1024;
+// Largest d at which the correction's idle warps compute W_g[:, :d] e.  They keep 24
+// KB per SM in flight, so above it they outlast the correction (d = 8192: 103 us of
+// a correction that takes 56 without them) and a launch of its own runs beside
+// it.  Rounds, V = 32000, B = 1 / 8 / 16, us, in idle warps and alone: d = 4096: 52
+// / 61 / 70 and 49 / 61 / 71; 4608: 62 / 72 / 80 and 56 / 71 / 78; 6144: 106 / 111 /
+// 119 and 91 / 104 / 113; 8192: 161 / 164 / 175 and 133 / 153 / 162.
+constexpr int kGateBiasAlone = 4096;
 
 // Row tiles of R rows for `clusters` resident clusters over `mtiles` weight
 // tiles: `ntiles` tiles of `tile_n` rows (a multiple of 16, at most 256).
@@ -1736,10 +1743,13 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
   }
 }
 
-// W_g[:, :d] e alone (a round whose gate follows verification: the raw variant).
+// W_g[:, :d] e alone: a round whose gate follows verification (the raw variant),
+// and beside the correction above kGateBiasAlone.  Few registers, so that its CTAs
+// fit on the SMs beside the correction's.
 __global__ void __launch_bounds__(256) swap_gemv_kernel(const GateBiasParams p) {
   pdl_launch_dependents();
-  gate_bias_share(p.e, p.Wg, p.ge, p.d, 2 * p.d, (int)blockIdx.x * 8 + (threadIdx.x >> 5), (int)gridDim.x * 8, threadIdx.x & 31);
+  gate_bias_share_small(p.e, p.Wg, p.ge, p.d, 2 * p.d, (int)blockIdx.x * 8 + (threadIdx.x >> 5), (int)gridDim.x * 8,
+                        threadIdx.x & 31);
   // Complete only after the previous kernel: the next kernel's programmatic
   // wait, which covers this kernel alone, then covers that one too.  One CTA
   // waiting is enough (the grid completes with its last CTA); the others
@@ -1911,7 +1921,7 @@ static int swap_cluster_capacity(int dev, int S, int smem, cudaError_t* err) {
 // costs its k-blocks (measured: 750 cycles each at N = 160, 830 at 177, 1070 at
 // 250; the issue of the MMAs and the stage's handshake make most of a small
 // one), 60 cycles per row of the tile (the drain and the sum over the splits),
-// 4000 to start and end, and with packed rows 700 per CTA of the cluster (they
+// `wave` to start and end (4000), and with packed rows 700 per CTA of the cluster (they
 // wait for each other).  Packed rows take four K splits at most: larger
 // clusters are not all placed at once beside the last CTAs of the kernel before
 // (a round, V = 2048, d = 3584, B = 32, 384 rows: 108 us with S = 5 for the
@@ -1919,8 +1929,11 @@ static int swap_cluster_capacity(int dev, int S, int smem, cudaError_t* err) {
 // d = 1024 to 4096 and 64 to 733 rows, and 33 pairs of standalone calls, each
 // timed with every S, the choice takes 1.5 % more than the best S of each (11 %
 // at most); one estimate at three quarters, 2 (128 + N) cycles per k-block, 24
-// per row, any S: 6 % (32 % at most).
-static cudaError_t swap_pick_splits(int dev, int smem, int rmax, bool direct, int parts, int mtiles, int nkb,
+// per row, any S: 6 % (32 % at most).  Above d = 4096 a further wave costs far more,
+// 20000: over 164 rounds of d = 4352 to 12288 the choice takes 1.9 % more than the
+// best S of each (15 % at most), with 4000 5.5 % (78 %).  Below, 20000 changes 5 of 80
+// choices, for 10 % more at one of two acceptance rates and 7 % less at the other.
+static cudaError_t swap_pick_splits(int dev, int smem, int rmax, bool direct, int parts, int mtiles, int nkb, int wave,
                                     int* S_out, int* clusters) {
   long long best = -1;
   cudaError_t err = cudaSuccess;
@@ -1935,7 +1948,7 @@ static cudaError_t swap_pick_splits(int dev, int smem, int rmax, bool direct, in
       const SwapCut cut = direct ? SwapCut{1, (rmax + 15) / 16 * 16} : swap_cut(rows, mtiles, cap);
       const long long waves = ((long long)mtiles * cut.ntiles + cap - 1) / cap;
       const int block = std::max(750, 17 * cut.tile_n / 4);
-      cost += waves * ((long long)((nkb + splits - 1) / splits) * block + 60 * cut.tile_n + 4000 + (direct ? 0 : 700 * S));
+      cost += waves * ((long long)((nkb + splits - 1) / splits) * block + 60 * cut.tile_n + wave + (direct ? 0 : 700 * S));
     }
     if (best < 0 || cost < best) {
       best = cost;
@@ -2019,6 +2032,8 @@ static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
   gp.e = reinterpret_cast<const __nv_bfloat16*>(a.e);
   gp.Wg = reinterpret_cast<const __nv_bfloat16*>(a.Wg);
   gp.ge = a.ge;
+  const bool bias_alone = d > kGateBiasAlone;
+  const int wave = d > 4096 && !a.e_dense ? 20000 : 4000;
   if (a.do_correct) {
     CUtensorMap mA, mA2;
     RowMaps mB;
@@ -2047,9 +2062,9 @@ static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
     c.beta = a.beta;
     c.r_out = reinterpret_cast<__nv_bfloat16*>(a.r_out);
     c.compact_out = a.compact_out;
-    if (a.do_gate && !a.e_dense) c.bias = gp;
+    if (a.do_gate && !a.e_dense && !bias_alone) c.bias = gp;
     int clusters = 0;
-    if ((err = swap_pick_splits(dev, smem, rmax, direct, 1, c.mtiles, c.nkb, &c.S, &clusters)) != cudaSuccess) return err;
+    if ((err = swap_pick_splits(dev, smem, rmax, direct, 1, c.mtiles, c.nkb, wave, &c.S, &clusters)) != cudaSuccess) return err;
     err = launch_dependent(direct ? swap_cluster_kernel<true> : swap_cluster_kernel<false>, grid_of(c, clusters),
                            dim3(SW_THREADS), (size_t)smem, stream, (unsigned)c.S, mA, mA2, mA, mB, mB, c);
     if (err != cudaSuccess) return err;
@@ -2065,7 +2080,7 @@ static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
         !encode_row_maps(&mB, a.rpack, du, rmax, rstride) ||
         (a.e_dense && !encode_row_maps(&mE, a.epack, du, rmax, 2 * du)))
       return cudaErrorInvalidValue;
-    if (!a.do_correct && !a.e_dense && !a.ge_ready) {  // no correction kernel to compute it: W_g[:, :d] e in its own launch
+    if ((!a.do_correct || bias_alone) && !a.e_dense && !a.ge_ready) {  // W_g[:, :d] e in its own launch
       err = launch_dependent(swap_gemv_kernel, dim3((unsigned)(info.sm_count * 4)), dim3(256), 0, stream, 1u, gp);
       if (err != cudaSuccess) return err;
     }
@@ -2082,7 +2097,8 @@ static cudaError_t launch_cond_swap(const TcCondArgs& a, cudaStream_t stream) {
     const int gsmem = a.last && rmax > 256 ? SW_SMEM_MAX : smem;
     g.stage_bytes = gsmem - 1024;
     int clusters = 0;
-    if ((err = swap_pick_splits(dev, gsmem, rmax, direct, a.e_dense ? 3 : 1, g.mtiles, g.nkb, &g.S, &clusters)) != cudaSuccess) return err;
+    if ((err = swap_pick_splits(dev, gsmem, rmax, direct, a.e_dense ? 3 : 1, g.mtiles, g.nkb, wave, &g.S, &clusters)) != cudaSuccess)
+      return err;
     err = launch_dependent(direct ? swap_cluster_kernel<true> : swap_cluster_kernel<false>, grid_of(g, clusters),
                            dim3(SW_THREADS), (size_t)gsmem, stream, (unsigned)g.S, mA, mA2, mA3, mB,
                            a.e_dense ? mE : mB, g);

@@ -375,3 +375,38 @@ def test_rounds_on_two_streams(rt, B, d):
     for ws, out, w in zip(wss, outs, want):
         assert ws.check() == 0
         assert torch.equal(out.accept_len, w.accept_len) and torch.equal(out.e_out, w.e_out)
+
+
+@pytest.mark.parametrize("B", [1, 4])
+@pytest.mark.parametrize("d", [6144, 7168])
+def test_round_of_few_sequences_at_large_hidden_sizes(rt, d, B):
+    """Hidden sizes above the ones the split-K rule was fitted to: a round that
+    reads its five d x d weight blocks once takes less time than copying them
+    (0.67 to 0.86 of it; with W_g e in the correction's idle warps and several
+    waves of clusters it took 1.01 to 1.17 times as long)."""
+    cfg = CONFIGS[2].__class__("large", B, 16, 32000, d, "bf16", 1.0, "uniform", seed_offset=d + B)
+    x = make_round_inputs(cfg, device="cuda")
+    ws = rt.Workspace(B, cfg.K, cfg.V, d, torch.bfloat16)
+    out = rt.RoundBuffers(B, cfg.K, d, torch.bfloat16)
+    a = torch.zeros((5, d, d), dtype=torch.bfloat16, device="cuda")
+    b = torch.empty_like(a)
+
+    def cost(f):
+        best = float("inf")
+        for _ in range(6):
+            start, stop = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda._sleep(1_000_000)  # the calls are enqueued before the first starts
+            start.record()
+            for _ in range(5):
+                f()
+            stop.record()
+            torch.cuda.synchronize()
+            best = min(best, start.elapsed_time(stop))
+        return best
+
+    round_cost, copy_cost = cost(lambda: rt.run_round(x, ws, out=out)), cost(lambda: b.copy_(a))
+    assert round_cost <= 0.95 * copy_cost, (round_cost, copy_cost)
+    assert ws.check() == 0
+    want = oracle_round(x)
+    assert_verify_exact(want, out.accept_len, out.committed, out.bonus)
+    assert_close(out.e_out, want["e_tilde"], f"d={d} B={B}")
