@@ -265,18 +265,19 @@ def test_verify_schedule_plan(lib):
 
 
 def test_workspace_holds_small_r_partials(lib):
-    """At most 1024 conditioned rows (and the gate GEMM's work tiles within 256
-    CTAs) the workspace also holds the split partials of the small-R GEMMs:
-    256 CTAs x 128 weight rows x min(256, rows rounded to 16) fp32."""
+    """At most 1024 conditioned rows (and 2 d / 128 weight tiles times their row
+    tiles of 256 within 256) the workspace also holds 256 x 128 x min(256, rows
+    rounded to 16) fp32 values: room for split partials, of which the library uses
+    a part (the corrected signal of a round of few sequences)."""
     ws = lib.retrace_workspace_bytes
     for B, K, d in ((1, 16, 2560), (8, 16, 4096), (64, 16, 2560), (64, 17, 4096)):
         rows = (B * (K - 1) + 15) // 16 * 16
         part = 256 * 128 * min(256, rows) * 4
         assert ws(B, K, 1000, d, BF16) >= part
-    small = ws(64, 17, 1000, 4096, BF16)   # 1024 rows: partials of 32 MiB
+    small = ws(64, 17, 1000, 4096, BF16)   # 1024 rows: a region of 32 MiB
     large = ws(65, 17, 1000, 4096, BF16)   # 1040 rows: the CTA-pair path, 4 MiB of split-tile halves
     assert (32 - 4 - 1) << 20 < small - large < (32 - 4) << 20
-    # fp32 takes the FFMA path: neither partial region
+    # fp32 takes the FFMA path: no split halves
     assert ws(65, 17, 1000, 4096, F32) < ws(64, 17, 1000, 4096, F32) - (30 << 20)
 
 
@@ -290,7 +291,7 @@ def test_workspace_holds_pair_split_halves(lib):
         rows = B * (K - 1)
         # r, apack, epack (bf16) and the row map come on top of the split halves
         assert ws(B, K, 1000, d, BF16) > split + rows * d * 2 * 4
-    # d not a multiple of 256 takes the FFMA path, without split halves: from
+    # d not a multiple of 256 has no split halves: from
     # d = 4096 to 4224 the d-sized buffers grow by half as much as from 3840 to
     # 4096, and the split region goes
     a, b, c = (ws(256, 16, 1000, dd, BF16) for dd in (3840, 4096, 4224))

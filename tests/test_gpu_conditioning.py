@@ -1,7 +1,7 @@
 """GPU parity of alignment/correction (Eq. 4-7) and gated fusion (Eq. 8) vs the oracle.
 
 Covers both kernel families: the tcgen05 tensor-core path (bf16, d a multiple
-of 256) and the FFMA path (fp32, and bf16 at other hidden sizes).
+of 8 and at least 128) and the FFMA path (fp32, and bf16 at other hidden sizes).
 """
 
 import math
@@ -48,13 +48,17 @@ SHAPES = [
     (5, 4, 512, torch.bfloat16),
     (19, 16, 256, torch.bfloat16),  # 19 * 15 = 285 rows: 3 M tiles, ragged last tile
     (3, 16, 2560, torch.bfloat16),
+    (4, 8, 192, torch.bfloat16),  # ragged feature tiles
+    (3, 12, 160, torch.bfloat16),
     # FFMA path
-    (4, 8, 192, torch.bfloat16),
     (3, 5, 100, torch.bfloat16),
+    (3, 12, 164, torch.bfloat16),
     (2, 8, 256, torch.float32),
     (6, 16, 96, torch.float32),
-    (4, 9, 160, torch.float32),  # B (K-1) = 32: the last shape of the warp-per-feature kernel
-    (3, 12, 160, torch.bfloat16),  # B (K-1) = 33: the first of the 32 x 64 tiles
+    (4, 9, 160, torch.float32),  # B (K-1) = 32: the last shape whose sums go by fours
+    (3, 12, 160, torch.float32),  # B (K-1) = 33
+    (2, 9, 223, torch.float32),  # the last hidden size whose sums go by fours
+    (2, 9, 224, torch.float32),
 ]
 
 
@@ -170,11 +174,8 @@ def accept_for_rows(B, K, R):
 
 @pytest.mark.parametrize("R", [1, 15, 16, 17, 127, 128, 129, 240, 241, 255, 256, 257, 384, 513, 769, 1023, 1200])
 def test_pair_tile_boundaries(rt, R):
-    """Row counts around the tile edges of the CTA-pair kernel: one to five
-    row tiles of 16 to 256 rows (a multiple of 16 chosen from R), halves of
-    8 to 128 rows in each CTA loaded as boxes of 64, 32, 16 and 8 rows, and
-    the last tile's padding.  B (K-1) = 1200 possible rows keeps the call off
-    the small-R path."""
+    """Row counts around the edges of 16- to 256-row tiles, with 1200 possible rows
+    (the small-R kernel; test_many_rows has the CTA-pair kernel's)."""
     B, K, d, dtype = 80, 16, 256, torch.bfloat16
     x = make_inputs(B, K, d, dtype, seed=R, accept=accept_for_rows(B, K, R))
     A = host_int(x["accept"])
@@ -199,12 +200,11 @@ def test_pair_tile_boundaries(rt, R):
 @pytest.mark.parametrize("B,K,d", [(1, 2, 256), (3, 6, 512), (16, 16, 256), (16, 17, 256), (8, 16, 2560),
                                    (17, 16, 256), (40, 16, 256), (64, 17, 256)])
 def test_small_r_path(rt, B, K, d):
-    """At most 1024 conditioned rows (B (K-1) <= 1024): the GEMMs run with the
-    weights as the 128-row side against N tiles of up to 256 rows, split over
-    K, the partials summed in a fixed order.  Every draft rejected at once
-    (A_b = 0), so all B (K-1) rows are carried: 1, 15, 240, 256, 255, 600 and
-    1024 rows (one to four N tiles, the last one partial) and d up to 2560;
-    both entry points against the oracle, repeatable bit for bit."""
+    """Small-R path: the GEMMs run with the weights as the 128-row side against row
+    tiles of up to 256 rows, split over K in clusters, the partials summed in a
+    fixed order.  Every draft rejected at once (A_b = 0), so all B (K-1) rows are
+    carried: 1, 15, 240, 256, 255, 600 and 1024 rows (the last tile partial) and d
+    up to 2560; both entry points against the oracle, repeatable bit for bit."""
     dtype = torch.bfloat16
     x = make_inputs(B, K, d, dtype, seed=B * 100 + K, accept=torch.zeros(B, dtype=torch.int32).cuda())
     A = host_int(x["accept"])
@@ -234,18 +234,16 @@ def test_small_r_path(rt, B, K, d):
 @pytest.mark.parametrize("B,K,d,R", [(1, 2, 256, 1), (1, 17, 512, 15), (2, 9, 256, 16), (17, 2, 1024, 17),
                                      (8, 16, 4096, 100), (16, 16, 256, 240), (17, 16, 2560, 255),
                                      (16, 17, 256, 256),
-                                     # more than 256 possible rows: N tiles of 256, split-K partials
+                                     # more than 256 possible rows
                                      (18, 16, 256, 16), (18, 16, 512, 257), (40, 16, 256, 511),
                                      (40, 16, 1024, 512), (35, 16, 4096, 513), (64, 16, 2560, 960),
                                      (64, 17, 256, 1000), (64, 17, 512, 1024)])
 def test_small_r_rows(rt, B, K, d, R):
-    """Exactly R carried rows on the small-R path (B (K-1) <= 1024).  At most
-    256 possible rows the GEMMs run as split-K clusters that sum their
-    partials through distributed shared memory; above that as split-K tiles
-    whose fp32 partials a reduction kernel sums.  R below, at and above
-    multiples of 16 and of 256 (one to four N tiles), cluster sizes that
-    differ between d = 256 and d = 4096: r and e~ against the oracle through
-    both standalone entry points, and repeated bit for bit."""
+    """Exactly R carried rows on the small-R path: split-K clusters that sum their
+    partials through distributed shared memory, in row tiles cut from R.  R below,
+    at and above multiples of 16 and of 256, cluster sizes that differ between d =
+    256 and d = 4096: r and e~ against the oracle through both standalone entry
+    points, and repeated bit for bit."""
     dtype = torch.bfloat16
     assert B * (K - 1) <= 1024 and R <= B * (K - 1)
     # carry exactly R rows: sequences reject at once (n_b = K - 1) until R is reached

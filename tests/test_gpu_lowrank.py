@@ -1,8 +1,8 @@
 """GPU parity of the low-rank conditioning path (retrace_round_lowrank) vs the oracle.
 
 Configs 1 (fp32, FFMA kernel), 3 and 4 (bf16, tensor cores) are checked in
-full; a bf16 shape with d not a multiple of 128 takes the FFMA kernel; the
-serving batch (config 5) is checked on its verification outputs, every
+full, and a bf16 shape with ragged blocks (test_lowrank_hidden_sizes has those
+that take the FFMA kernel); the serving batch (config 5) is checked on its verification outputs, every
 unconditioned row, and the conditioned rows of a seeded sample of sequences.
 """
 
@@ -16,7 +16,7 @@ from paper_2608_29748_gb300.workloads import CONFIGS, make_lowrank_weights, make
 
 pytestmark = pytest.mark.gpu
 
-SIMT_BF16 = CONFIGS[2].__class__("bf16 d=320 (FFMA path)", 6, 16, 5003, 320, "bf16", 1.0, "uniform", seed_offset=9)
+RAGGED_BF16 = CONFIGS[2].__class__("bf16 d=320 (ragged blocks)", 6, 16, 5003, 320, "bf16", 1.0, "uniform", seed_offset=9)
 
 
 @pytest.fixture(scope="module")
@@ -45,9 +45,9 @@ def oracle_lowrank(x, w, seqs=None):
         host_f64(w["Wg_lr"]), x["beta"], dtype)
 
 
-@pytest.mark.parametrize("cfg_id", [1, 3, 4, "simt-bf16"])
+@pytest.mark.parametrize("cfg_id", [1, 3, 4, "ragged-bf16"])
 def test_lowrank_round_full(rt, cfg_id):
-    cfg = SIMT_BF16 if cfg_id == "simt-bf16" else CONFIGS[cfg_id]
+    cfg = RAGGED_BF16 if cfg_id == "ragged-bf16" else CONFIGS[cfg_id]
     x = make_round_inputs(cfg, device="cuda")
     w = make_lowrank_weights(cfg, device="cuda")
     out, targ, ws = run(rt, x, w)

@@ -3,7 +3,7 @@
 Configs 1-4 are checked in full.  Config 5 (B = 256, 1.3 GB of logits) is
 checked twice: in full in the launch configuration the benchmark times
 (target_argmax not requested, so the default schedule verifies in row
-windows, copies and packs rows in the copy kernel and runs both projections
+windows, copies and packs rows in the finish kernel and runs both projections
 in cond_pair_kernel), and with target_argmax requested (one verification
 pass) on a seeded sample of conditioned rows.
 """
@@ -27,11 +27,10 @@ def rt():
 
 
 def small_r_path(B, K, d):
-    """Whether the conditioning of a bf16 round with a broadcast e takes the
-    small-R GEMMs: at most 1024 possible rows, and the gate GEMM's work tiles
-    (2d/128 weight tiles x N tiles of 256 rows) at most 256."""
-    rows = (B * (K - 1) + 15) // 16 * 16
-    return 0 < rows <= 1024 and (2 * d // 128) * ((rows + 255) // 256) <= 256
+    """Whether the conditioning of a bf16 round takes the small-R GEMMs: at most
+    4096 possible rows, and rows times features at most 2^22."""
+    rows = B * (K - 1)
+    return 0 < rows <= 4096 and rows * d <= 1 << 22
 
 
 def run(rt, x, ws=None, **kw):
@@ -64,7 +63,7 @@ def test_round_serving_batch_benched_path(rt):
     """Config 5 at full size (B=256, K=16, V=151936, d=4096) through exactly
     the call bench.py times: retrace_round with target_argmax NULL under the
     default schedule.  That composition is the row-window verification passes,
-    verify_copy_kernel (unconditioned rows of e~, packing of [m; u]) and
+    verify_finish_kernel (unconditioned rows of e~, packing of [m; u]) and
     cond_pair_kernel (both projections; R = 2876 rows, so the last 256-row
     pair block is partial).  Every output is compared with the oracle: the
     verification outputs and n bit-exact, every row of e~ within the bf16
@@ -248,7 +247,8 @@ def test_overlap_flag_rejects_what_the_kernel_does_not_cover(rt):
 
 # Ablation variants (component ablation, Table 3): raw conditioning gated,
 # raw conditioning overwrite, no conditioning.
-SMALL_SIMT_BF16 = CONFIGS[2].__class__("bf16 d=320 (FFMA path)", 6, 16, 5003, 320, "bf16", 1.0, "uniform", seed_offset=9)
+RAGGED_BF16 = CONFIGS[2].__class__("bf16 d=320 (ragged tiles)", 6, 16, 5003, 320, "bf16", 1.0, "uniform", seed_offset=9)
+FFMA_BF16 = CONFIGS[2].__class__("bf16 d=325 (FFMA path)", 6, 16, 5003, 325, "bf16", 1.0, "uniform", seed_offset=9)
 
 
 def _flag(rt, variant):
@@ -256,9 +256,9 @@ def _flag(rt, variant):
 
 
 @pytest.mark.parametrize("variant", ["raw", "overwrite", "none"])
-@pytest.mark.parametrize("cfg_id", [1, 3, 4, "simt-bf16"])
+@pytest.mark.parametrize("cfg_id", [1, 3, 4, "ragged-bf16", "ffma-bf16"])
 def test_ablation_variants(rt, cfg_id, variant):
-    cfg = SMALL_SIMT_BF16 if cfg_id == "simt-bf16" else CONFIGS[cfg_id]
+    cfg = {"ragged-bf16": RAGGED_BF16, "ffma-bf16": FFMA_BF16}.get(cfg_id) or CONFIGS[cfg_id]
     x = make_round_inputs(cfg, device="cuda")
     if variant != "raw":  # weights the variant does not use may be absent
         x = {**x, "Wc": None, "Wv": None, "Wg": None}
@@ -325,12 +325,16 @@ def test_small_r_round_with_almost_nothing_to_condition(rt, R):
 
 
 @pytest.mark.parametrize("accept", ["mixed", "none", "all"])
-@pytest.mark.parametrize("B,K,V,d", [(1, 5, 515, 128), (1, 16, 1003, 2560), (1, 120, 64, 256), (2, 63, 200, 264), (3, 9, 640, 136),
-                                     (5, 12, 333, 1160), (8, 16, 4099, 512), (8, 17, 129, 256), (16, 6, 77, 512)])
+@pytest.mark.parametrize("B,K,V,d", [(1, 5, 515, 128), (1, 16, 1003, 2560), (1, 65, 64, 256), (2, 33, 200, 264), (3, 9, 640, 136),
+                                     (3, 17, 333, 1160), (4, 16, 4099, 512), (8, 9, 129, 256), (8, 6, 77, 4352),
+                                     # above 64 tile rows
+                                     (1, 120, 64, 256), (2, 63, 200, 264), (5, 12, 333, 1160), (8, 16, 4099, 512),
+                                     (8, 17, 129, 256), (16, 6, 77, 512)])
 def test_round_of_few_sequences(rt, B, K, V, d, accept):
-    """Few sequences verified in one pass (no argmax output): the conditioning
-    decides them and reads the carried rows where they lie.  One to 16
-    sequences of 8 to 120 tile rows, all drafts accepted (nothing to
+    """Few sequences verified in one pass (no argmax output).  Up to 64 tile rows
+    (K - 1 rounded up to 8 per sequence) the conditioning decides them and reads
+    the carried rows where they lie: one to eight sequences of 8 to 64 tile rows;
+    above that verification packs them.  All drafts accepted (nothing to
     condition), none, and a mix with A = K-2, K-1 and K; twice on one workspace."""
     cfg = CONFIGS[2].__class__("few", B, K, V, d, "bf16", 1.0, "uniform", seed_offset=B + K)
     x = make_round_inputs(cfg, device="cuda")
@@ -353,6 +357,52 @@ def test_round_of_few_sequences(rt, B, K, V, d, accept):
             nb = int(want["n"][b])
             assert torch.equal(out.e_out[b, nb:], x["e"].expand(K - nb, d))
     assert torch.equal(outs[0].e_out, outs[1].e_out)
+
+
+@pytest.mark.parametrize("variant", ["corrected", "raw"])
+@pytest.mark.parametrize("dense_e", [False, True])
+@pytest.mark.parametrize("B,V,d", [(274, 515, 256), (274, 515, 264), (70, 2048, 4104)])
+def test_rounds_of_many_rows(rt, B, V, d, dense_e, variant):
+    """Whole rounds above the small-R line: both projections in one launch, r handed
+    from the correction to the gate inside it.  CTA pairs with whole and ragged
+    feature tiles, broadcast and per-position e, and one-SM tiles (per-position e,
+    d a multiple of 256), with and without every argmax as an output."""
+    cfg = CONFIGS[2].__class__("many", B, 16, V, d, "bf16", 1.0, "uniform", seed_offset=B + d)
+    x = make_round_inputs(cfg, device="cuda")
+    assert not small_r_path(cfg.B, cfg.K, cfg.d)
+    if dense_e:
+        x["e"] = (torch.randn((cfg.B, cfg.K, cfg.d), device="cuda") * 0.02).to(torch.bfloat16)
+    if variant == "raw":
+        x = {**x, "Wc": None}
+    flags = 0 if variant == "corrected" else rt.COND_RAW
+    out, targ, ws = run(rt, x, flags=flags)
+    again = rt.run_round(x, ws, flags=flags)
+    torch.cuda.synchronize()
+    assert ws.check() == 0
+    want = oracle_round(x, variant)
+    assert_verify_exact(want, out.accept_len, out.committed, out.bonus, targ)
+    np.testing.assert_array_equal(host_int(out.n), want["n"])
+    assert_close(out.e_out, want["e_tilde"], f"many rows, d={d} {variant}")
+    assert torch.equal(again.committed, out.committed) and torch.equal(again.n, out.n)
+    assert_close(again.e_out, want["e_tilde"], f"many rows, d={d} {variant}, no argmax")
+
+
+@pytest.mark.parametrize("dense_e", [False, True])
+@pytest.mark.parametrize("cfg", [RAGGED_BF16, FFMA_BF16], ids=["ragged", "ffma"])
+def test_round_hidden_sizes_off_the_tiles(rt, cfg, dense_e):
+    """bf16 rounds at a d that is a multiple of 8 only (tensor cores), and at an odd
+    one (FFMA: the correction's compact r, W_g e in further CTAs of its launch)."""
+    x = make_round_inputs(cfg, device="cuda")
+    if dense_e:
+        x["e"] = (torch.randn((cfg.B, cfg.K, cfg.d), device="cuda") * 0.02).to(torch.bfloat16)
+    out, targ, ws = run(rt, x)
+    again = rt.run_round(x, ws)
+    torch.cuda.synchronize()
+    assert ws.check() == 0
+    want = oracle_round(x)
+    for o in (out, again):
+        assert_verify_exact(want, o.accept_len, o.committed, o.bonus)
+        assert_close(o.e_out, want["e_tilde"], cfg.name)
 
 
 @pytest.mark.parametrize("B,d", [(70, 4096), (140, 2056)])

@@ -52,14 +52,15 @@ def check_conditioning(x, out, rows, dtype):
     assert_close(got, ref, "sampled round e~")
 
 
-def check_round(rt, x, s):
+def check_round(rt, x, s, ws=None):
     cfg_B, K1, _ = x["logits"].shape
     K = K1 - 1
     d = x["hD"].shape[2]
     dtype = "bf16" if x["logits"].dtype == torch.bfloat16 else "f32"
     tl, dl, draft, u, amb = conditioned_uniforms_for(x, s)
     s = dict(s, uniforms=torch.tensor(u, dtype=torch.float32, device="cuda"))
-    ws = rt.Workspace(cfg_B, K, x["logits"].shape[2], d, x["logits"].dtype)
+    if ws is None:
+        ws = rt.Workspace(cfg_B, K, x["logits"].shape[2], d, x["logits"].dtype)
     out = rt.run_round_sampled(x, s, ws)
     torch.cuda.synchronize()
     assert ws.check() == 0
@@ -100,8 +101,9 @@ def test_sampled_round_matches_the_oracle(rt, cfg_id):
 
 def test_sampled_round_dense_e_and_short_blocks(rt):
     """Per-position e (packed by the finalize kernel) and blocks of 1 and 2 drafts,
-    on the tensor-core (d = 512) and FFMA (d = 320) conditioning paths."""
-    for K, d in ((1, 512), (2, 512), (16, 512), (16, 320)):
+    on the tensor-core (d = 512, and 320: ragged tiles) and FFMA (d = 325)
+    conditioning paths."""
+    for K, d in ((1, 512), (2, 512), (16, 512), (16, 320), (16, 325)):
         cfg = CONFIGS[2].__class__("t", 9, K, 3001, d, "bf16", 1.0, "uniform", seed_offset=17)
         x = make_round_inputs(cfg, device="cuda")
         x["e"] = (torch.randn((cfg.B, K, cfg.d), device="cuda") * 0.02).to(torch.bfloat16)
@@ -109,6 +111,64 @@ def test_sampled_round_dense_e_and_short_blocks(rt):
         out = check_round(rt, x, s)
         if K == 1:
             assert torch.equal(out.e_out, x["e"])
+
+
+def planted_sampling(x, accept, seed):
+    """Drafts that the temperature-1 test accepts up to accept[b] whatever the
+    uniforms (the target's most likely tokens, then one outside the vocabulary)."""
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    B, K1, V = x["logits"].shape
+    K = K1 - 1
+    draft = torch.argmax(x["logits"][:, :K].float(), dim=-1).to(torch.int32)
+    for b, a in enumerate(accept):
+        if a < K:
+            draft[b, a] = V
+    noise = torch.randn((B, K, V), generator=g, device="cuda")
+    uniforms = torch.rand((B, K1), generator=g, device="cuda") * 0.01
+    uniforms[:, K] = torch.rand((B,), generator=g, device="cuda")
+    return {"draft_logits": (x["logits"][:, :K].float() + 0.1 * noise).to(x["logits"].dtype), "draft": draft,
+            "uniforms": uniforms, "temperature": 1.0, "top_k": 20, "top_p": 0.95}
+
+
+@pytest.mark.parametrize("windows", [False, True])
+@pytest.mark.parametrize("B,K,V,d", [(1, 16, 4099, 2560), (4, 16, 1003, 264), (8, 8, 515, 512), (2, 33, 300, 136), (1, 65, 64, 256),
+                                     (2, 8, 333, 4352)])
+def test_sampled_rounds_of_few_sequences(rt, B, K, V, d, windows):
+    """At most 64 tile rows and a broadcast e: the conditioning reads the carried
+    rows where they lie, by the accepted lengths that the finalize kernel wrote.
+    A = 0, K - 2, K - 1 and K, on one workspace with greedy rounds between (which
+    decide the sequences from the argmax keys there)."""
+    cfg = CONFIGS[2].__class__("few", B, K, V, d, "bf16", 1.0, "uniform", seed_offset=B + K)
+    x = make_round_inputs(cfg, device="cuda")
+    ws = rt.Workspace(B, K, V, d, torch.bfloat16)
+    prev = rt.retrace_set_verify_schedule(rt.VERIFY_WINDOWS if windows else rt.VERIFY_FULL)
+    try:
+        greedy = rt.run_round(x, rt.Workspace(B, K, V, d, torch.bfloat16))
+        for shift in range(4):
+            accept = [[0, K - 2, K - 1, K][(b + shift) % 4] for b in range(B)]
+            out = check_round(rt, x, planted_sampling(x, accept, shift), ws)
+            assert host_int(out.accept_len).tolist() == accept
+            between = rt.run_round(x, ws)
+            torch.cuda.synchronize()
+            assert torch.equal(between.committed, greedy.committed) and torch.equal(between.e_out, greedy.e_out)
+    finally:
+        rt.retrace_set_verify_schedule(prev)
+    assert ws.check() == 0
+
+
+@pytest.mark.parametrize("dense_e", [False, True])
+@pytest.mark.parametrize("d", [256, 264])
+def test_sampled_rounds_of_many_rows(rt, d, dense_e):
+    """Above the small-R line: the rows that the finalize kernel packed, in the
+    CTA-pair kernel (whole and ragged tiles, per-position e) and the one-SM kernel
+    (per-position e, d a multiple of 256)."""
+    cfg = CONFIGS[2].__class__("many", 274, 16, 515, d, "bf16", 1.0, "uniform", seed_offset=d)
+    x = make_round_inputs(cfg, device="cuda")
+    if dense_e:
+        x["e"] = (torch.randn((cfg.B, cfg.K, cfg.d), device="cuda") * 0.02).to(torch.bfloat16)
+    accept = [(5 * b) % (cfg.K + 1) for b in range(cfg.B)]
+    out = check_round(rt, x, planted_sampling(x, accept, d))
+    assert host_int(out.accept_len).tolist() == accept
 
 
 def test_sampled_round_serving_batch(rt):
