@@ -398,10 +398,11 @@ __device__ __forceinline__ void topk_part(const T* x, int V, int k, int parts, i
 
 // Clusters of p.parts CTAs.  The rows of a pass: the window's target rows of
 // each listed sequence, then its drafter rows (`row` is the row's slot in
-// p.keys).  A cluster takes one row at a time, each CTA a part of it, and
-// CTA 0 merges the parts; when a pass has many rows for its clusters, each
-// CTA takes whole rows instead (the merge and the shorter streams cost more
-// than they balance).  The live count of a later pass is known on the device
+// p.keys).  A cluster takes one row, each CTA a part of it, and CTA 0 merges
+// the parts; when a pass has more rows than clusters, each CTA takes whole rows
+// instead (rounds, V = 151936, d = 2560, of which a later pass has 192 / 228 / 432
+// rows for 114 clusters of four: 173 / 193 / 185 us, with up to two rows per
+// cluster 183 / 224 / 192, with up to four 182 / 222 / 236).  The live count of a later pass is known on the device
 // only, so its grid is resident CTAs that loop over the rows (LOOP; in the first
 // pass a CTA per row, which measured 158 us per round of 32 sequences, was
 // faster than resident ones, 165).
@@ -416,7 +417,7 @@ __global__ void __launch_bounds__(kThreads, 3) sampled_topk_kernel(const TopkPar
   }
   const int wt = p.i1 - p.i0, wd = min(p.i1, p.K) - p.i0;
   const int rows = n_live * (wt + wd);  // B (2K+1) at most, below 2^31
-  const int parts = rows > (int)gridDim.x ? 1 : p.parts;
+  const int parts = rows > (int)gridDim.x / p.parts ? 1 : p.parts;
   const int part = parts > 1 ? (int)cluster_rank() : 0;
   const int step = (int)gridDim.x / parts;
   auto row_of = [&](int r0, const T*& x) -> int {

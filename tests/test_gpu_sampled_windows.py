@@ -208,3 +208,41 @@ def test_greedy_and_sampled_windows_share_a_workspace(rt, windows):
         for a, b in zip(got, ref):
             assert torch.equal(a, b), it
     assert ws.check() == 0
+
+
+@pytest.mark.parametrize("second,third", [(36, 10), (19, 2)])
+def test_windows_that_read_half_the_rows_take_no_longer(rt, second, third):
+    """Row windows that read half of one pass's rows, with as many rows in a later
+    pass as its resident CTAs can take one each (432) or half of them (228): no
+    slower than the one pass (121 and 105 us against 129; with clusters that took
+    several rows in turn 160 and 130)."""
+    B, K = 64, 16
+    cfg = CONFIGS[2].__class__("half", B, K, 151936, 8, "bf16", 2.0, "uniform", seed_offset=5)
+    accept = torch.tensor([12] * third + [6] * (second - third) + [1] * (B - second))
+    x, s = planted(cfg, accept)
+    ws = rt.Workspace(B, K, cfg.V, cfg.d, cfg.torch_dtype)
+    outs = [torch.empty(B, dtype=torch.int32, device="cuda"), torch.empty((B, K + 1), dtype=torch.int32, device="cuda"),
+            torch.empty(B, dtype=torch.int32, device="cuda")]
+
+    def cost(mode):
+        prev = rt.retrace_set_verify_schedule(mode)
+        best = float("inf")
+        try:
+            for _ in range(6):
+                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                torch.cuda._sleep(2_000_000)  # the calls are enqueued before the first starts
+                a.record()
+                for _ in range(5):
+                    rt.retrace_verify_sampled(x["logits"], s["draft_logits"], s["draft"], s["uniforms"], 1.0, 20, 0.95,
+                                              *outs, ws)
+                b.record()
+                torch.cuda.synchronize()
+                best = min(best, a.elapsed_time(b))
+        finally:
+            rt.retrace_set_verify_schedule(prev)
+        assert host_int(outs[0]).tolist() == accept.tolist()
+        return best
+
+    full, windows = cost(rt.VERIFY_FULL), cost(rt.VERIFY_WINDOWS)
+    print(f"one pass {full / 5 * 1e3:.1f} us, windows {windows / 5 * 1e3:.1f} us")
+    assert windows <= full, (windows, full)
