@@ -35,6 +35,12 @@ namespace {
 
 constexpr int kThreads = 512;
 constexpr int kUnroll = 4;
+// Rows up to this many elements that vectors do not cover whole (they begin or end
+// off a 16-byte boundary) go by elements (SHORT): a CTA has the threads for it, and a
+// row takes one load latency instead of the vectors' and then the edges'.  K = 64, B =
+// 79, us, by vectors / by elements: V = 515 45.8 / 38.5, 1003 46.0 / 38.8, 2051 47.2
+// / 40.5; 4099 takes 50 either way.
+constexpr int kShortRow = 8 * kThreads;
 // Least logits bytes per active CTA: small problems spread one row or so per
 // CTA instead of streaming several rows one after another on a few CTAs.
 constexpr long long kMinCtaBytes = 4096;
@@ -127,11 +133,33 @@ struct Vec<float> {
 // odd vocabulary, an odd stride) begins with up to E - 1 elements before slot
 // 0.  Those and the elements after the last vector (fewer than 2 E together)
 // go one per thread, in the CTA that has the row's last slot.  At V = 32003
-// (B = 48, 11 rows, bf16) a call with element loads took 28.6 us, now 17.0.
-template <typename T>
+// (B = 48, 11 rows, bf16) a call with element loads took 28.6 us, now 15.5.
+// (Loading them ahead of the vectors made every row slower, V = 151936 by 4 %;
+// the last threads take them, which have no vector where the row is short.)
+// SHORT: slot q is elements q E .. q E + E - 1, loaded one by one.
+template <typename T, bool SHORT>
 __device__ __forceinline__ unsigned long long segment_key(const T* __restrict__ rowp, int v0, int v1, int slots,
                                                           int V) {
   constexpr int E = Vec<T>::E;
+  if constexpr (SHORT) {
+    const int end = min(v1 * E, V);
+    float best = -INFINITY;
+    int at = -1;
+    for (int v = v0 * E + (int)threadIdx.x; v < end; v += kUnroll * kThreads) {
+      T x[kUnroll];
+#pragma unroll
+      for (int u = 0; u < kUnroll; ++u)
+        if (v + u * kThreads < end) x[u] = rowp[v + u * kThreads];
+#pragma unroll
+      for (int u = 0; u < kUnroll; ++u) {
+        if (v + u * kThreads < end && (to_f32<T>(x[u]) > best || at < 0)) {
+          best = to_f32<T>(x[u]);
+          at = v + u * kThreads;
+        }
+      }
+    }
+    return at >= 0 ? make_key(best, (uint32_t)at) : 0ull;
+  }
   const int head = min(V, (int)((16u - (uint32_t)((uintptr_t)rowp & 15u)) & 15u) / (int)sizeof(T));
   const int full = (V - head) / E;  // at most `slots`
   const int hi = v1 < full ? v1 : full;
@@ -171,8 +199,9 @@ __device__ __forceinline__ unsigned long long segment_key(const T* __restrict__ 
     }
   }
   const int edges = V - full * E;  // head, then tail
-  if (v1 == slots && (int)threadIdx.x < edges) {
-    const int v = (int)threadIdx.x < head ? (int)threadIdx.x : (int)threadIdx.x + full * E;
+  const int et = kThreads - 1 - (int)threadIdx.x;
+  if (v1 == slots && et < edges) {
+    const int v = et < head ? et : et + full * E;
     key = umax64(key, make_key(to_f32<T>(rowp[v]), (uint32_t)v));
   }
   return key;
@@ -450,7 +479,7 @@ __device__ int begin_later_pass(const VerifyParams& p, int* s_stage, int* s_warp
   return n;
 }
 
-template <typename T>
+template <typename T, bool SHORT>
 __global__ void __launch_bounds__(kThreads, 2) verify_kernel(const VerifyParams p) {
   __shared__ unsigned long long s_red[kThreads / 32];
   __shared__ int s_t[kMaxK + 1];
@@ -494,7 +523,7 @@ __global__ void __launch_bounds__(kThreads, 2) verify_kernel(const VerifyParams 
     const T* rowp = reinterpret_cast<const T*>(p.logits) + (long long)b * p.batch_stride +
                     (long long)i * p.row_stride;
 
-    unsigned long long key = segment_key<T>(rowp, v0, v1, p.slots_per_row, p.V);
+    unsigned long long key = segment_key<T, SHORT>(rowp, v0, v1, p.slots_per_row, p.V);
     key = block_max_key(key, s_red);
     if (threadIdx.x == 0) atomicMax(&p.keys[(long long)b * K1 + i], key);
     s = seg_end;
@@ -772,9 +801,12 @@ cudaError_t launch_typed(const VerifyArgs& a, cudaStream_t stream) {
   static std::atomic<int> occ_cache[64];
   int occ = occ_cache[info.device & 63].load(std::memory_order_acquire);
   if (occ == 0) {
-    err = cudaFuncSetAttribute(verify_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCopyStageBytes);
-    if (err != cudaSuccess) return err;
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, verify_kernel<T>, kThreads, kCopyStageBytes);
+    for (auto kern : {verify_kernel<T, false>, verify_kernel<T, true>}) {
+      err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kCopyStageBytes);
+      if (err != cudaSuccess) return err;
+    }
+    // (the two forms have the same threads and shared memory, and registers for two CTAs per SM)
+    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, verify_kernel<T, false>, kThreads, kCopyStageBytes);
     if (err != cudaSuccess) return err;
     if (occ < 1) occ = 1;
     occ_cache[info.device & 63].store(occ, std::memory_order_release);
@@ -795,6 +827,8 @@ cudaError_t launch_typed(const VerifyArgs& a, cudaStream_t stream) {
   p.keys = a.keys;
   p.tickets = a.tickets;
   const int E = 16 / (int)sizeof(T);
+  const bool whole = a.V % E == 0 && (uintptr_t)a.logits % 16 == 0 && a.row_stride % E == 0 && a.batch_stride % E == 0;
+  auto kern = a.V <= kShortRow && !whole ? verify_kernel<T, true> : verify_kernel<T, false>;
   p.slots_per_row = (a.V + E - 1) / E;
   p.total_slots = (long long)a.B * (a.K + 1) * p.slots_per_row;
   p.e = a.e;
@@ -855,10 +889,10 @@ cudaError_t launch_typed(const VerifyArgs& a, cudaStream_t stream) {
     // stays with the finalisers).
     auto launch_first = [&]() -> cudaError_t {
       if (a.plain_first) {
-        verify_kernel<T><<<(unsigned)grid, kThreads, kCopyStageBytes, stream>>>(p);
+        kern<<<(unsigned)grid, kThreads, kCopyStageBytes, stream>>>(p);
         return cudaGetLastError();
       }
-      return launch_dependent(verify_kernel<T>, dim3((unsigned)grid), dim3(kThreads), kCopyStageBytes, stream, 1u, p);
+      return launch_dependent(kern, dim3((unsigned)grid), dim3(kThreads), kCopyStageBytes, stream, 1u, p);
     };
     if (a.keys_only) {
       p.windowed = 1;
@@ -912,10 +946,10 @@ cudaError_t launch_typed(const VerifyArgs& a, cudaStream_t stream) {
     p.count_out = k == 0 ? nullptr : a.pass_counts + k;
     p.base_out = k == 0 ? nullptr : bases + k;
     if (k == 0 && a.plain_first) {
-      verify_kernel<T><<<(unsigned)grid_full, kThreads, kCopyStageBytes, stream>>>(p);
+      kern<<<(unsigned)grid_full, kThreads, kCopyStageBytes, stream>>>(p);
       err = cudaGetLastError();
     } else {
-      err = launch_dependent(verify_kernel<T>, dim3((unsigned)grid_full), dim3(kThreads), kCopyStageBytes, stream, 1u,
+      err = launch_dependent(kern, dim3((unsigned)grid_full), dim3(kThreads), kCopyStageBytes, stream, 1u,
                              p);
     }
     if (err != cudaSuccess) return err;
