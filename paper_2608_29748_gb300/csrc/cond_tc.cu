@@ -1925,7 +1925,9 @@ static int swap_cluster_capacity(int dev, int S, int smem, cudaError_t* err) {
 // wait for each other).  Packed rows take four K splits at most: larger
 // clusters are not all placed at once beside the last CTAs of the kernel before
 // (a round, V = 2048, d = 3584, B = 32, 384 rows: 108 us with S = 5 for the
-// correction, which one wave should hold, 72 with S = 2).  Over 160 rounds of
+// correction, which one wave should hold, 72 with S = 2; direct rows, B = 8, K = 5,
+// whose larger clusters are counted as seven eighths: 61 us with S = 5, 48 with
+// S = 4).  Over 160 rounds of
 // d = 1024 to 4096 and 64 to 733 rows, and 33 pairs of standalone calls, each
 // timed with every S, the choice takes 1.5 % more than the best S of each (11 %
 // at most); one estimate at three quarters, 2 (128 + N) cycles per k-block, 24
@@ -1943,10 +1945,11 @@ static cudaError_t swap_pick_splits(int dev, int smem, int rmax, bool direct, in
     const int cap = swap_cluster_capacity(dev, S, smem, &err);
     if (err != cudaSuccess) return err;
     if (cap == 0) continue;
+    const int held = splits > 4 ? cap - cap / 8 : cap;  // at once, beside the kernel before
     long long cost = 0;
     for (const int rows : {(rmax + 1) / 2, (3 * rmax + 3) / 4}) {
       const SwapCut cut = direct ? SwapCut{1, (rmax + 15) / 16 * 16} : swap_cut(rows, mtiles, cap);
-      const long long waves = ((long long)mtiles * cut.ntiles + cap - 1) / cap;
+      const long long waves = ((long long)mtiles * cut.ntiles + held - 1) / held;
       const int block = std::max(750, 17 * cut.tile_n / 4);
       cost += waves * ((long long)((nkb + splits - 1) / splits) * block + 60 * cut.tile_n + wave + (direct ? 0 : 700 * S));
     }

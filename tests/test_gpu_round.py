@@ -460,3 +460,29 @@ def test_round_of_few_sequences_at_large_hidden_sizes(rt, d, B):
     want = oracle_round(x)
     assert_verify_exact(want, out.accept_len, out.committed, out.bonus)
     assert_close(out.e_out, want["e_tilde"], f"d={d} B={B}")
+
+
+def test_round_of_few_sequences_grows_with_the_weights(rt):
+    """From d = 3072 to 3584 a round of few sequences grows by no more than its
+    weights do (1.36; about 1.15.  With clusters of five that one wave just held on
+    an idle GPU, and not beside verification's last CTAs, it grew by 1.46)."""
+    B, K, V = 8, 5, 18880
+
+    def cost(d):
+        x = make_round_inputs(CONFIGS[2].__class__("few", B, K, V, d, "bf16", 1.0, "geometric", 0.3, seed_offset=d), device="cuda")
+        ws, out = rt.Workspace(B, K, V, d, torch.bfloat16), rt.RoundBuffers(B, K, d, torch.bfloat16)
+        best = float("inf")
+        for _ in range(8):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda._sleep(1_000_000)  # the calls are enqueued before the first starts
+            a.record()
+            for _ in range(5):
+                rt.run_round(x, ws, out=out)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        return best
+
+    small, large = cost(3072), cost(3584)
+    print(f"d = 3072 {small * 200:.1f} us, d = 3584 {large * 200:.1f} us")
+    assert large <= (3584 / 3072) ** 2 * small, (large, small)
