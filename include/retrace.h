@@ -170,15 +170,18 @@ retrace_status retrace_verify(const void* logits, retrace_dtype dtype, int B, in
 #define RETRACE_VERIFY_WINDOWS 2
 int retrace_set_verify_schedule(int mode);
 
-/* The greedy verification schedule a call with this shape takes under the
- * current mode, given a workspace: returns the number of passes n (1 = the
- * one-pass schedule; -1 for an invalid shape or dtype) and, when
- * window_starts is not NULL, writes the n + 1 window boundaries (at most 17
- * entries: pass k reads rows [window_starts[k], window_starts[k+1]) of the
- * sequences that matched every row before it).  A windowed greedy round
- * launches n verification kernels plus one for the row copies (one kernel in
- * one pass); at temperature T, 2n kernels (top-k scan and accept tests per
- * pass) plus the copies (two in one pass).  Host arithmetic only. */
+/* The verification schedule (greedy, or at temperature T with target_argmax 0)
+ * a call with this shape takes under the current mode, given a workspace:
+ * returns the number of passes n (1 = the one-pass schedule; -1 for an invalid
+ * shape or dtype) and, when window_starts is not NULL, writes the n + 1 window
+ * boundaries (at most 17 entries: pass k reads rows [window_starts[k],
+ * window_starts[k+1]) of the sequences that matched, or accepted, every row
+ * before it).  A windowed greedy verification launches n kernels plus the
+ * finish kernel; one pass is one kernel, plus the finish or copy kernel where
+ * the round packs rows for fewer sequences than SMs.  At temperature T, 2n
+ * kernels (top-k scan and accept tests per pass), plus the copies of a windowed
+ * round and of one that packs rows for fewer sequences than SMs.  Host
+ * arithmetic only. */
 int retrace_verify_plan(int B, int K, int V, retrace_dtype dtype, int target_argmax, int* window_starts);
 
 /* Rejected-trajectory alignment and target-aware correction (Eq. 3-7,

@@ -844,10 +844,12 @@ retrace_status retrace_round_lowrank(const void* logits, int64_t logits_row_stri
     va.gate_ld = d + RETRACE_LOWRANK_LATENT;
     va.gate_done = &ge_ready;
   }
-  // With several row blocks the next round's CTAs, launched ahead, take the room
-  // of lr_fuse_kernel's (B = 32 / 64, d = 2560, V = 151936: 60 / 77 us against 55 /
-  // 70); with one (128 rows) or on the FFMA kernel launching ahead wins (B = 1 /
-  // 8, d = 2560: 26.9 / 34.7 against 28.5 / 35.0; d = 1024, fp32, B = 4: 100.0 / 101.7).
+  // With several row blocks the next round's CTAs, launched ahead, take the room of
+  // lr_fuse_kernel's; with one (128 rows) or on the FFMA kernel launching ahead wins.
+  // Ahead / plain, us, d = 2560, V = 151936: 60 rows 31.3 / 32.9, 120 36.0 / 36.1, 135
+  // 36.8 / 37.3, 150 38.5 / 38.0, 240 44.8 / 42.8, 480 61.4 / 57.1, 960 79.1 / 73.8 (d =
+  // 4096 alike; V = 32000: 120 30.3 / 31.5, 480 38.3 / 39.0, 960 48.6 / 48.2); fp32,
+  // d = 1024, B = 4: 100.0 / 101.7.
   va.plain_first = tc && (long long)B * (K - 1) > 128;
   if (tc) {  // the finalising CTA of each sequence packs its [m; u] rows
     va.hT = hT;

@@ -3,7 +3,8 @@
 // Two steps per projection family:
 //
 // 1. pack_rows_kernel (standalone calls; in a round verification packs) lays
-//    the conditioned rows out contiguously, in sequence order (R = sum_b n_b rows, n_b = max(0, K-1-A_b)):
+//    the conditioned rows out contiguously, in sequence order (R = sum_b n_b
+//    rows, n_b = max(0, K-1-A_b)):
 //      correction operand  Apack[g] = [ hD[b, A_b+1+j] ; hT[b, A_b+j] ]  (Eq. 4-5),
 //      or the corrected signal rows r[b, j] for a standalone gate call,
 //      plus, for per-position e, Epack[g] = e[b, j];
@@ -42,7 +43,9 @@
 //   warp 0     tile scheduler + TMA producer (one elected lane);
 //   warp 1     MMA issuer (one lane);
 //   warp 2     TMEM allocation: 2 accumulators x 256 fp32 columns = 512 columns;
-//   warps 2-3  the broadcast-e GEMV W_g[:, :d] e, rows claimed from a counter;
+//   warps 2-3  (pair kernel) the broadcast-e GEMV W_g[:, :d] e, in static shares over
+//              the grid; the overlapped round's epilogue warps claim its rows from a
+//              counter before their first tile;
 //   warps 4-7  epilogue: tcgen05.ld of their 32 TMEM lanes (= tile rows).
 // The two accumulators alternate between tiles, so a tile's epilogue overlaps
 // the next tile's main loop.  Every mbarrier wait is bounded; on expiry the CTA
@@ -325,8 +328,8 @@ __device__ __forceinline__ void epilogue_gate(const CondParams& p, uint32_t tadd
 // sequence is finalised.
 // Not FUSED: a per-position e only.  Its 128-row tiles fill the last wave
 // better than the pair kernel's, whose gate tiles are long with the e half
-// added (a round, d = 2560, 1821 rows: 170 us here, 206 on pairs; d = 4096,
-// 1821: 337 / 365; 2802: 445 / 445).
+// added (a round, d = 2560, 1821 rows: 168 us here, 206 on pairs; d = 4096,
+// 1821: 335 / 365; 2802: 440 / 445).
 constexpr int kGateLag = 4;
 
 template <bool FUSED>
@@ -1166,8 +1169,8 @@ __global__ void wait_selftest_kernel(int kind, const uint32_t* flag, uint32_t ta
 // W_g,e e: a cluster then holds 128 features of all three, each product in
 // its own CTAs (S = 3 splits), and the sum adds the last two.  (As further
 // k-blocks of the stacked tiles, W_v's half zeros, a gate tile had twice the
-// k-blocks on as many CTAs: 36 us at B = 32, d = 2560.)  Nothing goes through global partials and no reduction kernel follows.  The partial
-// is stored row-major ([row][feature]) so that both the TMEM drain and the
+// k-blocks on as many CTAs: 36 us at B = 32, d = 2560.)  Nothing goes through
+// global partials and no reduction kernel follows.  The partial is stored row-major ([row][feature]) so that both the TMEM drain and the
 // cluster's reads move whole 128- and 256-byte rows.
 //
 // The row tiles are cut on the device from R (swap_cut): as many as the
@@ -1851,8 +1854,9 @@ static cudaError_t launch_cond_pair(const TcCondArgs& a, int clusters, cudaStrea
   p.split_max = (a.split_part && a.do_gate && !a.e_dense) ? kPairSplitTiles : 0;
   p.status = a.status;
   // clusters of two CTAs; set-up may overlap the previous kernel's end
-  return launch_dependent(d % 256 == 0 && !p.e_dense ? cond_pair_kernel<false> : cond_pair_kernel<true>, dim3(2 * (unsigned)clusters), dim3(P_THREADS), P_SMEM_BYTES, stream, 2,
-                          mApack, mWc, mR, mWv, mWg, mE, mWge, p);
+  auto kern = d % 256 == 0 && !p.e_dense ? cond_pair_kernel<false> : cond_pair_kernel<true>;
+  return launch_dependent(kern, dim3(2 * (unsigned)clusters), dim3(P_THREADS), P_SMEM_BYTES, stream, 2, mApack, mWc, mR,
+                          mWv, mWg, mE, mWge, p);
 }
 
 // Pairs of CTAs of cond_pair_kernel to launch: those the device keeps resident

@@ -40,7 +40,7 @@ constexpr int kLowRankLatent = 64;      // rank of the rejected-suffix latents
 constexpr int kLowRankCorrection = 32;  // rank of the target-aware correction
 constexpr int kLowRankSplits = 8;       // split-K parts per half of the [m; u] reduction
 //   skeys    uint64 [B*(2K+1), 64]  sampled verification: top-k keys per target and drafter row
-//   swp      fp32                   K halves of the CTA-pair kernel's split gate tiles
+//   swp      fp32                   K halves of the CTA-pair kernel's split gate tiles; r of direct rows
 constexpr int kMaxTopK = 64;            // largest top_k of sampled verification
 constexpr int kWindowRows = 4;          // rows per pass of windowed verification
 constexpr int kMaxWindowPasses = 16;    // most passes of windowed verification
@@ -72,8 +72,9 @@ inline CondPath cond_path(long long B, long long K, long long d, bool direct, bo
   if (gate_dense_e && d % 256 == 0) return kCondOneSm;
   return pairs > 0 ? kCondPair : kCondSwap;
 }
-// The region of swap_part_bytes in the workspace holds the corrected signal of a
-// round without packed rows (direct rows, below).
+// Small calls' region of the workspace, in the size it had when split partials went
+// through it (callers compute and pass that size); what is used of it is the
+// corrected signal of a round without packed rows (direct rows, below).
 constexpr int kSwapMaxRows = 1024;
 constexpr int kSwapMaxCtas = 256;
 inline size_t swap_part_bytes(long long B, long long K, long long d) {

@@ -2,10 +2,11 @@
 // commit steps; greedy decoding = top_k 1).
 //
 // The [B, K+1, V] logits are one flat stream of B*(K+1) rows.  The rows are
-// cut into "slots" (16-byte vectors: 8 bf16 or 4 fp32) and the slot range is split evenly over the grid, so every
-// CTA streams the same number of bytes whatever B, K and V are.  A CTA reduces
-// each row segment it owns to one 64-bit (value, ~index) key and folds it into
-// the row's key with atomicMax.  The last CTA to finish a sequence (per-
+// cut into "slots" (16-byte vectors: 8 bf16 or 4 fp32; short rows that vectors do
+// not cover whole go by elements) and the slot range is split evenly over the
+// grid, so every CTA streams the same number of bytes whatever B, K and V are.  A
+// CTA reduces each row segment it owns to one 64-bit (value, ~index) key and folds
+// it into the row's key with atomicMax.  The last CTA to finish a sequence (per-
 // sequence arrival ticket; nothing ever waits) decodes its K+1 argmaxes,
 // finds the first mismatch with a warp ballot and writes the accepted length,
 // committed tokens and bonus, resets the keys and ticket to zero for the next
@@ -23,8 +24,10 @@
 // offsets, after the rows of the sequences decided in earlier windows.  The
 // pass then streams only the listed sequences' rows.  Rows past the window
 // holding the first mismatch are never read.  verify_finish_kernel decides
-// the sequences of the last window the same way and does the row copies.  A one-pass round that packs rows for fewer sequences than
-// there are SMs leaves its copies to verify_copy_kernel, spread over the grid.
+// the sequences of the last window the same way and does the row copies.  A
+// one-pass round that packs rows for fewer sequences than there are SMs runs as
+// one such window; with every row's argmax as an output it keeps the finalisers
+// and leaves its copies to verify_copy_kernel, spread over the grid.
 #include <atomic>
 
 #include "common.cuh"
