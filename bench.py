@@ -61,9 +61,9 @@ L2_FLUSH_BYTES = 256 << 20
 # kernel sources it was measured on: `sources` is kernel_sources_hash() at the
 # time, and the line reports null traffic once the sources differ.
 TRAFFIC = {
-    ("verify", "qwen3-8b-B256-K16"): {"bytes": 311310080 + 2837248 + 184313856 + 146176 + 55402496 + 3840
-                                      + 47182336 + 4024320, "sources": "6513f6d371864d1a"},
-    ("conditioning", "qwen3-8b-B256-K16"): {"bytes": 486870528 + 36317184, "sources": "6513f6d371864d1a"},
+    ("verify", "qwen3-8b-B256-K16"): {"bytes": 311316480 + 2942464 + 184309504 + 106496 + 55402496 + 0
+                                      + 47184896 + 4111104, "sources": "99f8a58bce59fe79"},
+    ("conditioning", "qwen3-8b-B256-K16"): {"bytes": 502643456 + 37257216, "sources": "99f8a58bce59fe79"},
 }
 
 
